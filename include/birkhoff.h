@@ -118,9 +118,10 @@ bk_status birkhoff_apply(const bk_plan* plan, const void* v, void* out, int batc
 /* B v (trans = 0) or B^T v (trans = 1) for `count` plans of one dtype whose N may all differ,
  * e.g. the requests of a serving batch: entry i computes out[i] = B_i v[i] for batch[i]
  * vectors of plans[i], exactly as birkhoff_apply(_T)(plans[i], v[i], out[i], batch[i]) would
- * (bitwise the same values). Plans on the single-CTA path run in one launch, plans on the
- * unsplit four-step path in one launch per pass (five), each per 16 plans; dense, Bluestein,
- * split and double-float plans run their own launches within the call.
+ * (bitwise the same values). Plans on the single-CTA path run in one launch, four-step plans (up
+ * to 2^18 in FP32, 2^17 in FP64) in another, or in one launch per pass (four) when one of them is
+ * on the launch-per-pass path, each per 16 plans; dense, Bluestein and longer plans run their own
+ * launches within the call.
  *   plans, v, out, batch   host arrays of `count` entries (1 <= count <= 4096); v[i], out[i]
  *                          device arrays as for birkhoff_apply; v[i] == out[i] is allowed, but
  *                          different entries' vectors must not overlap
@@ -178,12 +179,13 @@ bk_status birkhoff_apply_b_T(const bk_plan* plan, const void* v, void* out, int 
  * the same plan in flight. */
 bk_status bk_plan_set_dense(bk_plan* plan, int on, void* stream);
 
-/* How a plan computes its products. *path: 0 one CTA per vector (small N), 1 four-step FFT,
- * 2 four-step with the split DCT-I, 3 dense product, 4 Bluestein convolution (N not a power of
- * two above 1024). For paths 1 and 2: the FFT
- * factors N1 x N2 of the (even-half) transform and the complex elements per CTA, as chosen by
- * the tile autotuner at plan creation (or by the occupancy heuristic when tuning is off:
- * environment BK_AUTOTUNE=0). Outputs may be NULL. */
+/* How a plan computes its products. *path: 0 one CTA per vector (small N), 1 four-step FFT in
+ * one launch (a cluster of CTAs per vector), 2 four-step FFT split into a launch per pass, 3 dense
+ * product, 4 Bluestein convolution (N not a power of two above 1024). For paths 1 and 2: the
+ * rows N1 and columns N2 that the real-even four-step transform keeps (half of its factors, N1 N2 =
+ * N / 2) and the complex elements per CTA, for path 2 as chosen by the tile autotuner at plan
+ * creation (or by the occupancy heuristic when tuning is off: environment BK_AUTOTUNE=0). Outputs
+ * may be NULL. */
 bk_status bk_plan_shape(const bk_plan* plan, int* path, int* N1, int* N2, int* elems);
 
 /* *on = 1 while the plan's products take the dense path, else 0. Plans of an N that is not a
@@ -193,7 +195,7 @@ bk_status bk_plan_shape(const bk_plan* plan, int* path, int* N1, int* N2, int* e
 bk_status bk_plan_dense_state(const bk_plan* plan, int* on);
 
 /* Arithmetic of the FP64 transforms for plans (and problems) created after the call:
- *   mode 1: four-step FP64 plans (powers of two, N >= 256) compute their DCTs in double-float
+ *   mode 1: FP64 plans of powers of two, N >= 256, compute their DCTs in double-float
  *           arithmetic, each value the unevaluated sum of two binary32 numbers (48 significand
  *           bits; Knuth's TwoSum, Dekker's FastTwoSum and an FMA product), on the FP32 pipe,
  *           which GB300 runs 64 times as fast as its FP64 pipe. Vectors stay binary64 in
@@ -201,7 +203,7 @@ bk_status bk_plan_dense_state(const bk_plan* plan, int* on);
  *   mode 0: IEEE binary64 arithmetic throughout.
  *   mode -1 (the default): double-float for N >= 2^18, where it measured faster (1.8x at
  *           2^20), binary64 below (the environment variable BK_F64_DF=0 selects mode 0).
- * Single-CTA plans (N <= 128) and dense products always use binary64. Host only; BK_ERR_ARG for
+ * Plans with N <= 128 and dense products always use binary64. Host only; BK_ERR_ARG for
  * any other mode. This is the library's choice of arithmetic; the paper's method is exact FP64. */
 bk_status bk_set_f64_transform(int mode);
 

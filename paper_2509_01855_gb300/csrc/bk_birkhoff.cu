@@ -26,8 +26,8 @@
 //   Y_k = P + Q,  Y_{N-k} = P - Q,  P = Re(Z_k + Z_{N-k}) / 2,
 //   Q = [cos(pi k/N) Im(Z_k + Z_{N-k}) - sin(pi k/N) Re(Z_k - Z_{N-k})] / 2.
 // N <= NSMALL: one CTA per vector does the whole chain in shared memory (one HBM read and one
-// write). Larger N: four-step FFT (N = N1 N2) in two passes per DCT, the integration stencil
-// fused into the load of the second DCT, and the node-0 value gathered from per-CTA partials.
+// write) with that FFT. Larger powers of two: the real-even four-step DFT of bk_dct.cuh in two
+// passes per DCT, the integration stencil fused into the load of the second DCT.
 #include <math.h>
 #include <stdarg.h>
 #include <stdlib.h>
@@ -52,7 +52,6 @@ namespace bk {
 // The kernels compute in T and keep their internal real vectors (the stage buffers between the
 // two DCTs) in T; the caller's vectors are User<T> (binary64 for double-float arithmetic, whose
 // products convert the input once in k_to_arith and the output in the last epilogue).
-template <typename T> using St = T;
 template <typename T> using Us = typename User<T>::t;
 // Conversion of a stored element S to the arithmetic type T and back (identity when S == T).
 template <typename T, typename S> struct Cv;
@@ -63,10 +62,6 @@ template <typename T> struct Cv<T, T> {
 template <> struct Cv<dfl, double> {
   static __device__ __forceinline__ dfl in(double x) { return d2df(x); }
   static __device__ __forceinline__ double out(dfl x) { return df2d(x); }
-};
-// Pass-B output type: the caller's type for the final epilogues, T for the stage buffer.
-template <typename T, int E> struct OutS {
-  typedef typename std::conditional<(E == 2 || E == 3), Us<T>, T>::type t;
 };
 template <typename T, typename S> __device__ __forceinline__ T rdv(const S* __restrict__ p, int64_t i) {
   return Cv<T, S>::in(p[i]);
@@ -155,18 +150,38 @@ __global__ void k_post_table(typename V2<T>::t* tp, int64_t N) {
   }
 }
 
-// Stage twiddle table of a length-2^log2n FFT (see bk_fft.cuh): entry off + (r-1) Ns + k of the
-// block of the stage with Ns = 2^l is omega_{16 Ns}^{r k}, from sincospi(2 r k / (16 Ns)).
+// Stage twiddle table of a length-2^log2n FFT of radix R = 2^e (see bk_fft.cuh): entry
+// off + (r-1) Ns + k of the block of the stage with Ns = 2^l is omega_{R Ns}^{r k}, from
+// sincospi(2 r k / (R Ns)).
 template <typename T>
-__global__ void k_stage_tw(typename V2<T>::t* stw, int log2n, int len) {
+__global__ void k_stage_tw(typename V2<T>::t* stw, int log2n, int e, int len) {
+  const int R1 = (1 << e) - 1;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < len; idx += gridDim.x * blockDim.x) {
-    int l = (log2n & 3) ? (log2n & 3) : 4, off = 0;
-    while (idx >= off + (15 << l)) { off += 15 << l; l += 4; }
-    const int e = idx - off;
-    const int r = (e >> l) + 1, k = e & ((1 << l) - 1);
+    int l = log2n % e ? log2n % e : e, off = 0;
+    while (idx >= off + (R1 << l)) { off += R1 << l; l += e; }
+    const int i = idx - off;
+    const int r = (i >> l) + 1, k = i & ((1 << l) - 1);
     double sn, cs;
-    sincospi((double)(2 * r * k) / (double)(16 << l), &sn, &cs);
+    sincospi((double)(2 * r * k) / (double)(1 << (l + e)), &sn, &cs);
     stw[idx] = mk2<T>((T)cs, (T)(-sn));
+  }
+}
+
+// Inter-pass twiddles of the real-even passes, [N1/2 + 1][N2/2 + 2] (2N = N1 N2; see bk_dct.cuh):
+// omega_2N^{n2 k} / 2 for a pair's first column (even positions; position 0 is column 0), times -i
+// for its second (odd positions; position 1 is column N2/2).
+template <typename T>
+__global__ void k_re_tw(typename V2<T>::t* tw, int N1, int N2) {
+  const int RS = N2 / 2 + 2;
+  const int64_t len = (int64_t)(N1 / 2 + 1) * RS;
+  const double N = 0.5 * (double)N1 * (double)N2;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = i / RS;
+    const int pos = (int)(i - k * RS);
+    const int64_t n2 = pos == 0 ? 0 : (pos == 1 ? N2 / 2 : pos - 1);
+    double sn, cs;
+    sincospi((double)(n2 * k) / N, &sn, &cs);
+    tw[i] = (pos & 1) ? mk2<T>((T)(-0.5 * sn), (T)(-0.5 * cs)) : mk2<T>((T)(0.5 * cs), (T)(-0.5 * sn));
   }
 }
 
@@ -289,111 +304,6 @@ __device__ __forceinline__ typename V2<T>::t load_z(const S* __restrict__ src, i
   return mk2<T>(load_x<T, K>(src, i1, N, invN, Y0, tb), load_x<T, K>(src, i2, N, invN, Y0, tb));
 }
 
-// Split DCT-I (four-step plans): the DCT-I of length N+1 of x is, at even indices, the DCT-I of
-// length M+1 (M = N/2) of the pair sums a_i = x_i + x_{N-i} (a_M = 2 x_M) and, at odd indices
-// 2m+1, the DCT-III of length M, sum_{i<M} u_i cos(pi i (2m+1) / (2M)), of the pair differences
-// u_0 = x_0 - x_N, u_i = 2 (x_i - x_{N-i}). Pass-A load modes:
-//   PM_FULL : the unsplit length-N FFT input (load_z)
-//   PM_PAIR : z_j of the length-M DCT-I of the pair sums (n = M)
-//   PM_DCT3 : conj Z_k (k < n = M/2) of the DCT-III by a length-M/2 inverse FFT (Makhoul):
-//             H_0 = u_0, H_k = e^{i theta k} (u_k - i u_{M-k}) / 2 (theta = pi / (2M) = pi / N,
-//             u_M = 0), Z_k = (H_k + conj H_{M/2-k}) + i e^{2 pi i k / M} (H_k - conj H_{M/2-k});
-//             the inverse FFT runs as conj(FFT(conj Z)).
-// Two-level split (largest plans): the even half's DCT-I of length M+1 of a is split once more,
-// so R(x)_{4m} is the DCT-I of length Q+1 (Q = N/4) of aa_i = a_i + a_{M-i}, R(x)_{4m+2} the
-// DCT-III of length Q of u'_0 = a_0 - a_M, u'_i = 2 (a_i - a_{M-i}), and R(x)_{2m+1} the
-// DCT-III of x's pair differences as above: FFTs of N/4 + N/8 + N/4 points instead of
-// N/2 + N/4. The pair sums a are formed on the fly from x in the loads:
-//   PM_PAIR2 : z_j of the length-Q DCT-I of aa (n = Q)
-//   PM_DCT3A : conj Z_k (k < n = Q/2) of the DCT-III of u' (as PM_DCT3, on a)
-//   PM_CPLX  : a plain complex vector (pairs of reals) of length n (Bluestein's convolution)
-enum { PM_FULL = 0, PM_PAIR = 1, PM_DCT3 = 2, PM_PAIR2 = 3, PM_DCT3A = 4, PM_CPLX = 5 };
-
-template <typename T, int K, typename S>
-__device__ __forceinline__ T pair_sum(const S* __restrict__ src, int i, int Ns) {
-  // a_i = x_i + x_{Ns-i}; IN_WINV halves interior samples (i = 0 pairs the two end samples)
-  const T a = rdv<T>(src, i) + rdv<T>(src, Ns - i);
-  return (K == IN_WINV && i != 0) ? T(0.5) * a : a;
-}
-
-template <typename T, int K, typename S>
-__device__ __forceinline__ typename V2<T>::t load_z_pair(const S* __restrict__ src, int j, int n, StencilTab<T> tb) {
-  const int Ns = 2 * n;
-  const int m1 = 2 * j, m2 = 2 * j + 1;
-  const int i1 = m1 <= n ? m1 : 2 * n - m1;
-  const int i2 = m2 <= n ? m2 : 2 * n - m2;
-  return mk2<T>(pair_sum<T, K>(src, i1, Ns), pair_sum<T, K>(src, i2, Ns));
-}
-
-// H_k of the DCT-III input (see above), with the factors folded: for k >= 1 every sample is an
-// interior one, so H_k = c e^{i theta k} ((x_k - x_{N-k}) - i (x_{M-k} - x_{M+k})) with c = 1
-// (IN_PLAIN) or 1/2 (IN_WINV halves interior samples); H_0 = u_0 = W-scaled x_0 - x_N.
-template <typename T, int K, typename S>
-__device__ __forceinline__ typename V2<T>::t dct3_H(const S* __restrict__ src, int i, int M,
-                                                   const typename V2<T>::t* __restrict__ tpost) {
-  const int N = 2 * M;
-  if (i == 0) return mk2<T>(rdv<T>(src, 0) - rdv<T>(src, N), T(0));
-  const T a = rdv<T>(src, i) - rdv<T>(src, N - i), b = rdv<T>(src, M - i) - rdv<T>(src, M + i);
-  typename V2<T>::t cs = tpost[i];  // (cos, sin)(pi i / N)
-  if (K == IN_WINV) { cs.x *= T(0.5); cs.y *= T(0.5); }
-  return mk2<T>(a * cs.x + b * cs.y, a * cs.y - b * cs.x);
-}
-
-template <typename T, int K, typename S>
-__device__ __forceinline__ typename V2<T>::t load_z_dct3(const S* __restrict__ src, int k, int n,
-                                                        const typename V2<T>::t* __restrict__ tpost,
-                                                        const typename V2<T>::t* __restrict__ eo, StencilTab<T> tb) {
-  typedef typename V2<T>::t C;
-  const int M = 2 * n;
-  const C Hk = dct3_H<T, K>(src, k, M, tpost);
-  const C Hm = dct3_H<T, K>(src, n - k, M, tpost);  // H_{M/2 - k}; conj taken below
-  const C E = mk2<T>(Hk.x + Hm.x, Hk.y - Hm.y);
-  const C D = mk2<T>(Hk.x - Hm.x, Hk.y + Hm.y);
-  const C w = eo[k];  // omega_M^k; e^{2 pi i k / M} = conj w
-  const C O = mk2<T>(D.x * w.x + D.y * w.y, D.y * w.x - D.x * w.y);
-  return mk2<T>(E.x - O.y, -(E.y + O.x));
-}
-
-// z_j of the length-Q DCT-I of aa (n = Q, x of length 4Q + 1): aa_i = a_i + a_{2Q-i}.
-template <typename T, int K, typename S>
-__device__ __forceinline__ typename V2<T>::t load_z_pair2(const S* __restrict__ src, int j, int n) {
-  const int Nf = 4 * n, M = 2 * n;
-  const int m1 = 2 * j, m2 = 2 * j + 1;
-  const int i1 = m1 <= n ? m1 : 2 * n - m1;
-  const int i2 = m2 <= n ? m2 : 2 * n - m2;
-  return mk2<T>(pair_sum<T, K>(src, i1, Nf) + pair_sum<T, K>(src, M - i1, Nf),
-                pair_sum<T, K>(src, i2, Nf) + pair_sum<T, K>(src, M - i2, Nf));
-}
-
-// H_k of the DCT-III of length Q of u' (pair differences of a, x of length 4Q + 1): as dct3_H on
-// a with theta = pi / (2Q), (cos, sin)(pi i / (2Q)) = tpost[2i]; a carries the W^{-1} scaling of
-// IN_WINV already, so the factor c is 1.
-template <typename T, int K, typename S>
-__device__ __forceinline__ typename V2<T>::t dct3_H_pairs(const S* __restrict__ src, int i, int Q,
-                                                         const typename V2<T>::t* __restrict__ tpost) {
-  const int M = 2 * Q, Nf = 4 * Q;
-  if (i == 0) return mk2<T>(pair_sum<T, K>(src, 0, Nf) - pair_sum<T, K>(src, M, Nf), T(0));
-  const T a = pair_sum<T, K>(src, i, Nf) - pair_sum<T, K>(src, M - i, Nf);
-  const T b = pair_sum<T, K>(src, Q - i, Nf) - pair_sum<T, K>(src, Q + i, Nf);
-  const typename V2<T>::t cs = tpost[2 * i];
-  return mk2<T>(a * cs.x + b * cs.y, a * cs.y - b * cs.x);
-}
-
-template <typename T, int K, typename S>
-__device__ __forceinline__ typename V2<T>::t load_z_dct3a(const S* __restrict__ src, int k, int n,
-                                                         const typename V2<T>::t* __restrict__ tpost,
-                                                         const typename V2<T>::t* __restrict__ eo) {
-  typedef typename V2<T>::t C;
-  const int Q = 2 * n;
-  const C Hk = dct3_H_pairs<T, K>(src, k, Q, tpost);
-  const C Hm = dct3_H_pairs<T, K>(src, n - k, Q, tpost);
-  const C E = mk2<T>(Hk.x + Hm.x, Hk.y - Hm.y);
-  const C D = mk2<T>(Hk.x - Hm.x, Hk.y + Hm.y);
-  const C w = eo[2 * k];  // the table is built for the DCT-III of length 2Q
-  const C O = mk2<T>(D.x * w.x + D.y * w.y, D.y * w.x - D.x * w.y);
-  return mk2<T>(E.x - O.y, -(E.y + O.x));
-}
-
 // Real-FFT split: from Z_k, Z_{N-k} and (cos, sin)(pi kk / N), kk = min(k, N - k).
 template <typename T>
 __device__ __forceinline__ void split_pair(typename V2<T>::t zk, typename V2<T>::t zc,
@@ -425,7 +335,7 @@ __device__ void dct1_block(const T* __restrict__ X, int kind, T* __restrict__ Y,
   }
   __syncthreads();
   if (N >= 16) {
-    fft16_any<T>(buf, N, log2N, 1, pad_stride(N), stw);
+    fft_any<T, SmallFft<T>::E, SmallFft<T>::EPT, 4, 12>(buf, log2N, 1, pad_stride(N), stw);
   } else {
     // N = 4 or 8: direct DFT (tw holds omega_N^i, n_tab = N)
     C zk = mk2<T>(T(0), T(0));
@@ -448,15 +358,6 @@ __device__ void dct1_block(const T* __restrict__ X, int kind, T* __restrict__ Y,
   __syncthreads();
 }
 
-// Thread cap of the transform kernels: each thread stages 16 complex values, so FP64 kernels
-// are limited to 256 threads (up to 255 registers each) and FP32 ones to 512.
-template <typename T> struct MaxThr { static constexpr int v = sizeof(T) == 8 ? 256 : 512; };
-// Resident CTAs per SM the pass kernels are compiled for (register cap 64K / (threads x this)).
-// Double-float: 3 (80 registers instead of 128, spills unchanged at ~50 bytes, 24 instead of 16
-// warps per SM for the 128-thread tiles; the latency-bound passes gained: 4-component products
-// 2^20 0.553 -> 0.519 ms, 2^22 2.48 -> 2.11 ms; 4 CTAs (64 registers) lost: 0.576, 2.33 ms).
-// binary32 at 3 would cap the 512-thread tiles at 42 registers and spill ~400 bytes.
-template <typename T> struct MinB { static constexpr int v = std::is_same<T, dfl>::value ? 3 : 2; };
 // Element loads each thread keeps in flight in the pass kernels' load phases.
 // FP32: 8 (latency-bound passes; 16 spilled under the 64-register cap of two 512-thread CTAs
 // per SM), FP64: 4 (FP64-pipe-bound, register-heavy).
@@ -500,7 +401,7 @@ __device__ __forceinline__ void small_body(int vec, const Us<T>* __restrict__ in
 }
 
 template <typename T, bool TRANS>
-__global__ void __launch_bounds__(MaxThr<T>::v)
+__global__ void __launch_bounds__(1024)
     k_birkhoff_small(const Us<T>* __restrict__ in, Us<T>* __restrict__ out, int N, int log2N, int64_t pitch,
                      T s, const typename V2<T>::t* __restrict__ tw, const typename V2<T>::t* __restrict__ stw,
                      const typename V2<T>::t* __restrict__ tpost, StencilTab<T> tb) {
@@ -508,86 +409,46 @@ __global__ void __launch_bounds__(MaxThr<T>::v)
 }
 
 // ---------------------------------------------------------------------------------------------
-// Four-step passes for large N (N = N1 * N2, j = N2 j1 + j2, k = k1 + N1 k2).
-// Pass A: per CTA, NB columns j2; FFT over j1 (length N1), twiddle omega_N^{j2 k1}; writes
-//         A[k1][j2]. Also writes the CTA's partial sum of Re z + Im z (the DC value of the DCT).
-// Pass B: per CTA, P row pairs {p, N1 - p} (p = 0 pairs rows 0 and N1/2); FFT over j2 (length
-//         N2), real-FFT split, epilogue.
+// Four-step passes of a plain complex FFT of length n = N1 N2 (Bluestein's convolution; j = N2 j1 +
+// j2, k = k1 + N1 k2). Pass A: per CTA, NB columns j2; FFT over j1 (length N1), twiddle
+// omega_n^{j2 k1}; writes A[k1][j2]. Pass B: per CTA, 2P rows k1; FFT over j2 (length N2); writes
+// the outputs in natural order.
 // ---------------------------------------------------------------------------------------------
-template <typename T, int K, int MODE>
-__device__ __forceinline__ void passA_body(
-            int bid, int nbid, const St<T>* __restrict__ src, int64_t src_stride, typename V2<T>::t* __restrict__ Aout,
-            T* __restrict__ partial, int N, int N1, int log2N1, int N2, int NB, int bs,
-            const typename V2<T>::t* __restrict__ stw,
-            const typename V2<T>::t* __restrict__ twN, T invN, StencilTab<T> tb,
-            const typename V2<T>::t* __restrict__ twLo,
-            const typename V2<T>::t* __restrict__ twHi, int tw_h,
-            const typename V2<T>::t* __restrict__ tpost, const typename V2<T>::t* __restrict__ eo,
-            int vec_in = -1, int nthr_in = 0) {
+template <typename T>
+__global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
+    k_passA(const T* __restrict__ src, int64_t src_stride, typename V2<T>::t* __restrict__ Aout, int N, int N1,
+            int log2N1, int N2, int NB, int bs, const typename V2<T>::t* __restrict__ stw,
+            const typename V2<T>::t* __restrict__ twN, const typename V2<T>::t* __restrict__ twLo,
+            const typename V2<T>::t* __restrict__ twHi, int tw_h) {
   typedef typename V2<T>::t C;
   extern __shared__ __align__(16) unsigned char smem[];
   C* buf = reinterpret_cast<C*>(smem);
   // FP32: sub-FFT twiddles in shared memory after the tile (FP64 reads the global table)
   C* tws = buf + (size_t)NB * bs;
   const bool smem_tw = sizeof(T) == 4;
-  if (smem_tw) load_tw_smem<T>(tws, stw, stage_tw_len(log2N1));
-  __shared__ T red[32];
-  // vector and working thread count: blockIdx.y and blockDim.x, or given by a batched launch
-  // (whose CTAs may have more threads than this plan's; the extra ones only meet the barriers,
-  // so that the DC partial sums keep this plan's order)
-  const int vec = vec_in >= 0 ? vec_in : (int)blockIdx.y;
-  const int nt = nthr_in > 0 ? nthr_in : (int)blockDim.x;
-  const St<T>* x = src + (int64_t)vec * src_stride;
-  const int c0 = bid * NB;
+  if (smem_tw) load_tw_smem<T>(tws, stw, stage_tw_len(log2N1, CplxFft<T>::E));
+  const int vec = blockIdx.y;
+  const C* x = reinterpret_cast<const C*>(src + (int64_t)vec * src_stride);
+  const int c0 = blockIdx.x * NB;
   const int log2NB = __ffs(NB) - 1, log2N2 = __ffs(N2) - 1;  // NB, N2 are powers of two
-  // The stage buffer read by the second DCT already holds Y / N (forward) or Y - Y0
-  // (transpose), so its stencils run with scale 1 and Y0 = 0 (constants the compiler folds).
-  const T Y0 = T(0);
-  const T sc = K == ST_FWD ? T(1) : invN;
-  // DC partials: consumed after IN_WINV (the transposed stage) and ST_FWD (the forward output);
-  // in split plans the DC value is the even half's (the DCT-III has none)
-  constexpr bool DC = (K == IN_WINV || K == ST_FWD) && MODE != PM_DCT3 && MODE != PM_DCT3A;
-  T dc = T(0);
   const int total = NB * N1;
   // independent element loads in flight per thread before the shared-memory stores
   constexpr int LD = InFlight<T>::v;
-  for (int idx0 = (int)threadIdx.x < nt ? (int)threadIdx.x : total; idx0 < total; idx0 += LD * nt) {
+  for (int idx0 = threadIdx.x; idx0 < total; idx0 += LD * blockDim.x) {
     C z[LD];
 #pragma unroll
     for (int u = 0; u < LD; ++u) {
-      const int idx = idx0 + u * nt;
-      if (idx < total) {
-        const int b = idx & (NB - 1);
-        const int j = ((idx >> log2NB) << log2N2) + c0 + b;
-        if (MODE == PM_FULL) z[u] = load_z<T, K>(x, j, N, sc, Y0, tb);
-        else if (MODE == PM_CPLX) z[u] = mk2<T>(x[2 * (int64_t)j], x[2 * (int64_t)j + 1]);
-        else if (MODE == PM_PAIR) z[u] = load_z_pair<T, K>(x, j, N, tb);
-        else if (MODE == PM_PAIR2) z[u] = load_z_pair2<T, K>(x, j, N);
-        else if (MODE == PM_DCT3A) z[u] = load_z_dct3a<T, K>(x, j, N, tpost, eo);
-        else z[u] = load_z_dct3<T, K>(x, j, N, tpost, eo, tb);
-      }
+      const int idx = idx0 + u * blockDim.x;
+      if (idx < total) z[u] = x[((idx >> log2NB) << log2N2) + c0 + (idx & (NB - 1))];
     }
 #pragma unroll
     for (int u = 0; u < LD; ++u) {
-      const int idx = idx0 + u * nt;
-      if (idx < total) {
-        if (DC) dc += z[u].x + z[u].y;
-        buf[(idx & (NB - 1)) * bs + padi(idx >> log2NB)] = z[u];
-      }
+      const int idx = idx0 + u * blockDim.x;
+      if (idx < total) buf[(idx & (NB - 1)) * bs + padi(idx >> log2NB)] = z[u];
     }
   }
-  if (DC) {
-    // block reduction of dc (deterministic order)
-    for (int o = 16; o > 0; o >>= 1) dc += shfl_xor(dc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = dc;
-  }
   __syncthreads();
-  if (DC && threadIdx.x < 32) {
-    T a = (int)threadIdx.x < (nt >> 5) ? red[threadIdx.x] : T(0);
-    for (int o = 16; o > 0; o >>= 1) a += shfl_xor(a, o);
-    if (threadIdx.x == 0) partial[(int64_t)vec * nbid + bid] = a;
-  }
-  fft16_any<T>(buf, N1, log2N1, NB, bs, smem_tw ? tws : stw);
+  fft_any<T, CplxFft<T>::E, CplxFft<T>::EPT>(buf, log2N1, NB, bs, smem_tw ? tws : stw);
   C* A = Aout + (int64_t)vec * N;
   // inter-pass twiddles omega_N^{j2 k1}, 4 independent table loads in flight per thread.
   // FP64: one table of omega_N^m (the FP64 pipe, not memory, bounds these kernels).
@@ -614,121 +475,34 @@ __device__ __forceinline__ void passA_body(
   }
 }
 
-#define BK_PASSA_PARAMS(S)                                                                           \
-  const St<T>* __restrict__ src##S, int64_t src_stride##S, typename V2<T>::t* __restrict__ Aout##S,          \
-      T* __restrict__ partial##S, int N##S, int N1##S, int log2N1##S, int N2##S, int NB##S, int bs##S,      \
-      const typename V2<T>::t* __restrict__ stw##S, const typename V2<T>::t* __restrict__ twN##S,           \
-      const typename V2<T>::t* __restrict__ twLo##S, const typename V2<T>::t* __restrict__ twHi##S, int tw_h##S
-#define BK_PASSA_ARGS(S)                                                                             \
-  src##S, src_stride##S, Aout##S, partial##S, N##S, N1##S, log2N1##S, N2##S, NB##S, bs##S, stw##S, twN##S
-#define BK_PASSA_TAIL(S) twLo##S, twHi##S, tw_h##S
-
-// Pass A of one transform (unsplit, or one half of a split DCT-I).
-template <typename T, int K, int MODE = PM_FULL>
-__global__ void __launch_bounds__(MaxThr<T>::v, MinB<T>::v)
-    k_passA(BK_PASSA_PARAMS(), T invN, StencilTab<T> tb, const typename V2<T>::t* __restrict__ tpost = nullptr,
-            const typename V2<T>::t* __restrict__ eo = nullptr) {
-  passA_body<T, K, MODE>(blockIdx.x, gridDim.x, BK_PASSA_ARGS(), invN, tb, BK_PASSA_TAIL(), tpost, eo);
-}
-
-// Pass A of both halves of a split DCT-I in one launch: CTAs [0, gE) run the even half (pair
-// sums), the rest the odd half (DCT-III); one launch fills the GPU better than two smaller ones.
+// Second-DCT input of a Bluestein product as its own elementwise pass: x_m of kind K (ST_FWD with
+// scale sc, or ST_TRN with Y0 = 0) for every m <= N, written to G.
 template <typename T, int K>
-__global__ void __launch_bounds__(MaxThr<T>::v, MinB<T>::v)
-    k_passA_split(int gE, BK_PASSA_PARAMS(E), BK_PASSA_PARAMS(O), T invN, StencilTab<T> tb,
-                  const typename V2<T>::t* __restrict__ tpost, const typename V2<T>::t* __restrict__ eo) {
-  if ((int)blockIdx.x < gE)
-    passA_body<T, K, PM_PAIR>(blockIdx.x, gE, BK_PASSA_ARGS(E), invN, tb, BK_PASSA_TAIL(E), tpost, eo);
-  else
-    passA_body<T, K, PM_DCT3>(blockIdx.x - gE, gridDim.x - gE, BK_PASSA_ARGS(O), invN, tb, BK_PASSA_TAIL(O), tpost, eo);
-}
-
-// Pass A of the three parts of a two-level split DCT-I in one launch: CTAs [0, g1) the DCT-I of
-// aa, [g1, g1 + g2) the DCT-III of a's pair differences, the rest the DCT-III of x's.
-template <typename T, int K>
-__global__ void __launch_bounds__(MaxThr<T>::v, MinB<T>::v)
-    k_passA_split3(int g1, int g2, BK_PASSA_PARAMS(E), BK_PASSA_PARAMS(D), BK_PASSA_PARAMS(O), T invN,
-                   StencilTab<T> tb, const typename V2<T>::t* __restrict__ tpost,
-                   const typename V2<T>::t* __restrict__ eo) {
-  const int b = blockIdx.x;
-  if (b < g1)
-    passA_body<T, K, PM_PAIR2>(b, g1, BK_PASSA_ARGS(E), invN, tb, BK_PASSA_TAIL(E), tpost, eo);
-  else if (b < g1 + g2)
-    passA_body<T, K, PM_DCT3A>(b - g1, g2, BK_PASSA_ARGS(D), invN, tb, BK_PASSA_TAIL(D), tpost, eo);
-  else
-    passA_body<T, K, PM_DCT3>(b - g1 - g2, gridDim.x - g1 - g2, BK_PASSA_ARGS(O), invN, tb, BK_PASSA_TAIL(O), tpost,
-                              eo);
-}
-
-// Second-DCT input as its own elementwise pass (planned applies): x_m of kind K (ST_FWD with
-// scale sc, or ST_TRN) for every m <= N, written to G, with per-CTA partial sums of W_m x_m
-// (the DC value R(x)_0 of the DCT, W = 1 at the ends, 2 inside) when `partial` is given. Fusing
-// the stencil into the pass-A loads instead exposes its neighbour loads: those passes ran
-// 25-40% longer than plain-load ones.
-// (bid, nbid, vec: block, blocks per vector and vector, from the launch or a batched launch;
-// 256 threads.)
-template <typename T, int K>
-__device__ __forceinline__ void stencil_body(int bid, int nbid, int vec, const St<T>* __restrict__ stage, int64_t Ls,
-                                             St<T>* __restrict__ G, int N, T sc, StencilTab<T> tb,
-                                             T* __restrict__ partial) {
-  __shared__ T red[8];
-  const St<T>* Y = stage + (int64_t)vec * Ls;
-  St<T>* g = G + (int64_t)vec * Ls;
-  typedef Cv<T, St<T>> CV;
-  T acc = T(0);
+__global__ void __launch_bounds__(256) k_stencil(const T* __restrict__ stage, int64_t Ls, T* __restrict__ G, int N, T sc,
+                                                 StencilTab<T> tb) {
+  const T* Y = stage + (int64_t)blockIdx.y * Ls;
+  T* g = G + (int64_t)blockIdx.y * Ls;
   // interior nodes 2..N-2 by the plain three-point formulas (the boundary cases, if-converted
   // into the same loop, tripled its FP64 instructions); the four boundary nodes by one thread
   const T* __restrict__ rk = tb.rk;
-  for (int m = 2 + bid * blockDim.x + threadIdx.x; m <= N - 2; m += nbid * blockDim.x) {
-    const T ym = CV::in(Y[m - 1]), yp = CV::in(Y[m + 1]);
-    const T x = K == ST_FWD ? (yp - ym) * (sc * rk[m]) : ym * rk[m - 1] - yp * rk[m + 1];
-    g[m] = CV::out(x);
-    acc += T(2) * x;
+  for (int m = 2 + blockIdx.x * blockDim.x + threadIdx.x; m <= N - 2; m += gridDim.x * blockDim.x) {
+    const T ym = Y[m - 1], yp = Y[m + 1];
+    g[m] = K == ST_FWD ? (yp - ym) * (sc * rk[m]) : ym * rk[m - 1] - yp * rk[m + 1];
   }
-  if (bid == 0 && threadIdx.x == 0) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     const int mb[4] = {0, 1, N - 1, N};
-    for (int i = 0; i < 4; ++i) {
-      const T x = load_x<T, K>(Y, mb[i], N, sc, T(0), tb);
-      g[mb[i]] = CV::out(x);
-      acc += (mb[i] == 0 || mb[i] == N) ? x : T(2) * x;
-    }
-  }
-  if (partial) {
-    for (int o = 16; o > 0; o >>= 1) acc += shfl_xor(acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      T a = T(0);
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a += red[w];
-      partial[(int64_t)vec * nbid + bid] = a;
-    }
+    for (int i = 0; i < 4; ++i) g[mb[i]] = load_x<T, K>(Y, mb[i], N, sc, T(0), tb);
   }
 }
 
-template <typename T, int K>
-__global__ void __launch_bounds__(256) k_stencil(const St<T>* __restrict__ stage, int64_t Ls, St<T>* __restrict__ G, int N,
-                                                 T sc, StencilTab<T> tb, T* __restrict__ partial) {
-  stencil_body<T, K>(blockIdx.x, gridDim.x, blockIdx.y, stage, Ls, G, N, sc, tb, partial);
-}
-
-// Caller's vectors (pitch apart) converted to the arithmetic type T, Ls apart (double-float
-// products: one conversion per element instead of one per load in the transform passes).
-template <typename T>
-__global__ void __launch_bounds__(256) k_to_arith(const Us<T>* __restrict__ v, int64_t pitch, T* __restrict__ x,
-                                                  int64_t Ls) {
-  const Us<T>* src = v + (int64_t)blockIdx.y * pitch;
-  T* dst = x + (int64_t)blockIdx.y * Ls;
-  for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < Ls; m += (int64_t)gridDim.x * blockDim.x)
-    dst[m] = Cv<T, Us<T>>::in(src[m]);
-}
-
-// Epilogue kinds of pass B:
-//   EP_STORE     : stage[k] = Y_k / N                      (after the first DCT, forward)
-//   EP_STORE_TRN : stage[k] = Y_k - Y0, Y0 from partials   (after the first DCT, transpose)
-//   EP_FWD_OUT   : out[k] = s (Y_k - Y0), Y0 from partials (after the second DCT, forward)
-//   EP_TRN_OUT   : out[k] = (s/N) W_k Y_k                   (after the second DCT, transpose)
-//   EP_CPLX      : dst[k] = Z_k                          (PB_CPLX: a plain complex FFT)
-//   EP_CPLX_MC   : dst[k] = conj(Z_k tab[k])             (PB_CPLX: spectral product, conjugated)
+// Epilogue kinds of a DCT-I's outputs R_k:
+//   EP_STORE     : stage[k] = R_k / N                      (after the first DCT, forward)
+//   EP_STORE_TRN : stage of the transposed product         (after the first DCT, transpose)
+//   EP_FWD_OUT   : out[k] = s (R_k - R_0)                  (after the second DCT, forward)
+//   EP_TRN_OUT   : out[k] = (s/N) W_k R_k                  (after the second DCT, transpose)
+// and of the plain complex FFT's pass B:
+//   EP_CPLX      : dst[k] = Z_k
+//   EP_CPLX_MC   : dst[k] = conj(Z_k tab[k])             (spectral product, conjugated)
 enum { EP_STORE = 0, EP_STORE_TRN = 1, EP_FWD_OUT = 2, EP_TRN_OUT = 3, EP_CPLX = 4, EP_CPLX_MC = 5 };
 
 template <typename T, int E, typename S>
@@ -739,6 +513,12 @@ __device__ __forceinline__ void ep_write(S* __restrict__ dst, int k, T yk, int N
   else if (E == EP_FWD_OUT) dst[k] = CV::out(s * (yk - Y0));
   else dst[k] = CV::out((k == 0 || k == N) ? s * invN * yk : T(2) * s * invN * yk);
 }
+
+}  // namespace bk
+
+#include "bk_dct.cuh"
+
+namespace bk {
 
 // ---------------------------------------------------------------------------------------------
 // N that is not a power of two (N > 1024): Bluestein's identity j k = (j^2 + k^2 - (k - j)^2)/2
@@ -754,10 +534,10 @@ __device__ __forceinline__ void ep_write(S* __restrict__ dst, int k, T yk, int N
 // ---------------------------------------------------------------------------------------------
 // a = z w zero-padded to M (one complex per element), z_j from the input kind K (IN_PLAIN / IN_WINV).
 template <typename T, int K>
-__global__ void __launch_bounds__(256) k_bs_pre(const St<T>* __restrict__ src, int64_t sstride, int N, int64_t M,
+__global__ void __launch_bounds__(256) k_bs_pre(const T* __restrict__ src, int64_t sstride, int N, int64_t M,
                                                 const typename V2<T>::t* __restrict__ w, T* __restrict__ a) {
   typedef typename V2<T>::t C;
-  const St<T>* x = src + (int64_t)blockIdx.y * sstride;
+  const T* x = src + (int64_t)blockIdx.y * sstride;
   T* dst = a + (int64_t)blockIdx.y * 2 * M;
   StencilTab<T> tb;
   tb.rk = nullptr;
@@ -776,11 +556,11 @@ template <typename T, int E>
 __global__ void __launch_bounds__(256) k_bs_post(const T* __restrict__ y, int64_t M, int N,
                                                  const typename V2<T>::t* __restrict__ w,
                                                  const typename V2<T>::t* __restrict__ tpost,
-                                                 typename OutS<T, E>::t* __restrict__ dst, int64_t dstride,
+                                                 T* __restrict__ dst, int64_t dstride,
                                                  int64_t zero_to, T s, T invN) {
   typedef typename V2<T>::t C;
   const T* yv = y + (int64_t)blockIdx.y * 2 * M;
-  typename OutS<T, E>::t* out = dst + (int64_t)blockIdx.y * dstride;
+  T* out = dst + (int64_t)blockIdx.y * dstride;
   auto Z = [&](int k) {  // w_k conj(y_k)
     const C yk = mk2<T>(yv[2 * (int64_t)k], -yv[2 * (int64_t)k + 1]);
     return cmul(w[k], yk);
@@ -795,56 +575,26 @@ __global__ void __launch_bounds__(256) k_bs_post(const T* __restrict__ y, int64_
     if (N - k != k) ep_write<T, E>(out, N - k, ynk, N, s, Y0, invN);
   }
   if ((E == EP_FWD_OUT || E == EP_TRN_OUT) && blockIdx.x == 0) {
-    for (int64_t m = N + 1 + threadIdx.x; m < zero_to; m += blockDim.x) out[m] = typename OutS<T, E>::t(0);
+    for (int64_t m = N + 1 + threadIdx.x; m < zero_to; m += blockDim.x) out[m] = T(0);
   }
 }
 
-// Pass-B modes: PB_PAIRS, row pairs {p, N1 - p} and the real-FFT split of a DCT-I (outputs at
-// ostride k of a transform of parent size Npar; (cos, sin)(pi k / n) read as tpost[tps k]);
-// PB_ROWS, plain rows of the DCT-III's inverse FFT (outputs unpacked to the odd indices of the
-// sub-transform, ostride (2m+1) of the whole one).
-// PB_CPLX, plain rows of a complex FFT written in natural order k = k1 + N1 k2 as complex pairs
-// (epilogues EP_CPLX, EP_CPLX_MC; `tpost` then holds the spectral table).
-enum { PB_PAIRS = 0, PB_ROWS = 1, PB_CPLX = 2 };
-
-template <typename T, int E, int MODE>
-__device__ __forceinline__ void passB_body(
-            int bid, const typename V2<T>::t* __restrict__ Ain, typename OutS<T, E>::t* __restrict__ dst, int64_t dst_stride,
-            int64_t pitch_zero_to, const T* __restrict__ partial, int n_partial, int N, int N1,
-            int N2, int log2N2, int P, const typename V2<T>::t* __restrict__ stw,
-            const typename V2<T>::t* __restrict__ tpost, T s, T invN, int ostride, int tps, int Npar,
-            int vec_in = -1, int nthr_in = 0) {
+// Pass B of the plain complex FFT: outputs as complex pairs in natural order; EP_CPLX_MC multiplies
+// by the spectral table and conjugates.
+template <typename T, int E>
+__global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
+    k_passB(const typename V2<T>::t* __restrict__ Ain, T* __restrict__ dst, int64_t dst_stride, int N, int N1, int N2,
+            int log2N2, int P, const typename V2<T>::t* __restrict__ stw, const typename V2<T>::t* __restrict__ tab) {
   typedef typename V2<T>::t C;
   extern __shared__ __align__(16) unsigned char smem[];
   const int bs = pad_stride(N2);
   C* buf = reinterpret_cast<C*>(smem);
   C* tws = buf + (size_t)2 * P * bs;
   const bool smem_tw = sizeof(T) == 4;
-  if (smem_tw) load_tw_smem<T>(tws, stw, stage_tw_len(log2N2));
-  __shared__ T red[32];
-  // as in passA_body: a batched launch gives the vector and this plan's thread count
-  const int vec = vec_in >= 0 ? vec_in : (int)blockIdx.y;
-  const int nt = nthr_in > 0 ? nthr_in : (int)blockDim.x;
-  const C* A = Ain + (int64_t)vec * N;
-  typename OutS<T, E>::t* out = dst + (int64_t)vec * dst_stride;
-  const int p0 = bid * P;
-  T Y0 = T(0);
-  if (E == EP_STORE_TRN || E == EP_FWD_OUT) {
-    T acc = T(0);
-    const T* pp = partial + (int64_t)vec * n_partial;
-    for (int i = (int)threadIdx.x < nt ? (int)threadIdx.x : n_partial; i < n_partial; i += nt) acc += pp[i];
-    for (int o = 16; o > 0; o >>= 1) acc += shfl_xor(acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      T a = (int)threadIdx.x < (nt >> 5) ? red[threadIdx.x] : T(0);
-      for (int o = 16; o > 0; o >>= 1) a += shfl_xor(a, o);
-      if (threadIdx.x == 0) red[0] = a;
-    }
-    __syncthreads();
-    Y0 = red[0];
-  }
-  // load 2P rows: PB_PAIRS local row q = 2 i (+1) for pair p0 + i; PB_ROWS rows 2 p0 + q
+  if (smem_tw) load_tw_smem<T>(tws, stw, stage_tw_len(log2N2, CplxFft<T>::E));
+  const C* A = Ain + (int64_t)blockIdx.y * N;
+  C* out = reinterpret_cast<C*>(dst + (int64_t)blockIdx.y * dst_stride);
+  const int p0 = blockIdx.x * P;
   const int total = 2 * P * N2;
   constexpr int LD = InFlight<T>::v;
   for (int idx0 = threadIdx.x; idx0 < total; idx0 += LD * blockDim.x) {
@@ -852,176 +602,38 @@ __device__ __forceinline__ void passB_body(
 #pragma unroll
     for (int u = 0; u < LD; ++u) {
       const int idx = idx0 + u * blockDim.x;
-      if (idx < total) {
-        const int q = idx >> log2N2;
-        int row;
-        if (MODE == PB_ROWS || MODE == PB_CPLX) {
-          row = 2 * p0 + q;
-        } else {
-          const int p = p0 + (q >> 1);
-          row = (q & 1) == 0 ? p : (p == 0 ? N1 / 2 : N1 - p);
-        }
-        z[u] = A[((int64_t)row << log2N2) + (idx & (N2 - 1))];
-      }
+      if (idx < total) z[u] = A[((int64_t)(2 * p0 + (idx >> log2N2)) << log2N2) + (idx & (N2 - 1))];
     }
 #pragma unroll
     for (int u = 0; u < LD; ++u) {
       const int idx = idx0 + u * blockDim.x;
-      if (idx < total) {
-        const int q = idx >> log2N2;
-        buf[q * bs + padi(idx & (N2 - 1))] = z[u];
-      }
+      if (idx < total) buf[(idx >> log2N2) * bs + padi(idx & (N2 - 1))] = z[u];
     }
   }
   __syncthreads();
-  fft16_any<T>(buf, N2, log2N2, 2 * P, bs, smem_tw ? tws : stw);
-  if constexpr (MODE == PB_CPLX) {
-    // lanes take consecutive rows, so each store run covers 2P consecutive outputs
-    const int log2R = __ffs(2 * P) - 1;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-      const int q = idx & (2 * P - 1);
-      const int k2 = idx >> log2R;
-      C R = buf[q * bs + padi(k2)];
-      const int64_t k = (int64_t)(2 * p0 + q) + (int64_t)N1 * k2;
-      if (E == EP_CPLX_MC) {
-        const C t = cmul(R, tpost[k]);
-        R.x = t.x;
-        R.y = -t.y;
-      }
-      out[2 * k] = R.x;
-      out[2 * k + 1] = R.y;
+  fft_any<T, CplxFft<T>::E, CplxFft<T>::EPT>(buf, log2N2, 2 * P, bs, smem_tw ? tws : stw);
+  // lanes take consecutive rows, so each store run covers 2P consecutive outputs
+  const int log2R = __ffs(2 * P) - 1;
+  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    const int q = idx & (2 * P - 1);
+    const int k2 = idx >> log2R;
+    C R = buf[q * bs + padi(k2)];
+    const int64_t k = (int64_t)(2 * p0 + q) + (int64_t)N1 * k2;
+    if (E == EP_CPLX_MC) {
+      const C t = cmul(R, tab[k]);
+      R.x = t.x;
+      R.y = -t.y;
     }
-    return;
+    out[k] = R;
   }
-  if (MODE == PB_ROWS) {
-    // output p = k1 + N1 k2 of the inverse FFT is z_p = conj(result): r_{2p} = Re, r_{2p+1} = -Im;
-    // X_{2j} = r_j, X_{2j+1} = r_{M-1-j} (j < M/2 = N), and Y_{2m+1} = X_m
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-      const int q = idx >> log2N2;
-      const int k2 = idx & (N2 - 1);
-      const C R = buf[q * bs + padi(k2)];
-      const int64_t pz = (int64_t)(2 * p0 + q) + (int64_t)N1 * k2;
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int64_t r = 2 * pz + t;
-        const int64_t m = r < N ? 2 * r : 2 * (2 * (int64_t)N - 1 - r) + 1;
-        ep_write<T, E>(out, (int)(ostride * (2 * m + 1)), t == 0 ? R.x : -R.y, Npar, s, Y0, invN);
-      }
-    }
-    return;
-  }
-  const int half = N / 2;
-  // Row pair i of the CTA and column k2 give outputs k = p0 + i + N1 k2 and N - k: lanes take
-  // consecutive i (P-long runs of consecutive outputs) and load 4 split twiddles at a time.
-  const int log2P = __ffs(P) - 1;  // P is a power of two
-  for (int idx0 = threadIdx.x; idx0 < P * N2; idx0 += 4 * blockDim.x) {
-    C cs[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int idx = idx0 + u * blockDim.x;
-      const int k = p0 + (idx & (P - 1)) + N1 * (idx >> log2P);
-      if (idx < P * N2 && p0 + (idx & (P - 1)) != 0) cs[u] = tpost[(k <= half ? k : N - k) * tps];
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int idx = idx0 + u * blockDim.x;
-      if (idx >= P * N2) continue;
-      const int i = idx & (P - 1);
-      const int k2 = idx >> log2P;
-      const int p = p0 + i;
-      const C* ra = buf + (2 * i) * bs;
-      const C* rb = buf + (2 * i + 1) * bs;
-      if (p == 0) {
-        // row 0 pairs internally (k2 <-> N2 - k2); row N1/2 pairs k2 <-> N2 - 1 - k2
-        if (k2 <= N2 / 2) {
-          const int k = N1 * k2;
-          T yk, ynk;
-          split_pair<T>(ra[padi(k2)], ra[padi((N2 - k2) & (N2 - 1))], tpost[k * tps], yk, ynk);
-          ep_write<T, E>(out, k * ostride, yk, Npar, s, Y0, invN);
-          if (k != half) ep_write<T, E>(out, (N - k) * ostride, ynk, Npar, s, Y0, invN);
-        }
-        if (k2 < N2 / 2) {
-          const int k = N1 / 2 + N1 * k2;
-          T yk, ynk;
-          split_pair<T>(rb[padi(k2)], rb[padi(N2 - 1 - k2)], tpost[k * tps], yk, ynk);
-          ep_write<T, E>(out, k * ostride, yk, Npar, s, Y0, invN);
-          ep_write<T, E>(out, (N - k) * ostride, ynk, Npar, s, Y0, invN);
-        }
-      } else {
-        const int k = p + N1 * k2;
-        const C zk = ra[padi(k2)];
-        const C zc = rb[padi(N2 - 1 - k2)];
-        T yk, ynk;
-        if (k <= half) {
-          split_pair<T>(zk, zc, cs[u], yk, ynk);
-        } else {
-          split_pair<T>(zc, zk, cs[u], ynk, yk);
-        }
-        ep_write<T, E>(out, k * ostride, yk, Npar, s, Y0, invN);
-        ep_write<T, E>(out, (N - k) * ostride, ynk, Npar, s, Y0, invN);
-      }
-    }
-  }
-  // zero the padding of the output vectors (final epilogues only)
-  if ((E == EP_FWD_OUT || E == EP_TRN_OUT) && bid == 0) {
-    for (int64_t m = Npar + 1 + threadIdx.x; m < pitch_zero_to; m += blockDim.x) out[m] = typename OutS<T, E>::t(0);
-  }
-}
-
-#define BK_PASSB_PARAMS(S)                                                                           \
-  const typename V2<T>::t* __restrict__ Ain##S, int N##S, int N1##S, int N2##S, int log2N2##S, int P##S, \
-      const typename V2<T>::t* __restrict__ stw##S
-
-template <typename T, int E, int MODE = PB_PAIRS>
-__global__ void __launch_bounds__(MaxThr<T>::v, MinB<T>::v)
-    k_passB(const typename V2<T>::t* __restrict__ Ain, typename OutS<T, E>::t* __restrict__ dst, int64_t dst_stride,
-            int64_t pitch_zero_to, const T* __restrict__ partial, int n_partial, int N, int N1,
-            int N2, int log2N2, int P, const typename V2<T>::t* __restrict__ stw,
-            const typename V2<T>::t* __restrict__ tpost, T s, T invN, int ostride, int tps, int Npar) {
-  passB_body<T, E, MODE>(blockIdx.x, Ain, dst, dst_stride, pitch_zero_to, partial, n_partial, N, N1, N2, log2N2, P, stw,
-                         tpost, s, invN, ostride, tps, Npar);
-}
-
-// Pass B of both halves of a split DCT-I in one launch: CTAs [0, gE) the even half's row pairs
-// and real split (outputs at even indices), the rest the odd half's rows (odd indices).
-template <typename T, int E>
-__global__ void __launch_bounds__(MaxThr<T>::v, MinB<T>::v)
-    k_passB_split(int gE, BK_PASSB_PARAMS(E), BK_PASSB_PARAMS(O), typename OutS<T, E>::t* __restrict__ dst, int64_t dst_stride,
-                  int64_t pitch_zero_to, const T* __restrict__ partial, int n_partial,
-                  const typename V2<T>::t* __restrict__ tpost, T s, T invN, int Npar) {
-  if ((int)blockIdx.x < gE)
-    passB_body<T, E, PB_PAIRS>(blockIdx.x, AinE, dst, dst_stride, pitch_zero_to, partial, n_partial, NE, N1E, N2E,
-                               log2N2E, PE, stwE, tpost, s, invN, 2, 2, Npar);
-  else
-    passB_body<T, E, PB_ROWS>(blockIdx.x - gE, AinO, dst, dst_stride, 0, partial, n_partial, NO, N1O, N2O, log2N2O,
-                              PO, stwO, tpost, s, invN, 1, 1, Npar);
-}
-
-// Pass B of a two-level split: the DCT-I of aa (outputs 4k), the DCT-III of a's pair
-// differences (outputs 4m + 2) and the DCT-III of x's (outputs 2m + 1).
-template <typename T, int E>
-__global__ void __launch_bounds__(MaxThr<T>::v, MinB<T>::v)
-    k_passB_split3(int h1, int h2, BK_PASSB_PARAMS(E), BK_PASSB_PARAMS(D), BK_PASSB_PARAMS(O), typename OutS<T, E>::t* __restrict__ dst,
-                   int64_t dst_stride, int64_t pitch_zero_to, const T* __restrict__ partial, int n_partial,
-                   const typename V2<T>::t* __restrict__ tpost, T s, T invN, int Npar) {
-  const int b = blockIdx.x;
-  if (b < h1)
-    passB_body<T, E, PB_PAIRS>(b, AinE, dst, dst_stride, pitch_zero_to, partial, n_partial, NE, N1E, N2E, log2N2E, PE,
-                               stwE, tpost, s, invN, 4, 4, Npar);
-  else if (b < h1 + h2)
-    passB_body<T, E, PB_ROWS>(b - h1, AinD, dst, dst_stride, 0, partial, n_partial, ND, N1D, N2D, log2N2D, PD, stwD,
-                              tpost, s, invN, 2, 2, Npar);
-  else
-    passB_body<T, E, PB_ROWS>(b - h1 - h2, AinO, dst, dst_stride, 0, partial, n_partial, NO, N1O, N2O, log2N2O, PO,
-                              stwO, tpost, s, invN, 1, 1, Npar);
 }
 
 // ---------------------------------------------------------------------------------------------
-// Batched launches over plans of different N (birkhoff_apply_batch): one launch per pass covers
-// up to BATCH_MAX plans. A job is one plan's part of a launch (its vectors, CTAs per vector and
-// shapes); CTA b of the launch belongs to the job q with start[q] <= b < start[q + 1] and runs
-// that job's body with that plan's own thread count, so every value it writes is the one the
-// plan's own launch writes. The descriptors travel as __grid_constant__ kernel parameters.
+// Batched launches over plans of different N (birkhoff_apply_batch): one launch covers up to
+// BATCH_MAX plans. A job is one plan's part of a launch (its vectors and shapes); CTA (or cluster)
+// b of the launch belongs to the job q with start[q] <= b < start[q + 1] and runs that job's body,
+// whose results do not depend on the launch's thread count or cluster size. The descriptors travel
+// as __grid_constant__ kernel parameters.
 // ---------------------------------------------------------------------------------------------
 constexpr int BATCH_MAX = 16;
 
@@ -1035,40 +647,6 @@ template <typename T> struct SmallJob {
   StencilTab<T> tb;
   T s;
   int N, log2N, nblk;
-};
-
-template <typename T> struct PassAJob {
-  const T* src;
-  int64_t sstride;
-  typename V2<T>::t* A;
-  T* partial;
-  const typename V2<T>::t* stw;
-  const typename V2<T>::t* twN;
-  const typename V2<T>::t* twLo;
-  const typename V2<T>::t* twHi;
-  StencilTab<T> tb;
-  T invN;
-  int N, N1, log2N1, N2, NB, bs, tw_h, nthr, nblk;
-};
-
-template <typename T> struct PassBJob {
-  const typename V2<T>::t* A;
-  T* dst;
-  int64_t dstride, zero_to;
-  const T* partial;
-  const typename V2<T>::t* stw;
-  const typename V2<T>::t* tpost;
-  T s, invN;
-  int npartial, N, N1, N2, log2N2, P, nthr, nblk;
-};
-
-template <typename T> struct StencilJob {
-  const T* stage;
-  T* G;
-  T* partial;
-  int64_t Ls;
-  StencilTab<T> tb;
-  int N, nblk;
 };
 
 template <typename J> struct Batch {
@@ -1085,59 +663,66 @@ __device__ __forceinline__ int batch_job(const Batch<J>& b, int cta) {
 }
 
 template <typename T, bool TRANS>
-__global__ void __launch_bounds__(MaxThr<T>::v) k_small_batch(const __grid_constant__ Batch<SmallJob<T>> b) {
+__global__ void __launch_bounds__(1024) k_small_batch(const __grid_constant__ Batch<SmallJob<T>> b) {
   const int q = batch_job(b, blockIdx.x);
   const SmallJob<T>& J = b.j[q];
   small_body<T, TRANS>((int)blockIdx.x - b.start[q], J.in, J.out, J.N, J.log2N, J.pitch, J.s, J.tw, J.stw, J.tpost,
                        J.tb);
 }
 
-template <typename T, int K>
-__global__ void __launch_bounds__(MaxThr<T>::v, MinB<T>::v) k_passA_batch(const __grid_constant__ Batch<PassAJob<T>> b) {
+// Launch-per-pass plans of one radix F: CTA b of a job runs vector b % nvec of tile b / nvec.
+template <typename T, bool TRANS, bool SECOND, typename F>
+__global__ void __launch_bounds__(F::MT, F::MINB) k_re_passA_batch(const __grid_constant__ Batch<ReJob<T>> b) {
   const int q = batch_job(b, blockIdx.x);
-  const PassAJob<T>& J = b.j[q];
-  const int local = (int)blockIdx.x - b.start[q];
-  const int vec = local / J.nblk;
-  passA_body<T, K, PM_FULL>(local - vec * J.nblk, J.nblk, J.src, J.sstride, J.A, J.partial, J.N, J.N1, J.log2N1, J.N2,
-                            J.NB, J.bs, J.stw, J.twN, J.invN, J.tb, J.twLo, J.twHi, J.tw_h, nullptr, nullptr, vec,
-                            J.nthr);
+  const ReJob<T>& J = b.j[q];
+  const int l = (int)blockIdx.x - b.start[q];
+  if constexpr (SECOND)
+    re_passA_cta<T, TRANS ? ST_TRN : ST_FWD, F, T>(J.g, l % J.nvec, l / J.nvec, J.NB, J.bsA, J.Y, J.ystride, J.A, J.astride,
+                                                   J.part);
+  else
+    re_passA_cta<T, TRANS ? IN_WINV : IN_PLAIN, F, T>(J.g, l % J.nvec, l / J.nvec, J.NB, J.bsA, J.in, J.pitch, J.A,
+                                                      J.astride, J.part);
+}
+template <typename T, bool TRANS, bool SECOND, typename F>
+__global__ void __launch_bounds__(F::MT, F::MINB) k_re_passB_batch(const __grid_constant__ Batch<ReJob<T>> b) {
+  const int q = batch_job(b, blockIdx.x);
+  const ReJob<T>& J = b.j[q];
+  const int l = (int)blockIdx.x - b.start[q];
+  if constexpr (SECOND)
+    re_passB_cta<T, TRANS ? EP_TRN_OUT : EP_FWD_OUT, F, T>(J.g, l % J.nvec, l / J.nvec, J.P, J.bsB, J.A, J.astride, J.out,
+                                                           J.pitch, J.pitch, J.part, J.s, J.invN);
+  else
+    re_passB_cta<T, TRANS ? EP_STORE_TRN : EP_STORE, F, T>(J.g, l % J.nvec, l / J.nvec, J.P, J.bsB, J.A, J.astride, J.Y,
+                                                           J.ystride, 0, J.part, J.s, J.invN);
 }
 
-template <typename T, int E>
-__global__ void __launch_bounds__(MaxThr<T>::v, MinB<T>::v) k_passB_batch(const __grid_constant__ Batch<PassBJob<T>> b) {
-  const int q = batch_job(b, blockIdx.x);
-  const PassBJob<T>& J = b.j[q];
-  const int local = (int)blockIdx.x - b.start[q];
-  const int vec = local / J.nblk;
-  passB_body<T, E, PB_PAIRS>(local - vec * J.nblk, J.A, J.dst, J.dstride, J.zero_to, J.partial, J.npartial, J.N, J.N1,
-                             J.N2, J.log2N2, J.P, J.stw, J.tpost, J.s, J.invN, 1, 1, J.N, vec, J.nthr);
-}
-
-template <typename T, int K>
-__global__ void __launch_bounds__(256) k_stencil_batch(const __grid_constant__ Batch<StencilJob<T>> b) {
-  const int q = batch_job(b, blockIdx.x);
-  const StencilJob<T>& J = b.j[q];
-  const int local = (int)blockIdx.x - b.start[q];
-  const int vec = local / J.nblk;
-  stencil_body<T, K>(local - vec * J.nblk, J.nblk, vec, J.stage, J.Ls, J.G, J.N, T(1), J.tb, J.partial);
+template <typename T, bool TRANS>
+__global__ void __launch_bounds__(512, sizeof(T) == 8 ? 1 : 2) k_re_cluster_batch(const __grid_constant__ Batch<ReJob<T>> b, int csize) {
+  const int cl = blockIdx.x / csize;
+  const int q = batch_job(b, cl);
+  re_cluster_body<T, TRANS>(b.j[q], cl - b.start[q], blockIdx.x % csize, csize);
 }
 
 // ---------------------------------------------------------------------------------------------
 // Plan creation / destruction and the apply entry points
 // ---------------------------------------------------------------------------------------------
-// Stage tables and the inter-pass twiddle table of one four-step layout.
+template <typename T>
+static bk_status build_stage_table(void** dst, int64_t n, int e, cudaStream_t st) {
+  typedef typename V2<T>::t C;
+  const int len = stage_tw_len(ilog2(n), e);
+  if (len == 0) return BK_OK;
+  BK_TRY(dmalloc(dst, sizeof(C) * len));
+  k_stage_tw<T><<<(len + 255) / 256, 256, 0, st>>>((C*)*dst, ilog2(n), e, len);
+  BK_CHECK_LAUNCH();
+  return BK_OK;
+}
+
+// Tables of the plain complex layout: stage tables and the inter-pass twiddles.
 template <typename T>
 static bk_status build_fs_tables(FourStep& f, cudaStream_t st) {
   typedef typename V2<T>::t C;
-  for (int w = 0; w < 2; ++w) {
-    const int n = w == 0 ? f.N1 : f.N2;
-    void** dst = w == 0 ? &f.stw1 : &f.stw2;
-    const int len = stage_tw_len(ilog2(n));
-    if (len == 0) continue;
-    BK_TRY(dmalloc(dst, sizeof(C) * len));
-    k_stage_tw<T><<<(len + 255) / 256, 256, 0, st>>>((C*)*dst, ilog2(n), len);
-    BK_CHECK_LAUNCH();
-  }
+  BK_TRY(build_stage_table<T>(&f.stw1, f.N1, CplxFft<T>::E, st));
+  BK_TRY(build_stage_table<T>(&f.stw2, f.N2, CplxFft<T>::E, st));
   const int64_t n = f.n;
   if (sizeof(T) == 8) {
     BK_TRY(dmalloc(&f.twN, sizeof(C) * n));
@@ -1166,20 +751,14 @@ static void free_fs(FourStep& f) {
   f = FourStep();
 }
 
+static int re_tw_blocks(const FourStep& f) { return (int)std::min<int64_t>((f.a_len() + 255) / 256, 8192); }
+
 template <typename T>
 static bk_status build_tables(Plan* p, cudaStream_t st) {
   typedef typename V2<T>::t C;
   const int64_t N = p->N;
   // FFT twiddles: single-CTA plans keep omega_N^i (direct DFT for N < 16) and the stage table of
-  // N; four-step plans the stage tables of N1 and N2.
-  auto stage_table = [&](void** dst, int64_t n) -> bk_status {
-    const int len = stage_tw_len(ilog2(n));
-    if (len == 0) return BK_OK;
-    BK_TRY(dmalloc(dst, sizeof(C) * len));
-    k_stage_tw<T><<<(len + 255) / 256, 256, 0, st>>>((C*)*dst, ilog2(n), len);
-    BK_CHECK_LAUNCH();
-    return BK_OK;
-  };
+  // N; four-step plans the stage tables of N1 and N2 and the inter-pass table.
   if (p->blue) {
     BK_TRY(build_fs_tables<T>(p->fsM, st));
     BK_TRY(dmalloc(&p->chirp, sizeof(C) * N));
@@ -1190,25 +769,23 @@ static bk_status build_tables(Plan* p, cudaStream_t st) {
     BK_TRY(dmalloc(&p->tw, sizeof(C) * N));
     k_tw_table<T><<<(int)std::min<int64_t>((N + 255) / 256, 4096), 256, 0, st>>>((C*)p->tw, N, (double)N);
     BK_CHECK_LAUNCH();
-    if (N >= 16) BK_TRY(stage_table(&p->stwS, N));
+    if (N >= 16) BK_TRY(build_stage_table<T>(&p->stwS, N, SmallFft<T>::E, st));
   } else {
-    BK_TRY(build_fs_tables<T>(p->fs, st));
-    if (p->split) {
-      BK_TRY(build_fs_tables<T>(p->fso, st));
-      if (p->split == 2) BK_TRY(build_fs_tables<T>(p->fse, st));
-      const int64_t M = N / 2;
-      BK_TRY(dmalloc(&p->eo, sizeof(C) * (M / 2)));
-      // exp(+2 pi i k / M) = conj(omega_M^k)
-      k_tw_table<T><<<(int)std::min<int64_t>((M / 2 + 255) / 256, 4096), 256, 0, st>>>((C*)p->eo, M / 2, (double)M);
-      BK_CHECK_LAUNCH();
-    }
+    const int e = p->split ? p->fe : SmallFft<T>::E;
+    BK_TRY(build_stage_table<T>(&p->fs.stw1, p->fs.N1, e, st));
+    BK_TRY(build_stage_table<T>(&p->fs.stw2, p->fs.N2, e, st));
+    BK_TRY(dmalloc(&p->fs.twN, sizeof(C) * p->fs.a_len()));
+    k_re_tw<T><<<re_tw_blocks(p->fs), 256, 0, st>>>((C*)p->fs.twN, p->fs.N1, p->fs.N2);
+    BK_CHECK_LAUNCH();
   }
   BK_TRY(dmalloc(&p->rk, sizeof(T) * (N + 2)));
   k_rk_table<T><<<(int)std::min<int64_t>((N + 2 + 255) / 256, 4096), 256, 0, st>>>((T*)p->rk, N + 2);
   BK_CHECK_LAUNCH();
-  BK_TRY(dmalloc(&p->tpost, sizeof(C) * (N / 2 + 1)));
-  k_post_table<T><<<(int)std::min<int64_t>((N / 2 + 256) / 256, 4096), 256, 0, st>>>((C*)p->tpost, N);
-  BK_CHECK_LAUNCH();
+  if (p->blue || p->small) {
+    BK_TRY(dmalloc(&p->tpost, sizeof(C) * (N / 2 + 1)));
+    k_post_table<T><<<(int)std::min<int64_t>((N / 2 + 256) / 256, 4096), 256, 0, st>>>((C*)p->tpost, N);
+    BK_CHECK_LAUNCH();
+  }
   return BK_OK;
 }
 
@@ -1254,14 +831,14 @@ static bk_status compute_weights(Plan* p, cudaStream_t st) {
 }
 #endif  // BK_TRANSFORM_KERNEL_UNIT
 
-// Largest N run by the single-CTA kernel (one CTA per vector): 128 in FP64, whose single CTA
-// runs on one SM's FP64 pipe (4 components, cold L2, B / four-step ms: 2^8 0.062 / 0.056,
-// 2^10 0.089 / 0.068, 2^11 0.097 / 0.074), 4096 in FP32 (2^12 0.034 / 0.038, 2^13 0.044 /
-// 0.042). BK_SMALL_MAX_LOG2 overrides it for tuning (at least 2^4; at most the shared-memory
-// limit of 4096 in FP64, 8192 in FP32). The four-step kernels need N >= 256.
-static int small_default(int dtype) { return dtype == BK_F64 ? 128 : 4096; }
+// Largest N run by the single-CTA kernel (one CTA per vector): 256 in FP64, whose single CTA runs
+// on one SM's FP64 pipe, 4096 in FP32. Measured (4 components, warm, us per product, one CTA /
+// cluster): FP64 2^8 18.6 / 24.7, 2^10 35.1 / 26.8; FP32 2^11 13.5 / 15.5, 2^12 16.7 / 17.2.
+// BK_SMALL_MAX_LOG2 overrides it for tuning (at least 2^4; at most the shared-memory limit of
+// 4096). The four-step kernels need N >= 128.
+static int small_default(int dtype) { return dtype == BK_F64 ? 256 : 4096; }
 static int small_limit(int dtype) {
-  const int cap = dtype == BK_F64 ? 4096 : 8192;
+  const int cap = 4096;
   const char* e = getenv("BK_SMALL_MAX_LOG2");
   if (e) {
     const long v = atol(e);
@@ -1277,7 +854,7 @@ static size_t smem_small(int64_t N) {
   return sizeof(T) * 2 * Lp + sizeof(typename V2<T>::t) * (size_t)pad_stride((int)N);
 }
 
-static int round_threads(int64_t t) {
+static int round_threads(int64_t t) {  // whole warps
   t = (t + 31) / 32 * 32;
   return (int)std::min<int64_t>(1024, std::max<int64_t>(32, t));
 }
@@ -1301,7 +878,7 @@ static int sm_count() {
 // transforms thus run many one-warp CTAs instead of a few full ones (at 2^14 x 4 components the
 // full-size tiles gave 16 CTAs per pass). BK_FOURSTEP_ELEMS fixes it (tuning).
 static int fourstep_elems(int dtype, int64_t n, int nvec, int N1, int N2, int Eforce = 0) {
-  const int cap = dtype == BK_F64 ? 4096 : 8192;  // 16 per thread at the thread cap
+  const int cap = dtype == BK_F64 ? 4096 : 8192;  // values per thread x the thread cap
   if (Eforce > 0) return std::min(cap, std::max(Eforce, std::max(N1, 2 * N2)));
   const char* e = getenv("BK_FOURSTEP_ELEMS");
   if (e) {
@@ -1315,48 +892,34 @@ static int fourstep_elems(int dtype, int64_t n, int nvec, int N1, int N2, int Ef
   return (int)std::min<int64_t>(E, cap);
 }
 
-// Smallest log2 N planned with the two-level split: 2^18 in FP64, 2^24 in FP32
-// (BK_SPLIT2_MIN_LOG2 overrides both; 30 disables). Measured products (4 components, two-level
-// vs one-level ms): FP64 2^17 0.181 vs 0.178, 2^18 0.272 vs 0.313, 2^20 0.978 vs 1.084, 2^22
-// 3.88 vs 4.38, 2^24 17.6 vs 19.3; FP32 2^23 1.557 vs 1.556, 2^24 4.02 vs 4.17.
-static int split2_min_log2(int dtype) {
-  const char* e = getenv("BK_SPLIT2_MIN_LOG2");
-  if (e) {
-    const long v = atol(e);
-    if (v >= 13 && v <= 30) return (int)v;
-  }
-  return dtype == BK_F64 ? 18 : 24;
-}
-
-// Smallest log2 N planned with the split DCT-I: 2^17 in FP64, 2^23 in FP32 (BK_SPLIT_MIN_LOG2
-// overrides both for tuning; 30 disables the split). Below them the half-size launches fill the
-// GPU poorly. Measured products (tuned tiles, 4 components, split vs unsplit ms): FP64 2^16
-// 0.158 vs 0.124, 2^17 0.179 vs 0.189, 2^18 0.316 vs 0.351, 2^19 0.570 vs 0.638, 2^20 1.09
-// vs 1.27; FP32 2^20 0.21 vs 0.166, 2^21 0.349 vs 0.322, 2^22 0.715 vs 0.713, 2^23 1.55 vs
-// 1.88. At 2^24 both precisions need the split (the unsplit length-2^24 FFT exceeds the
-// four-step shapes).
+// Smallest log2 N whose four passes run as a launch each instead of as one cluster launch: 14 in
+// FP64, whose sixteen CTAs per vector leave most FP64 pipes idle, 15 in FP32. Measured (4
+// components, warm, us per product, cluster / launch per pass): FP64 2^12 30.9 / 40.2, 2^13 39.1 /
+// 42.2, 2^14 49.4 / 45.3, 2^15 72 / 46.3; FP32 2^13 21.3 / 26.9, 2^14 22.8 / 25.8, 2^16 49.0 / 30.7.
+// BK_SPLIT_MIN_LOG2 overrides it for tuning.
 static int split_min_log2(int dtype) {
   const char* e = getenv("BK_SPLIT_MIN_LOG2");
   if (e) {
     const long v = atol(e);
-    if (v >= 13 && v <= 30) return (int)v;
+    if (v >= 7 && v <= 30) return (int)v;
   }
-  return dtype == BK_F64 ? 17 : 23;
+  return dtype == BK_F64 ? 14 : 15;
 }
 
 // Shapes of one four-step layout (tables untouched, so a built plan can be re-shaped); Eforce
 // > 0 fixes the elements per CTA (the autotuner's candidates), 0 takes fourstep_elems.
 static bk_status configure_fourstep(FourStep& f, int64_t n, int dtype, int nvec, int Eforce = 0) {
+  const int ept = dtype == BK_F64 ? CplxFft<double>::EPT : CplxFft<float>::EPT;
   const int log2n = ilog2(n);
   f.n = n;
-  // balanced factors, with the rows short enough for one row pair per CTA (2 N2 / 16 threads)
-  // and the columns for one column per CTA (N1 / 16 threads) under the thread cap
-  const int maxthr = dtype == BK_F64 ? 256 : 512;
+  // balanced factors, with the rows short enough for one row pair per CTA (2 N2 / EPT threads)
+  // and the columns for one column per CTA (N1 / EPT threads) under the thread cap
+  const int maxthr = dtype == BK_F64 ? CplxFft<double>::MT : CplxFft<float>::MT;
   int l2 = log2n - log2n / 2;
-  while (l2 > 0 && (2 << l2) / 16 > maxthr) --l2;
+  while (l2 > 0 && (2 << l2) / ept > maxthr) --l2;
   f.N2 = 1 << l2;
   f.N1 = 1 << (log2n - l2);
-  if (f.N1 / 16 > maxthr) {
+  if (f.N1 / ept > maxthr) {
     set_error("four-step configuration failed for n=%lld (transform too long for this precision)", (long long)n);
     return BK_ERR_UNSUPPORTED;
   }
@@ -1378,14 +941,93 @@ static bk_status configure_fourstep(FourStep& f, int64_t n, int dtype, int nvec,
   f.bsA = f.N1 + f.N1 / 16 + padA;
   f.smemA = csz * ((size_t)NB * f.bsA + (dtype == BK_F32 ? f.N1 : 0));
   f.smemB = csz * ((size_t)2 * P * pad_stride(f.N2) + (dtype == BK_F32 ? f.N2 : 0));
-  f.thrA = round_threads((int64_t)NB * f.N1 / 16);
-  f.thrB = round_threads((int64_t)2 * P * f.N2 / 16);
-  if ((int64_t)NB * f.N1 / 16 > maxthr || (int64_t)2 * P * f.N2 / 16 > maxthr || f.smemA > FOURSTEP_SMEM_BUDGET ||
+  f.thrA = round_threads((int64_t)NB * f.N1 / ept);
+  f.thrB = round_threads((int64_t)2 * P * f.N2 / ept);
+  if ((int64_t)NB * f.N1 / ept > maxthr || (int64_t)2 * P * f.N2 / ept > maxthr || f.smemA > FOURSTEP_SMEM_BUDGET ||
       f.smemB > FOURSTEP_SMEM_BUDGET) {
     set_error("four-step configuration failed for n=%lld", (long long)n);
     return BK_ERR_UNSUPPORTED;
   }
-  f.nPartA = f.N2 / f.NB;
+  return BK_OK;
+}
+
+// Batch stride of a tile of nb transforms of length n in shared memory: when a warp's FFT stays
+// inside one transform (n / 16 >= 32 threads), the accesses with the transform as the fastest lane
+// index hit distinct banks if the stride is = W / nb modulo the W complex elements of a 128-byte
+// wavefront.
+static int re_stride(int dtype, int n, int nb) {
+  const int W = dtype == BK_F64 ? 8 : 16;
+  return n + n / 16 + (n / 16 >= 32 && nb < W ? W / nb : 1);
+}
+
+// Factors of the real-even passes, 2N = N1 N2 (both >= 16 for N >= 128). At N = 2^24 the FP64 rows
+// have 8192 points (the BIG instances of pass B).
+static void re_factors(FourStep& f, int64_t N) {
+  const int l = ilog2(N) + 1;
+  f.n = 2 * N;
+  f.N1 = 1 << (l / 2);
+  f.N2 = 1 << (l - l / 2);
+}
+
+static bool re_big(const FourStep& f, int dtype) { return dtype == BK_F64 && f.N2 > 4096; }
+
+// log2 radix of the launch-per-pass kernels (the reasons and figures are in bk_fft.cuh), and the
+// complex elements per CTA their thread cap admits.
+static int re_radix(int64_t N, int dtype, bool df) {
+  if (dtype == BK_F64) return df ? 3 : 2;
+  return N <= (int64_t(1) << 18) ? 2 : 4;
+}
+static int re_elems_max(const FourStep& f, int dtype, int fe) {
+  if (dtype == BK_F32) return fe == 4 ? FftShape<float, 4>::MT * FftShape<float, 4>::EPT : FftShape<float, 2>::MT * FftShape<float, 2>::EPT;
+  return std::max(4096, f.N2);   // 1024 threads of 4 or 512 of 8; one longer row takes BigFft
+}
+
+// Tiles of the launch-per-pass form for E complex elements per CTA (0: enough CTAs for two per SM
+// over the plan's vectors).
+static bk_status configure_re(FourStep& f, int64_t N, int dtype, int fe, int nvec, int Eforce = 0) {
+  re_factors(f, N);
+  const int E = std::min(re_elems_max(f, dtype, fe), fourstep_elems(dtype, N / 2, nvec, f.N1, f.N2 / 2, Eforce));
+  f.NB = std::max(1, E / f.N1);
+  f.P = std::max(1, E / f.N2);
+  const size_t csz = 2 * dtype_size(dtype);
+  f.bsA = re_stride(dtype, f.N1, f.NB);
+  f.bsB = re_stride(dtype, f.N2, f.P);
+  f.smemA = csz * ((size_t)f.NB * f.bsA + (dtype == BK_F32 ? stage_tw_len(ilog2(f.N1), fe) : 0));
+  f.smemB = csz * ((size_t)f.P * f.bsB + (dtype == BK_F32 ? stage_tw_len(ilog2(f.N2), fe) : 0));
+  const int64_t tA = (int64_t)f.NB * f.N1 >> fe, tB = re_big(f, dtype) ? 512 : (int64_t)f.P * f.N2 >> fe;
+  f.thrA = round_threads(tA);
+  f.thrB = round_threads(tB);
+  if (f.smemA > FOURSTEP_SMEM_BUDGET || f.smemB > FOURSTEP_SMEM_BUDGET || f.thrA < tA || f.thrB < tB) {
+    set_error("four-step configuration failed for N=%lld", (long long)N);
+    return BK_ERR_UNSUPPORTED;
+  }
+  return BK_OK;
+}
+
+// Tiles of the one-launch form: a cluster of at most 16 CTAs per vector, its column and row pairs
+// spread over all of them.
+static bk_status configure_cluster(Plan* p) {
+  FourStep& f = p->fs;
+  re_factors(f, p->N);
+  p->csize = std::min(16, f.N2 / 4);
+  const int maxthr = 512;
+  auto per = [&](int pairs, int n) {   // pairs per CTA, in as few equal rounds as the thread cap allows
+    const int each = (pairs + p->csize - 1) / p->csize;
+    const int rounds = (int)(((int64_t)each * n / SmallFft<float>::EPT + maxthr - 1) / maxthr);
+    return (each + rounds - 1) / rounds;
+  };
+  f.NB = per(f.N2 / 4 + 1, f.N1);
+  f.P = per(f.N1 / 4 + 1, f.N2);
+  f.bsA = re_stride(p->dtype, f.N1, f.NB);
+  f.bsB = re_stride(p->dtype, f.N2, f.P);
+  const size_t csz = 2 * dtype_size(p->dtype);
+  p->csmem = csz * (size_t)(std::max(f.NB * f.bsA, f.P * f.bsB) + stage_tw_len(ilog2(f.N1), SmallFft<float>::E) +
+                               stage_tw_len(ilog2(f.N2), SmallFft<float>::E));
+  p->cthr = std::max(128, round_threads(std::max(f.NB * f.N1, f.P * f.N2) / SmallFft<float>::EPT));
+  if (p->csmem > FOURSTEP_SMEM_BUDGET || p->cthr > maxthr) {
+    set_error("cluster configuration failed for N=%lld", (long long)p->N);
+    return BK_ERR_UNSUPPORTED;
+  }
   return BK_OK;
 }
 
@@ -1402,53 +1044,78 @@ static bk_status smem_attr(K* fn, int cap) {
   return BK_OK;
 }
 
+template <typename T, typename F>
+static bk_status re_attrs_B(int cap) {
+  BK_TRY(smem_attr(k_re_passB<T, EP_STORE, F, T>, cap));
+  BK_TRY(smem_attr(k_re_passB<T, EP_STORE_TRN, F, T>, cap));
+  BK_TRY(smem_attr(k_re_passB<T, EP_FWD_OUT, F, Us<T>>, cap));
+  BK_TRY(smem_attr(k_re_passB<T, EP_TRN_OUT, F, Us<T>>, cap));
+  return BK_OK;
+}
+
+template <typename T, typename F>
+static bk_status re_attrs_AB(int cap) {
+  BK_TRY(smem_attr(k_re_passA<T, IN_PLAIN, F, Us<T>>, cap));
+  BK_TRY(smem_attr(k_re_passA<T, IN_WINV, F, Us<T>>, cap));
+  BK_TRY(smem_attr(k_re_passA<T, ST_FWD, F, T>, cap));
+  BK_TRY(smem_attr(k_re_passA<T, ST_TRN, F, T>, cap));
+  return re_attrs_B<T, F>(cap);
+}
+
+template <typename F>
+static bk_status cluster_attr(F* fn, int cap) {
+  BK_TRY(smem_attr(fn, cap));
+  BK_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  return BK_OK;
+}
+
+template <typename T>
+bk_status re_attrs() {
+  const int cap = (int)FOURSTEP_SMEM_BUDGET;
+  if constexpr (sizeof(T) == 4) {
+    BK_TRY((re_attrs_AB<T, FftShape<T, 2>>(cap)));
+    BK_TRY((re_attrs_AB<T, FftShape<T, 4>>(cap)));
+  } else {
+    BK_TRY((re_attrs_AB<T, FftShape<T, std::is_same<T, dfl>::value ? 3 : 2>>(cap)));
+    BK_TRY((re_attrs_B<T, BigFft<T>>(cap)));
+  }
+  if constexpr (!std::is_same<T, dfl>::value) {
+    BK_TRY(cluster_attr(k_re_cluster<T, false>, cap));
+    BK_TRY(cluster_attr(k_re_cluster<T, true>, cap));
+    BK_TRY(cluster_attr(k_re_cluster_batch<T, false>, cap));
+    BK_TRY(cluster_attr(k_re_cluster_batch<T, true>, cap));
+    typedef FftShape<T, 2> F;
+    BK_TRY(smem_attr(k_re_passA_batch<T, false, false, F>, cap));
+    BK_TRY(smem_attr(k_re_passA_batch<T, false, true, F>, cap));
+    BK_TRY(smem_attr(k_re_passA_batch<T, true, false, F>, cap));
+    BK_TRY(smem_attr(k_re_passA_batch<T, true, true, F>, cap));
+    BK_TRY(smem_attr(k_re_passB_batch<T, false, false, F>, cap));
+    BK_TRY(smem_attr(k_re_passB_batch<T, false, true, F>, cap));
+    BK_TRY(smem_attr(k_re_passB_batch<T, true, false, F>, cap));
+    BK_TRY(smem_attr(k_re_passB_batch<T, true, true, F>, cap));
+  }
+  return BK_OK;
+}
+
 template <typename T>
 bk_status set_smem_attrs(const Plan* p) {
   if (p->small) {
-    const int cap = (int)smem_small<T>(p->dtype == BK_F64 ? 4096 : 8192);
-    BK_TRY(smem_attr(k_birkhoff_small<T, false>, cap));
-    BK_TRY(smem_attr(k_birkhoff_small<T, true>, cap));
     if constexpr (!std::is_same<T, dfl>::value) {
+      const int cap = (int)smem_small<T>(4096);
+      BK_TRY(smem_attr(k_birkhoff_small<T, false>, cap));
+      BK_TRY(smem_attr(k_birkhoff_small<T, true>, cap));
       BK_TRY(smem_attr(k_small_batch<T, false>, cap));
       BK_TRY(smem_attr(k_small_batch<T, true>, cap));
     }
+  } else if (p->blue) {
+    if constexpr (!std::is_same<T, dfl>::value) {
+      const int cap = (int)FOURSTEP_SMEM_BUDGET;
+      BK_TRY(smem_attr(k_passA<T>, cap));
+      BK_TRY(smem_attr(k_passB<T, EP_CPLX>, cap));
+      BK_TRY(smem_attr(k_passB<T, EP_CPLX_MC>, cap));
+    }
   } else {
-    const int cap = (int)FOURSTEP_SMEM_BUDGET;
-    if constexpr (!std::is_same<T, dfl>::value) {
-      BK_TRY(smem_attr(k_passA_batch<T, IN_PLAIN>, cap));
-      BK_TRY(smem_attr(k_passA_batch<T, IN_WINV>, cap));
-      BK_TRY(smem_attr(k_passB_batch<T, EP_STORE>, cap));
-      BK_TRY(smem_attr(k_passB_batch<T, EP_STORE_TRN>, cap));
-      BK_TRY(smem_attr(k_passB_batch<T, EP_FWD_OUT>, cap));
-      BK_TRY(smem_attr(k_passB_batch<T, EP_TRN_OUT>, cap));
-    }
-    BK_TRY(smem_attr(k_passA<T, IN_PLAIN>, cap));
-    BK_TRY(smem_attr(k_passA<T, IN_WINV>, cap));
-    if constexpr (std::is_same<T, double>::value) {
-      BK_TRY(smem_attr(k_passA<T, ST_FWD>, cap));
-      BK_TRY(smem_attr(k_passA<T, ST_TRN>, cap));
-    }
-    BK_TRY(smem_attr(k_passB<T, EP_STORE>, cap));
-    BK_TRY(smem_attr(k_passB<T, EP_STORE_TRN>, cap));
-    BK_TRY(smem_attr(k_passB<T, EP_FWD_OUT>, cap));
-    BK_TRY(smem_attr(k_passB<T, EP_TRN_OUT>, cap));
-    BK_TRY(smem_attr(k_passA_split<T, IN_PLAIN>, cap));
-    BK_TRY(smem_attr(k_passA_split<T, IN_WINV>, cap));
-    BK_TRY(smem_attr(k_passB_split<T, EP_STORE>, cap));
-    BK_TRY(smem_attr(k_passB_split<T, EP_STORE_TRN>, cap));
-    BK_TRY(smem_attr(k_passB_split<T, EP_FWD_OUT>, cap));
-    BK_TRY(smem_attr(k_passB_split<T, EP_TRN_OUT>, cap));
-    BK_TRY(smem_attr(k_passA_split3<T, IN_PLAIN>, cap));
-    BK_TRY(smem_attr(k_passA_split3<T, IN_WINV>, cap));
-    BK_TRY(smem_attr(k_passB_split3<T, EP_STORE>, cap));
-    BK_TRY(smem_attr(k_passB_split3<T, EP_STORE_TRN>, cap));
-    BK_TRY(smem_attr(k_passB_split3<T, EP_FWD_OUT>, cap));
-    BK_TRY(smem_attr(k_passB_split3<T, EP_TRN_OUT>, cap));
-    if constexpr (!std::is_same<T, dfl>::value) {
-      BK_TRY(smem_attr(k_passA<T, IN_PLAIN, PM_CPLX>, cap));
-      BK_TRY(smem_attr(k_passB<T, EP_CPLX, PB_CPLX>, cap));
-      BK_TRY(smem_attr(k_passB<T, EP_CPLX_MC, PB_CPLX>, cap));
-    }
+    BK_TRY(re_attrs<T>());
   }
   return BK_OK;
 }
@@ -1460,6 +1127,7 @@ static int64_t blue_max(int dtype) { return dtype == BK_F64 ? (int64_t(1) << 22)
 // The instances of set_smem_attrs and apply_impl (and with them every transform kernel) are
 // compiled in bk_birkhoff_f64.cu and bk_birkhoff_f32.cu, in parallel with this unit.
 extern template bk_status set_smem_attrs<double>(const Plan* p);
+extern template bk_status re_attrs<double>();
 extern template bk_status set_smem_attrs<float>(const Plan* p);
 extern template bk_status set_smem_attrs<dfl>(const Plan* p);
 template <typename T> bk_status blue_spectrum(Plan* p, cudaStream_t st);
@@ -1468,19 +1136,15 @@ extern template bk_status blue_spectrum<float>(Plan* p, cudaStream_t st);
 #endif
 
 // Power-of-two plans take the FFT chain unless BK_DENSE=1 (read at plan creation; then every
-// plan with N <= 1024 and at most 16 vectors per product starts on the dense product). The dense
-// product is faster per call (4 vectors, cold L2, FFT / dense ms: FP32 2^10 0.027 / 0.019, FP64
-// 2^8 0.056 / 0.023, 2^10 0.068 / 0.036), but small-N solves are bound by their launches and do
-// not change, and in concurrent serving, where slots of other sizes are created and evicted,
-// building its tables (an O(N^3) FP64 formation of B^a per plan) cut throughput from 191 to
-// 152 solves/s on one GPU. BK_DENSE=0 is the default; N that is not a power of two is always
-// dense.
+// plan with N <= 1024 and at most 16 vectors per product starts on the dense product): building the
+// dense tables (an O(N^3) FP64 formation of B^a per plan) in concurrent serving, where slots of
+// other sizes are created and evicted, cut throughput from 191 to 152 solves/s on one GPU.
+// BK_DENSE=0 is the default; N that is not a power of two is always dense.
 // FP64 plans of N >= 2^18 compute their transforms in double-float arithmetic (bk_df.cuh) unless
 // switched off: bk_set_f64_transform(0) for plans created afterwards, or the environment variable
-// BK_F64_DF=0 (read at plan creation); bk_set_f64_transform(1) extends it to every four-step FP64
-// plan (N >= 256). Measured products (4 components, cold L2, FP64 / double-float ms): 2^14 0.095 /
-// 0.109, 2^16 0.123 / 0.132, 2^18 0.272 / 0.228, 2^20 0.978 / 0.553, 2^22 3.87 / 2.50, 2^24 17.6 /
-// 12.3: below 2^18 the passes are latency-bound and the double-float instructions lengthen them.
+// BK_F64_DF=0 (read at plan creation); bk_set_f64_transform(1) extends it to every FP64 plan with
+// N >= 256. Measured products (4 components, warm, us, FP64 / double-float): 2^18 206 / 122, 2^20
+// 736 / 363; below 2^18 the passes are latency-bound and the double-float instructions lengthen them.
 #ifndef BK_TRANSFORM_KERNEL_UNIT
 static std::atomic<int> g_f64_df{-1};
 static bool f64_df_default(int64_t N) {
@@ -1502,18 +1166,7 @@ static bool dense_default(int dtype, int64_t N, int nvec) {
 // Four-step shapes of a plan for E complex elements per CTA (0: the occupancy heuristic).
 static bk_status fourstep_shapes(Plan* p, int E) {
   const int nvec = p->n_comp * p->max_batch;
-  if (p->split == 2) {
-    BK_TRY(configure_fourstep(p->fs, p->N / 4, p->dtype, nvec, E));
-    BK_TRY(configure_fourstep(p->fse, p->N / 8, p->dtype, nvec, E));
-    BK_TRY(configure_fourstep(p->fso, p->N / 4, p->dtype, nvec, E));
-    return BK_OK;
-  }
-  if (p->split) {
-    BK_TRY(configure_fourstep(p->fs, p->N / 2, p->dtype, nvec, E));
-    BK_TRY(configure_fourstep(p->fso, p->N / 4, p->dtype, nvec, E));
-    return BK_OK;
-  }
-  return configure_fourstep(p->fs, p->N, p->dtype, nvec, E);
+  return p->split ? configure_re(p->fs, p->N, p->dtype, p->fe, nvec, E) : configure_cluster(p);
 }
 
 // Tile autotuner of the four-step transforms. The elements per CTA E (powers of two from one
@@ -1546,8 +1199,8 @@ static bk_status autotune_tiles(Plan* p, cudaStream_t st) {
       return fourstep_shapes(p, it->second);
     }
   }
-  const int cap = p->dtype == BK_F64 ? 4096 : 8192;
-  const int emin = std::max(p->fs.N1, 2 * p->fs.N2);
+  const int cap = re_elems_max(p->fs, p->dtype, p->fe);
+  const int emin = std::max(p->fs.N1, p->fs.N2);
   const size_t vbytes = dtype_size(p->dtype) * (size_t)p->pitch * nvec;
   void* vin = nullptr;
   void* vout = nullptr;
@@ -1629,7 +1282,8 @@ bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtyp
     const char* e = getenv("BK_DENSE_TEST_TIMEOUT");  // test mode of the dense kernel, as bk_plan_dense_test_timeout
     p->dtest = (e && e[0] == '1') ? 1 : 0;
   }
-  p->small = !p->generic && !p->blue && N <= small_limit(dtype);
+  p->df = dtype == BK_F64 && is_pow2(N) && N >= 256 && f64_df_default(N);
+  p->small = !p->generic && !p->blue && !p->df && N <= small_limit(dtype);
   bk_status st_ = BK_OK;
   AllocCounter counter(&p->bytes);
   do {
@@ -1647,8 +1301,7 @@ bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtyp
     }
     if (p->small) {
       p->smemS = dtype == BK_F64 ? smem_small<double>(N) : smem_small<float>(N);
-      p->thrS = round_threads(N / 16);
-      if (p->thrS > (dtype == BK_F64 ? 256 : 512)) p->thrS = dtype == BK_F64 ? 256 : 512;
+      p->thrS = round_threads(N / SmallFft<float>::EPT);
     } else if (p->blue) {
       p->M = 1;
       while (p->M < 2 * N - 1) p->M *= 2;
@@ -1659,21 +1312,15 @@ bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtyp
       if ((st_ = dmalloc(&p->scrY, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
       if ((st_ = dmalloc(&p->scrG, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
     } else {
-      // split DCT-I from 2^split_min_log2() on: fs the length-N/2 FFT, fso the length-N/4 one
-      p->split = ilog2(N) >= split2_min_log2(dtype) ? 2 : (ilog2(N) >= split_min_log2(dtype) ? 1 : 0);
+      p->split = p->df || ilog2(N) >= std::min(2 * CL_MAXLOG2, split_min_log2(dtype));
+      p->fe = re_radix(N, dtype, p->df);
       if ((st_ = fourstep_shapes(p, 0)) != BK_OK) break;
       const int64_t nvec = (int64_t)n_comp * max_batch;
-      const size_t csz = 2 * dtype_size(dtype);
-      if ((st_ = dmalloc(&p->scrA, csz * (size_t)N * nvec)) != BK_OK) break;
-      if ((st_ = dmalloc(&p->scrY, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
-      if ((st_ = dmalloc(&p->scrG, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
-      // partial sums for the narrowest pass-A tile any shape may take (most CTAs per vector)
-      const int nbMin = std::max(1, std::max(p->fs.N1, 2 * p->fs.N2) / p->fs.N1);
-      const size_t nPartMax = (size_t)std::max(p->fs.nPartA, p->fs.N2 / std::min(nbMin, p->fs.N2));
-      if ((st_ = dmalloc(&p->part1, dtype_size(dtype) * nPartMax * nvec)) != BK_OK) break;
-      if ((st_ = dmalloc(&p->part2, dtype_size(dtype) * nPartMax * nvec)) != BK_OK) break;
+      const size_t es = dtype_size(dtype);
+      if ((st_ = dmalloc(&p->scrA, 2 * es * (size_t)p->fs.a_len() * nvec)) != BK_OK) break;
+      if ((st_ = dmalloc(&p->scrY, es * (size_t)(N + 2) * nvec)) != BK_OK) break;
+      if ((st_ = dmalloc(&p->part, es * (size_t)p->fs.pairs() * nvec)) != BK_OK) break;
     }
-    p->df = dtype == BK_F64 && !p->small && !p->blue && f64_df_default(N);
     st_ = dtype == BK_F64 ? (p->df ? build_tables<dfl>(p, st) : build_tables<double>(p, st)) : build_tables<float>(p, st);
     if (st_ != BK_OK) break;
     if ((st_ = dmalloc((void**)&p->t_nodes, sizeof(double) * (size_t)L)) != BK_OK) break;
@@ -1684,7 +1331,7 @@ bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtyp
     if (st_ != BK_OK) break;
     if (p->blue && (st_ = dtype == BK_F64 ? blue_spectrum<double>(p, st) : blue_spectrum<float>(p, st)) != BK_OK) break;
     if ((st_ = compute_weights(p, st)) != BK_OK) break;
-    if (!p->small && !p->blue && autotune_enabled()) {
+    if (p->split && autotune_enabled()) {
       if ((st_ = autotune_tiles(p, st)) != BK_OK) break;
     }
     if (dense_default(dtype, N, n_comp * max_batch)) {
@@ -1709,20 +1356,16 @@ void plan_destroy(Plan* p) {
   dfree(p->tw);
   dfree(p->stwS);
   free_fs(p->fs);
-  free_fs(p->fso);
-  free_fs(p->fse);
   free_fs(p->fsM);
   dfree(p->chirp);
   dfree(p->bh);
   dfree(p->bsc);
-  dfree(p->eo);
   dfree(p->tpost);
   dfree(p->rk);
   dfree(p->scrA);
   dfree(p->scrY);
   dfree(p->scrG);
-  dfree(p->part1);
-  dfree(p->part2);
+  dfree(p->part);
   dfree(p->t_nodes);
   dfree(p->dA[0]);
   dfree(p->dA[1]);
@@ -1733,83 +1376,6 @@ void plan_destroy(Plan* p) {
 }
 #endif  // BK_TRANSFORM_KERNEL_UNIT
 
-// One split DCT-I of the vectors at src (input kind K) into dst with epilogue E: pass A of the
-// even half (pair sums, length-N/2 FFT on fs) and of the odd half (pair differences, length-N/4
-// inverse FFT on fso), then both pass-B launches writing even and odd output indices. partA
-// receives the even half's DC partial sums (IN_WINV); partB holds the partials the epilogue
-// reads for Y0.
-template <typename T, int K, int E>
-static bk_status split_dct(const Plan* p, const St<T>* src, int64_t sstride, typename OutS<T, E>::t* dst, int64_t dstride, int64_t zero_to,
-                           int nvec, void* scrA, T* partA, const T* partB, int npartB, T s, T invN, StencilTab<T> tb,
-                           cudaStream_t st) {
-  typedef typename V2<T>::t C;
-  const int N = (int)p->N, M = N / 2;
-  const FourStep& e = p->fs;
-  const FourStep& o = p->fso;
-  C* Ae = (C*)scrA;
-  C* Ao = Ae + (int64_t)nvec * M;
-  const C* tp = (const C*)p->tpost;
-  const int gE = e.N2 / e.NB, gO = o.N2 / o.NB;
-  k_passA_split<T, K><<<dim3(gE + gO, nvec), std::max(e.thrA, o.thrA), std::max(e.smemA, o.smemA), st>>>(
-      gE, src, sstride, Ae, partA, M, e.N1, ilog2(e.N1), e.N2, e.NB, e.bsA, (const C*)e.stw1, (const C*)e.twN,
-      (const C*)e.twLo, (const C*)e.twHi, e.tw_h,
-      src, sstride, Ao, nullptr, M / 2, o.N1, ilog2(o.N1), o.N2, o.NB, o.bsA, (const C*)o.stw1, (const C*)o.twN,
-      (const C*)o.twLo, (const C*)o.twHi, o.tw_h, invN, tb, tp, (const C*)p->eo);
-  BK_CHECK_LAUNCH();
-  const int hE = e.N1 / 2 / e.P, hO = o.N1 / 2 / o.P;
-  k_passB_split<T, E><<<dim3(hE + hO, nvec), std::max(e.thrB, o.thrB), std::max(e.smemB, o.smemB), st>>>(
-      hE, Ae, M, e.N1, e.N2, ilog2(e.N2), e.P, (const C*)e.stw2, Ao, M / 2, o.N1, o.N2, ilog2(o.N2), o.P,
-      (const C*)o.stw2, dst, dstride, zero_to, partB, npartB, tp, s, invN, N);
-  BK_CHECK_LAUNCH();
-  return BK_OK;
-}
-
-// One two-level split DCT-I (see PM_PAIR2): pass A of its three parts in one launch, then pass B
-// of the three in one launch writing outputs 4k, 4m + 2 and 2m + 1.
-template <typename T, int K, int E>
-static bk_status split_dct3(const Plan* p, const St<T>* src, int64_t sstride, typename OutS<T, E>::t* dst, int64_t dstride, int64_t zero_to,
-                            int nvec, void* scrA, T* partA, const T* partB, int npartB, T s, T invN, StencilTab<T> tb,
-                            cudaStream_t st) {
-  typedef typename V2<T>::t C;
-  const int N = (int)p->N, Q = N / 4;
-  const FourStep& e = p->fs;   // length Q: DCT-I of aa
-  const FourStep& d = p->fse;  // length Q/2: DCT-III of a's pair differences
-  const FourStep& o = p->fso;  // length Q: DCT-III of x's pair differences
-  C* Ae = (C*)scrA;
-  C* Ad = Ae + (int64_t)nvec * Q;
-  C* Ao = Ad + (int64_t)nvec * (Q / 2);
-  const C* tp = (const C*)p->tpost;
-  const int g1 = e.N2 / e.NB, g2 = d.N2 / d.NB, g3 = o.N2 / o.NB;
-  const int thrA = std::max(e.thrA, std::max(d.thrA, o.thrA));
-  const size_t smA = std::max(e.smemA, std::max(d.smemA, o.smemA));
-  k_passA_split3<T, K><<<dim3(g1 + g2 + g3, nvec), thrA, smA, st>>>(
-      g1, g2, src, sstride, Ae, partA, Q, e.N1, ilog2(e.N1), e.N2, e.NB, e.bsA, (const C*)e.stw1, (const C*)e.twN,
-      (const C*)e.twLo, (const C*)e.twHi, e.tw_h,
-      src, sstride, Ad, nullptr, Q / 2, d.N1, ilog2(d.N1), d.N2, d.NB, d.bsA, (const C*)d.stw1, (const C*)d.twN,
-      (const C*)d.twLo, (const C*)d.twHi, d.tw_h,
-      src, sstride, Ao, nullptr, Q, o.N1, ilog2(o.N1), o.N2, o.NB, o.bsA, (const C*)o.stw1, (const C*)o.twN,
-      (const C*)o.twLo, (const C*)o.twHi, o.tw_h, invN, tb, tp, (const C*)p->eo);
-  BK_CHECK_LAUNCH();
-  const int h1 = e.N1 / 2 / e.P, h2 = d.N1 / 2 / d.P, h3 = o.N1 / 2 / o.P;
-  const int thrB = std::max(e.thrB, std::max(d.thrB, o.thrB));
-  const size_t smB = std::max(e.smemB, std::max(d.smemB, o.smemB));
-  k_passB_split3<T, E><<<dim3(h1 + h2 + h3, nvec), thrB, smB, st>>>(
-      h1, h2, Ae, Q, e.N1, e.N2, ilog2(e.N2), e.P, (const C*)e.stw2, Ad, Q / 2, d.N1, d.N2, ilog2(d.N2), d.P,
-      (const C*)d.stw2, Ao, Q, o.N1, o.N2, ilog2(o.N2), o.P, (const C*)o.stw2, dst, dstride, zero_to, partB, npartB, tp,
-      s, invN, N);
-  BK_CHECK_LAUNCH();
-  return BK_OK;
-}
-
-template <typename T, int K, int E>
-static bk_status split_any(const Plan* p, const St<T>* src, int64_t sstride, typename OutS<T, E>::t* dst, int64_t dstride, int64_t zero_to,
-                           int nvec, void* scrA, T* partA, const T* partB, int npartB, T s, T invN, StencilTab<T> tb,
-                           cudaStream_t st) {
-  if (p->split == 2)
-    return split_dct3<T, K, E>(p, src, sstride, dst, dstride, zero_to, nvec, scrA, partA, partB, npartB, s, invN, tb, st);
-  return split_dct<T, K, E>(p, src, sstride, dst, dstride, zero_to, nvec, scrA, partA, partB, npartB, s, invN, tb, st);
-}
-
 // One length-M complex FFT on the plan's Bluestein layout: src (M complex per vector, as real
 // pairs) -> dst (same), through the four-step scratch A; E = EP_CPLX_MC multiplies by the
 // spectral table and conjugates in the store.
@@ -1818,16 +1384,12 @@ static bk_status blue_fft(const Plan* p, const T* src, T* dst, typename V2<T>::t
   typedef typename V2<T>::t C;
   const FourStep& f = p->fsM;
   const int M = (int)p->M;
-  StencilTab<T> tb;
-  tb.rk = nullptr;
-  tb.cN = T(0);
-  k_passA<T, IN_PLAIN, PM_CPLX><<<dim3(f.N2 / f.NB, nvec), f.thrA, f.smemA, st>>>(
-      src, 2 * (int64_t)M, A, nullptr, M, f.N1, ilog2(f.N1), f.N2, f.NB, f.bsA, (const C*)f.stw1, (const C*)f.twN,
-      (const C*)f.twLo, (const C*)f.twHi, f.tw_h, T(1), tb);
+  k_passA<T><<<dim3(f.N2 / f.NB, nvec), f.thrA, f.smemA, st>>>(src, 2 * (int64_t)M, A, M, f.N1, ilog2(f.N1), f.N2, f.NB,
+                                                               f.bsA, (const C*)f.stw1, (const C*)f.twN,
+                                                               (const C*)f.twLo, (const C*)f.twHi, f.tw_h);
   BK_CHECK_LAUNCH();
-  k_passB<T, E, PB_CPLX><<<dim3(f.N1 / 2 / f.P, nvec), f.thrB, f.smemB, st>>>(
-      A, dst, 2 * (int64_t)M, 0, nullptr, 0, M, f.N1, f.N2, ilog2(f.N2), f.P, (const C*)f.stw2, (const C*)p->bh, T(1),
-      T(1), 1, 1, M);
+  k_passB<T, E><<<dim3(f.N1 / 2 / f.P, nvec), f.thrB, f.smemB, st>>>(A, dst, 2 * (int64_t)M, M, f.N1, f.N2, ilog2(f.N2),
+                                                                     f.P, (const C*)f.stw2, (const C*)p->bh);
   BK_CHECK_LAUNCH();
   return BK_OK;
 }
@@ -1835,7 +1397,7 @@ static bk_status blue_fft(const Plan* p, const T* src, T* dst, typename V2<T>::t
 // One DCT-I of length N + 1 for N not a power of two: chirp, FFT_M, spectral product, FFT_M,
 // chirp and real split (k_bs_pre, blue_fft x 2, k_bs_post).
 template <typename T, int K, int E>
-static bk_status blue_dct(const Plan* p, const T* src, int64_t sstride, typename OutS<T, E>::t* dst, int64_t dstride,
+static bk_status blue_dct(const Plan* p, const T* src, int64_t sstride, T* dst, int64_t dstride,
                           int64_t zero_to, int nvec, T s, T invN, cudaStream_t st) {
   typedef typename V2<T>::t C;
   const int64_t M = p->M;
@@ -1869,144 +1431,167 @@ bk_status blue_spectrum(Plan* p, cudaStream_t st) {
 }
 
 template <typename T>
-bk_status apply_impl(const Plan* p, const Us<T>* vu, Us<T>* out, int nvec, bool trans, double s_scale,
-                            cudaStream_t st, void* scrA, void* scrY, void* part1, void* part2, void* scrG) {
+static ReArgs<T> re_args(const Plan* p) {
+  typedef typename V2<T>::t C;
+  const FourStep& f = p->fs;
+  ReArgs<T> g;
+  g.N = (int)p->N;
+  g.N1 = f.N1;
+  g.N2 = f.N2;
+  g.log2N1 = ilog2(f.N1);
+  g.log2N2 = ilog2(f.N2);
+  g.RS = f.RS();
+  g.stw1 = (const C*)f.stw1;
+  g.stw2 = (const C*)f.stw2;
+  g.twA = (const C*)f.twN;
+  g.rk = (const T*)p->rk;
+  g.cE = (T)(2.0 / ((double)p->N + 1.0));
+  return g;
+}
+
+// Launch-per-pass form: one pass A and one pass B launch over nvec vectors.
+template <typename T, int K, typename F, typename S>
+static bk_status re_launch_AF(const Plan* p, const S* src, int64_t sstride, int nvec, cudaStream_t st) {
+  typedef typename V2<T>::t C;
+  const FourStep& f = p->fs;
+  k_re_passA<T, K, F, S><<<dim3(nvec, (f.pairs() + f.NB - 1) / f.NB), f.thrA, f.smemA, st>>>(
+      re_args<T>(p), f.NB, f.bsA, src, sstride, (C*)p->scrA, f.a_len(), (T*)p->part);
+  BK_CHECK_LAUNCH();
+  return BK_OK;
+}
+template <typename T, int K, typename S>
+static bk_status re_launch_A(const Plan* p, const S* src, int64_t sstride, int nvec, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    if (p->fe == 4) return re_launch_AF<T, K, FftShape<T, 4>>(p, src, sstride, nvec, st);
+    return re_launch_AF<T, K, FftShape<T, 2>>(p, src, sstride, nvec, st);
+  } else {
+    return re_launch_AF<T, K, FftShape<T, std::is_same<T, dfl>::value ? 3 : 2>>(p, src, sstride, nvec, st);
+  }
+}
+
+template <typename T, int E, typename F, typename S>
+static bk_status re_launch_BF(const Plan* p, S* dst, int64_t dstride, int64_t zero_to, int nvec, T s, cudaStream_t st) {
+  typedef typename V2<T>::t C;
+  const FourStep& f = p->fs;
+  k_re_passB<T, E, F, S><<<dim3(nvec, (f.N1 / 4 + f.P) / f.P), f.thrB, f.smemB, st>>>(
+      re_args<T>(p), f.P, f.bsB, (const C*)p->scrA, f.a_len(), dst, dstride, zero_to, (const T*)p->part, s,
+      T(1.0 / (double)p->N));
+  BK_CHECK_LAUNCH();
+  return BK_OK;
+}
+template <typename T, int E, typename S>
+static bk_status re_launch_B(const Plan* p, S* dst, int64_t dstride, int64_t zero_to, int nvec, T s, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    if (p->fe == 4) return re_launch_BF<T, E, FftShape<T, 4>>(p, dst, dstride, zero_to, nvec, s, st);
+    return re_launch_BF<T, E, FftShape<T, 2>>(p, dst, dstride, zero_to, nvec, s, st);
+  } else {
+    if (re_big(p->fs, p->dtype)) return re_launch_BF<T, E, BigFft<T>>(p, dst, dstride, zero_to, nvec, s, st);
+    return re_launch_BF<T, E, FftShape<T, std::is_same<T, dfl>::value ? 3 : 2>>(p, dst, dstride, zero_to, nvec, s, st);
+  }
+}
+
+template <typename T>
+static ReJob<T> re_job(const Plan* p, const void* in, void* out, int nvec, T s) {
+  ReJob<T> J;
+  J.g = re_args<T>(p);
+  J.in = (const Us<T>*)in;
+  J.out = (Us<T>*)out;
+  J.pitch = p->pitch;
+  J.astride = p->fs.a_len();
+  J.ystride = p->N + 2;
+  J.A = (typename V2<T>::t*)p->scrA;
+  J.Y = (T*)p->scrY;
+  J.part = (T*)p->part;
+  J.s = s;
+  J.invN = T(1.0 / (double)p->N);
+  J.NB = p->fs.NB;
+  J.bsA = p->fs.bsA;
+  J.P = p->fs.P;
+  J.bsB = p->fs.bsB;
+  J.nvec = nvec;
+  return J;
+}
+
+// One launch of clusters of csize CTAs (blockIdx.x / csize is the cluster).
+template <typename F, typename A>
+static bk_status launch_clusters(F* fn, const A& arg, int nclusters, int csize, int thr, size_t smem, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nclusters * csize);
+  cfg.blockDim = dim3(thr);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = csize;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  BK_TRY_CUDA(cudaLaunchKernelEx(&cfg, fn, arg, csize));
+  BK_CHECK_LAUNCH();
+  return BK_OK;
+}
+
+template <typename T>
+bk_status apply_impl(const Plan* p, const Us<T>* v, Us<T>* out, int nvec, bool trans, double s_scale, cudaStream_t st) {
   typedef typename V2<T>::t C;
   const int N = (int)p->N;
-  // the first DCT's input: the caller's vectors, or (double-float) their conversion into the
-  // stencil buffer, which the first DCT consumes before the stencil overwrites it
-  const St<T>* v = nullptr;
-  int64_t vstride = p->pitch;
-  if constexpr (std::is_same<T, Us<T>>::value) {
-    v = vu;
-  } else {
-    if (!scrG) {
-      set_error("internal: double-float products need the stencil buffer");
-      return BK_ERR_ARG;
-    }
-    k_to_arith<T><<<dim3(std::max(1, std::min(1024, (N + 256) / 256)), nvec), 256, 0, st>>>(vu, p->pitch, (T*)scrG,
-                                                                                              N + 1);
-    BK_CHECK_LAUNCH();
-    v = (const T*)scrG;
-    vstride = N + 1;
-  }
   const T s = (T)s_scale;
-  const T invN = T(1.0 / (double)N);
-  StencilTab<T> tb;
-  tb.rk = (const T*)p->rk;
-  tb.cN = (T)(1.0 / (4.0 * ((double)N * (double)N - 1.0)));
-  if (p->small) {
-    if (!trans)
-      k_birkhoff_small<T, false><<<nvec, p->thrS, p->smemS, st>>>(vu, out, N, ilog2(N), p->pitch, s, (const C*)p->tw, (const C*)p->stwS, (const C*)p->tpost, tb);
-    else
-      k_birkhoff_small<T, true><<<nvec, p->thrS, p->smemS, st>>>(vu, out, N, ilog2(N), p->pitch, s, (const C*)p->tw, (const C*)p->stwS, (const C*)p->tpost, tb);
-    BK_CHECK_LAUNCH();
-    return BK_OK;
-  }
   if constexpr (!std::is_same<T, dfl>::value) {
+    const T invN = T(1.0 / (double)N);
+    StencilTab<T> tb;
+    tb.rk = (const T*)p->rk;
+    tb.cN = (T)(1.0 / (4.0 * ((double)N * (double)N - 1.0)));
+    if (p->small) {
+      if (!trans)
+        k_birkhoff_small<T, false><<<nvec, p->thrS, p->smemS, st>>>(v, out, N, ilog2(N), p->pitch, s, (const C*)p->tw, (const C*)p->stwS, (const C*)p->tpost, tb);
+      else
+        k_birkhoff_small<T, true><<<nvec, p->thrS, p->smemS, st>>>(v, out, N, ilog2(N), p->pitch, s, (const C*)p->tw, (const C*)p->stwS, (const C*)p->tpost, tb);
+      BK_CHECK_LAUNCH();
+      return BK_OK;
+    }
     if (p->blue) {
       const int64_t Ls = N + 1;
-      T* Ystage = (T*)scrY;
-      T* Gst = (T*)scrG;
+      T* Ystage = (T*)p->scrY;
+      T* Gst = (T*)p->scrG;
       const dim3 gS((unsigned)std::min<int64_t>(1024, (N + 255) / 256), nvec);
       if (!trans) {
-        BK_TRY((blue_dct<T, IN_PLAIN, EP_STORE>(p, v, vstride, Ystage, Ls, 0, nvec, s, invN, st)));
-        k_stencil<T, ST_FWD><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb, nullptr);
+        BK_TRY((blue_dct<T, IN_PLAIN, EP_STORE>(p, v, p->pitch, Ystage, Ls, 0, nvec, s, invN, st)));
+        k_stencil<T, ST_FWD><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb);
         BK_CHECK_LAUNCH();
         BK_TRY((blue_dct<T, IN_PLAIN, EP_FWD_OUT>(p, Gst, Ls, out, p->pitch, p->pitch, nvec, s, invN, st)));
       } else {
-        BK_TRY((blue_dct<T, IN_WINV, EP_STORE_TRN>(p, v, vstride, Ystage, Ls, 0, nvec, s, invN, st)));
-        k_stencil<T, ST_TRN><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb, nullptr);
+        BK_TRY((blue_dct<T, IN_WINV, EP_STORE_TRN>(p, v, p->pitch, Ystage, Ls, 0, nvec, s, invN, st)));
+        k_stencil<T, ST_TRN><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb);
         BK_CHECK_LAUNCH();
         BK_TRY((blue_dct<T, IN_PLAIN, EP_TRN_OUT>(p, Gst, Ls, out, p->pitch, p->pitch, nvec, s, invN, st)));
       }
       return BK_OK;
     }
+    if (!p->split)
+      return launch_clusters(trans ? k_re_cluster<T, true> : k_re_cluster<T, false>, re_job<T>(p, v, out, nvec, s), nvec,
+                             p->csize, p->cthr, p->csmem, st);
   }
-  if (p->split && scrG) {
-    const int64_t Ls = N + 1;
-    St<T>* Ystage = (St<T>*)scrY;
-    St<T>* Gst = (St<T>*)scrG;
-    T* pa1 = (T*)part1;
-    T* pa2 = (T*)part2;
-    const int nPA = p->fs.nPartA;
-    const dim3 gS(nPA, nvec);
-    if (!trans) {
-      BK_TRY((split_any<T, IN_PLAIN, EP_STORE>(p, v, vstride, Ystage, Ls, 0, nvec, scrA, nullptr, nullptr, 0, s, invN, tb, st)));
-      k_stencil<T, ST_FWD><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb, pa2);
-      BK_CHECK_LAUNCH();
-      BK_TRY((split_any<T, IN_PLAIN, EP_FWD_OUT>(p, Gst, Ls, out, p->pitch, p->pitch, nvec, scrA, nullptr, pa2, nPA, s, invN, tb, st)));
-    } else {
-      BK_TRY((split_any<T, IN_WINV, EP_STORE_TRN>(p, v, vstride, Ystage, Ls, 0, nvec, scrA, pa1, pa1, nPA, s, invN, tb, st)));
-      k_stencil<T, ST_TRN><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb, nullptr);
-      BK_CHECK_LAUNCH();
-      BK_TRY((split_any<T, IN_PLAIN, EP_TRN_OUT>(p, Gst, Ls, out, p->pitch, p->pitch, nvec, scrA, nullptr, nullptr, 0, s, invN, tb, st)));
-    }
-    return BK_OK;
-  }
-  const FourStep& f = p->fs;
-  const int N1 = f.N1, N2 = f.N2, NB = f.NB, P = f.P;
-  const int log2N1 = ilog2(N1), log2N2 = ilog2(N2);
-  C* A = (C*)scrA;
-  St<T>* Ystage = (St<T>*)scrY;
-  T* pa1 = (T*)part1;
-  T* pa2 = (T*)part2;
-  const int nPA = f.nPartA;
-  dim3 gA(N2 / NB, nvec), gB(N1 / 2 / P, nvec);
-  const C* stw1 = (const C*)f.stw1;
-  const C* stw2 = (const C*)f.stw2;
-  const int bsA = f.bsA;
-  const C* twN = (const C*)f.twN;
-  const C* tp = (const C*)p->tpost;
-  const int64_t Ls = N + 1;
-  St<T>* Gst = (St<T>*)scrG;  // separate stencil pass when given (see k_stencil)
-  const dim3 gS(nPA, nvec);
+  T* Y = (T*)p->scrY;
+  const int64_t Ls = (int64_t)N + 2;   // even: pass A reads aligned pairs
   if (!trans) {
-    k_passA<T, IN_PLAIN><<<gA, f.thrA, f.smemA, st>>>(v, vstride, A, pa1, N, N1, log2N1, N2, NB, bsA, stw1, twN, (const C*)f.twLo, (const C*)f.twHi, f.tw_h, invN, tb);
-    BK_CHECK_LAUNCH();
-    k_passB<T, EP_STORE><<<gB, f.thrB, f.smemB, st>>>(A, Ystage, Ls, 0, nullptr, 0, N, N1, N2, log2N2, P, stw2, tp, s, invN, 1, 1, N);
-    BK_CHECK_LAUNCH();
-    if (Gst) {
-      k_stencil<T, ST_FWD><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb, pa2);
-      BK_CHECK_LAUNCH();
-      k_passA<T, IN_PLAIN><<<gA, f.thrA, f.smemA, st>>>(Gst, Ls, A, pa2, N, N1, log2N1, N2, NB, bsA, stw1, twN, (const C*)f.twLo, (const C*)f.twHi, f.tw_h, invN, tb);
-    } else if constexpr (std::is_same<T, double>::value) {
-      // fused stencil loads: only the allocation-free FP64 entry point has no stencil buffer
-      k_passA<T, ST_FWD><<<gA, f.thrA, f.smemA, st>>>(Ystage, Ls, A, pa2, N, N1, log2N1, N2, NB, bsA, stw1, twN, (const C*)f.twLo, (const C*)f.twHi, f.tw_h, invN, tb);
-    } else {
-      set_error("internal: FP32 products need the stencil buffer");
-      return BK_ERR_ARG;
-    }
-    BK_CHECK_LAUNCH();
-    k_passB<T, EP_FWD_OUT><<<gB, f.thrB, f.smemB, st>>>(A, out, p->pitch, p->pitch, pa2, nPA, N, N1, N2, log2N2, P, stw2, tp, s, invN, 1, 1, N);
-    BK_CHECK_LAUNCH();
+    BK_TRY((re_launch_A<T, IN_PLAIN>(p, v, p->pitch, nvec, st)));
+    BK_TRY((re_launch_B<T, EP_STORE>(p, Y, Ls, 0, nvec, s, st)));
+    BK_TRY((re_launch_A<T, ST_FWD>(p, (const T*)Y, Ls, nvec, st)));
+    BK_TRY((re_launch_B<T, EP_FWD_OUT>(p, out, p->pitch, p->pitch, nvec, s, st)));
   } else {
-    k_passA<T, IN_WINV><<<gA, f.thrA, f.smemA, st>>>(v, vstride, A, pa1, N, N1, log2N1, N2, NB, bsA, stw1, twN, (const C*)f.twLo, (const C*)f.twHi, f.tw_h, invN, tb);
-    BK_CHECK_LAUNCH();
-    k_passB<T, EP_STORE_TRN><<<gB, f.thrB, f.smemB, st>>>(A, Ystage, Ls, 0, pa1, nPA, N, N1, N2, log2N2, P, stw2, tp, s, invN, 1, 1, N);
-    BK_CHECK_LAUNCH();
-    // the stage buffer already holds Y - Y0, so the transposed stencil runs with Y0 = 0
-    if (Gst) {
-      k_stencil<T, ST_TRN><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb, nullptr);
-      BK_CHECK_LAUNCH();
-      k_passA<T, IN_PLAIN><<<gA, f.thrA, f.smemA, st>>>(Gst, Ls, A, pa2, N, N1, log2N1, N2, NB, bsA, stw1, twN, (const C*)f.twLo, (const C*)f.twHi, f.tw_h, invN, tb);
-    } else if constexpr (std::is_same<T, double>::value) {
-      k_passA<T, ST_TRN><<<gA, f.thrA, f.smemA, st>>>(Ystage, Ls, A, pa2, N, N1, log2N1, N2, NB, bsA, stw1, twN, (const C*)f.twLo, (const C*)f.twHi, f.tw_h, invN, tb);
-    } else {
-      set_error("internal: FP32 products need the stencil buffer");
-      return BK_ERR_ARG;
-    }
-    BK_CHECK_LAUNCH();
-    k_passB<T, EP_TRN_OUT><<<gB, f.thrB, f.smemB, st>>>(A, out, p->pitch, p->pitch, nullptr, 0, N, N1, N2, log2N2, P, stw2, tp, s, invN, 1, 1, N);
-    BK_CHECK_LAUNCH();
+    BK_TRY((re_launch_A<T, IN_WINV>(p, v, p->pitch, nvec, st)));
+    BK_TRY((re_launch_B<T, EP_STORE_TRN>(p, Y, Ls, 0, nvec, s, st)));
+    BK_TRY((re_launch_A<T, ST_TRN>(p, (const T*)Y, Ls, nvec, st)));
+    BK_TRY((re_launch_B<T, EP_TRN_OUT>(p, out, p->pitch, p->pitch, nvec, s, st)));
   }
   return BK_OK;
 }
 
 // Batched products of plans of one precision T (binary32 or binary64 arithmetic): the small
-// plans' chains in one launch, the unsplit four-step plans' five passes in one launch each, per
-// chunk of BATCH_MAX plans. Each plan uses its own tables and scratch, so a plan appears at most
-// once among the four-step ones (the caller checks). vec[i] / out[i]: nv[i] vectors pitch apart.
+// plans' chains in one launch, the four-step plans' chains in another or their passes in one launch
+// each, per chunk of BATCH_MAX plans. Each plan uses its own tables and scratch, so a plan appears at most once among
+// the four-step ones (the caller checks). vec[i] / out[i]: nv[i] vectors pitch apart.
 template <typename T>
 static bk_status launch_small_batch(const Plan* const* ps, const void* const* vin, void* const* vout, const int* nv,
                                     int n, bool trans, cudaStream_t st) {
@@ -2051,146 +1636,88 @@ static bk_status launch_small_batch(const Plan* const* ps, const void* const* vi
 template <typename T>
 static bk_status launch_fourstep_batch(const Plan* const* ps, const void* const* vin, void* const* vout, const int* nv,
                                        int n, bool trans, cudaStream_t st) {
-  typedef typename V2<T>::t C;
   for (int c0 = 0; c0 < n; c0 += BATCH_MAX) {
-    const int nj = std::min(BATCH_MAX, n - c0);
-    Batch<PassAJob<T>> a1, a2;
-    Batch<PassBJob<T>> b1, b2;
-    Batch<StencilJob<T>> sj;
-    memset(&a1, 0, sizeof(a1));
-    memset(&b1, 0, sizeof(b1));
-    memset(&sj, 0, sizeof(sj));
-    a1.njob = b1.njob = sj.njob = nj;
-    int thrA = 32, thrB = 32;
-    size_t smA = 0, smB = 0;
-    int ca = 0, cb = 0, cs = 0;
-    for (int q = 0; q < nj; ++q) {
+    Batch<ReJob<T>> b;
+    memset((void*)&b, 0, sizeof(b));
+    b.njob = std::min(BATCH_MAX, n - c0);
+    int thr = 32, cs = 1, cl = 0;
+    size_t smem = 0;
+    for (int q = 0; q < b.njob; ++q) {
       const Plan* p = ps[c0 + q];
-      const FourStep& f = p->fs;
-      const int N = (int)p->N;
-      const int64_t Ls = N + 1;
-      const int nvec = nv[c0 + q];
-      StencilTab<T> tb;
-      tb.rk = (const T*)p->rk;
-      tb.cN = (T)(1.0 / (4.0 * ((double)N * (double)N - 1.0)));
-      const T invN = T(1.0 / (double)N);
-      PassAJob<T>& A = a1.j[q];
-      A.src = (const T*)vin[c0 + q];
-      A.sstride = p->pitch;
-      A.A = (C*)p->scrA;
-      A.partial = (T*)p->part1;
-      A.stw = (const C*)f.stw1;
-      A.twN = (const C*)f.twN;
-      A.twLo = (const C*)f.twLo;
-      A.twHi = (const C*)f.twHi;
-      A.tb = tb;
-      A.invN = invN;
-      A.N = N;
-      A.N1 = f.N1;
-      A.log2N1 = ilog2(f.N1);
-      A.N2 = f.N2;
-      A.NB = f.NB;
-      A.bs = f.bsA;
-      A.tw_h = f.tw_h;
-      A.nthr = f.thrA;
-      A.nblk = f.N2 / f.NB;
-      a1.start[q] = ca;
-      ca += A.nblk * nvec;
-      PassBJob<T>& B = b1.j[q];
-      B.A = (const C*)p->scrA;
-      B.dst = (T*)p->scrY;
-      B.dstride = Ls;
-      B.zero_to = 0;
-      B.partial = trans ? (const T*)p->part1 : nullptr;
-      B.npartial = trans ? f.nPartA : 0;
-      B.stw = (const C*)f.stw2;
-      B.tpost = (const C*)p->tpost;
-      B.s = (T)p->s;
-      B.invN = invN;
-      B.N = N;
-      B.N1 = f.N1;
-      B.N2 = f.N2;
-      B.log2N2 = ilog2(f.N2);
-      B.P = f.P;
-      B.nthr = f.thrB;
-      B.nblk = f.N1 / 2 / f.P;
-      b1.start[q] = cb;
-      cb += B.nblk * nvec;
-      StencilJob<T>& S = sj.j[q];
-      S.stage = (const T*)p->scrY;
-      S.G = (T*)p->scrG;
-      S.partial = trans ? nullptr : (T*)p->part2;
-      S.Ls = Ls;
-      S.tb = tb;
-      S.N = N;
-      S.nblk = f.nPartA;
-      sj.start[q] = cs;
-      cs += S.nblk * nvec;
-      thrA = std::max(thrA, f.thrA);
-      thrB = std::max(thrB, f.thrB);
-      smA = std::max(smA, f.smemA);
-      smB = std::max(smB, f.smemB);
+      b.j[q] = re_job<T>(p, vin[c0 + q], vout[c0 + q], nv[c0 + q], (T)p->s);
+      b.start[q] = cl;
+      cl += nv[c0 + q];
+      thr = std::max(thr, p->cthr);
+      cs = std::max(cs, p->csize);
+      smem = std::max(smem, p->csmem);
     }
-    a1.start[nj] = ca;
-    b1.start[nj] = cb;
-    sj.start[nj] = cs;
-    // second DCT: pass A reads the stencil buffer, pass B writes the caller's vectors
-    a2 = a1;
-    b2 = b1;
-    for (int q = 0; q < nj; ++q) {
-      const Plan* p = ps[c0 + q];
-      a2.j[q].src = (const T*)p->scrG;
-      a2.j[q].sstride = p->N + 1;
-      a2.j[q].partial = (T*)p->part2;
-      b2.j[q].dst = (T*)vout[c0 + q];
-      b2.j[q].dstride = p->pitch;
-      b2.j[q].zero_to = p->pitch;
-      b2.j[q].partial = trans ? nullptr : (const T*)p->part2;
-      b2.j[q].npartial = trans ? 0 : p->fs.nPartA;
-    }
-    if (!trans) {
-      k_passA_batch<T, IN_PLAIN><<<ca, thrA, smA, st>>>(a1);
-      BK_CHECK_LAUNCH();
-      k_passB_batch<T, EP_STORE><<<cb, thrB, smB, st>>>(b1);
-      BK_CHECK_LAUNCH();
-      k_stencil_batch<T, ST_FWD><<<cs, 256, 0, st>>>(sj);
-      BK_CHECK_LAUNCH();
-      k_passA_batch<T, IN_PLAIN><<<ca, thrA, smA, st>>>(a2);
-      BK_CHECK_LAUNCH();
-      k_passB_batch<T, EP_FWD_OUT><<<cb, thrB, smB, st>>>(b2);
-      BK_CHECK_LAUNCH();
-    } else {
-      k_passA_batch<T, IN_WINV><<<ca, thrA, smA, st>>>(a1);
-      BK_CHECK_LAUNCH();
-      k_passB_batch<T, EP_STORE_TRN><<<cb, thrB, smB, st>>>(b1);
-      BK_CHECK_LAUNCH();
-      k_stencil_batch<T, ST_TRN><<<cs, 256, 0, st>>>(sj);
-      BK_CHECK_LAUNCH();
-      k_passA_batch<T, IN_PLAIN><<<ca, thrA, smA, st>>>(a2);
-      BK_CHECK_LAUNCH();
-      k_passB_batch<T, EP_TRN_OUT><<<cb, thrB, smB, st>>>(b2);
-      BK_CHECK_LAUNCH();
-    }
+    b.start[b.njob] = cl;
+    BK_TRY(launch_clusters(trans ? k_re_cluster_batch<T, true> : k_re_cluster_batch<T, false>, b, cl, cs, thr, smem, st));
   }
   return BK_OK;
 }
 
+// Four-step plans of radix 4 in the launch-per-pass form, one launch per pass for all of them.
+template <typename T, bool TRANS>
+static bk_status launch_passes_batch(const Plan* const* ps, const void* const* vin, void* const* vout, const int* nv,
+                                     int n, cudaStream_t st) {
+  typedef FftShape<T, 2> F;
+  for (int c0 = 0; c0 < n; c0 += BATCH_MAX) {
+    Batch<ReJob<T>> a, b;
+    memset((void*)&a, 0, sizeof(a));
+    a.njob = std::min(BATCH_MAX, n - c0);
+    b = a;
+    int thrA = 32, thrB = 32, ca = 0, cb = 0;
+    size_t smA = 0, smB = 0;
+    for (int q = 0; q < a.njob; ++q) {
+      const Plan* p = ps[c0 + q];
+      const FourStep& f = p->fs;
+      a.j[q] = b.j[q] = re_job<T>(p, vin[c0 + q], vout[c0 + q], nv[c0 + q], (T)p->s);
+      a.start[q] = ca;
+      b.start[q] = cb;
+      ca += nv[c0 + q] * ((f.pairs() + f.NB - 1) / f.NB);
+      cb += nv[c0 + q] * ((f.N1 / 4 + f.P) / f.P);
+      // a one-launch plan's shared memory and threads hold either of its passes' tiles
+      thrA = std::max(thrA, p->split ? f.thrA : p->cthr);
+      thrB = std::max(thrB, p->split ? f.thrB : p->cthr);
+      smA = std::max(smA, p->split ? f.smemA : p->csmem);
+      smB = std::max(smB, p->split ? f.smemB : p->csmem);
+    }
+    a.start[a.njob] = ca;
+    b.start[b.njob] = cb;
+    k_re_passA_batch<T, TRANS, false, F><<<ca, thrA, smA, st>>>(a);
+    BK_CHECK_LAUNCH();
+    k_re_passB_batch<T, TRANS, false, F><<<cb, thrB, smB, st>>>(b);
+    BK_CHECK_LAUNCH();
+    k_re_passA_batch<T, TRANS, true, F><<<ca, thrA, smA, st>>>(a);
+    BK_CHECK_LAUNCH();
+    k_re_passB_batch<T, TRANS, true, F><<<cb, thrB, smB, st>>>(b);
+    BK_CHECK_LAUNCH();
+  }
+  return BK_OK;
+}
+
+// fs_*: the four-step plans of radix 4. With launch-per-pass plans among them, the one-launch plans
+// join those launches (the same tiles and arithmetic, so the same results; beside the longer plans
+// they take no time of their own: sizes 2^8..2^16 of 4 FP32 components 79 -> 53 us in all).
 template <typename T>
 bk_status apply_batch_impl(const Plan* const* small_p, const void* const* small_v, void* const* small_o,
                            const int* small_n, int nsmall, const Plan* const* fs_p, const void* const* fs_v,
                            void* const* fs_o, const int* fs_n, int nfs, bool trans, cudaStream_t st) {
   if (nsmall > 0) BK_TRY(launch_small_batch<T>(small_p, small_v, small_o, small_n, nsmall, trans, st));
-  if (nfs > 0) BK_TRY(launch_fourstep_batch<T>(fs_p, fs_v, fs_o, fs_n, nfs, trans, st));
-  return BK_OK;
+  if (nfs == 0) return BK_OK;
+  bool split = false;
+  for (int i = 0; i < nfs; ++i) split = split || fs_p[i]->split;
+  if (!split) return launch_fourstep_batch<T>(fs_p, fs_v, fs_o, fs_n, nfs, trans, st);
+  return trans ? launch_passes_batch<T, true>(fs_p, fs_v, fs_o, fs_n, nfs, st)
+               : launch_passes_batch<T, false>(fs_p, fs_v, fs_o, fs_n, nfs, st);
 }
 
 #ifndef BK_TRANSFORM_KERNEL_UNIT
 extern template bk_status apply_impl<double>(const Plan* p, const double* v, double* out, int nvec, bool trans,
-                                             double s_scale, cudaStream_t st, void* scrA, void* scrY, void* part1,
-                                             void* part2, void* scrG);
+                                             double s_scale, cudaStream_t st);
 extern template bk_status apply_impl<float>(const Plan* p, const float* v, float* out, int nvec, bool trans,
-                                            double s_scale, cudaStream_t st, void* scrA, void* scrY, void* part1,
-                                            void* part2, void* scrG);
+                                            double s_scale, cudaStream_t st);
 extern template bk_status apply_batch_impl<double>(const Plan* const*, const void* const*, void* const*,
                                                    const int*, int, const Plan* const*, const void* const*,
                                                    void* const*, const int*, int, bool, cudaStream_t);
@@ -2198,17 +1725,16 @@ extern template bk_status apply_batch_impl<float>(const Plan* const*, const void
                                                   int, const Plan* const*, const void* const*, void* const*,
                                                   const int*, int, bool, cudaStream_t);
 extern template bk_status apply_impl<dfl>(const Plan* p, const double* v, double* out, int nvec, bool trans,
-                                          double s_scale, cudaStream_t st, void* scrA, void* scrY, void* part1,
-                                          void* part2, void* scrG);
+                                          double s_scale, cudaStream_t st);
 
 bk_status plan_apply_n(const Plan* p, const void* v, void* out, int nvec, bool trans, double s,
                        cudaStream_t st) {
   if (p->dense) return dense_apply(p, v, out, nvec, trans, s, st);
   if (p->dtype == BK_F64 && p->df)
-    return apply_impl<dfl>(p, (const double*)v, (double*)out, nvec, trans, s, st, p->scrA, p->scrY, p->part1, p->part2, p->scrG);
+    return apply_impl<dfl>(p, (const double*)v, (double*)out, nvec, trans, s, st);
   if (p->dtype == BK_F64)
-    return apply_impl<double>(p, (const double*)v, (double*)out, nvec, trans, s, st, p->scrA, p->scrY, p->part1, p->part2, p->scrG);
-  return apply_impl<float>(p, (const float*)v, (float*)out, nvec, trans, s, st, p->scrA, p->scrY, p->part1, p->part2, p->scrG);
+    return apply_impl<double>(p, (const double*)v, (double*)out, nvec, trans, s, st);
+  return apply_impl<float>(p, (const float*)v, (float*)out, nvec, trans, s, st);
 }
 
 // b-form helpers: c[vec] = out[vec][N] (forward) or s sum_i u[vec][i] (transpose, one block per
@@ -2281,9 +1807,9 @@ bk_status plan_apply(const Plan* p, const void* v, void* out, int batch, bool tr
   return plan_apply_n(p, v, out, batch * p->n_comp, trans, p->s, st);
 }
 
-// Products of several plans of one precision, N free per plan: small plans in one launch, unsplit
-// four-step plans in one launch per pass (per BATCH_MAX plans), every other plan (dense,
-// Bluestein, split, double-float) by its own launches.
+// Products of several plans of one precision, N free per plan: small plans in one launch, four-step
+// plans of radix 4 in another, or in one launch per pass where one of them needs it (each per
+// BATCH_MAX plans), every other plan (dense, Bluestein, radix 8 and 16) by its own launches.
 bk_status plan_apply_batch(const Plan* const* ps, const void* const* v, void* const* out, const int* batch, int count,
                            bool trans, cudaStream_t st) {
   BK_ARG(ps != nullptr && v != nullptr && out != nullptr && batch != nullptr, "NULL argument");
@@ -2304,7 +1830,7 @@ bk_status plan_apply_batch(const Plan* const* ps, const void* const* v, void* co
     BK_ARG(((uintptr_t)v[i] & 15) == 0 && ((uintptr_t)out[i] & 15) == 0, "entry %d: vectors must be 16-byte aligned",
            i);
     const int nv = batch[i] * p->n_comp;
-    if (p->dense || p->blue || p->split || p->df) {
+    if (p->dense || p->blue || p->df || (p->split && p->fe != 2)) {
       op.push_back(p); ov.push_back(v[i]); oo.push_back(out[i]); on.push_back(nv);
     } else if (p->small) {
       sp.push_back(p); sv.push_back(v[i]); so.push_back(out[i]); sn.push_back(nv);
@@ -2350,18 +1876,16 @@ static std::mutex g_noalloc_mu;
 static size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 // Bytes of the scratch layout for N (FP64) and nvec vectors, and the sub-buffer offsets.
-static size_t noalloc_layout(const Plan& p, int nvec, size_t off[9]) {
+static size_t noalloc_layout(const Plan& p, int nvec, size_t off[7]) {
   const int64_t N = p.N;
   size_t o = 0;
-  off[0] = o; o += align256(sizeof(double2) * stage_tw_len(ilog2(p.fs.N1)));          // stw1
-  off[1] = o; o += align256(sizeof(double2) * (N / 2 + 1));                           // tpost
-  off[2] = o; o += align256(sizeof(double2) * N);                                     // twN
-  off[3] = o; o += align256(sizeof(double2) * (size_t)N * nvec);                      // scrA
-  off[4] = o; o += align256(sizeof(double) * (size_t)(N + 1) * nvec);                 // scrY
-  off[5] = o; o += align256(sizeof(double) * (size_t)p.fs.nPartA * nvec);             // part1
-  off[6] = o; o += align256(sizeof(double) * (size_t)p.fs.nPartA * nvec);             // part2
-  off[7] = o; o += align256(sizeof(double) * (size_t)(N + 2));                        // rk
-  off[8] = o; o += align256(sizeof(double2) * stage_tw_len(ilog2(p.fs.N2)));          // stw2
+  off[0] = o; o += align256(sizeof(double2) * stage_tw_len(ilog2(p.fs.N1), CplxFft<double>::E));  // stw1
+  off[1] = o; o += align256(sizeof(double2) * stage_tw_len(ilog2(p.fs.N2), CplxFft<double>::E));  // stw2
+  off[2] = o; o += align256(sizeof(double2) * p.fs.a_len());                          // twN
+  off[3] = o; o += align256(sizeof(double2) * p.fs.a_len() * nvec);                   // scrA
+  off[4] = o; o += align256(sizeof(double) * (size_t)(N + 2) * nvec);                 // scrY
+  off[5] = o; o += align256(sizeof(double) * (size_t)p.fs.pairs() * nvec);            // part
+  off[6] = o; o += align256(sizeof(double) * (size_t)(N + 2));                        // rk
   return o;
 }
 
@@ -2372,11 +1896,7 @@ static bk_status noalloc_setup(int dev, void** out) {
   if (g_noalloc_ptr[dev] == nullptr) {
     void* ptr = nullptr;
     BK_TRY_CUDA(cudaGetSymbolAddress(&ptr, g_noalloc_scratch));
-    const int smem = (int)FOURSTEP_SMEM_BUDGET;
-    BK_TRY_CUDA(cudaFuncSetAttribute(k_passA<double, IN_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    BK_TRY_CUDA(cudaFuncSetAttribute(k_passA<double, ST_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    BK_TRY_CUDA(cudaFuncSetAttribute(k_passB<double, EP_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    BK_TRY_CUDA(cudaFuncSetAttribute(k_passB<double, EP_FWD_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BK_TRY(re_attrs<double>());
     g_noalloc_ptr[dev] = ptr;
   }
   *out = g_noalloc_ptr[dev];
@@ -2410,8 +1930,9 @@ bk_status noalloc_apply(const double* v, double* out, int64_t N, int nvec, int64
   p.tf = tf;
   p.s = 0.5 * (tf - t0);
   p.small = false;
-  BK_TRY(configure_fourstep(p.fs, N, BK_F64, nvec));
-  size_t off[9];
+  p.split = 1;
+  BK_TRY(configure_re(p.fs, N, BK_F64, 2, nvec));
+  size_t off[7];
   const size_t need = noalloc_layout(p, nvec, off);
   BK_ARG(need <= NOALLOC_BYTES, "N=%lld with %d vectors needs %zu bytes of scratch, more than the %zu reserved",
          (long long)N, nvec, need, NOALLOC_BYTES);
@@ -2419,23 +1940,24 @@ bk_status noalloc_apply(const double* v, double* out, int64_t N, int nvec, int64
   BK_TRY(noalloc_setup(dev, &base));
   unsigned char* b = (unsigned char*)base;
   p.fs.stw1 = b + off[0];
-  p.fs.stw2 = b + off[8];
-  p.tpost = b + off[1];
+  p.fs.stw2 = b + off[1];
   p.fs.twN = b + off[2];
-  p.rk = b + off[7];
+  p.scrA = b + off[3];
+  p.scrY = b + off[4];
+  p.part = b + off[5];
+  p.rk = b + off[6];
   // every table is rewritten by each call: nothing in the array has to start at zero
   k_rk_table<double><<<(int)std::min<int64_t>((N + 2 + 255) / 256, 4096), 256, 0, st>>>((double*)p.rk, N + 2);
   BK_CHECK_LAUNCH();
-  const int len1 = stage_tw_len(ilog2(p.fs.N1)), len2 = stage_tw_len(ilog2(p.fs.N2));
-  k_stage_tw<double><<<(len1 + 255) / 256, 256, 0, st>>>((double2*)p.fs.stw1, ilog2(p.fs.N1), len1);
+  constexpr int e = CplxFft<double>::E;
+  const int len1 = stage_tw_len(ilog2(p.fs.N1), e), len2 = stage_tw_len(ilog2(p.fs.N2), e);
+  k_stage_tw<double><<<(len1 + 255) / 256, 256, 0, st>>>((double2*)p.fs.stw1, ilog2(p.fs.N1), e, len1);
   BK_CHECK_LAUNCH();
-  k_stage_tw<double><<<(len2 + 255) / 256, 256, 0, st>>>((double2*)p.fs.stw2, ilog2(p.fs.N2), len2);
+  k_stage_tw<double><<<(len2 + 255) / 256, 256, 0, st>>>((double2*)p.fs.stw2, ilog2(p.fs.N2), e, len2);
   BK_CHECK_LAUNCH();
-  k_post_table<double><<<(int)std::min<int64_t>((N / 2 + 256) / 256, 4096), 256, 0, st>>>((double2*)p.tpost, N);
+  k_re_tw<double><<<re_tw_blocks(p.fs), 256, 0, st>>>((double2*)p.fs.twN, p.fs.N1, p.fs.N2);
   BK_CHECK_LAUNCH();
-  k_tw_table<double><<<(int)std::min<int64_t>((N + 255) / 256, 8192), 256, 0, st>>>((double2*)p.fs.twN, N, (double)N);
-  BK_CHECK_LAUNCH();
-  return apply_impl<double>(&p, v, out, nvec, false, p.s, st, b + off[3], b + off[4], b + off[5], b + off[6], nullptr);
+  return apply_impl<double>(&p, v, out, nvec, false, p.s, st);
 }
 
 }  // namespace bk
@@ -2533,9 +2055,9 @@ bk_status bk_plan_shape(const bk_plan* plan, int* path, int* N1, int* N2, int* e
   const bk::Plan* p = reinterpret_cast<const bk::Plan*>(plan);
   const int pth = p->dense ? 3 : (p->blue ? 4 : (p->small ? 0 : (p->split ? 2 : 1)));
   if (path) *path = pth;
-  if (N1) *N1 = (pth == 1 || pth == 2) ? p->fs.N1 : 0;
-  if (N2) *N2 = (pth == 1 || pth == 2) ? p->fs.N2 : 0;
-  if (elems) *elems = (pth == 1 || pth == 2) ? p->fs.NB * p->fs.N1 : 0;
+  if (N1) *N1 = (pth == 1 || pth == 2) ? p->fs.N1 / 2 : 0;
+  if (N2) *N2 = (pth == 1 || pth == 2) ? p->fs.N2 / 2 : 0;
+  if (elems) *elems = (pth == 1 || pth == 2) ? std::max(p->fs.NB * p->fs.N1, p->fs.P * p->fs.N2) : 0;
   return BK_OK;
 }
 

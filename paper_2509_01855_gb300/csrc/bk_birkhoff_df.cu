@@ -9,6 +9,6 @@ namespace bk {
 
 template bk_status set_smem_attrs<dfl>(const Plan* p);
 template bk_status apply_impl<dfl>(const Plan* p, const double* v, double* out, int nvec, bool trans, double s_scale,
-                                   cudaStream_t st, void* scrA, void* scrY, void* part1, void* part2, void* scrG);
+                                   cudaStream_t st);
 
 }  // namespace bk

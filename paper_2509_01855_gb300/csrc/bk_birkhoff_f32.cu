@@ -13,6 +13,6 @@ template bk_status apply_batch_impl<float>(const Plan* const*, const void* const
                                         const Plan* const*, const void* const*, void* const*, const int*, int, bool,
                                         cudaStream_t);
 template bk_status apply_impl<float>(const Plan* p, const float* v, float* out, int nvec, bool trans, double s_scale,
-                                     cudaStream_t st, void* scrA, void* scrY, void* part1, void* part2, void* scrG);
+                                     cudaStream_t st);
 
 }  // namespace bk

@@ -61,11 +61,17 @@ template <typename T> __host__ __device__ __forceinline__ typename V2<T>::t mk2(
   typename V2<T>::t r; r.x = x; r.y = y; return r;
 }
 
+// a b + c d and a b - c d with the contraction written out, so that every kernel a value may be
+// computed in (a plan's own or a batched launch) rounds it alike.
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ double dot2(double a, double b, double c, double d) { return __fma_rn(a, b, __dmul_rn(c, d)); }
+__device__ __forceinline__ dfl dot2(dfl a, dfl b, dfl c, dfl d) { return a * b + c * d; }
+
 // Complex product a * b.
 template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
   C r;
-  r.x = a.x * b.x - a.y * b.y;
-  r.y = a.x * b.y + a.y * b.x;
+  r.x = dot2(a.x, b.x, -a.y, b.y);
+  r.y = dot2(a.x, b.y, a.y, b.x);
   return r;
 }
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { C r; r.x = a.x + b.x; r.y = a.y + b.y; return r; }

@@ -1,15 +1,23 @@
 // Shared-memory batched complex FFT used by the DCT-I transforms of the Birkhoff products.
 // Forward transform, omega_n = exp(-2 pi i / n).
 //
-// In-place Stockham autosort with radix 16 (one mixed radix 2/4/8 stage first when log2 n is
-// not a multiple of 4). Every thread stages exactly 16 values per stage in registers (one
-// radix-16 butterfly, or 16/R butterflies of radix R), so one buffer suffices: read, barrier,
-// compute, write, barrier. Shared addresses are padded, a -> a + a/16, which makes the Stockham
-// writes conflict-free for 8- and 16-byte complex values; batches sit bs >= n + n/16 + 1 apart.
+// In-place Stockham autosort with radix 2^E (one smaller mixed-radix stage first when log2 n is not
+// a multiple of E). Every thread stages EPT values per stage in registers (EPT / R butterflies of
+// radix R), so one buffer suffices: read, barrier, compute, write, barrier. Shared addresses are
+// padded, a -> a + a/16; batches sit bs >= n + n/16 + 1 apart.
+//
+// The radix follows what bounds the kernel. FP64: GB300 issues a warp's FP64 instruction every 64
+// cycles per SM sub-partition, whatever its active lanes, and radix 4 needs as many FP64
+// instructions per point as radix 16 (28 per 4 points and 2 bits against 220 per 16 points and 4
+// bits), so radix 4 with 4 values per thread spreads the same work over four times the warps
+// (products of 4 components, radix 16 / radix 4, us: N = 2^10 55 / 27, 2^14 90 / 47, 2^16 122 / 70).
+// FP32 while latency bounds it: radix 4 as well (2^14 35 / 26, 2^16 47 / 31, 2^18 50 / 41); from
+// 2^19 on, bound by issue and shared memory: radix 16 (2^20 87 / 81). Double-float: radix 8, whose
+// code and registers are half of radix 16's (2^18 130 / 90, 2^20 339 / 260 radix 16 / radix 8).
 //
 // Twiddles come from a per-size stage table built on the device with sincospi at plan creation:
-// for each radix-16 stage with Ns > 1 (in stage order) a block stw[off + (r - 1) Ns + k] =
-// omega_{16 Ns}^{r k}, r = 1..15, k < Ns. Lanes hold consecutive k, so a warp reads consecutive
+// for each radix-R stage with Ns > 1 (in stage order) a block stw[off + (r - 1) Ns + k] =
+// omega_{R Ns}^{r k}, r = 1..R-1, k < Ns. Lanes hold consecutive k, so a warp reads consecutive
 // entries: no shared-memory bank conflicts, coalesced global loads. (Indexing one table of
 // omega_n^i by r k instead gave stride-r lane patterns, up to 16-way conflicts.) The table may
 // be the global one or a copy in shared memory (load_tw_smem).
@@ -24,12 +32,23 @@ namespace bk {
 __device__ __forceinline__ int padi(int a) { return a + (a >> 4); }
 __host__ __device__ inline int pad_stride(int n) { return n + (n >> 4) + 1; }
 
-// Entries of the stage twiddle table of a length-2^log2n FFT (radix-16 stages with Ns > 1).
-__host__ __device__ inline int stage_tw_len(int log2n) {
+// Entries of the stage twiddle table of a length-2^log2n FFT of radix 2^e (stages with Ns > 1).
+__host__ __device__ inline int stage_tw_len(int log2n, int e) {
   int len = 0;
-  for (int l = (log2n & 3) ? (log2n & 3) : 4; l < log2n; l += 4) len += 15 << l;
+  for (int l = log2n % e ? log2n % e : e; l < log2n; l += e) len += ((1 << e) - 1) << l;
   return len;
 }
+
+// Shape of the transform kernels of a type and log2 radix E: values per thread, thread cap and
+// resident CTAs per SM they are compiled for (64K registers / (threads x this) per thread).
+template <typename T, int E_> struct FftShape {
+  static constexpr int E = E_, EPT = 1 << E_, MT = E_ == 4 ? 512 : (E_ == 3 ? 512 : 1024), MINB = MT == 512 ? 2 : 1;
+};
+// Radix of the launch-per-pass kernels (re_radix) and of the plain complex passes, and of the
+// one-CTA and one-launch kernels, whose few CTAs are bound by latency.
+template <typename T> struct CplxFft : FftShape<T, sizeof(T) == 4 ? 4 : 2> {};
+template <typename T> struct SmallFft : FftShape<T, 2> {};
+template <typename T> struct BigFft { static constexpr int E = std::is_same<T, dfl>::value ? 3 : 2, EPT = 16, MT = 512, MINB = 1; };
 
 // Radix-R DFT of v[0..R-1] in registers (forward, natural order in and out).
 template <typename C, typename T, int R> struct Radix;
@@ -115,42 +134,40 @@ template <typename C, typename T> struct Radix<C, T, 16> {
   }
 };
 
-// One in-place stage of radix R (16/R butterflies per thread) of a length-2^LOG2N FFT whose
-// previous radices multiply to Ns = 2^LOG2NS. Threads t < nbatch * n/16 work; all threads must
+// One in-place stage of radix R (EPT/R butterflies per thread) of a length-2^LOG2N FFT whose
+// previous radices multiply to Ns = 2^LOG2NS. Threads t < nbatch * n/EPT work; all threads must
 // reach the barriers.
 //
-// Addressing. padi(a + c) = padi(a) + padi(c) whenever (a mod 16) + (c mod 16) < 16, so with
+// Addressing. padi(a + c) = padi(a) + padi(c) whenever the low four bits do not carry, so with
 // n and Ns known at compile time every shared address of a stage is one per-thread base plus an
 // immediate offset:
-//   reads  tt + q n/16 + r n/R : all offsets multiples of 16 once n >= 256 (smaller n: generic);
-//   writes idxD + r Ns, idxD = (j / Ns) 16 Ns + (j mod Ns): idxD mod 16 = j mod Ns < Ns when
-//          Ns < 16 and r Ns mod 16 <= 16 - Ns, or both offsets multiples of 16 (Ns >= 16); in
-//          the first stage (Ns = 1) idxD = R j is a multiple of R and r < R;
+//   reads  tt + q n/EPT + r n/R : offsets that are multiples of 16 (else generic);
+//   writes idxD + r Ns, idxD = (j / Ns) R Ns + (j mod Ns): the two terms share no bits;
 //   twiddles stw[(r - 1) Ns + k] from stw + k.
-template <typename T, int LOG2N, int R, int LOG2NS>
+template <typename T, int LOG2N, int R, int LOG2NS, int EPT>
 __device__ __forceinline__ void stage_ct(typename V2<T>::t* __restrict__ buf, int nbatch, int bs,
                                          const typename V2<T>::t* __restrict__ stw) {
   typedef typename V2<T>::t C;
   constexpr int log2R = R == 16 ? 4 : (R == 8 ? 3 : (R == 4 ? 2 : 1));
-  constexpr int PER = 16 / R;
-  constexpr int LOG2NB16 = LOG2N - 4;
-  constexpr int nb16 = 1 << LOG2NB16;
+  constexpr int log2EPT = EPT == 16 ? 4 : (EPT == 8 ? 3 : 2);
+  constexpr int PER = EPT / R;
+  constexpr int LOG2TP = LOG2N - log2EPT;
+  constexpr int nTP = 1 << LOG2TP;
   constexpr int nR = (1 << LOG2N) >> log2R;
   constexpr int Ns = 1 << LOG2NS;
-  constexpr bool lin_rd = (nR % 16 == 0) && (PER == 1 || nb16 % 16 == 0);
-  static_assert(PER == 1 || LOG2NS == 0, "mixed radix only as the first stage");
+  constexpr bool lin_rd = (nR % 16 == 0) && (PER == 1 || nTP % 16 == 0);
   const int t = threadIdx.x;
-  const bool active = t < (nbatch << LOG2NB16);
-  const int tt = t & (nb16 - 1);
-  C* base = buf + (size_t)(t >> LOG2NB16) * bs;
-  C v[16];
+  const bool active = t < (nbatch << LOG2TP);
+  const int tt = t & (nTP - 1);
+  C* base = buf + (size_t)(t >> LOG2TP) * bs;
+  C v[EPT];
   if (active) {
     const C* src = base + padi(tt);
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        const int c = q * nb16 + r * nR;
+        const int c = q * nTP + r * nR;
         v[q * R + r] = lin_rd ? src[c + (c >> 4)] : base[padi(tt + c)];
       }
     }
@@ -159,7 +176,7 @@ __device__ __forceinline__ void stage_ct(typename V2<T>::t* __restrict__ buf, in
   if (active) {
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-      const int j = tt + q * nb16;
+      const int j = tt + q * nTP;
       const int k = j & (Ns - 1);
       C* u = v + q * R;
       if (Ns > 1) {
@@ -179,44 +196,33 @@ __device__ __forceinline__ void stage_ct(typename V2<T>::t* __restrict__ buf, in
   __syncthreads();
 }
 
-// Radix-16 stages from Ns = 2^LOG2NS on; OFF is the stage table offset of the first of them.
-template <typename T, int LOG2N, int LOG2NS, int OFF>
-__device__ __forceinline__ void fft_ct_r16(typename V2<T>::t* buf, int nbatch, int bs,
-                                           const typename V2<T>::t* __restrict__ stw) {
+// Radix-2^E stages from Ns = 2^LOG2NS on; OFF is the stage table offset of the first of them.
+template <typename T, int LOG2N, int E, int EPT, int LOG2NS, int OFF>
+__device__ __forceinline__ void fft_ct_stages(typename V2<T>::t* buf, int nbatch, int bs,
+                                              const typename V2<T>::t* __restrict__ stw) {
   if constexpr (LOG2NS < LOG2N) {
-    stage_ct<T, LOG2N, 16, LOG2NS>(buf, nbatch, bs, stw + OFF);
-    fft_ct_r16<T, LOG2N, LOG2NS + 4, OFF + (LOG2NS > 0 ? (15 << LOG2NS) : 0)>(buf, nbatch, bs, stw);
+    stage_ct<T, LOG2N, (1 << E), LOG2NS, EPT>(buf, nbatch, bs, stw + OFF);
+    fft_ct_stages<T, LOG2N, E, EPT, LOG2NS + E, OFF + (LOG2NS > 0 ? (((1 << E) - 1) << LOG2NS) : 0)>(buf, nbatch, bs,
+                                                                                                      stw);
   }
 }
 
-// Length-2^LOG2N FFT: one mixed radix-2/4/8 stage when LOG2N is not a multiple of 4, then
-// radix-16 stages.
-template <typename T, int LOG2N>
+// Length-2^LOG2N FFT: one mixed-radix stage when LOG2N is not a multiple of E, then radix 2^E.
+template <typename T, int LOG2N, int E, int EPT>
 __device__ __forceinline__ void fft_ct(typename V2<T>::t* buf, int nbatch, int bs,
                                        const typename V2<T>::t* __restrict__ stw) {
-  constexpr int rem = LOG2N & 3;
-  if constexpr (rem != 0) stage_ct<T, LOG2N, (1 << rem), 0>(buf, nbatch, bs, stw);
-  fft_ct_r16<T, LOG2N, rem, 0>(buf, nbatch, bs, stw);
+  constexpr int rem = LOG2N % E;
+  if constexpr (rem != 0) stage_ct<T, LOG2N, (1 << rem), 0, EPT>(buf, nbatch, bs, stw);
+  fft_ct_stages<T, LOG2N, E, EPT, rem, 0>(buf, nbatch, bs, stw);
 }
 
-template <typename T, int LO, int HI>
+template <typename T, int E, int EPT, int LO, int HI>
 __device__ __forceinline__ void fft_ct_dispatch(typename V2<T>::t* buf, int log2n, int nbatch, int bs,
                                                 const typename V2<T>::t* __restrict__ stw) {
   if constexpr (LO <= HI) {
-    if (log2n == LO) fft_ct<T, LO>(buf, nbatch, bs, stw);
-    else fft_ct_dispatch<T, LO + 1, HI>(buf, log2n, nbatch, bs, stw);
+    if (log2n == LO) fft_ct<T, LO, E, EPT>(buf, nbatch, bs, stw);
+    else fft_ct_dispatch<T, E, EPT, LO + 1, HI>(buf, log2n, nbatch, bs, stw);
   }
-}
-
-// Batched in-place forward FFT of length n = 2^log2n (16 <= n <= 8192) over `nbatch` padded
-// transforms bs apart in shared memory (element i of batch b at buf[b * bs + padi(i)]), stw the
-// stage table of length n. The block needs at least nbatch * n / 16 threads. Input complete
-// before the call (barrier); result complete on return, in natural order, in place. Each length
-// is its own compile-time instance (log2n is uniform over the block).
-template <typename T>
-__device__ __forceinline__ void fft16(typename V2<T>::t* buf, int n, int log2n, int nbatch, int bs,
-                                      const typename V2<T>::t* __restrict__ stw) {
-  fft_ct_dispatch<T, 4, 13>(buf, log2n, nbatch, bs, stw);
 }
 
 // Copy a stage table (len entries) into shared memory.
@@ -235,33 +241,34 @@ namespace bk {
 // stage. Used by the double-float kernels, whose butterflies are an order of magnitude longer
 // than binary32 or binary64 ones, so that compile time and code size stay bounded; the address
 // arithmetic is generic (padi per element), which costs little next to double-float arithmetic.
-template <typename T, int R>
+template <typename T, int R, int EPT>
 __device__ __forceinline__ void stage_rt(typename V2<T>::t* __restrict__ buf, int nbatch, int bs,
                                          const typename V2<T>::t* __restrict__ stw, int log2n, int log2ns) {
   typedef typename V2<T>::t C;
   constexpr int log2R = R == 16 ? 4 : (R == 8 ? 3 : (R == 4 ? 2 : 1));
-  constexpr int PER = 16 / R;
-  const int log2nb16 = log2n - 4;
-  const int nb16 = 1 << log2nb16;
+  constexpr int log2EPT = EPT == 16 ? 4 : (EPT == 8 ? 3 : 2);
+  constexpr int PER = EPT / R;
+  const int log2tp = log2n - log2EPT;
+  const int ntp = 1 << log2tp;
   const int nR = (1 << log2n) >> log2R;
   const int Ns = 1 << log2ns;
   const int t = threadIdx.x;
-  const bool active = t < (nbatch << log2nb16);
-  const int tt = t & (nb16 - 1);
-  C* base = buf + (size_t)(t >> log2nb16) * bs;
-  C v[16];
+  const bool active = t < (nbatch << log2tp);
+  const int tt = t & (ntp - 1);
+  C* base = buf + (size_t)(t >> log2tp) * bs;
+  C v[EPT];
   if (active) {
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[q * R + r] = base[padi(tt + q * nb16 + r * nR)];
+      for (int r = 0; r < R; ++r) v[q * R + r] = base[padi(tt + q * ntp + r * nR)];
     }
   }
   __syncthreads();
   if (active) {
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-      const int j = tt + q * nb16;
+      const int j = tt + q * ntp;
       const int k = j & (Ns - 1);
       C* u = v + q * R;
       if (Ns > 1) {
@@ -278,27 +285,31 @@ __device__ __forceinline__ void stage_rt(typename V2<T>::t* __restrict__ buf, in
   __syncthreads();
 }
 
-// Run-time-length form of fft16 (same contract: 16 <= n <= 8192, nbatch * n / 16 threads).
-template <typename T>
-__device__ __forceinline__ void fft16_rt(typename V2<T>::t* buf, int n, int log2n, int nbatch, int bs,
-                                         const typename V2<T>::t* __restrict__ stw) {
-  const int rem = log2n & 3;
-  if (rem == 1) stage_rt<T, 2>(buf, nbatch, bs, stw, log2n, 0);
-  else if (rem == 2) stage_rt<T, 4>(buf, nbatch, bs, stw, log2n, 0);
-  else if (rem == 3) stage_rt<T, 8>(buf, nbatch, bs, stw, log2n, 0);
+template <typename T, int E, int EPT>
+__device__ __forceinline__ void fft_rt(typename V2<T>::t* buf, int log2n, int nbatch, int bs,
+                                       const typename V2<T>::t* __restrict__ stw) {
+  const int rem = log2n % E;
+  if (rem == 1) stage_rt<T, 2, EPT>(buf, nbatch, bs, stw, log2n, 0);
+  else if (E > 2 && rem == 2) stage_rt<T, 4, EPT>(buf, nbatch, bs, stw, log2n, 0);
+  else if (E > 3 && rem == 3) stage_rt<T, (E > 3 ? 8 : 2), EPT>(buf, nbatch, bs, stw, log2n, 0);
   int off = 0;
-  for (int l = rem; l < log2n; l += 4) {
-    stage_rt<T, 16>(buf, nbatch, bs, stw + off, log2n, l);
-    if (l > 0) off += 15 << l;
+  for (int l = rem; l < log2n; l += E) {
+    stage_rt<T, (1 << E), EPT>(buf, nbatch, bs, stw + off, log2n, l);
+    if (l > 0) off += ((1 << E) - 1) << l;
   }
 }
 
-// fft16 for binary32 / binary64, fft16_rt for double-float.
-template <typename T>
-__device__ __forceinline__ void fft16_any(typename V2<T>::t* buf, int n, int log2n, int nbatch, int bs,
-                                          const typename V2<T>::t* __restrict__ stw) {
-  if constexpr (std::is_same<T, dfl>::value) fft16_rt<T>(buf, n, log2n, nbatch, bs, stw);
-  else fft16<T>(buf, n, log2n, nbatch, bs, stw);
+// Batched in-place forward FFT of length n = 2^log2n (16 <= n <= 8192) over `nbatch` padded
+// transforms bs apart in shared memory (element i of batch b at buf[b * bs + padi(i)]), stw the
+// radix-2^E stage table of length n. The block needs at least nbatch * n / EPT threads. Input
+// complete before the call (barrier); result complete on return, in natural order, in place. Each
+// length 2^LO..2^HI is its own compile-time instance (log2n is uniform over the block); double-float
+// takes the run-time form.
+template <typename T, int E, int EPT, int LO = 4, int HI = 13>
+__device__ __forceinline__ void fft_any(typename V2<T>::t* buf, int log2n, int nbatch, int bs,
+                                        const typename V2<T>::t* __restrict__ stw) {
+  if constexpr (std::is_same<T, dfl>::value) fft_rt<T, E, EPT>(buf, log2n, nbatch, bs, stw);
+  else fft_ct_dispatch<T, E, EPT, LO, HI>(buf, log2n, nbatch, bs, stw);
 }
 
 }  // namespace bk

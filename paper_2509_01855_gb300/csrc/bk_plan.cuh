@@ -5,22 +5,27 @@
 
 namespace bk {
 
-// One four-step complex FFT layout of length n = N1 * N2 (pass A: columns of length N1, pass B:
-// rows of length N2) and its tables in the working type.
+// One four-step layout, n = N1 * N2 (pass A: columns of length N1, pass B: rows of length N2), and
+// its tables in the working type. Power-of-two plans: the real-even passes of bk_dct.cuh, n = 2N
+// (NB column pairs and P row pairs per CTA). Bluestein plans: a plain complex FFT of length n (NB
+// columns and 2P rows per CTA).
 struct FourStep {
   int64_t n = 0;
   int N1 = 0, N2 = 0;
-  int NB = 0, P = 0;          // pass A columns per CTA, pass B rows (or row pairs) per CTA
-  int bsA = 0;                // pass-A batch stride in shared memory (complex elements)
+  int NB = 0, P = 0;
+  int bsA = 0, bsB = 0;       // batch strides in shared memory (complex elements)
   size_t smemA = 0, smemB = 0;
   int thrA = 256, thrB = 256; // threads of the pass kernels (16 complex values each)
-  int nPartA = 0;             // pass-A CTAs per vector (partials per vector)
   void* stw1 = nullptr;       // stage twiddle table of the length-N1 FFT
   void* stw2 = nullptr;       // stage twiddle table of the length-N2 FFT
-  void* twN = nullptr;        // omega_n^m, m < n (FP64)
-  void* twLo = nullptr;       // omega_n^m, m < 2^tw_h (FP32)
-  void* twHi = nullptr;       // omega_n^{m 2^tw_h}, m < n / 2^tw_h (FP32)
+  void* twN = nullptr;        // real-even: the [N1/2 + 1][N2/2 + 2] table; else omega_n^m, m < n (FP64)
+  void* twLo = nullptr;       // omega_n^m, m < 2^tw_h (FP32, plain complex)
+  void* twHi = nullptr;       // omega_n^{m 2^tw_h}, m < n / 2^tw_h (FP32, plain complex)
   int tw_h = 0;
+  // real-even sizes per vector: row length and total of the scratch A, column pairs
+  int RS() const { return N2 / 2 + 2; }
+  int64_t a_len() const { return (int64_t)(N1 / 2 + 1) * RS(); }
+  int pairs() const { return N2 / 4 + 1; }
 };
 
 struct Plan {
@@ -43,21 +48,19 @@ struct Plan {
   int thrS = 256;             // threads of the single-CTA kernel
   void* tw = nullptr;         // omega_N^i, i < N (single-CTA plans; the N < 16 direct DFT)
   void* stwS = nullptr;       // stage twiddle table of the length-N FFT (single-CTA plans)
-  // Four-step plans. Unsplit: fs is the length-N FFT of the DCT-I. Split (split = 1): each DCT-I
-  // of length N+1 is the DCT-I of length N/2+1 of its pair sums (even outputs; fs, length N/2)
-  // and the DCT-III of length N/2 of its pair differences (odd outputs; fso, length N/4).
-  // Two-level split (split = 2): the even half split once more, fs the length-N/4 FFT of the
-  // DCT-I of length N/4+1, fse the length-N/8 FFT of the DCT-III of length N/4, fso as above.
-  FourStep fs, fso, fse;
+  // Four-step plans: the layout fs of the length-2N real-even DFT. split: the four passes run as
+  // a launch each; else as one launch, a cluster of csize CTAs per vector.
+  FourStep fs;
   int split = 0;
-  void* eo = nullptr;         // split: exp(2 pi i k / (N/2)), k < N/4 (DCT-III pre-processing)
-  void* tpost = nullptr;      // (cos, sin)(pi k / N), k = 0..N/2 (working type)
+  int fe = 2;                 // log2 radix of the launch-per-pass kernels
+  int csize = 0, cthr = 0;
+  size_t csmem = 0;
+  void* tpost = nullptr;      // (cos, sin)(pi k / N), k = 0..N/2 (working type; not four-step)
   void* rk = nullptr;         // 1 / (4k), k = 0..N+1 (working type; rk[0] = 0)
-  void* scrA = nullptr;       // four-step complex scratch, N per vector
-  void* scrY = nullptr;       // stage buffer between the two DCTs, N + 1 per vector
-  void* scrG = nullptr;       // second-DCT input (stencil output), N + 1 per vector
-  void* part1 = nullptr;      // pass-A partial sums, first DCT
-  void* part2 = nullptr;      // pass-A partial sums, second DCT
+  void* scrA = nullptr;       // scratch between passes A and B, fs.a_len() complex per vector
+  void* scrY = nullptr;       // stage buffer between the two DCTs, N + 2 per vector (Bluestein N + 1)
+  void* scrG = nullptr;       // Bluestein: second-DCT input (stencil output), N + 1 per vector
+  void* part = nullptr;       // pass-A shares of R_0, fs.pairs() per vector
   double* t_nodes = nullptr;  // node times t_j (FP64, device)
   double* w64 = nullptr;      // Clenshaw-Curtis weights (FP64, device, tau-domain)
   void* wT = nullptr;         // Clenshaw-Curtis weights in the working type (device)
