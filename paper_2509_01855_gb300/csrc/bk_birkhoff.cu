@@ -405,6 +405,7 @@ __global__ void __launch_bounds__(1024)
     k_birkhoff_small(const Us<T>* __restrict__ in, Us<T>* __restrict__ out, int N, int log2N, int64_t pitch,
                      T s, const typename V2<T>::t* __restrict__ tw, const typename V2<T>::t* __restrict__ stw,
                      const typename V2<T>::t* __restrict__ tpost, StencilTab<T> tb) {
+  pdl_wait();
   small_body<T, TRANS>(blockIdx.x, in, out, N, log2N, pitch, s, tw, stw, tpost, tb);
 }
 
@@ -420,6 +421,7 @@ __global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
             int log2N1, int N2, int NB, int bs, const typename V2<T>::t* __restrict__ stw,
             const typename V2<T>::t* __restrict__ twN, const typename V2<T>::t* __restrict__ twLo,
             const typename V2<T>::t* __restrict__ twHi, int tw_h) {
+  pdl_wait();
   typedef typename V2<T>::t C;
   extern __shared__ __align__(16) unsigned char smem[];
   C* buf = reinterpret_cast<C*>(smem);
@@ -480,6 +482,7 @@ __global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
 template <typename T, int K>
 __global__ void __launch_bounds__(256) k_stencil(const T* __restrict__ stage, int64_t Ls, T* __restrict__ G, int N, T sc,
                                                  StencilTab<T> tb) {
+  pdl_wait();
   const T* Y = stage + (int64_t)blockIdx.y * Ls;
   T* g = G + (int64_t)blockIdx.y * Ls;
   // interior nodes 2..N-2 by the plain three-point formulas (the boundary cases, if-converted
@@ -536,6 +539,7 @@ namespace bk {
 template <typename T, int K>
 __global__ void __launch_bounds__(256) k_bs_pre(const T* __restrict__ src, int64_t sstride, int N, int64_t M,
                                                 const typename V2<T>::t* __restrict__ w, T* __restrict__ a) {
+  pdl_wait();
   typedef typename V2<T>::t C;
   const T* x = src + (int64_t)blockIdx.y * sstride;
   T* dst = a + (int64_t)blockIdx.y * 2 * M;
@@ -558,6 +562,7 @@ __global__ void __launch_bounds__(256) k_bs_post(const T* __restrict__ y, int64_
                                                  const typename V2<T>::t* __restrict__ tpost,
                                                  T* __restrict__ dst, int64_t dstride,
                                                  int64_t zero_to, T s, T invN) {
+  pdl_wait();
   typedef typename V2<T>::t C;
   const T* yv = y + (int64_t)blockIdx.y * 2 * M;
   T* out = dst + (int64_t)blockIdx.y * dstride;
@@ -585,6 +590,7 @@ template <typename T, int E>
 __global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
     k_passB(const typename V2<T>::t* __restrict__ Ain, T* __restrict__ dst, int64_t dst_stride, int N, int N1, int N2,
             int log2N2, int P, const typename V2<T>::t* __restrict__ stw, const typename V2<T>::t* __restrict__ tab) {
+  pdl_wait();
   typedef typename V2<T>::t C;
   extern __shared__ __align__(16) unsigned char smem[];
   const int bs = pad_stride(N2);
@@ -664,6 +670,7 @@ __device__ __forceinline__ int batch_job(const Batch<J>& b, int cta) {
 
 template <typename T, bool TRANS>
 __global__ void __launch_bounds__(1024) k_small_batch(const __grid_constant__ Batch<SmallJob<T>> b) {
+  pdl_wait();
   const int q = batch_job(b, blockIdx.x);
   const SmallJob<T>& J = b.j[q];
   small_body<T, TRANS>((int)blockIdx.x - b.start[q], J.in, J.out, J.N, J.log2N, J.pitch, J.s, J.tw, J.stw, J.tpost,
@@ -673,6 +680,7 @@ __global__ void __launch_bounds__(1024) k_small_batch(const __grid_constant__ Ba
 // Launch-per-pass plans of one radix F: CTA b of a job runs vector b % nvec of tile b / nvec.
 template <typename T, bool TRANS, bool SECOND, typename F>
 __global__ void __launch_bounds__(F::MT, F::MINB) k_re_passA_batch(const __grid_constant__ Batch<ReJob<T>> b) {
+  pdl_wait();
   const int q = batch_job(b, blockIdx.x);
   const ReJob<T>& J = b.j[q];
   const int l = (int)blockIdx.x - b.start[q];
@@ -685,6 +693,7 @@ __global__ void __launch_bounds__(F::MT, F::MINB) k_re_passA_batch(const __grid_
 }
 template <typename T, bool TRANS, bool SECOND, typename F>
 __global__ void __launch_bounds__(F::MT, F::MINB) k_re_passB_batch(const __grid_constant__ Batch<ReJob<T>> b) {
+  pdl_wait();
   const int q = batch_job(b, blockIdx.x);
   const ReJob<T>& J = b.j[q];
   const int l = (int)blockIdx.x - b.start[q];
@@ -698,6 +707,7 @@ __global__ void __launch_bounds__(F::MT, F::MINB) k_re_passB_batch(const __grid_
 
 template <typename T, bool TRANS>
 __global__ void __launch_bounds__(512, sizeof(T) == 8 ? 1 : 2) k_re_cluster_batch(const __grid_constant__ Batch<ReJob<T>> b, int csize) {
+  pdl_wait();
   const int cl = blockIdx.x / csize;
   const int q = batch_job(b, cl);
   re_cluster_body<T, TRANS>(b.j[q], cl - b.start[q], blockIdx.x % csize, csize);
@@ -1384,13 +1394,11 @@ static bk_status blue_fft(const Plan* p, const T* src, T* dst, typename V2<T>::t
   typedef typename V2<T>::t C;
   const FourStep& f = p->fsM;
   const int M = (int)p->M;
-  k_passA<T><<<dim3(f.N2 / f.NB, nvec), f.thrA, f.smemA, st>>>(src, 2 * (int64_t)M, A, M, f.N1, ilog2(f.N1), f.N2, f.NB,
+  BK_TRY(launch(k_passA<T>, dim3(f.N2 / f.NB, nvec), f.thrA, f.smemA, st, src, 2 * (int64_t)M, A, M, f.N1, ilog2(f.N1), f.N2, f.NB,
                                                                f.bsA, (const C*)f.stw1, (const C*)f.twN,
-                                                               (const C*)f.twLo, (const C*)f.twHi, f.tw_h);
-  BK_CHECK_LAUNCH();
-  k_passB<T, E><<<dim3(f.N1 / 2 / f.P, nvec), f.thrB, f.smemB, st>>>(A, dst, 2 * (int64_t)M, M, f.N1, f.N2, ilog2(f.N2),
-                                                                     f.P, (const C*)f.stw2, (const C*)p->bh);
-  BK_CHECK_LAUNCH();
+                                                               (const C*)f.twLo, (const C*)f.twHi, f.tw_h));
+  BK_TRY(launch(k_passB<T, E>, dim3(f.N1 / 2 / f.P, nvec), f.thrB, f.smemB, st, A, dst, 2 * (int64_t)M, M, f.N1, f.N2, ilog2(f.N2),
+                                                                     f.P, (const C*)f.stw2, (const C*)p->bh));
   return BK_OK;
 }
 
@@ -1405,14 +1413,12 @@ static bk_status blue_dct(const Plan* p, const T* src, int64_t sstride, T* dst, 
   T* Ma = (T*)p->scrA;
   C* Mb = (C*)(Ma + 2 * M * (int64_t)p->n_comp * p->max_batch);
   const int gp = (int)std::min<int64_t>(1024, (M + 255) / 256);
-  k_bs_pre<T, K><<<dim3(gp, nvec), 256, 0, st>>>(src, sstride, N, M, (const C*)p->chirp, Ma);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_bs_pre<T, K>, dim3(gp, nvec), 256, 0, st, src, sstride, N, M, (const C*)p->chirp, Ma));
   BK_TRY((blue_fft<T, EP_CPLX_MC>(p, Ma, Ma, Mb, nvec, st)));
   BK_TRY((blue_fft<T, EP_CPLX>(p, Ma, Ma, Mb, nvec, st)));
   const int gq = (int)std::min<int64_t>(1024, (N / 2 + 256) / 256);
-  k_bs_post<T, E><<<dim3(gq, nvec), 256, 0, st>>>(Ma, M, N, (const C*)p->chirp, (const C*)p->tpost, dst, dstride,
-                                                  zero_to, s, invN);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_bs_post<T, E>, dim3(gq, nvec), 256, 0, st, Ma, M, N, (const C*)p->chirp, (const C*)p->tpost, dst, dstride,
+                                                  zero_to, s, invN));
   return BK_OK;
 }
 
@@ -1454,9 +1460,8 @@ template <typename T, int K, typename F, typename S>
 static bk_status re_launch_AF(const Plan* p, const S* src, int64_t sstride, int nvec, cudaStream_t st) {
   typedef typename V2<T>::t C;
   const FourStep& f = p->fs;
-  k_re_passA<T, K, F, S><<<dim3(nvec, (f.pairs() + f.NB - 1) / f.NB), f.thrA, f.smemA, st>>>(
-      re_args<T>(p), f.NB, f.bsA, src, sstride, (C*)p->scrA, f.a_len(), (T*)p->part);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_re_passA<T, K, F, S>, dim3(nvec, (f.pairs() + f.NB - 1) / f.NB), f.thrA, f.smemA, st, 
+      re_args<T>(p), f.NB, f.bsA, src, sstride, (C*)p->scrA, f.a_len(), (T*)p->part));
   return BK_OK;
 }
 template <typename T, int K, typename S>
@@ -1473,10 +1478,9 @@ template <typename T, int E, typename F, typename S>
 static bk_status re_launch_BF(const Plan* p, S* dst, int64_t dstride, int64_t zero_to, int nvec, T s, cudaStream_t st) {
   typedef typename V2<T>::t C;
   const FourStep& f = p->fs;
-  k_re_passB<T, E, F, S><<<dim3(nvec, (f.N1 / 4 + f.P) / f.P), f.thrB, f.smemB, st>>>(
+  BK_TRY(launch(k_re_passB<T, E, F, S>, dim3(nvec, (f.N1 / 4 + f.P) / f.P), f.thrB, f.smemB, st, 
       re_args<T>(p), f.P, f.bsB, (const C*)p->scrA, f.a_len(), dst, dstride, zero_to, (const T*)p->part, s,
-      T(1.0 / (double)p->N));
-  BK_CHECK_LAUNCH();
+      T(1.0 / (double)p->N)));
   return BK_OK;
 }
 template <typename T, int E, typename S>
@@ -1512,26 +1516,6 @@ static ReJob<T> re_job(const Plan* p, const void* in, void* out, int nvec, T s) 
   return J;
 }
 
-// One launch of clusters of csize CTAs (blockIdx.x / csize is the cluster).
-template <typename F, typename A>
-static bk_status launch_clusters(F* fn, const A& arg, int nclusters, int csize, int thr, size_t smem, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)nclusters * csize);
-  cfg.blockDim = dim3(thr);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = csize;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  BK_TRY_CUDA(cudaLaunchKernelEx(&cfg, fn, arg, csize));
-  BK_CHECK_LAUNCH();
-  return BK_OK;
-}
-
 template <typename T>
 bk_status apply_impl(const Plan* p, const Us<T>* v, Us<T>* out, int nvec, bool trans, double s_scale, cudaStream_t st) {
   typedef typename V2<T>::t C;
@@ -1542,14 +1526,9 @@ bk_status apply_impl(const Plan* p, const Us<T>* v, Us<T>* out, int nvec, bool t
     StencilTab<T> tb;
     tb.rk = (const T*)p->rk;
     tb.cN = (T)(1.0 / (4.0 * ((double)N * (double)N - 1.0)));
-    if (p->small) {
-      if (!trans)
-        k_birkhoff_small<T, false><<<nvec, p->thrS, p->smemS, st>>>(v, out, N, ilog2(N), p->pitch, s, (const C*)p->tw, (const C*)p->stwS, (const C*)p->tpost, tb);
-      else
-        k_birkhoff_small<T, true><<<nvec, p->thrS, p->smemS, st>>>(v, out, N, ilog2(N), p->pitch, s, (const C*)p->tw, (const C*)p->stwS, (const C*)p->tpost, tb);
-      BK_CHECK_LAUNCH();
-      return BK_OK;
-    }
+    if (p->small)
+      return launch(trans ? k_birkhoff_small<T, true> : k_birkhoff_small<T, false>, nvec, p->thrS, p->smemS, st, v, out,
+                    N, ilog2(N), p->pitch, s, (const C*)p->tw, (const C*)p->stwS, (const C*)p->tpost, tb);
     if (p->blue) {
       const int64_t Ls = N + 1;
       T* Ystage = (T*)p->scrY;
@@ -1557,20 +1536,18 @@ bk_status apply_impl(const Plan* p, const Us<T>* v, Us<T>* out, int nvec, bool t
       const dim3 gS((unsigned)std::min<int64_t>(1024, (N + 255) / 256), nvec);
       if (!trans) {
         BK_TRY((blue_dct<T, IN_PLAIN, EP_STORE>(p, v, p->pitch, Ystage, Ls, 0, nvec, s, invN, st)));
-        k_stencil<T, ST_FWD><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb);
-        BK_CHECK_LAUNCH();
+        BK_TRY(launch(k_stencil<T, ST_FWD>, gS, 256, 0, st, Ystage, Ls, Gst, N, T(1), tb));
         BK_TRY((blue_dct<T, IN_PLAIN, EP_FWD_OUT>(p, Gst, Ls, out, p->pitch, p->pitch, nvec, s, invN, st)));
       } else {
         BK_TRY((blue_dct<T, IN_WINV, EP_STORE_TRN>(p, v, p->pitch, Ystage, Ls, 0, nvec, s, invN, st)));
-        k_stencil<T, ST_TRN><<<gS, 256, 0, st>>>(Ystage, Ls, Gst, N, T(1), tb);
-        BK_CHECK_LAUNCH();
+        BK_TRY(launch(k_stencil<T, ST_TRN>, gS, 256, 0, st, Ystage, Ls, Gst, N, T(1), tb));
         BK_TRY((blue_dct<T, IN_PLAIN, EP_TRN_OUT>(p, Gst, Ls, out, p->pitch, p->pitch, nvec, s, invN, st)));
       }
       return BK_OK;
     }
     if (!p->split)
-      return launch_clusters(trans ? k_re_cluster<T, true> : k_re_cluster<T, false>, re_job<T>(p, v, out, nvec, s), nvec,
-                             p->csize, p->cthr, p->csmem, st);
+      return launch_cl(p->csize, trans ? k_re_cluster<T, true> : k_re_cluster<T, false>, nvec * p->csize, p->cthr,
+                       p->csmem, st, re_job<T>(p, v, out, nvec, s), p->csize);
   }
   T* Y = (T*)p->scrY;
   const int64_t Ls = (int64_t)N + 2;   // even: pass A reads aligned pairs
@@ -1624,11 +1601,7 @@ static bk_status launch_small_batch(const Plan* const* ps, const void* const* vi
       smem = std::max(smem, p->smemS);
     }
     b.start[b.njob] = cta;
-    if (!trans)
-      k_small_batch<T, false><<<cta, thr, smem, st>>>(b);
-    else
-      k_small_batch<T, true><<<cta, thr, smem, st>>>(b);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(trans ? k_small_batch<T, true> : k_small_batch<T, false>, cta, thr, smem, st, b));
   }
   return BK_OK;
 }
@@ -1652,7 +1625,7 @@ static bk_status launch_fourstep_batch(const Plan* const* ps, const void* const*
       smem = std::max(smem, p->csmem);
     }
     b.start[b.njob] = cl;
-    BK_TRY(launch_clusters(trans ? k_re_cluster_batch<T, true> : k_re_cluster_batch<T, false>, b, cl, cs, thr, smem, st));
+    BK_TRY(launch_cl(cs, trans ? k_re_cluster_batch<T, true> : k_re_cluster_batch<T, false>, cl * cs, thr, smem, st, b, cs));
   }
   return BK_OK;
 }
@@ -1685,14 +1658,10 @@ static bk_status launch_passes_batch(const Plan* const* ps, const void* const* v
     }
     a.start[a.njob] = ca;
     b.start[b.njob] = cb;
-    k_re_passA_batch<T, TRANS, false, F><<<ca, thrA, smA, st>>>(a);
-    BK_CHECK_LAUNCH();
-    k_re_passB_batch<T, TRANS, false, F><<<cb, thrB, smB, st>>>(b);
-    BK_CHECK_LAUNCH();
-    k_re_passA_batch<T, TRANS, true, F><<<ca, thrA, smA, st>>>(a);
-    BK_CHECK_LAUNCH();
-    k_re_passB_batch<T, TRANS, true, F><<<cb, thrB, smB, st>>>(b);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_re_passA_batch<T, TRANS, false, F>, ca, thrA, smA, st, a));
+    BK_TRY(launch(k_re_passB_batch<T, TRANS, false, F>, cb, thrB, smB, st, b));
+    BK_TRY(launch(k_re_passA_batch<T, TRANS, true, F>, ca, thrA, smA, st, a));
+    BK_TRY(launch(k_re_passB_batch<T, TRANS, true, F>, cb, thrB, smB, st, b));
   }
   return BK_OK;
 }
@@ -1741,11 +1710,13 @@ bk_status plan_apply_n(const Plan* p, const void* v, void* out, int nvec, bool t
 // vector, fixed order), then out[vec][i] -= c[vec] (forward) or c[vec] w_i (transpose), i <= N.
 template <typename T>
 __global__ void k_bform_last(const T* __restrict__ out, int64_t pitch, int64_t N, T* __restrict__ c) {
+  pdl_wait();
   if (threadIdx.x == 0) c[blockIdx.x] = out[(int64_t)blockIdx.x * pitch + N];
 }
 template <typename T>
 __global__ void __launch_bounds__(256) k_bform_sum(const T* __restrict__ u, int64_t pitch, int64_t L, double s,
                                                    T* __restrict__ c) {
+  pdl_wait();
   __shared__ double red[8];
   const T* x = u + (int64_t)blockIdx.x * pitch;
   double a = 0.0;
@@ -1762,6 +1733,7 @@ __global__ void __launch_bounds__(256) k_bform_sum(const T* __restrict__ u, int6
 template <typename T>
 __global__ void k_bform_sub(T* __restrict__ out, int64_t pitch, int64_t L, const T* __restrict__ c,
                             const T* __restrict__ w) {
+  pdl_wait();
   const T cv = c[blockIdx.y];
   T* o = out + (int64_t)blockIdx.y * pitch;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < L; i += (int64_t)gridDim.x * blockDim.x)
@@ -1775,17 +1747,14 @@ static bk_status apply_b_impl(const Plan* p, const void* v, void* out, int nvec,
   const T* w = p->dtype == BK_F64 ? (const T*)p->w64 : (const T*)p->wT;
   if (trans) {
     // the sum first: v may alias out
-    k_bform_sum<T><<<nvec, 256, 0, st>>>((const T*)v, p->pitch, p->L, p->s, c);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_bform_sum<T>, nvec, 256, 0, st, (const T*)v, p->pitch, p->L, p->s, c));
     BK_TRY(plan_apply_n(p, v, out, nvec, true, p->s, st));
-    k_bform_sub<T><<<g, 256, 0, st>>>((T*)out, p->pitch, p->L, c, w);
+    BK_TRY(launch(k_bform_sub<T>, g, 256, 0, st, (T*)out, p->pitch, p->L, c, w));
   } else {
     BK_TRY(plan_apply_n(p, v, out, nvec, false, p->s, st));
-    k_bform_last<T><<<nvec, 32, 0, st>>>((const T*)out, p->pitch, p->N, c);
-    BK_CHECK_LAUNCH();
-    k_bform_sub<T><<<g, 256, 0, st>>>((T*)out, p->pitch, p->L, c, nullptr);
+    BK_TRY(launch(k_bform_last<T>, nvec, 32, 0, st, (const T*)out, p->pitch, p->N, c));
+    BK_TRY(launch(k_bform_sub<T>, g, 256, 0, st, (T*)out, p->pitch, p->L, c, nullptr));
   }
-  BK_CHECK_LAUNCH();
   return BK_OK;
 }
 

@@ -24,9 +24,9 @@ void set_error(const char* fmt, ...);
     }                                                                                 \
   } while (0)
 
-#define BK_TRY(expr)                       \
+#define BK_TRY(...)                        \
   do {                                     \
-    bk_status s_ = (expr);                 \
+    bk_status s_ = (__VA_ARGS__);          \
     if (s_ != BK_OK) return s_;            \
   } while (0)
 
@@ -42,6 +42,54 @@ void note_launches(long long n);
     bk::note_launch();             \
     BK_TRY_CUDA(cudaGetLastError()); \
   } while (0)
+
+// Programmatic dependent launch. Every kernel of the library's call chains starts with
+// pdl_wait(): it waits until the kernels before it in the stream have completed and their writes
+// are visible (at once when it was launched plainly). Launches through launch() may then be set up
+// while the kernel before them still runs, which hides most of the launch latency of these chains;
+// order and results are those of plain launches. Measured on GB300, plain / dependent launches, us:
+// FP64 products of 4 components 2^14 43 / 34, 2^16 64 / 56, KKT preconditioner at 2^17 146 / 120,
+// FP32 orbit solve at 2^12 4990 / 3870. The kernels do not trigger the next launch early: its CTAs
+// then took their places beside the running kernel's, where those of the FP64-bound sweeps crowded
+// onto the SMs that happened to be free (the preconditioner took 181 us).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch k on st, counted like BK_CHECK_LAUNCH(). Under stream capture (and where the capture
+// state cannot be read) the launch is a plain one. cluster > 0: clusters of that many CTAs.
+template <typename... KA, typename... A>
+inline bk_status launch_cl(int cluster, void (*k)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    (void)cudaGetLastError();
+    cs = cudaStreamCaptureStatusActive;
+  }
+  if (cs == cudaStreamCaptureStatusNone) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 0) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = (unsigned)cluster;
+    at[n].val.clusterDim.y = 1;
+    at[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = (unsigned)n;
+  BK_TRY_CUDA(cudaLaunchKernelEx(&cfg, k, static_cast<KA>(a)...));
+  note_launch();
+  return BK_OK;
+}
+template <typename... KA, typename... A>
+inline bk_status launch(void (*k)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... a) {
+  return launch_cl(0, k, grid, block, smem, st, static_cast<KA>(a)...);
+}
 
 #define BK_ARG(cond, ...)                  \
   do {                                     \

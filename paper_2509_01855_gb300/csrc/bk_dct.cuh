@@ -388,6 +388,7 @@ template <typename T, int K, typename F, typename S>
 __global__ void __launch_bounds__(F::MT, F::MINB)
     k_re_passA(const __grid_constant__ ReArgs<T> g, int NB, int bs, const S* __restrict__ src, int64_t sstride,
                typename V2<T>::t* __restrict__ A, int64_t astride, T* __restrict__ part) {
+  pdl_wait();
   re_passA_cta<T, K, F, S>(g, blockIdx.x, blockIdx.y, NB, bs, src, sstride, A, astride, part);
 }
 
@@ -397,6 +398,7 @@ __global__ void __launch_bounds__(F::MT, F::MINB)
     k_re_passB(const __grid_constant__ ReArgs<T> g, int P, int bs, const typename V2<T>::t* __restrict__ A,
                int64_t astride, S* __restrict__ dst, int64_t dstride, int64_t zero_to, const T* __restrict__ part,
                T s, T invN) {
+  pdl_wait();
   re_passB_cta<T, E, F, S>(g, blockIdx.x, blockIdx.y, P, bs, A, astride, dst, dstride, zero_to, part, s, invN);
 }
 
@@ -464,6 +466,7 @@ __device__ __forceinline__ void re_cluster_body(const ReJob<T>& J, int vec, int 
 
 template <typename T, bool TRANS>
 __global__ void __launch_bounds__(512, sizeof(T) == 8 ? 1 : 2) k_re_cluster(const __grid_constant__ ReJob<T> J, int csize) {
+  pdl_wait();
   re_cluster_body<T, TRANS>(J, blockIdx.x / csize, blockIdx.x % csize, csize);
 }
 

@@ -133,6 +133,7 @@ __device__ void node_deviation(const Tc* x, const Tc* u, Tc h, Tc* D, Tc pa) {
 template <typename T, int KIND, int NX, int NU>
 __global__ void k_lin_nodes(const double* __restrict__ z, int64_t P, int64_t L, const double* __restrict__ w,
                             double s, T* __restrict__ Dn, T* __restrict__ xu, double pa) {
+  pdl_wait();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
     T x[NXM], u[NUM];
 #pragma unroll
@@ -185,6 +186,7 @@ __device__ __forceinline__ void dev_mul(const Tm* A, const Tm* B, Tm* C) {
 // thread per segment: A <- (I + 2 D)(I + A) - I = A + 2 (D + D A), from A = 2 D of its first node.
 template <typename T, int NX>
 __global__ void k_lin_seg(const T* __restrict__ Dn, int64_t L, int nseg, T* __restrict__ A0) {
+  pdl_wait();
   const int seg = blockIdx.x * blockDim.x + threadIdx.x;
   if (seg >= nseg) return;
   constexpr int SEG = Seg<T>::v;
@@ -225,6 +227,7 @@ __global__ void k_lin_seg(const T* __restrict__ Dn, int64_t L, int nseg, T* __re
 // M_4(31) M_4(15), which is the map of the parent item at the next level.
 template <typename T, int NX>
 __global__ void __launch_bounds__(32) k_lin_level(T* __restrict__ m, int n, T* __restrict__ parent) {
+  pdl_wait();
   constexpr int NC = NX * NX;
   __shared__ T S[5][32][NC + 1];
   const int lane = threadIdx.x;
@@ -297,6 +300,7 @@ __global__ void __launch_bounds__(32) k_lin_level(T* __restrict__ m, int n, T* _
 
 template <typename Tin, typename Tout>
 __global__ void k_convert(const Tin* __restrict__ a, Tout* __restrict__ b, int64_t n) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     b[i] = (Tout)a[i];
 }
@@ -647,6 +651,7 @@ __device__ __forceinline__ void sw_down0_warp(int g, SweepTiles<T, NX>& tl, cons
 template <typename T, int NX, int DIR, int W>
 __global__ void __launch_bounds__(32 * W) k_sw_up0(const T* __restrict__ Dn, const T* __restrict__ Y, const T* __restrict__ G, int64_t P,
                                                    int64_t L, const T* __restrict__ w, T s, Levels<T> lv) {
+  pdl_wait();
   __shared__ SweepTiles<T, NX> tiles[W];
   const int g = blockIdx.x * W + (threadIdx.x >> 5);
   if (g >= ((lv.n[0] + 31) >> 5)) return;  // whole warps
@@ -655,6 +660,7 @@ __global__ void __launch_bounds__(32 * W) k_sw_up0(const T* __restrict__ Dn, con
 
 template <typename T, int NX, int DIR, int W>
 __global__ void __launch_bounds__(32 * W) k_sw_upL(Levels<T> lv, int l) {
+  pdl_wait();
   const int b = blockIdx.x * W + (threadIdx.x >> 5);
   if (b >= ((lv.n[l] + 31) >> 5)) return;
   sw_upL_warp<T, NX, DIR>(b, lv, l);
@@ -664,6 +670,7 @@ template <typename T, int NX, int DIR, int W>
 __global__ void __launch_bounds__(32 * W) k_sw_down0(const T* __restrict__ Dn, const T* __restrict__ Y, const T* __restrict__ G, int64_t P,
                                                      int64_t L, const T* __restrict__ w, T s, Levels<T> lv,
                                                      T* __restrict__ out, T* __restrict__ bout) {
+  pdl_wait();
   __shared__ SweepTiles<T, NX> tiles[W];
   const int g = blockIdx.x * W + (threadIdx.x >> 5);
   if (g >= ((lv.n[0] + 31) >> 5)) return;  // whole warps
@@ -679,6 +686,7 @@ template <typename T, int NX, int DIR>
 __global__ void __launch_bounds__(32 * SW1_MAXW) k_sw_one(const T* __restrict__ Dn, const T* __restrict__ Y, const T* __restrict__ G,
                                                           int64_t P, int64_t L, const T* __restrict__ w, T s,
                                                           Levels<T> lv, T* __restrict__ out, T* __restrict__ bout) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char sw1_smem[];
   SweepTiles<T, NX>* tiles = reinterpret_cast<SweepTiles<T, NX>*>(sw1_smem);
   const int warp = threadIdx.x >> 5;
@@ -744,15 +752,12 @@ template <typename T, int NX, int DIR, int W>
 static bk_status run_sweep_multi(Problem* pr, OpData& d, const T* Y, const T* G, T* out, T* bout, const T* w, T s,
                                  const Levels<T>& lv, cudaStream_t st) {
   const int g0 = (((pr->lvn[0] + 31) >> 5) + W - 1) / W;
-  k_sw_up0<T, NX, DIR, W><<<g0, 32 * W, 0, st>>>((const T*)d.Dn, Y, G, pr->P, pr->L, w, s, lv);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_sw_up0<T, NX, DIR, W>, g0, 32 * W, 0, st, (const T*)d.Dn, Y, G, pr->P, pr->L, w, s, lv));
   for (int l = 1; l < pr->nlev; ++l) {
     const int gl = (((pr->lvn[l] + 31) >> 5) + W - 1) / W;
-    k_sw_upL<T, NX, DIR, W><<<gl, 32 * W, 0, st>>>(lv, l);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_sw_upL<T, NX, DIR, W>, gl, 32 * W, 0, st, lv, l));
   }
-  k_sw_down0<T, NX, DIR, W><<<g0, 32 * W, 0, st>>>((const T*)d.Dn, Y, G, pr->P, pr->L, w, s, lv, out, bout);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_sw_down0<T, NX, DIR, W>, g0, 32 * W, 0, st, (const T*)d.Dn, Y, G, pr->P, pr->L, w, s, lv, out, bout));
   return BK_OK;
 }
 
@@ -774,9 +779,8 @@ static bk_status run_sweep(Problem* pr, OpData& d, const T* Y, const T* G, T* ou
   if (form == 1 && !(pr->nlev <= 2 && nblk0 <= SW1_MAXW)) form = 0;
   if (form == 0) form = nblk0 < 4 * 152 ? 2 : 3;
   if (form == 1) {
-    k_sw_one<T, NX, DIR><<<1, 32 * nblk0, nblk0 * sizeof(SweepTiles<T, NX>), st>>>(
-        (const T*)d.Dn, Y, G, pr->P, pr->L, w, s, lv, out, bout);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_sw_one<T, NX, DIR>, 1, 32 * nblk0, nblk0 * sizeof(SweepTiles<T, NX>), st, 
+        (const T*)d.Dn, Y, G, pr->P, pr->L, w, s, lv, out, bout));
     return BK_OK;
   }
   if (form == 2) return run_sweep_multi<T, NX, DIR, 1>(pr, d, Y, G, out, bout, w, s, lv, st);
@@ -791,6 +795,7 @@ static bk_status run_sweep(Problem* pr, OpData& d, const T* Y, const T* G, T* ou
 template <typename T, int KIND>
 __global__ void k_jvp(const T* __restrict__ xu, const T* __restrict__ dX, const T* __restrict__ dU, int64_t P,
                       int64_t L, T* __restrict__ t, T pa, const T* __restrict__ ds, T inv_s) {
+  pdl_wait();
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
   const T dss = ds ? ds[0] * inv_s : T(0);
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
@@ -822,6 +827,7 @@ __global__ void k_jvp(const T* __restrict__ xu, const T* __restrict__ dX, const 
 template <typename T, int NX>
 __global__ void k_state_post(const T* __restrict__ chi, const T* __restrict__ Bt, int64_t P, int64_t L,
                              T* __restrict__ out, const double* __restrict__ sdev) {
+  pdl_wait();
   const T s = sdev ? T(*sdev) : T(1);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < NX * P; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t k = i % P;
@@ -840,6 +846,7 @@ __global__ void k_kkt_post(const T* __restrict__ xu, const T* __restrict__ mu, c
                            int64_t L, TermSpec ts, T cost_uu, T* __restrict__ out, T pa, int64_t s_idx,
                            double* __restrict__ part, const double* __restrict__ sdev,
                            const T* __restrict__ hbar) {
+  pdl_wait();
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NV = NX + NU;
   __shared__ double red[32];
   // sdev: Bt and Mu arrive unscaled (B^a, B^aT products) and take the device time scale here;
@@ -941,6 +948,7 @@ __global__ void k_kkt_post(const T* __restrict__ xu, const T* __restrict__ mu, c
 // One block: *out = scale * sum of n partials (fixed order).
 template <typename T>
 __global__ void k_free_finish(const double* __restrict__ part, int n, double scale, T* __restrict__ out) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a += part[i];
@@ -953,6 +961,7 @@ __global__ void k_free_finish(const double* __restrict__ part, int n, double sca
 template <typename T, int KIND>
 __global__ void k_border(const T* __restrict__ xu, const T* __restrict__ mu, const T* __restrict__ Baf, T inv_s,
                          int64_t P, int64_t L, T pa, T* __restrict__ a) {
+  pdl_wait();
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NV = NX + NU;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
     if (k < 32) a[(NV + NX) * P + k] = T(0);
@@ -991,6 +1000,7 @@ __global__ void k_border(const T* __restrict__ xu, const T* __restrict__ mu, con
 // f at the linearisation point, working type (padding left unwritten: products ignore it).
 template <typename T, int KIND>
 __global__ void k_fT(const T* __restrict__ xu, int64_t P, int64_t L, T pa, T* __restrict__ f) {
+  pdl_wait();
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
     T x[NXM], u[NUM], fx[NXM];
@@ -1007,6 +1017,7 @@ __global__ void k_fT(const T* __restrict__ xu, int64_t P, int64_t L, T pa, T* __
 // Partials of x . y over n elements (FP64 accumulation), one per block.
 template <typename T>
 __global__ void k_dot_part(const T* __restrict__ x, const T* __restrict__ y, int64_t n, double* __restrict__ part) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -1017,6 +1028,7 @@ __global__ void k_dot_part(const T* __restrict__ x, const T* __restrict__ y, int
 
 // gam[0] = 1 / sum(part) (the border's a . q), one block.
 __global__ void k_border_gamma(const double* __restrict__ part, int n, double* __restrict__ gam) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a += part[i];
@@ -1027,6 +1039,7 @@ __global__ void k_border_gamma(const double* __restrict__ part, int n, double* _
 // Bordered solve, step 2 (one block): ds = (a . t - r_s) / (a . q) into gam[1].
 template <typename T>
 __global__ void k_border_ds(const double* __restrict__ part, int n, const T* __restrict__ rs, double* __restrict__ gam) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a += part[i];
@@ -1038,6 +1051,7 @@ __global__ void k_border_ds(const double* __restrict__ part, int n, const T* __r
 template <typename T>
 __global__ void k_border_fix(const T* __restrict__ q, const double* __restrict__ gam, int64_t n, int64_t s_idx,
                              T* __restrict__ y) {
+  pdl_wait();
   const T ds = (T)gam[1];
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = i == s_idx ? ds : y[i] - ds * q[i];
@@ -1052,6 +1066,7 @@ __global__ void k_pre_u(const T* __restrict__ xu, const T* __restrict__ w, T s, 
                         const T* __restrict__ b, int64_t P, int64_t L, T* __restrict__ yu, T* __restrict__ g,
                         T gsign, const T* __restrict__ mu, T pa, const double* __restrict__ sdev,
                         const T* __restrict__ hbar) {
+  pdl_wait();
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
   if (sdev) s = T(*sdev);
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
@@ -1116,6 +1131,7 @@ __global__ void k_pre_u(const T* __restrict__ xu, const T* __restrict__ w, T s, 
 template <typename T>
 __global__ void k_pre_nu(const T* __restrict__ q, const T* __restrict__ rnu, const T* __restrict__ Sinv, int64_t P,
                          int64_t L, TermSpec ts, T* __restrict__ ynu) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   T rhs[NEM];
   for (int r = 0; r < ts.n_e; ++r) rhs[r] = T(ts.ea[r]) * q[ts.idx[r] * P + (L - 1)] - rnu[r];
@@ -1132,6 +1148,7 @@ template <typename T, int NX, int NU>
 __global__ void k_pre_fix(const T* __restrict__ Zc, const T* __restrict__ HWc, const T* __restrict__ Qc,
                           const T* __restrict__ ynu, int n_e, int64_t P, int64_t L, T* __restrict__ yx,
                           T* __restrict__ yu, T* __restrict__ yl) {
+  pdl_wait();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
     // the node's outputs stay in registers over the n_e columns (one read and one write each)
     T ax[NX], al[NX], au[NU];
@@ -1158,6 +1175,7 @@ __global__ void k_pre_fix(const T* __restrict__ Zc, const T* __restrict__ HWc, c
 
 template <typename T>
 __global__ void k_unit(T* v, int64_t n, int64_t idx) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     v[i] = i == idx ? T(1) : T(0);
 }
@@ -1167,6 +1185,7 @@ __global__ void k_unit(T* v, int64_t n, int64_t idx) {
 // ---------------------------------------------------------------------------------------------
 template <int KIND>
 __global__ void k_feval(const double* __restrict__ z, int64_t P, int64_t L, double* __restrict__ fout, double pa) {
+  pdl_wait();
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
     if (k >= L) {
@@ -1195,6 +1214,7 @@ __global__ void k_resid_post(const double* __restrict__ z, const double* __restr
                              const double* __restrict__ Bf, const double* __restrict__ Mu, int64_t P, int64_t L,
                              TermSpec ts, X0Spec x0, double cost_uu, double* __restrict__ F,
                              double* __restrict__ partial, double pa, double* __restrict__ partial2, BarSpec bs) {
+  pdl_wait();
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NV = NX + NU;
   __shared__ double red[32];
   const double* X = z;
@@ -1299,6 +1319,7 @@ __global__ void k_resid_post(const double* __restrict__ z, const double* __restr
 // squared weighted norm sum(partial) + g_s^2 into out.
 __global__ void k_resid_free(const double* __restrict__ partial, const double* __restrict__ partial2, int n,
                              double inv_s, double* __restrict__ Fs, double* __restrict__ out) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0, b = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) { a += partial[i]; b += partial2[i]; }
@@ -1315,6 +1336,7 @@ __global__ void k_resid_free(const double* __restrict__ partial, const double* _
 template <int NX, int NU>
 __global__ void k_wnorm(const double* __restrict__ F, const double* __restrict__ w, int64_t P, int64_t L, int n_e,
                         double* __restrict__ partial) {
+  pdl_wait();
   constexpr int NV = NX + NU;
   __shared__ double red[32];
   double acc = 0.0;
@@ -1332,6 +1354,7 @@ __global__ void k_wnorm(const double* __restrict__ F, const double* __restrict__
 }
 
 __global__ void k_sum_partials(const double* __restrict__ partial, int n, double* __restrict__ out) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a += partial[i];
@@ -1414,6 +1437,7 @@ static void free_opdata(OpData& d) {
 template <typename T, int NU>
 __global__ void k_lin_bar(const double* __restrict__ z, const double* __restrict__ w, double s, int64_t P, int64_t L,
                           int nx, BarSpec b, T* __restrict__ hbar) {
+  pdl_wait();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
     if (k >= L) {
 #pragma unroll
@@ -1447,12 +1471,10 @@ static const T* bar_hbar(const Problem* pr, const OpData& d) {
 // Segment maps and scan levels from the node factors N_k (level data of the sweeps).
 template <typename T, int NX>
 static bk_status lin_levels(Problem* pr, OpData& d, cudaStream_t st) {
-  k_lin_seg<T, NX><<<(pr->nseg + 127) / 128, 128, 0, st>>>((const T*)d.Dn, pr->L, pr->nseg, (T*)d.lvm[0]);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_lin_seg<T, NX>, (pr->nseg + 127) / 128, 128, 0, st, (const T*)d.Dn, pr->L, pr->nseg, (T*)d.lvm[0]));
   for (int l = 0; l < pr->nlev; ++l) {
-    k_lin_level<T, NX><<<(pr->lvn[l] + 31) / 32, 32, 0, st>>>((T*)d.lvm[l], pr->lvn[l],
-                                                              l + 1 < pr->nlev ? (T*)d.lvm[l + 1] : nullptr);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_lin_level<T, NX>, (pr->lvn[l] + 31) / 32, 32, 0, st, (T*)d.lvm[l], pr->lvn[l],
+                                                              l + 1 < pr->nlev ? (T*)d.lvm[l + 1] : nullptr));
   }
   return BK_OK;
 }
@@ -1460,14 +1482,14 @@ static bk_status lin_levels(Problem* pr, OpData& d, cudaStream_t st) {
 template <typename T, int KIND>
 static bk_status lin_factors(Problem* pr, OpData& d, const double* z, cudaStream_t st) {
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
-  k_lin_nodes<T, KIND, NX, NU><<<nblk(pr->L), 256, 0, st>>>(z, pr->P, pr->L, pr->d64.plan->w64, pr->s, (T*)d.Dn, (T*)d.xu,
-                                                             pr->dyn_param());
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_lin_nodes<T, KIND, NX, NU>, nblk(pr->L), 256, 0, st, z, pr->P, pr->L, pr->d64.plan->w64, pr->s, (T*)d.Dn, (T*)d.xu,
+                                                             pr->dyn_param()));
   return lin_levels<T, NX>(pr, d, st);
 }
 
 template <typename T>
 __global__ void k_negate(T* v, int64_t n) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) v[i] = -v[i];
 }
 
@@ -1487,25 +1509,21 @@ static bk_status lin_schur_launch(Problem* pr, OpData& d, cudaStream_t st) {
   T* bz = (T*)d.t2;     // n_x * P : B-tilde^T Z_r
   T* g = (T*)d.t3;      // n_x * P : forcing
   for (int r = 0; r < ne; ++r) {
-    k_unit<T><<<nblk(NX * P), 256, 0, st>>>(unit, NX * P, (int64_t)pr->term_idx[r] * P + (L - 1));
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_unit<T>, nblk(NX * P), 256, 0, st, unit, NX * P, (int64_t)pr->term_idx[r] * P + (L - 1)));
     T* Z = Zc + (int64_t)r * NX * P;
     BK_TRY((run_sweep<T, NX, 1>(pr, d, unit, nullptr, Z, bz, st)));
     // W = Pu^T Z = -s Ju^T (B-tilde^T Z). k_pre_u with r_u = 0 and b = B-tilde^T Z gives
     // yu = s Ju^T b / (s w) = -H~^{-1} W and g = Ju yu = -Ju H~^{-1} W.
     T* HW = HWc + (int64_t)r * NU * P;
-    k_pre_u<T, KIND><<<nblk(P), 256, 0, st>>>((const T*)d.xu, (const T*)d.w, s, (T)1, nullptr, bz, P, L, HW, g, T(1),
-                                              (const T*)d.mu, (T)pr->dyn_param(), nullptr, bar_hbar<T>(pr, d));
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_pre_u<T, KIND>, nblk(P), 256, 0, st, (const T*)d.xu, (const T*)d.w, s, (T)1, nullptr, bz, P, L, HW, g, T(1),
+                                              (const T*)d.mu, (T)pr->dyn_param(), nullptr, bar_hbar<T>(pr, d)));
     // Q = P^{-1} Pu HW: forward sweep with Y = 0 and forcing -Ju HW = Ju (-HW) = g
-    k_unit<T><<<nblk(NX * P), 256, 0, st>>>(unit, NX * P, -1);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_unit<T>, nblk(NX * P), 256, 0, st, unit, NX * P, -1));
     T* Q = Qc + (int64_t)r * NX * P;
     BK_TRY((run_sweep<T, NX, 0>(pr, d, unit, g, Q, nullptr, st)));
   }
   // HWc holds -H~^{-1} W: negate it
-  k_negate<T><<<nblk((int64_t)ne * NU * P), 256, 0, st>>>(HWc, (int64_t)ne * NU * P);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_negate<T>, nblk((int64_t)ne * NU * P), 256, 0, st, HWc, (int64_t)ne * NU * P));
   // S = E Q: S[r][c] = Q_c[term_idx[r]][N], into pinned host memory
   T* hq = reinterpret_cast<T*>(pr->red_host + 256);
   for (int c = 0; c < ne; ++c)
@@ -1559,6 +1577,7 @@ static bk_status lin_border(Problem* pr, OpData& d, cudaStream_t st);
 // x_{idx_r}(t_f) and nu_r of a KKT vector (one thread)
 __global__ void k_term_vals(const double* __restrict__ z, int64_t P, int64_t L, int64_t nu_off, TermSpec ts,
                             double* __restrict__ out) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   for (int r = 0; r < ts.n_e; ++r) {
     out[r] = z[ts.idx[r] * P + (L - 1)];
@@ -1572,8 +1591,7 @@ static bk_status lin_end_rows(Problem* pr, const double* z, cudaStream_t st) {
   const TermSpec ts = term_spec(pr);
   double* dv = pr->red + 1800;
   double* hv = pr->red_host + 320;
-  k_term_vals<<<1, 32, 0, st>>>(z, pr->P, pr->L, (int64_t)(2 * pr->n_x + pr->n_u) * pr->P, ts, dv);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_term_vals, 1, 32, 0, st, z, pr->P, pr->L, (int64_t)(2 * pr->n_x + pr->n_u) * pr->P, ts, dv));
   BK_TRY_CUDA(cudaMemcpyAsync(hv, dv, sizeof(double) * 2 * NEM, cudaMemcpyDeviceToHost, st));
   BK_TRY_CUDA(cudaStreamSynchronize(st));
   for (int r = 0; r < pr->n_e; ++r) {
@@ -1614,22 +1632,18 @@ static bk_status linearize_kind(Problem* pr, const double* z, const double* mu, 
   else
     BK_TRY_CUDA(cudaMemcpyAsync(pr->d64.xu, z, sizeof(double) * (NX + NU) * P, cudaMemcpyDeviceToDevice, st));
   if (pr->d32.plan) {
-    k_convert<double, float><<<nblk(NX * P), 256, 0, st>>>((const double*)pr->d64.mu, (float*)pr->d32.mu, NX * P);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_convert<double, float>, nblk(NX * P), 256, 0, st, (const double*)pr->d64.mu, (float*)pr->d32.mu, NX * P));
     if (keep != LIN_KEEP_PRECOND) {
       BK_TRY((lin_factors<float, KIND>(pr, pr->d32, z, st)));
     } else {
-      k_convert<double, float><<<nblk((NX + NU) * P), 256, 0, st>>>(z, (float*)pr->d32.xu, (NX + NU) * P);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_convert<double, float>, nblk((NX + NU) * P), 256, 0, st, z, (float*)pr->d32.xu, (NX + NU) * P));
     }
   }
   if (pr->has_ubounds && pr->bar_mu > 0.0) {
     const BarSpec b = bar_spec(pr);
-    k_lin_bar<double, NU><<<nblk(P), 256, 0, st>>>(z, pr->d64.plan->w64, pr->s, P, pr->L, NX, b, (double*)pr->d64.hbar);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_lin_bar<double, NU>, nblk(P), 256, 0, st, z, pr->d64.plan->w64, pr->s, P, pr->L, NX, b, (double*)pr->d64.hbar));
     if (pr->d32.plan) {
-      k_lin_bar<float, NU><<<nblk(P), 256, 0, st>>>(z, pr->d64.plan->w64, pr->s, P, pr->L, NX, b, (float*)pr->d32.hbar);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_lin_bar<float, NU>, nblk(P), 256, 0, st, z, pr->d64.plan->w64, pr->s, P, pr->L, NX, b, (float*)pr->d32.hbar));
     }
   }
   pr->linearized = true;
@@ -1661,32 +1675,27 @@ static bk_status apply_typed(Problem* pr, OpData& d, int op, const T* in, T* out
   T* t3 = (T*)d.t3;
   if (op == BK_OP_STATE) {
     // the product ignores t1's padding (elements L..P-1), so it is never written
-    k_jvp<T, KIND><<<nblk(L), 256, 0, st>>>((const T*)d.xu, in, nullptr, P, L, t1, (T)pr->dyn_param(), nullptr, T(0));
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_jvp<T, KIND>, nblk(L), 256, 0, st, (const T*)d.xu, in, nullptr, P, L, t1, (T)pr->dyn_param(), nullptr, T(0)));
     const double* sd = sdev_of(pr);
     BK_TRY(plan_apply_n(d.plan, t1, t2, NX, false, sd ? 1.0 : pr->s, st));
-    k_state_post<T, NX><<<nblk(NX * P), 256, 0, st>>>(in, t2, P, L, out, sd);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_state_post<T, NX>, nblk(NX * P), 256, 0, st, in, t2, P, L, out, sd));
     return BK_OK;
   }
   const bool ft = pr->free_time;
   const T pa = (T)pr->dyn_param();
-  k_jvp<T, KIND><<<nblk(L), 256, 0, st>>>((const T*)d.xu, in, in + NX * P, P, L, t1, pa,
-                                          ft ? in + pr->s_idx() : nullptr, (T)(1.0 / pr->s));
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_jvp<T, KIND>, nblk(L), 256, 0, st, (const T*)d.xu, in, in + NX * P, P, L, t1, pa,
+                                          ft ? in + pr->s_idx() : nullptr, (T)(1.0 / pr->s)));
   // fixed final time: both products unscaled, k_kkt_post applies s from the device (so that a
   // captured GMRES step does not hold s); free final time: s (which changes within a step) by value
   const double* sd = sdev_of(pr);
   BK_TRY(plan_apply_n(d.plan, t1, t2, NX, false, sd ? 1.0 : pr->s, st));
   T* Mu = mu_out ? mu_out : t3;
   BK_TRY(plan_apply_n(d.plan, in + (NX + NU) * P, Mu, NX, true, sd ? 1.0 : pr->s, st));
-  k_kkt_post<T, KIND><<<ft ? FT_NB : nblk(P), 256, 0, st>>>((const T*)d.xu, (const T*)d.mu, (const T*)d.w, (T)pr->s, in,
+  BK_TRY(launch(k_kkt_post<T, KIND>, ft ? FT_NB : nblk(P), 256, 0, st, (const T*)d.xu, (const T*)d.mu, (const T*)d.w, (T)pr->s, in,
                                                             t2, Mu, P, L, term_spec(pr), (T)pr->cost_uu(), out, pa,
-                                                            pr->s_idx(), ft ? pr->sred : nullptr, sd, bar_hbar<T>(pr, d));
-  BK_CHECK_LAUNCH();
+                                                            pr->s_idx(), ft ? pr->sred : nullptr, sd, bar_hbar<T>(pr, d)));
   if (ft) {
-    k_free_finish<T><<<1, 256, 0, st>>>(pr->sred, FT_NB, -1.0 / pr->s, out + pr->s_idx());
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_free_finish<T>, 1, 256, 0, st, pr->sred, FT_NB, -1.0 / pr->s, out + pr->s_idx()));
   }
   return BK_OK;
 }
@@ -1733,15 +1742,12 @@ static bk_status precond_typed(Problem* pr, OpData& d, int op, const T* in, T* o
   T* b = (T*)d.t1;
   T* g = (T*)d.t2;
   BK_TRY((run_sweep<T, NX, 1>(pr, d, rx, nullptr, yl, b, st)));
-  k_pre_u<T, KIND><<<nblk(P), 256, 0, st>>>((const T*)d.xu, (const T*)d.w, (T)pr->s, (T)1, ru, b, P, L, yu, g, T(1),
-                                            (const T*)d.mu, (T)pr->dyn_param(), sdev_of(pr), bar_hbar<T>(pr, d));
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_pre_u<T, KIND>, nblk(P), 256, 0, st, (const T*)d.xu, (const T*)d.w, (T)pr->s, (T)1, ru, b, P, L, yu, g, T(1),
+                                            (const T*)d.mu, (T)pr->dyn_param(), sdev_of(pr), bar_hbar<T>(pr, d)));
   BK_TRY((run_sweep<T, NX, 0>(pr, d, rl, g, yx, nullptr, st)));
   if (pr->n_e > 0) {
-    k_pre_nu<T><<<1, 32, 0, st>>>(yx, rnu, (const T*)d.Sinv, P, L, term_spec(pr), ynu);
-    BK_CHECK_LAUNCH();
-    k_pre_fix<T, NX, NU><<<nblk(L), 256, 0, st>>>((const T*)d.Zc, (const T*)d.HWc, (const T*)d.Qc, ynu, pr->n_e, P, L, yx, yu, yl);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_pre_nu<T>, 1, 32, 0, st, yx, rnu, (const T*)d.Sinv, P, L, term_spec(pr), ynu));
+    BK_TRY(launch(k_pre_fix<T, NX, NU>, nblk(L), 256, 0, st, (const T*)d.Zc, (const T*)d.HWc, (const T*)d.Qc, ynu, pr->n_e, P, L, yx, yu, yl));
   } else {
     BK_TRY_CUDA(cudaMemsetAsync(ynu, 0, sizeof(T) * 32, st));
   }
@@ -1749,12 +1755,9 @@ static bk_status precond_typed(Problem* pr, OpData& d, int op, const T* in, T* o
     // bordered by the s row and column a (zero diagonal): with t = K-tilde^{-1} r (above) and
     // q = K-tilde^{-1} a, ds = (a . t - r_s) / (a . q), y = t - ds q, y_s = ds
     const int64_t n = pr->kkt_len();
-    k_dot_part<T><<<FT_NB, 256, 0, st>>>((const T*)d.brd, out, n, pr->sred);
-    BK_CHECK_LAUNCH();
-    k_border_ds<T><<<1, 256, 0, st>>>(pr->sred, FT_NB, in + pr->s_idx(), d.bgam);
-    BK_CHECK_LAUNCH();
-    k_border_fix<T><<<nblk(n), 256, 0, st>>>((const T*)d.brq, d.bgam, n, pr->s_idx(), out);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_dot_part<T>, FT_NB, 256, 0, st, (const T*)d.brd, out, n, pr->sred));
+    BK_TRY(launch(k_border_ds<T>, 1, 256, 0, st, pr->sred, FT_NB, in + pr->s_idx(), d.bgam));
+    BK_TRY(launch(k_border_fix<T>, nblk(n), 256, 0, st, (const T*)d.brq, d.bgam, n, pr->s_idx(), out));
   }
   return BK_OK;
 }
@@ -1767,17 +1770,13 @@ static bk_status lin_border(Problem* pr, OpData& d, cudaStream_t st) {
   const int64_t P = pr->P, L = pr->L;
   T* f = (T*)d.t1;
   T* Baf = (T*)d.t2;
-  k_fT<T, KIND><<<nblk(L), 256, 0, st>>>((const T*)d.xu, P, L, (T)pr->dyn_param(), f);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_fT<T, KIND>, nblk(L), 256, 0, st, (const T*)d.xu, P, L, (T)pr->dyn_param(), f));
   BK_TRY(plan_apply_n(d.plan, f, Baf, NX, false, 1.0, st));
-  k_border<T, KIND><<<nblk(P), 256, 0, st>>>((const T*)d.xu, (const T*)d.mu, Baf, (T)(1.0 / pr->s), P, L,
-                                             (T)pr->dyn_param(), (T*)d.brd);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_border<T, KIND>, nblk(P), 256, 0, st, (const T*)d.xu, (const T*)d.mu, Baf, (T)(1.0 / pr->s), P, L,
+                                             (T)pr->dyn_param(), (T*)d.brd));
   BK_TRY((precond_typed<T, KIND>(pr, d, BK_OP_KKT, (const T*)d.brd, (T*)d.brq, 0, st, false)));
-  k_dot_part<T><<<FT_NB, 256, 0, st>>>((const T*)d.brd, (const T*)d.brq, pr->kkt_len(), pr->sred);
-  BK_CHECK_LAUNCH();
-  k_border_gamma<<<1, 256, 0, st>>>(pr->sred, FT_NB, d.bgam);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_dot_part<T>, FT_NB, 256, 0, st, (const T*)d.brd, (const T*)d.brq, pr->kkt_len(), pr->sred));
+  BK_TRY(launch(k_border_gamma, 1, 256, 0, st, pr->sred, FT_NB, d.bgam));
   return BK_OK;
 }
 
@@ -1799,11 +1798,9 @@ bk_status op_precond(Problem* pr, OpData& d, int op, const void* in, void* out, 
   // FP64 vectors, FP32 preconditioner: round the input, apply in FP32, widen the result
   BK_ARG(d.dtype == BK_F64 && pr->pdtype == BK_F32 && pr->pcin, "preconditioner precision mismatch");
   const int64_t n = op == BK_OP_KKT ? pr->kkt_len() : pr->state_len();
-  k_convert<double, float><<<nblk(n), 256, 0, st>>>((const double*)in, (float*)pr->pcin, n);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_convert<double, float>, nblk(n), 256, 0, st, (const double*)in, (float*)pr->pcin, n));
   BK_TRY(op_precond_direct(pr, pr->d32, op, pr->pcin, pr->pcout, transpose, st));
-  k_convert<float, double><<<nblk(n), 256, 0, st>>>((const float*)pr->pcout, (double*)out, n);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_convert<float, double>, nblk(n), 256, 0, st, (const float*)pr->pcout, (double*)out, n));
   return BK_OK;
 }
 
@@ -1817,26 +1814,22 @@ static bk_status residual_launch(Problem* pr, const double* z, double* F, bool w
   double* f = (double*)d.t1;
   double* Bf = (double*)d.t2;
   if (!Mu) Mu = (double*)d.t3;
-  k_feval<KIND><<<nblk(P), 256, 0, st>>>(z, P, L, f, pr->dyn_param());
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_feval<KIND>, nblk(P), 256, 0, st, z, P, L, f, pr->dyn_param()));
   BK_TRY(plan_apply_n(d.plan, f, Bf, NX, false, pr->s, st));
   if (!mu_given) BK_TRY(plan_apply_n(d.plan, z + (NX + NU) * P, Mu, NX, true, pr->s, st));
   X0Spec x0;
   for (int m = 0; m < NXM; ++m) x0.x0[m] = pr->x0[m];
   const int nb = 592;
-  k_resid_post<KIND><<<nb, 256, 0, st>>>(z, pr->d64.plan->w64, pr->s, Bf, Mu, P, L, term_spec(pr), x0,
+  BK_TRY(launch(k_resid_post<KIND>, nb, 256, 0, st, z, pr->d64.plan->w64, pr->s, Bf, Mu, P, L, term_spec(pr), x0,
                                          pr->cost_uu(), F, pr->red, pr->dyn_param(),
-                                         pr->free_time ? pr->sred : nullptr, bar_spec(pr));
-  BK_CHECK_LAUNCH();
+                                         pr->free_time ? pr->sred : nullptr, bar_spec(pr)));
   if (pr->free_time) {
     // the time gradient g_s goes into F whether or not the norm is wanted
-    k_resid_free<<<1, 256, 0, st>>>(pr->red, pr->sred, nb, 1.0 / pr->s, F + pr->s_idx(), pr->red + 1024);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_resid_free, 1, 256, 0, st, pr->red, pr->sred, nb, 1.0 / pr->s, F + pr->s_idx(), pr->red + 1024));
     if (want_norm)
       BK_TRY_CUDA(cudaMemcpyAsync(pr->red_host, pr->red + 1024, sizeof(double), cudaMemcpyDeviceToHost, st));
   } else if (want_norm) {
-    k_sum_partials<<<1, 256, 0, st>>>(pr->red, nb, pr->red + 1024);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_sum_partials, 1, 256, 0, st, pr->red, nb, pr->red + 1024));
     BK_TRY_CUDA(cudaMemcpyAsync(pr->red_host, pr->red + 1024, sizeof(double), cudaMemcpyDeviceToHost, st));
   }
   return BK_OK;
@@ -1869,10 +1862,8 @@ static bk_status wnorm_kind(Problem* pr, const double* F, double* wnorm, cudaStr
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
   const int nb = 592;
   // the tail holds e and, for a free final time, g_s right after it
-  k_wnorm<NX, NU><<<nb, 256, 0, st>>>(F, pr->d64.plan->w64, pr->P, pr->L, pr->n_e + (pr->free_time ? 1 : 0), pr->red);
-  BK_CHECK_LAUNCH();
-  k_sum_partials<<<1, 256, 0, st>>>(pr->red, nb, pr->red + 1024);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_wnorm<NX, NU>, nb, 256, 0, st, F, pr->d64.plan->w64, pr->P, pr->L, pr->n_e + (pr->free_time ? 1 : 0), pr->red));
+  BK_TRY(launch(k_sum_partials, 1, 256, 0, st, pr->red, nb, pr->red + 1024));
   BK_TRY_CUDA(cudaMemcpyAsync(pr->red_host, pr->red + 1024, sizeof(double), cudaMemcpyDeviceToHost, st));
   BK_TRY_CUDA(cudaStreamSynchronize(st));
   *wnorm = sqrt(pr->red_host[0]);
@@ -2036,6 +2027,7 @@ static bk_status sync_time_scale(Problem* pr, const double* z, cudaStream_t st) 
 // pitch): X and lambda copied, u = atan2(u_r, u_theta) (the thrust direction as the angle of
 // a (sin u, cos u)), nu copied, s from the minimum-energy problem.
 __global__ void k_seed_mt(const double* __restrict__ zme, int64_t P, int64_t L, double s, double* __restrict__ zmt) {
+  pdl_wait();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -2048,6 +2040,7 @@ __global__ void k_seed_mt(const double* __restrict__ zme, int64_t P, int64_t L, 
 }
 
 __global__ void k_scale64(double* __restrict__ v, int64_t n, double a) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     v[i] *= a;
 }
@@ -2060,8 +2053,7 @@ static bk_status min_time_seed(Problem* mt, const Problem* me, const double* z_m
   BK_ARG(mt->N == me->N && mt->P == me->P, "the two problems must have the same N");
   BK_ARG(mt->t0 == me->t0, "the two problems must start at the same t0");
   const int64_t P = mt->P;
-  k_seed_mt<<<nblk(P), 256, 0, st>>>(z_me, P, mt->L, me->s, z_mt);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_seed_mt, nblk(P), 256, 0, st, z_me, P, mt->L, me->s, z_mt));
   mt->s = me->s;
   double wn = 0.0;
   BK_TRY(problem_residual(mt, z_mt, mt->F, &wn, st));
@@ -2073,8 +2065,7 @@ static bk_status min_time_seed(Problem* mt, const Problem* me, const double* z_m
     set_error("minimum-energy multipliers give a non-positive time gradient (%g)", S);
     return BK_ERR_ARG;
   }
-  k_scale64<<<nblk(4 * P + 3), 256, 0, st>>>(z_mt + 5 * P, 4 * P + 3, 2.0 / S);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_scale64, nblk(4 * P + 3), 256, 0, st, z_mt + 5 * P, 4 * P + 3, 2.0 / S));
   BK_TRY_CUDA(cudaStreamSynchronize(st));
   return BK_OK;
 }

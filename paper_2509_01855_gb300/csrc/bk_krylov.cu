@@ -230,6 +230,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_multidot(const T* __restrict__ V, int64_t ld, int nv, const T* __restrict__ w,
                                                   int64_t n, double* __restrict__ partial, double* __restrict__ out,
                                                   unsigned* __restrict__ cnt) {
+  pdl_wait();
   multidot_body<T>(V, ld, nv, w, n, partial, out, cnt);
 }
 
@@ -371,6 +372,7 @@ __global__ void __launch_bounds__(256) k_multiaxpy(const T* __restrict__ V, int6
                                                    double alpha, int64_t n, double* __restrict__ partial,
                                                    double* __restrict__ sq_out = nullptr,
                                                    unsigned* __restrict__ cnt = nullptr) {
+  pdl_wait();
   multiaxpy_body<T>(V, ld, nv, c, cscale, w, alpha, n, partial, sq_out, cnt);
 }
 
@@ -392,6 +394,7 @@ struct GmState {
 };
 
 __global__ void k_gm_init(GmState* s, double beta, double target, int jmax, int m) {
+  pdl_wait();
   const int t = threadIdx.x;
   if (t == 0) {
     s->j = 0;
@@ -412,6 +415,7 @@ __global__ void __launch_bounds__(256) k_multidot_s(const T* __restrict__ V, int
                                                     const GmState* __restrict__ s, const int* __restrict__ gate,
                                                     int64_t n, double* __restrict__ partial, double* __restrict__ out,
                                                     unsigned* __restrict__ cnt) {
+  pdl_wait();
   if (gate && *gate == 0) return;
   const int j = s->j;
   multidot_body<T>(V, ld, j + add, V + (int64_t)(j + woff) * ld, n, partial, out, cnt);
@@ -426,6 +430,7 @@ __global__ void __launch_bounds__(256) k_multiaxpy_s(const T* __restrict__ V, in
                                                      double cscale, double alpha, int64_t n,
                                                      double* __restrict__ partial, double* __restrict__ sq_out,
                                                      unsigned* __restrict__ cnt) {
+  pdl_wait();
   if (gate && *gate == 0) return;
   const int j = s->j;
   T* w = woff >= 0 ? const_cast<T*>(V) + (int64_t)(j + woff) * ld : x;
@@ -435,6 +440,7 @@ __global__ void __launch_bounds__(256) k_multiaxpy_s(const T* __restrict__ V, in
 // After the first Gram-Schmidt pass: column j of H from h = V^T w, and the DGKS test (|w|^2
 // after the pass below half of |w|^2 before it).
 __global__ void k_gm_a(GmState* s, const double* __restrict__ h1, const double* __restrict__ w2) {
+  pdl_wait();
   const int j = s->j, m = s->m;
   for (int i = threadIdx.x; i <= j; i += blockDim.x) s->H[i * m + j] = h1[i];
   if (threadIdx.x == 0) s->need2 = w2[0] < 0.5 * h1[j + 1] ? 1 : 0;
@@ -444,6 +450,7 @@ __global__ void k_gm_a(GmState* s, const double* __restrict__ h1, const double* 
 // the residual estimate and the stop test; j advances. In a graph, the WHILE condition follows.
 __global__ void k_gm_b(GmState* s, const double* __restrict__ h2, const double* __restrict__ w2,
                        cudaGraphConditionalHandle cond, int in_graph) {
+  pdl_wait();
   if (threadIdx.x != 0) return;
   const int j = s->j, m = s->m;
   double* H = s->H;
@@ -479,6 +486,7 @@ __global__ void k_gm_b(GmState* s, const double* __restrict__ h2, const double* 
 // V_j <- V_j / hn (j after k_gm_b, i.e. the new basis vector), unless hn == 0.
 template <typename T>
 __global__ void k_scale_inv_s(T* __restrict__ V, int64_t ld, const GmState* __restrict__ s, int64_t n) {
+  pdl_wait();
   const double hn = s->hn;
   if (!(hn > 0.0)) return;
   T* v = V + (int64_t)s->j * ld;
@@ -489,6 +497,7 @@ __global__ void k_scale_inv_s(T* __restrict__ V, int64_t ld, const GmState* __re
 
 // y = H(0:j, 0:j)^{-1} g (back substitution, one thread).
 __global__ void k_gm_solve(GmState* s) {
+  pdl_wait();
   if (threadIdx.x != 0) return;
   const int j = s->j, m = s->m;
   for (int i = j - 1; i >= 0; --i) {
@@ -502,6 +511,7 @@ __global__ void k_gm_solve(GmState* s) {
 template <typename T>
 __global__ void k_gm_pick(const T* __restrict__ V, int64_t ld, const GmState* __restrict__ s, T* __restrict__ dst,
                           int64_t n) {
+  pdl_wait();
   const T* v = V + (int64_t)s->j * ld;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
     dst[k] = v[k];
@@ -512,6 +522,7 @@ template <typename T>
 __global__ void k_gm_place(T* __restrict__ V, T* __restrict__ Z, int64_t ld, const GmState* __restrict__ s,
                            const T* __restrict__ w, const T* __restrict__ z, int64_t n, double* __restrict__ Tr,
                            int64_t tld, const double* __restrict__ a, int64_t an) {
+  pdl_wait();
   const int j = s->j;
   T* vd = V + (int64_t)(j + 1) * ld;
   T* zd = Z ? Z + (int64_t)j * ld : nullptr;
@@ -528,6 +539,7 @@ __global__ void k_gm_place(T* __restrict__ V, T* __restrict__ Z, int64_t ld, con
 // y <- a * x + b * y  (a, b host scalars)
 template <typename T>
 __global__ void k_axpby(const T* __restrict__ x, double a, T* __restrict__ y, double b, int64_t n) {
+  pdl_wait();
   const T aa = (T)a, bb = (T)b;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
     y[k] = b == 0.0 ? aa * x[k] : aa * x[k] + bb * y[k];
@@ -536,6 +548,7 @@ __global__ void k_axpby(const T* __restrict__ x, double a, T* __restrict__ y, do
 // y <- x * (1 / c[0])  (scale by a device scalar)
 template <typename T>
 __global__ void k_scale_inv(const T* __restrict__ x, const double* __restrict__ c, T* __restrict__ y, int64_t n) {
+  pdl_wait();
   const T inv = (T)(1.0 / c[0]);
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
     y[k] = x[k] * inv;
@@ -544,8 +557,7 @@ __global__ void k_scale_inv(const T* __restrict__ x, const double* __restrict__ 
 template <typename T>
 static bk_status dots(const T* V, int64_t ld, int nv, const T* w, int64_t n, double* partial, double* out,
                       unsigned* cnt, cudaStream_t st) {
-  k_multidot<T><<<DOT_BLOCKS, 256, 0, st>>>(V, ld, nv, w, n, partial, out, cnt);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_multidot<T>, DOT_BLOCKS, 256, 0, st, V, ld, nv, w, n, partial, out, cnt));
   return BK_OK;
 }
 
@@ -572,6 +584,7 @@ size_t gmres_workspace_bytes(int64_t n, int m, int dtype) {
 template <typename T>
 __global__ void k_wscale(const T* __restrict__ in, T* __restrict__ out, const T* __restrict__ w, int64_t P,
                          int64_t L, int nz, int nl, int64_t n, int inv) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t blk = i / P, k = i - blk * P;
     T f = T(1);
@@ -619,15 +632,13 @@ static bk_status arnoldi_step(const GmCtx<T>& c, int jh, bool graph, cudaGraphCo
   const T* vin = c.V + (int64_t)jh * ld;
   if (graph) {
     T* dst = c.weighted ? c.r : c.z;
-    k_gm_pick<T><<<c.g, 256, 0, st>>>(c.V, ld, c.gs, dst, n);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_gm_pick<T>, c.g, 256, 0, st, c.V, ld, c.gs, dst, n));
     vin = dst;
   }
   if (c.precond) {
     T* zout = graph ? c.zc : c.Zb + (int64_t)jh * ld;
     if (c.weighted) {
-      k_wscale<T><<<c.g, 256, 0, st>>>(vin, c.z, (const T*)d.w, pr->P, pr->L, wz, wl, n, 1);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_wscale<T>, c.g, 256, 0, st, vin, c.z, (const T*)d.w, pr->P, pr->L, wz, wl, n, 1));
       BK_TRY(op_precond(pr, d, c.op, c.z, zout, 0, st));
     } else {
       BK_TRY(op_precond(pr, d, c.op, vin, zout, 0, st));
@@ -637,34 +648,25 @@ static bk_status arnoldi_step(const GmCtx<T>& c, int jh, bool graph, cudaGraphCo
     BK_TRY(op_apply(pr, d, c.op, vin, wout, st, aout));
   }
   if (c.weighted) {
-    k_wscale<T><<<c.g, 256, 0, st>>>(wout, wout, (const T*)d.w, pr->P, pr->L, wz, wl, n, 0);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_wscale<T>, c.g, 256, 0, st, wout, wout, (const T*)d.w, pr->P, pr->L, wz, wl, n, 0));
   }
   if (graph) {
-    k_gm_place<T><<<c.g, 256, 0, st>>>(c.V, c.precond ? c.Zb : nullptr, ld, c.gs, c.r, c.zc, n,
+    BK_TRY(launch(k_gm_place<T>, c.g, 256, 0, st, c.V, c.precond ? c.Zb : nullptr, ld, c.gs, c.r, c.zc, n,
                                        c.aux ? c.aux->T : nullptr, c.aux ? c.aux->ld : 0, c.ac,
-                                       c.aux ? c.aux->n : 0);
-    BK_CHECK_LAUNCH();
+                                       c.aux ? c.aux->n : 0));
   }
   // Gram-Schmidt (DGKS): h1 = [V_0..V_j]^T w and |w|^2 (w = V_{j+1}), w <- w - V h1 with the new
   // |w|^2; the second pass runs (its kernels do work) only when k_gm_a asked for it.
   double* w2 = c.h2 + (MAXM + 1);
-  k_multidot_s<T><<<DOT_BLOCKS, 256, 0, st>>>(c.V, ld, 2, 1, c.gs, nullptr, n, c.partial, c.h1, c.cnt);
-  BK_CHECK_LAUNCH();
-  k_multiaxpy_s<T><<<DOT_BLOCKS, 256, 0, st>>>(c.V, ld, 1, 1, nullptr, c.gs, nullptr, c.h1, -1.0, 1.0, n, c.partial,
-                                               w2, c.cnt + 1);
-  BK_CHECK_LAUNCH();
-  k_gm_a<<<1, 128, 0, st>>>(c.gs, c.h1, w2);
-  BK_CHECK_LAUNCH();
-  k_multidot_s<T><<<DOT_BLOCKS, 256, 0, st>>>(c.V, ld, 1, 1, c.gs, &c.gs->need2, n, c.partial, c.h2, c.cnt);
-  BK_CHECK_LAUNCH();
-  k_multiaxpy_s<T><<<DOT_BLOCKS, 256, 0, st>>>(c.V, ld, 1, 1, nullptr, c.gs, &c.gs->need2, c.h2, -1.0, 1.0, n,
-                                               c.partial, w2, c.cnt + 1);
-  BK_CHECK_LAUNCH();
-  k_gm_b<<<1, 32, 0, st>>>(c.gs, c.h2, w2, cond, graph ? 1 : 0);
-  BK_CHECK_LAUNCH();
-  k_scale_inv_s<T><<<c.g, 256, 0, st>>>(c.V, ld, c.gs, n);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_multidot_s<T>, DOT_BLOCKS, 256, 0, st, c.V, ld, 2, 1, c.gs, nullptr, n, c.partial, c.h1, c.cnt));
+  BK_TRY(launch(k_multiaxpy_s<T>, DOT_BLOCKS, 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, nullptr, c.h1, -1.0, 1.0, n, c.partial,
+                                               w2, c.cnt + 1));
+  BK_TRY(launch(k_gm_a, 1, 128, 0, st, c.gs, c.h1, w2));
+  BK_TRY(launch(k_multidot_s<T>, DOT_BLOCKS, 256, 0, st, c.V, ld, 1, 1, c.gs, &c.gs->need2, n, c.partial, c.h2, c.cnt));
+  BK_TRY(launch(k_multiaxpy_s<T>, DOT_BLOCKS, 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, &c.gs->need2, c.h2, -1.0, 1.0, n,
+                                               c.partial, w2, c.cnt + 1));
+  BK_TRY(launch(k_gm_b, 1, 32, 0, st, c.gs, c.h2, w2, cond, graph ? 1 : 0));
+  BK_TRY(launch(k_scale_inv_s<T>, c.g, 256, 0, st, c.V, ld, c.gs, n));
   return BK_OK;
 }
 
@@ -862,8 +864,7 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
   weighted = weighted && op == BK_OP_KKT && o.use_precond;
   const int wz = pr->n_x + pr->n_u, wl = pr->n_x;
   auto wscale = [&](const T* in, T* out, int inv) -> bk_status {
-    k_wscale<T><<<g, 256, 0, st>>>(in, out, (const T*)d.w, pr->P, pr->L, wz, wl, n, inv);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_wscale<T>, g, 256, 0, st, in, out, (const T*)d.w, pr->P, pr->L, wz, wl, n, inv));
     return BK_OK;
   };
   // the right-hand side the iteration sees: D b (weighted) or b
@@ -898,13 +899,11 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
     // r = b - A x (x = 0 on the first cycle)
     if (first) {
       if (!weighted) {  // weighted: r already holds D b
-        k_axpby<T><<<g, 256, 0, st>>>(b, 1.0, r, 0.0, n);
-        BK_CHECK_LAUNCH();
+        BK_TRY(launch(k_axpby<T>, g, 256, 0, st, b, 1.0, r, 0.0, n));
       }
     } else {
       BK_TRY(op_apply(pr, d, op, x, r, st));
-      k_axpby<T><<<g, 256, 0, st>>>(b, 1.0, r, -1.0, n);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_axpby<T>, g, 256, 0, st, b, 1.0, r, -1.0, n));
       if (weighted) BK_TRY(wscale(r, r, 0));
     }
     double beta = bnorm;  // r = b on the first cycle
@@ -917,11 +916,9 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
     first = false;
     resid = beta;
     if (beta <= target || total >= o.max_iter) break;
-    k_axpby<T><<<g, 256, 0, st>>>(r, 1.0 / beta, V, 0.0, n);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_axpby<T>, g, 256, 0, st, r, 1.0 / beta, V, 0.0, n));
     const int jmax = std::min(m, o.max_iter - total);
-    k_gm_init<<<1, 128, 0, st>>>(gs, beta, target, jmax, m);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_gm_init, 1, 128, 0, st, gs, beta, target, jmax, m));
     if (gg) {
       BK_TRY_CUDA(cudaGraphLaunch(gg->x, st));
     } else {
@@ -934,15 +931,12 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
       }
     }
     // x += Z y (flexible form; Z = V without preconditioning), y = H^{-1} g on the device
-    k_gm_solve<<<1, 32, 0, st>>>(gs);
-    BK_CHECK_LAUNCH();
-    k_multiaxpy_s<T><<<g, 256, 0, st>>>(o.use_precond ? Zb : V, ld, 0, -1, x, gs, nullptr, gs->y, 1.0, 1.0, n,
-                                        nullptr, nullptr, nullptr);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_gm_solve, 1, 32, 0, st, gs));
+    BK_TRY(launch(k_multiaxpy_s<T>, g, 256, 0, st, o.use_precond ? Zb : V, ld, 0, -1, x, gs, nullptr, gs->y, 1.0, 1.0, n,
+                                        nullptr, nullptr, nullptr));
     if (aux) {
-      k_multiaxpy_s<double><<<grid_for(aux->n), 256, 0, st>>>(aux->T, aux->ld, 0, -1, aux->Td, gs, nullptr, gs->y,
-                                                              1.0, 1.0, aux->n, nullptr, nullptr, nullptr);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_multiaxpy_s<double>, grid_for(aux->n), 256, 0, st, aux->T, aux->ld, 0, -1, aux->Td, gs, nullptr, gs->y,
+                                                              1.0, 1.0, aux->n, nullptr, nullptr, nullptr));
     }
     if (gg) {
       BK_TRY_CUDA(cudaMemcpyAsync(hostbuf, gs, sizeof(GmHead), cudaMemcpyDeviceToHost, st));
@@ -962,8 +956,7 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
     if (total >= o.max_iter) {
       // final explicit residual
       BK_TRY(op_apply(pr, d, op, x, r, st));
-      k_axpby<T><<<g, 256, 0, st>>>(b, 1.0, r, -1.0, n);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_axpby<T>, g, 256, 0, st, b, 1.0, r, -1.0, n));
       if (weighted) BK_TRY(wscale(r, r, 0));
       BK_TRY(dots<T>(r, ld, 1, r, n, partial, h1, cnt, st));
       BK_TRY_CUDA(cudaMemcpyAsync(hostbuf, h1, sizeof(double), cudaMemcpyDeviceToHost, st));

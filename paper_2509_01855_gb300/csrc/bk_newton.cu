@@ -51,18 +51,21 @@ namespace bk {
 
 template <typename Tin, typename Tout>
 __global__ void k_cast(const Tin* __restrict__ a, Tout* __restrict__ b, int64_t n) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     b[i] = (Tout)a[i];
 }
 
 // y = a x + b y (FP64)
 __global__ void k_axpby64(const double* __restrict__ x, double a, double* __restrict__ y, double b, int64_t n) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = a * x[i] + (b == 0.0 ? 0.0 : b * y[i]);
 }
 
 // y += (double) x (x float)
 __global__ void k_acc32(const float* __restrict__ x, double* __restrict__ y, int64_t n) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] += (double)x[i];
 }
@@ -70,12 +73,14 @@ __global__ void k_acc32(const float* __restrict__ x, double* __restrict__ y, int
 // z_t = z + alpha d
 __global__ void k_step(const double* __restrict__ z, const double* __restrict__ d, double alpha,
                        double* __restrict__ zt, int64_t n) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     zt[i] = z[i] + alpha * d[i];
 }
 
 // sum of squares partials (FP64)
 __global__ void k_sumsq(const double* __restrict__ x, int64_t n, double* __restrict__ partial) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -97,6 +102,7 @@ constexpr double kTau = 0.995;   // fraction-to-boundary
 // of ts.mu, nu_r = psi_r'(x) (-mu / (x - elo) or mu / (ehi - x)).
 __global__ void k_interior(double* __restrict__ z, int64_t P, int64_t L, int nx, BarSpec b, TermSpec ts,
                            int64_t nu_off, double margin) {
+  pdl_wait();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
     if (k == L - 1) {
 #pragma unroll
@@ -126,6 +132,7 @@ __global__ void k_interior(double* __restrict__ z, int64_t P, int64_t L, int nx,
 // (zero for an absent bound and in the padding).
 __global__ void k_pd_init(const double* __restrict__ z, const double* __restrict__ w, double s, int64_t P, int64_t L,
                           int nx, int nu, BarSpec b, double* __restrict__ zb) {
+  pdl_wait();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
     for (int q = 0; q < NUM; ++q) {
@@ -142,6 +149,7 @@ __global__ void k_pd_init(const double* __restrict__ z, const double* __restrict
 // C_l = (u - lo) z_l - mu s w, C_h = (hi - u) z_h - mu s w.
 __global__ void k_pd_rhs(const double* __restrict__ z, const double* __restrict__ zb, const double* __restrict__ w,
                          double s, int64_t P, int64_t L, int nx, int nu, BarSpec b, double* __restrict__ rhs) {
+  pdl_wait();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
     const double c = b.mu * s * w[k];
 #pragma unroll
@@ -167,6 +175,7 @@ __global__ void k_pd_rhs(const double* __restrict__ z, const double* __restrict_
 __global__ void k_pd_dz(const double* __restrict__ z, const double* __restrict__ d, const double* __restrict__ zb,
                         const double* __restrict__ w, double s, int64_t P, int64_t L, int nx, int nu, BarSpec b,
                         double* __restrict__ dzb) {
+  pdl_wait();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
     for (int q = 0; q < NUM; ++q) {
@@ -195,6 +204,7 @@ __global__ void k_pd_dz(const double* __restrict__ z, const double* __restrict__
 __global__ void k_max_step(const double* __restrict__ z, const double* __restrict__ d, const double* __restrict__ zb,
                            const double* __restrict__ dzb, int64_t P, int64_t L, int nx, int nu, BarSpec b,
                            TermSpec ts, int64_t nu_off, double* __restrict__ partial) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 1.0 / kTau;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
@@ -237,6 +247,7 @@ __global__ void k_max_step(const double* __restrict__ z, const double* __restric
 }
 
 __global__ void k_min_block(const double* __restrict__ partial, int n, double* __restrict__ out) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 1.0 / kTau;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a = fmin(a, partial[i]);
@@ -256,6 +267,7 @@ static inline int g1(int64_t n) {
 }
 
 __global__ void k_sum_block(const double* __restrict__ partial, int n, double* __restrict__ out) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a += partial[i];
@@ -272,10 +284,8 @@ __global__ void k_sum_block(const double* __restrict__ partial, int n, double* _
 // ||x||_2 (FP64, fixed reduction order), synchronous.
 static bk_status norm2(Problem* pr, const double* x, int64_t n, double* out, cudaStream_t st) {
   const int nb = 592;
-  k_sumsq<<<nb, 256, 0, st>>>(x, n, pr->red);
-  BK_CHECK_LAUNCH();
-  k_sum_block<<<1, 256, 0, st>>>(pr->red, nb, pr->red + 1024);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_sumsq, nb, 256, 0, st, x, n, pr->red));
+  BK_TRY(launch(k_sum_block, 1, 256, 0, st, pr->red, nb, pr->red + 1024));
   BK_TRY_CUDA(cudaMemcpyAsync(pr->red_host, pr->red + 1024, sizeof(double), cudaMemcpyDeviceToHost, st));
   BK_TRY_CUDA(cudaStreamSynchronize(st));
   *out = sqrt(pr->red_host[0]);
@@ -286,11 +296,9 @@ static bk_status norm2(Problem* pr, const double* x, int64_t n, double* out, cud
 static bk_status max_step(Problem* pr, const double* z, const double* d, const double* zb, const double* dzb,
                           double* out, cudaStream_t st) {
   const int nb = (int)((pr->L + 255) / 256 < 592 ? (pr->L + 255) / 256 : 592);
-  k_max_step<<<nb, 256, 0, st>>>(z, d, zb, dzb, pr->P, pr->L, pr->n_x, pr->n_u, bar_spec(pr), term_spec(pr),
-                                 (int64_t)(2 * pr->n_x + pr->n_u) * pr->P, pr->red);
-  BK_CHECK_LAUNCH();
-  k_min_block<<<1, 256, 0, st>>>(pr->red, nb, pr->red + 1024);
-  BK_CHECK_LAUNCH();
+  BK_TRY(launch(k_max_step, nb, 256, 0, st, z, d, zb, dzb, pr->P, pr->L, pr->n_x, pr->n_u, bar_spec(pr), term_spec(pr),
+                                 (int64_t)(2 * pr->n_x + pr->n_u) * pr->P, pr->red));
+  BK_TRY(launch(k_min_block, 1, 256, 0, st, pr->red, nb, pr->red + 1024));
   BK_TRY_CUDA(cudaMemcpyAsync(pr->red_host, pr->red + 1024, sizeof(double), cudaMemcpyDeviceToHost, st));
   BK_TRY_CUDA(cudaStreamSynchronize(st));
   *out = fmin(1.0, kTau * pr->red_host[0]);
@@ -383,13 +391,11 @@ static bk_status newton_impl(Problem* pr, double* z, const bk_newton_opts& o, bk
   if (bar) {
     pr->bar_mu = mu;
     pr->bar_z = nullptr;
-    k_interior<<<g1(pr->L), 256, 0, st>>>(z, pr->P, pr->L, pr->n_x, bar_spec(pr), term_spec(pr),
-                                          (int64_t)(2 * pr->n_x + pr->n_u) * pr->P, 1e-3);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_interior, g1(pr->L), 256, 0, st, z, pr->P, pr->L, pr->n_x, bar_spec(pr), term_spec(pr),
+                                          (int64_t)(2 * pr->n_x + pr->n_u) * pr->P, 1e-3));
   }
   if (pd) {
-    k_pd_init<<<g1(pr->P), 256, 0, st>>>(z, pr->d64.plan->w64, pr->s, pr->P, pr->L, pr->n_x, pr->n_u, bar_spec(pr), zb);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_pd_init, g1(pr->P), 256, 0, st, z, pr->d64.plan->w64, pr->s, pr->P, pr->L, pr->n_x, pr->n_u, bar_spec(pr), zb));
     pr->bar_z = zb;
   }
   BK_TRY(problem_residual(pr, z, F, &phi, st, Mu, false));
@@ -436,8 +442,7 @@ static bk_status newton_impl(Problem* pr, double* z, const bk_newton_opts& o, bk
                                                   : LIN_FULL;
     if (keep == LIN_FULL) ++info->precond_builds;
     BK_TRY(problem_linearize(pr, z, st, Mu, keep));
-    k_axpby64<<<g, 256, 0, st>>>(F, -1.0, rhs, 0.0, n);
-    BK_CHECK_LAUNCH();
+    BK_TRY(launch(k_axpby64, g, 256, 0, st, F, -1.0, rhs, 0.0, n));
     // Primal-dual form: GMRES in the merit's norm, to a residual of (forcing term) x the merit.
     // The eliminated right-hand side carries C / (distance to the bound), which near an active
     // bound is far larger than the merit's C / sqrt(w): a tolerance relative to it alone gave
@@ -449,9 +454,8 @@ static bk_status newton_impl(Problem* pr, double* z, const bk_newton_opts& o, bk
     // merit's norm it took 20 Newton steps at N = 2^6, 2^10 and 2^14.
     const bool weighted = o.weighted_inner != 0 || pd || pr->has_ebounds;
     if (pd) {
-      k_pd_rhs<<<g1(pr->L), 256, 0, st>>>(z, zb, pr->d64.plan->w64, pr->s, pr->P, pr->L, pr->n_x, pr->n_u,
-                                          bar_spec(pr), rhs);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_pd_rhs, g1(pr->L), 256, 0, st, z, zb, pr->d64.plan->w64, pr->s, pr->P, pr->L, pr->n_x, pr->n_u,
+                                          bar_spec(pr), rhs));
       if (o.krylov_rtol <= 0) {
         double bw = 0.0;
         BK_TRY(problem_wnorm(pr, rhs, &bw, st));
@@ -469,21 +473,17 @@ static bk_status newton_impl(Problem* pr, double* z, const bk_newton_opts& o, bk
       double rn0 = 0.0;
       BK_TRY(norm2(pr, rhs, n, &rn0, st));
       BK_TRY_CUDA(cudaMemsetAsync(d, 0, sizeof(double) * n, st));
-      k_axpby64<<<g, 256, 0, st>>>(rhs, 1.0, r, 0.0, n);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_axpby64, g, 256, 0, st, rhs, 1.0, r, 0.0, n));
       for (int sweep = 0; sweep < o.max_refine; ++sweep) {
-        k_cast<double, float><<<g, 256, 0, st>>>(r, r32, n);
-        BK_CHECK_LAUNCH();
+        BK_TRY(launch(k_cast<double, float>, g, 256, 0, st, r, r32, n));
         BK_TRY(gmres(pr, pr->d32, BK_OP_KKT, r32, d32, ko, &ki, gws, st, nullptr, weighted));
         info->krylov_iterations += ki.iterations;
         info->kkt_solves += 1;
-        k_acc32<<<g, 256, 0, st>>>(d32, d, n);
-        BK_CHECK_LAUNCH();
+        BK_TRY(launch(k_acc32, g, 256, 0, st, d32, d, n));
         if (sweep + 1 == o.max_refine) break;  // last sweep: the Newton residual checks d
         // r = rhs - K d (FP64)
         BK_TRY(op_apply(pr, pr->d64, BK_OP_KKT, d, r, st));
-        k_axpby64<<<g, 256, 0, st>>>(rhs, 1.0, r, -1.0, n);
-        BK_CHECK_LAUNCH();
+        BK_TRY(launch(k_axpby64, g, 256, 0, st, rhs, 1.0, r, -1.0, n));
         double rn = 0.0;
         BK_TRY(norm2(pr, r, n, &rn, st));
         if (rn <= o.ir_rtol * rn0) break;
@@ -500,19 +500,16 @@ static bk_status newton_impl(Problem* pr, double* z, const bk_newton_opts& o, bk
     // backtracking line search on ||F||_W, from the fraction-to-boundary bound under control bounds
     double alpha = 1.0, phit = 0.0;
     if (pd) {
-      k_pd_dz<<<g1(pr->P), 256, 0, st>>>(z, d, zb, pr->d64.plan->w64, pr->s, pr->P, pr->L, pr->n_x, pr->n_u,
-                                         bar_spec(pr), dzb);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_pd_dz, g1(pr->P), 256, 0, st, z, d, zb, pr->d64.plan->w64, pr->s, pr->P, pr->L, pr->n_x, pr->n_u,
+                                         bar_spec(pr), dzb));
     }
     if (bar) BK_TRY(max_step(pr, z, d, zb, dzb, &alpha, st));
     int bt = 0;
     const double phi2 = phi * phi;
     for (;;) {
-      k_step<<<g, 256, 0, st>>>(z, d, alpha, zt, n);
-      BK_CHECK_LAUNCH();
+      BK_TRY(launch(k_step, g, 256, 0, st, z, d, alpha, zt, n));
       if (pd) {
-        k_step<<<g1(nzb), 256, 0, st>>>(zb, dzb, alpha, zbt, nzb);
-        BK_CHECK_LAUNCH();
+        BK_TRY(launch(k_step, g1(nzb), 256, 0, st, zb, dzb, alpha, zbt, nzb));
         pr->bar_z = zbt;
       }
       if (ft) {
@@ -523,8 +520,7 @@ static bk_status newton_impl(Problem* pr, double* z, const bk_newton_opts& o, bk
           BK_TRY(problem_residual(pr, zt, F, &phit, st, Mut, false));
         }
       } else {
-        k_step<<<g1(nxP), 256, 0, st>>>(Mu, Mud, alpha, Mut, nxP);
-        BK_CHECK_LAUNCH();
+        BK_TRY(launch(k_step, g1(nxP), 256, 0, st, Mu, Mud, alpha, Mut, nxP));
         BK_TRY(problem_residual(pr, zt, F, &phit, st, Mut, true));
       }
       if (phit <= (1.0 - 1e-4 * alpha) * phi || bt >= 30) break;
