@@ -800,6 +800,9 @@ static bk_status build_tables(Plan* p, cudaStream_t st) {
 }
 
 #ifndef BK_TRANSFORM_KERNEL_UNIT
+static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_batch, int dtype, double t0, double tf,
+                                   int64_t pitch, cudaStream_t st, bool weights_only);
+
 __global__ void k_unit_last(double* e, int64_t L, int64_t pitch) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < pitch; i += (int64_t)gridDim.x * blockDim.x)
     e[i] = (i == L - 1) ? 1.0 : 0.0;
@@ -809,14 +812,21 @@ __global__ void k_d2f(const double* a, float* b, int64_t n) {
     b[i] = (float)a[i];
 }
 
-// Clenshaw-Curtis weights as the last row of B^a: w = (B^a)^T e_N, computed in FP64 with the
-// transpose product itself (O(N log N)). A BK_F32 plan uses a temporary FP64 plan.
+// The end weights of an even N are 1 / (N^2 - 1) exactly. The transpose product gives them to its
+// absolute rounding, N times larger relative to them than to the others, and the control block of
+// the KKT preconditioner divides by them.
+__global__ void k_weight_ends(double* w, int64_t N) {
+  if (threadIdx.x < 2) w[threadIdx.x * N] = 1.0 / ((double)N * (double)N - 1.0);
+}
+
+// Clenshaw-Curtis weights as the last row of B^a: w = (B^a)^T e_N, computed in binary64 with the
+// transpose product itself (O(N log N)). FP32 and double-float plans use a temporary binary64 plan.
 static bk_status compute_weights(Plan* p, cudaStream_t st) {
   const int64_t L = p->L;
   Plan* q = p;
   Plan* tmp = nullptr;
-  if (p->dtype != BK_F64) {
-    BK_TRY(plan_create(&tmp, p->N, 1, 1, BK_F64, 0.0, 2.0, 0, st));
+  if (p->dtype != BK_F64 || p->df) {
+    BK_TRY(plan_create_arith(&tmp, p->N, 1, 1, BK_F64, 0.0, 2.0, 0, st, true));
     q = tmp;
   }
   double* e = nullptr;
@@ -826,6 +836,10 @@ static bk_status compute_weights(Plan* p, cudaStream_t st) {
     k_unit_last<<<(int)((q->pitch + 255) / 256), 256, 0, st>>>(e, L, q->pitch);
     note_launch();
     r = cudaGetLastError() == cudaSuccess ? plan_apply_n(q, e, p->w64, 1, true, 1.0, st) : BK_ERR_CUDA;
+  }
+  if (r == BK_OK && p->N % 2 == 0) {
+    k_weight_ends<<<1, 32, 0, st>>>(p->w64, p->N);
+    note_launch();
   }
   if (r == BK_OK && p->dtype == BK_F32) {
     r = dmalloc(&p->wT, sizeof(float) * L);
@@ -1261,8 +1275,15 @@ bool plan_n_supported(int64_t N, int dtype) {
   return N >= 4 && (is_pow2(N) ? N <= (int64_t(1) << 24) : (dense_supported(N) || N <= blue_max(dtype)));
 }
 
-bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtype, double t0,
-                      double tf, int64_t pitch, cudaStream_t st) {
+bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtype, double t0, double tf, int64_t pitch,
+                      cudaStream_t st) {
+  return plan_create_arith(out, N, n_comp, max_batch, dtype, t0, tf, pitch, st, false);
+}
+
+// weights_only: a plan for compute_weights' one product, in binary64, with the default tiles and
+// without weights of its own.
+static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_batch, int dtype, double t0, double tf,
+                                   int64_t pitch, cudaStream_t st, bool weights_only) {
   *out = nullptr;
   BK_ARG(plan_n_supported(N, dtype),
          "N must be a power of two in [4, 2^24] or any N in [4, %lld] (this precision), got %lld",
@@ -1292,7 +1313,7 @@ bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtyp
     const char* e = getenv("BK_DENSE_TEST_TIMEOUT");  // test mode of the dense kernel, as bk_plan_dense_test_timeout
     p->dtest = (e && e[0] == '1') ? 1 : 0;
   }
-  p->df = dtype == BK_F64 && is_pow2(N) && N >= 256 && f64_df_default(N);
+  p->df = dtype == BK_F64 && is_pow2(N) && N >= 256 && !weights_only && f64_df_default(N);
   p->small = !p->generic && !p->blue && !p->df && N <= small_limit(dtype);
   bk_status st_ = BK_OK;
   AllocCounter counter(&p->bytes);
@@ -1340,6 +1361,7 @@ bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtyp
     st_ = dtype == BK_F64 ? (p->df ? set_smem_attrs<dfl>(p) : set_smem_attrs<double>(p)) : set_smem_attrs<float>(p);
     if (st_ != BK_OK) break;
     if (p->blue && (st_ = dtype == BK_F64 ? blue_spectrum<double>(p, st) : blue_spectrum<float>(p, st)) != BK_OK) break;
+    if (weights_only) break;
     if ((st_ = compute_weights(p, st)) != BK_OK) break;
     if (p->split && autotune_enabled()) {
       if ((st_ = autotune_tiles(p, st)) != BK_OK) break;

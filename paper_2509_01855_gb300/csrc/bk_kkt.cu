@@ -21,6 +21,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 #include <vector>
 
 #include "bk_problem.cuh"
@@ -311,335 +312,340 @@ __global__ void k_convert(const Tin* __restrict__ a, Tout* __restrict__ b, int64
 // (I + N_j^T) rho_j + K_j^T r_j, output y_j = K_j^T r_j + N_j^T rho_j, optional b_j =
 // w_j (y_j / 2 + rho_j).
 //
-// A sweep scans the affine maps sigma -> A sigma + b level by level. The up kernels form each
+// A sweep scans the affine maps sigma -> A sigma + b level by level. The up kernel forms each
 // item's offset b (its map applied to a zero state) and the inclusive scan e of the offsets
 // within its block of 32: a Kogge-Stone scan over the lanes of a warp with the span matrices,
 // so that every FP64 instruction runs on all 32 lanes (a warp instruction occupies the FP64
 // pipe for its full width whatever its active mask). The down kernel composes, for its segment,
-// the incoming state from the top level down, S <- Pre(i) S + e(i-1) (backward:
-// S <- Suf(i)^T S + e(i+1)), and reruns the segment's nodes from it.
+// the incoming state from the top level down and reruns the segment's nodes from it.
 // ---------------------------------------------------------------------------------------------
 template <typename T> struct Levels {
   const T* m[MAXLEV];  // matrix slots per level
-  T* o[MAXLEV];        // item offsets from zero, levels >= 1
-  T* e[MAXLEV];        // inclusive in-block scan values
+  T* o[MAXLEV];        // item offsets from zero, levels >= 1 (os apart per column)
+  T* e[MAXLEV];        // inclusive in-block scan values (es apart per column)
+  int64_t es[MAXLEV];
   int n[MAXLEV];       // items per level
+  int cnt0[MAXLEV];    // first arrival counter of a level's blocks, levels >= 1
+  int ncnt;            // counters per column
+  unsigned* cnt;       // arrival counters (zero between sweeps)
   int nlev;
   const double* sdev;  // the time scale on the device (null: the kernel argument s)
 };
 
-// One node of a sweep with the node's deviation D (K = I + D, N = 2 D):
-//   DIR 0: v = y + h g + st,  out = K v = v + D v,  st <- st + 2 h g + N v = st + 2 h g + 2 D v
-//   DIR 1: y = K^T yin + N^T st = yin + D^T (yin + 2 st),  out = y and y / 2 + st,  st <- st + y
-template <typename T, int NX, int DIR>
-__device__ __forceinline__ void node_step(const T* __restrict__ Dn, int64_t k, const T* yin, const T* gin, T h,
-                                          T* st, T* out, bool want_out) {
-  T Dm[NX * NX];   // entries in a zero column (ZeroCols) are neither loaded nor used
+// Operands of a sweep over up to NEM columns (blockIdx.y).
+template <typename T> struct SweepArgs {
+  Levels<T> lv;
+  const T* Dn;
+  const T* w;
+  const T* Y;          // input, ys apart per column; null: zero, or (DIR 1) the unit vector of
+  int64_t ys;          // component unit[col] at the last node
+  const T* G[NEM];     // DIR 0: forcing per column (null: none)
+  T* out;              // os apart per column
+  int64_t os;
+  T* bout;             // DIR 1: B-tilde^T out, bs apart per column (null: not wanted)
+  int64_t bs;
+  T* last;             // DIR 0: out at the last node, n_x per column (null: not wanted)
+  int64_t P, L;
+  T s;
+  int unit[NEM];
+  int vec;             // Y, G, out, bout are 16-byte aligned
+};
+
+// N consecutive values at p (N a multiple of the 16-byte vector's length).
+template <typename T> struct V16;
+template <> struct V16<float> { typedef float4 t; static constexpr int n = 4; };
+template <> struct V16<double> { typedef double2 t; static constexpr int n = 2; };
+template <typename T, int N>
+__device__ __forceinline__ void ld_run(const T* __restrict__ p, bool vec, T* v) {
+  if (vec) {
+    typedef typename V16<T>::t VT;
 #pragma unroll
-  for (int c = 0; c < NX * NX; ++c) Dm[c] = zcol<NX>(c % NX) ? T(0) : Dn[il_index<Seg<T>::v>(k, c, NX * NX)];
-  if (DIR == 0) {
-    T v[NX], dv[NX];
-#pragma unroll
-    for (int m = 0; m < NX; ++m) v[m] = yin[m] + h * gin[m] + st[m];
-#pragma unroll
-    for (int r = 0; r < NX; ++r) {
-      T a = T(0);
-#pragma unroll
-      for (int c = 0; c < NX; ++c)
-        if (!zcol<NX>(c)) a += Dm[r * NX + c] * v[c];
-      dv[r] = a;
-    }
-    if (want_out) {
-#pragma unroll
-      for (int r = 0; r < NX; ++r) out[r] = v[r] + dv[r];
-    }
-#pragma unroll
-    for (int r = 0; r < NX; ++r) st[r] = (st[r] + T(2) * h * gin[r]) + T(2) * dv[r];
+    for (int q = 0; q < N / V16<T>::n; ++q) *reinterpret_cast<VT*>(v + q * V16<T>::n) = reinterpret_cast<const VT*>(p)[q];
   } else {
-    T q[NX], y[NX];
 #pragma unroll
-    for (int c = 0; c < NX; ++c) q[c] = yin[c] + T(2) * st[c];
+    for (int q = 0; q < N; ++q) v[q] = p[q];
+  }
+}
+template <typename T, int N>
+__device__ __forceinline__ void st_run(T* p, bool vec, const T* v) {
+  if (vec) {
+    typedef typename V16<T>::t VT;
 #pragma unroll
-    for (int r = 0; r < NX; ++r) {
-      T a = T(0);
+    for (int q = 0; q < N / V16<T>::n; ++q) reinterpret_cast<VT*>(p)[q] = *reinterpret_cast<const VT*>(v + q * V16<T>::n);
+  } else {
 #pragma unroll
-      for (int c = 0; c < NX; ++c)
-        if (!zcol<NX>(r)) a += Dm[c * NX + r] * q[c];
-      y[r] = yin[r] + a;
-    }
-    if (want_out) {
-#pragma unroll
-      for (int r = 0; r < NX; ++r) { out[r] = y[r]; out[NX + r] = y[r] * T(0.5) + st[r]; }
-    }
-#pragma unroll
-    for (int r = 0; r < NX; ++r) st[r] += y[r];
+    for (int q = 0; q < N; ++q) p[q] = v[q];
   }
 }
 
+// r = D v or D^T v (TR), skipping the zero columns of D. The products are summed on their own and
+// added to the states once: starting the FMA chains from the states would round at the states'
+// magnitude in every term (FP32 KKT preconditioner at N = 2^10: error 1.3e-6 instead of 2e-7).
+template <typename T, int NX, bool TR>
+__device__ __forceinline__ void dev_apply(const T* D, const T* v, T* r) {
+#pragma unroll
+  for (int i = 0; i < NX; ++i) {
+    T t = T(0);
+    bool first = true;
+#pragma unroll
+    for (int c = 0; c < NX; ++c)
+      if (!zcol<NX>(TR ? i : c)) {
+        const T m = TR ? D[c * NX + i] : D[i * NX + c];
+        t = first ? m * v[c] : fma(m, v[c], t);
+        first = false;
+      }
+    r[i] = t;
+  }
+}
+
+// One node of a sweep with the node's deviation D (K = I + D, N = 2 D), h = s w / 2:
+//   DIR 0: v = y + h g + st,  out = K v = v + D v,  st <- st + 2 h g + N v = st + 2 h g + 2 D v
+//   DIR 1: y = K^T yin + N^T st = yin + D^T (yin + 2 st),  out = y, bo = w (y / 2 + st),  st <- st + y
+template <typename T, int NX, int DIR, bool HASG, bool OUT>
+__device__ __forceinline__ void node_step(const T* Dm, const T* yin, const T* gin, T h, T w, T* st, T* out, T* bo) {
+  T q[NX], dv[NX];
+  if (DIR == 0) {
+#pragma unroll
+    for (int m = 0; m < NX; ++m) q[m] = (HASG ? fma(h, gin[m], yin[m]) : yin[m]) + st[m];
+    dev_apply<T, NX, false>(Dm, q, dv);
+#pragma unroll
+    for (int r = 0; r < NX; ++r) {
+      if (OUT) out[r] = q[r] + dv[r];
+      st[r] = fma(T(2), dv[r], HASG ? fma(T(2) * h, gin[r], st[r]) : st[r]);
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < NX; ++c) q[c] = fma(T(2), st[c], yin[c]);
+    dev_apply<T, NX, true>(Dm, q, dv);
+#pragma unroll
+    for (int r = 0; r < NX; ++r) {
+      const T y = zcol<NX>(r) ? yin[r] : yin[r] + dv[r];
+      if (OUT) {
+        out[r] = y;
+        bo[r] = w * fma(T(0.5), y, st[r]);
+      }
+      st[r] += y;
+    }
+  }
+}
+
+// Nonzero test on the bit pattern (integer pipe; +0 and -0 count as zero): scans whose offsets are
+// all zero are skipped without spending FP64 instructions on the test.
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ bool nonzero(float x) { return (__float_as_int(x) << 1) != 0; }
+
 // Inclusive scan of the offsets e within block blk (lane i holds item 32 blk + i), level slot
 // size `slot`. DIR 0: e_i += M_k(i) e_{i-2^k}; DIR 1 (reverse order, transposed maps):
-// e_i += M_k(i + 2^k - 1)^T e_{i+2^k}.
+// e_i += M_k(i + 2^k - 1)^T e_{i+2^k}. A step's matrix is loaded while the step before it runs.
 template <typename T, int NX, int DIR>
 __device__ __forceinline__ void warp_scan(const T* __restrict__ m, int64_t slot, int64_t blk, T* e) {
   constexpr int NC = NX * NX;
   const int lane = threadIdx.x & 31;
+  T Mv[2][NC];
+  auto load = [&](int k, T* M) {
+    const int d = 1 << k;
+    const int it = DIR == 0 ? lane : min(lane + d - 1, 31);
+    const T* mp = m + k * slot + il32(blk * 32 + it, 0, NC);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) M[c] = zcol<NX>(c % NX) ? T(0) : mp[c << 5];
+  };
+  load(0, Mv[0]);
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
+    if (k < 4) load(k + 1, Mv[(k + 1) & 1]);
     const int d = 1 << k;
-    T pe[NX];
+    T pe[NX], r[NX];
 #pragma unroll
-    for (int r = 0; r < NX; ++r)
-      pe[r] = DIR == 0 ? shfl_up(e[r], d) : shfl_down(e[r], d);
+    for (int q = 0; q < NX; ++q) pe[q] = DIR == 0 ? shfl_up(e[q], d) : shfl_down(e[q], d);
+    dev_apply<T, NX, DIR == 1>(Mv[k & 1], pe, r);
     const bool act = DIR == 0 ? lane >= d : lane + d < 32;
-    if (act) {
-      const int64_t item = blk * 32 + (DIR == 0 ? lane : lane + d - 1);
-      const T* M = m + k * slot;
-      T Mv[NC];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) Mv[c] = zcol<NX>(c % NX) ? T(0) : M[il32(item, c, NC)];
-#pragma unroll
-      for (int r = 0; r < NX; ++r) {
-        T a = T(0);   // (I + D) pe = pe + D pe
-#pragma unroll
-        for (int c = 0; c < NX; ++c)
-          if (!zcol<NX>(DIR == 0 ? c : r)) a += (DIR == 0 ? Mv[r * NX + c] : Mv[c * NX + r]) * pe[c];
-        e[r] = e[r] + (pe[r] + a);
-      }
-    }
+    for (int q = 0; q < NX; ++q) e[q] = act ? e[q] + (pe[q] + r[q]) : e[q];
   }
 }
 
-// Per-node vectors of a warp's 32 segments move through shared memory in chunks of CH nodes
-// (one 32-byte sector per segment and component), so that every global access is sector-
-// coalesced: lane l of staging instruction q handles element q*32 + l of the [segment][node]
-// chunk. Reading them lane-by-segment directly (a 16-node stride) wasted most of each sector.
+// Nodes per register chunk: 32 bytes per component.
 template <typename T> struct SweepChunk {
-  static constexpr int CH = 32 / (int)sizeof(T);   // nodes per chunk
-  static constexpr int TS = CH + 1;                // padded row (bank spread)
-  static_assert(Seg<T>::v % CH == 0, "segment length must be a multiple of the staging chunk");
+  static constexpr int CH = 32 / (int)sizeof(T);
+  static_assert(Seg<T>::v % CH == 0, "segment length must be a multiple of the chunk");
 };
 
-template <typename T>
-__device__ __forceinline__ void stage_in(const T* __restrict__ src, int64_t P, int nc, int64_t L, int64_t seg0,
-                                         int i0, T* __restrict__ tile) {
-  constexpr int CH = SweepChunk<T>::CH, TS = SweepChunk<T>::TS, SEG = Seg<T>::v;
-  const int lane = threadIdx.x & 31;
-  for (int c = 0; c < nc; ++c) {
-#pragma unroll
-    for (int q = 0; q < CH; ++q) {
-      const int e = q * 32 + lane;
-      const int sl = e / CH, nd = e - (e / CH) * CH;
-      const int64_t k = (seg0 + sl) * SEG + i0 + nd;
-      tile[(c * 32 + sl) * TS + nd] = k < L ? src[c * P + k] : T(0);
-    }
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ void stage_out(const T* __restrict__ tile, int nc, int64_t P, int64_t L, int64_t seg0,
-                                          int i0, T* __restrict__ dst) {
-  constexpr int CH = SweepChunk<T>::CH, TS = SweepChunk<T>::TS, SEG = Seg<T>::v;
-  const int lane = threadIdx.x & 31;
-  for (int c = 0; c < nc; ++c) {
-#pragma unroll
-    for (int q = 0; q < CH; ++q) {
-      const int e = q * 32 + lane;
-      const int sl = e / CH, nd = e - (e / CH) * CH;
-      const int64_t k = (seg0 + sl) * SEG + i0 + nd;
-      if (k < L) dst[c * P + k] = tile[(c * 32 + sl) * TS + nd];
-    }
-  }
-}
-
-// Shared tiles of one warp: A (n_x components), B (n_x components), W (1 component).
-template <typename T, int NX> struct SweepTiles {
-  static constexpr int ROWS = 32 * SweepChunk<T>::TS;
-  T a[NX * ROWS], b[NX * ROWS], w[ROWS];
-};
-
-// Nonzero test on the bit pattern (integer pipe; +0 and -0 count as zero): the sweeps use it to
-// skip work whose inputs are all zero without spending FP64 instructions on the test.
-__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
-__device__ __forceinline__ bool nonzero(float x) { return (__float_as_int(x) << 1) != 0; }
-
-// Up, level 0 (one warp per block of 32 segments, 4 warps per CTA): each lane runs its segment
-// from a zero state (the segment's offset), then the warp scans the block. A chunk whose inputs
-// and states are zero on every lane leaves the states zero and is skipped, and a block whose
-// offsets are all zero has zero scan values: the terminal Schur columns' right-hand sides are
-// unit vectors at the last node, so their up passes do almost no FP64 work.
-template <typename T, int NX, int DIR>
-__device__ __forceinline__ void sw_up0_warp(int g, SweepTiles<T, NX>& tl, const T* __restrict__ Dn,
-                                            const T* __restrict__ Y,
-                                            const T* __restrict__ G, int64_t P, int64_t L, const T* __restrict__ w,
-                                            T s, const Levels<T>& lv) {
-  constexpr int CH = SweepChunk<T>::CH, TS = SweepChunk<T>::TS, SEG = Seg<T>::v;
-  const int nblk = (lv.n[0] + 31) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int64_t seg0 = (int64_t)g * 32;
-  const int64_t seg = seg0 + lane;
-  if (lv.sdev) s = T(*lv.sdev);
-  T st[NX];
-#pragma unroll
-  for (int m = 0; m < NX; ++m) st[m] = T(0);
+// A lane's segment moves through registers in chunks of CH consecutive nodes: its runs of 32 bytes
+// per component are whole sectors, its deviations are interleaved over the warp's lanes, and every
+// load of a chunk is unconditional and independent of the states, so they are all in flight before
+// the chain of node steps needs them. (Staged through shared memory, with loads behind per-node
+// conditions, an FP32 sweep of N = 4096 spent 20 us per pass waiting for one load after another.)
+// Lanes past the last segment read its data again and drop their results.
+template <typename T, int NX, int DIR, bool HASG, bool OUT>
+__device__ __forceinline__ void sweep_segment(const SweepArgs<T>& a, int col, int64_t seg, T* st) {
+  constexpr int CH = SweepChunk<T>::CH, SEG = Seg<T>::v, NC = NX * NX;
+  const int nseg = a.lv.n[0];
+  const int64_t sc = seg < nseg ? seg : nseg - 1;
+  const bool alive = seg < nseg;
+  const int64_t k0 = sc * SEG;
+  const int64_t P = a.P;
+  const bool vec = a.vec != 0;
+  const T hs = T(0.5) * (a.lv.sdev ? T(*a.lv.sdev) : a.s);
+  const T* Y = a.Y ? a.Y + col * a.ys : nullptr;
+  const T* G = HASG ? a.G[col] : nullptr;
+  const T* Dp = a.Dn + (((sc >> 5) * SEG * NC) << 5) + (sc & 31);
+  const bool wantb = OUT && DIR == 1 && a.bout != nullptr;
+#pragma unroll 1
   for (int c = 0; c < SEG / CH; ++c) {
     const int i0 = (DIR == 0 ? c : SEG / CH - 1 - c) * CH;
-    __syncwarp();
-    stage_in<T>(Y, P, NX, L, seg0, i0, tl.a);
-    if (G) stage_in<T>(G, P, NX, L, seg0, i0, tl.b);
-    stage_in<T>(w, P, 1, L, seg0, i0, tl.w);
-    __syncwarp();
-    bool act = false;
+    T y[NX][CH], g[HASG ? NX : 1][CH], b[OUT && DIR == 1 ? NX : 1][CH], wv[CH];
 #pragma unroll
     for (int m = 0; m < NX; ++m) {
-      act |= nonzero(st[m]);
+      if (Y) {
+        ld_run<T, CH>(Y + m * P + k0 + i0, vec, y[m]);
+      } else {
 #pragma unroll
-      for (int jj = 0; jj < CH; ++jj) {
-        act |= nonzero(tl.a[(m * 32 + lane) * TS + jj]);
-        if (G) act |= nonzero(tl.b[(m * 32 + lane) * TS + jj]);
+        for (int q = 0; q < CH; ++q) y[m][q] = DIR == 1 && k0 + i0 + q == a.L - 1 && m == a.unit[col] ? T(1) : T(0);
       }
+      if (HASG) ld_run<T, CH>(G + m * P + k0 + i0, vec, g[m]);
     }
-    if (!__any_sync(0xffffffffu, act)) continue;
+    if (HASG || wantb) {   // the weights end at L
+#pragma unroll
+      for (int q = 0; q < CH; ++q) wv[q] = k0 + i0 + q < a.L ? a.w[k0 + i0 + q] : T(0);
+    }
+    T Dm[CH][NC];
+#pragma unroll
+    for (int nd = 0; nd < CH; ++nd)
+#pragma unroll
+      for (int q = 0; q < NC; ++q) Dm[nd][q] = zcol<NX>(q % NX) ? T(0) : __ldg(Dp + (((i0 + nd) * NC + q) << 5));
 #pragma unroll
     for (int jj = 0; jj < CH; ++jj) {
       const int nd = DIR == 0 ? jj : CH - 1 - jj;
-      const int64_t k = seg * SEG + i0 + nd;
-      if (seg < lv.n[0] && k < L) {
-        T yin[NX], gin[NX], dummy[2 * NX];
+      const bool live = alive && k0 + i0 + nd < a.L;
+      T yin[NX], gin[NX], ns[NX], o[NX], bo[NX];
 #pragma unroll
-        for (int m = 0; m < NX; ++m) {
-          yin[m] = tl.a[(m * 32 + lane) * TS + nd];
-          gin[m] = G ? tl.b[(m * 32 + lane) * TS + nd] : T(0);
-        }
-        node_step<T, NX, DIR>(Dn, k, yin, gin, T(0.5) * s * tl.w[lane * TS + nd], st, dummy, false);
+      for (int m = 0; m < NX; ++m) {
+        yin[m] = y[m][nd];
+        gin[m] = HASG ? g[m][nd] : T(0);
+        ns[m] = st[m];
+      }
+      const T w = HASG || wantb ? wv[nd] : T(0);
+      node_step<T, NX, DIR, HASG, OUT>(Dm[nd], yin, gin, hs * w, w, ns, o, bo);
+#pragma unroll
+      for (int m = 0; m < NX; ++m) {
+        st[m] = live ? ns[m] : st[m];
+        if (OUT) y[m][nd] = live ? o[m] : T(0);
+        if (OUT && DIR == 1) b[m][nd] = live ? bo[m] : T(0);
+      }
+      if (OUT && DIR == 0 && a.last && live && k0 + i0 + nd == a.L - 1) {
+#pragma unroll
+        for (int m = 0; m < NX; ++m) a.last[col * NX + m] = o[m];
       }
     }
-  }
-  T e[NX];
-  bool any = false;
+    if (OUT && alive) {
 #pragma unroll
-  for (int m = 0; m < NX; ++m) {
-    e[m] = st[m];
-    any |= nonzero(st[m]);
-  }
-  if (__any_sync(0xffffffffu, any)) warp_scan<T, NX, DIR>(lv.m[0], (int64_t)nblk * 32 * NX * NX, g, e);
+      for (int m = 0; m < NX; ++m) st_run<T, CH>(a.out + col * a.os + m * P + k0 + i0, vec, y[m]);
+    }
+    if (wantb && alive) {
 #pragma unroll
-  for (int m = 0; m < NX; ++m) lv.e[0][il32(seg, m, NX)] = e[m];
-  if (lv.nlev > 1 && lane == (DIR == 0 ? 31 : 0)) {
-#pragma unroll
-    for (int m = 0; m < NX; ++m) lv.o[1][il32(g, m, NX)] = e[m];
+      for (int m = 0; m < NX; ++m) st_run<T, CH>(a.bout + col * a.bs + m * P + k0 + i0, vec, b[OUT && DIR == 1 ? m : 0]);
+    }
   }
 }
 
-// Up, level l >= 1 (one warp per block of 32 items): scan of the items' offsets.
-template <typename T, int NX, int DIR>
-__device__ __forceinline__ void sw_upL_warp(int b, const Levels<T>& lv, int l) {
-  const int n = lv.n[l];
-  const int nblk = (n + 31) >> 5;
+// Up pass, one warp per block g of 32 segments: each lane runs its segment from a zero state (the
+// segment's offset), then the warp scans the block. Upper levels follow in the same launch: the
+// warp that completes a block of 32 items (by the block's arrival counter) scans it, writes its
+// parent's offset and goes on to the next level, so the result does not depend on which warp that is.
+template <typename T, int NX, int DIR, bool HASG>
+__device__ __forceinline__ void sw_up_warp(const SweepArgs<T>& a, int col, int g) {
+  const Levels<T>& lv = a.lv;
   const int lane = threadIdx.x & 31;
-  const int64_t i = (int64_t)b * 32 + lane;
-  const T* o = lv.o[l];
+  const int64_t seg = (int64_t)g * 32 + lane;
   T e[NX];
-  bool any = false;
 #pragma unroll
-  for (int m = 0; m < NX; ++m) {
-    e[m] = i < n ? o[il32(i, m, NX)] : T(0);
-    any |= nonzero(e[m]);
+  for (int m = 0; m < NX; ++m) e[m] = T(0);
+  // without input or forcing only the last node's unit entry is nonzero
+  const bool idle = !a.Y && !HASG && (DIR == 0 || g != (lv.n[0] - 1) >> 5);
+  if (!idle) {
+    sweep_segment<T, NX, DIR, HASG, false>(a, col, seg, e);
+#pragma unroll
+    for (int m = 0; m < NX; ++m) e[m] = seg < lv.n[0] ? e[m] : T(0);
   }
-  if (__any_sync(0xffffffffu, any)) warp_scan<T, NX, DIR>(lv.m[l], (int64_t)nblk * 32 * NX * NX, b, e);
-  T* el = lv.e[l];
+  int64_t b = g;
+  for (int l = 0;; ++l) {
+    bool any = false;
 #pragma unroll
-  for (int m = 0; m < NX; ++m) el[il32(i, m, NX)] = e[m];
-  if (l + 1 < lv.nlev && lane == (DIR == 0 ? 31 : 0)) {
-    T* op = lv.o[l + 1];
+    for (int m = 0; m < NX; ++m) any |= nonzero(e[m]);
+    if (__any_sync(0xffffffffu, any))
+      warp_scan<T, NX, DIR>(lv.m[l], (int64_t)((lv.n[l] + 31) >> 5) * 32 * NX * NX, b, e);
+    T* el = lv.e[l] + col * lv.es[l];
 #pragma unroll
-    for (int m = 0; m < NX; ++m) op[il32(b, m, NX)] = e[m];
+    for (int m = 0; m < NX; ++m) el[il32(b * 32 + lane, m, NX)] = e[m];
+    if (l + 1 >= lv.nlev) return;
+    T* o = lv.o[l + 1] + col * lv.es[l + 1];
+    if (lane == (DIR == 0 ? 31 : 0)) {
+#pragma unroll
+      for (int m = 0; m < NX; ++m) o[il32(b, m, NX)] = e[m];
+    }
+    __threadfence();
+    __syncwarp();
+    const int64_t nb = b >> 5;
+    const int n = lv.n[l + 1];
+    unsigned* cnt = lv.cnt + col * lv.ncnt + lv.cnt0[l + 1] + nb;
+    unsigned old = 0;
+    if (lane == 0) {
+      old = atomicAdd(cnt, 1u);
+      if (old + 1 == (unsigned)min(32, n - 32 * (int)nb)) *cnt = 0u;   // zero for the next sweep
+    }
+    old = __shfl_sync(0xffffffffu, old, 0);
+    if (old + 1 != (unsigned)min(32, n - 32 * (int)nb)) return;
+    __threadfence();
+    b = nb;
+#pragma unroll
+    for (int m = 0; m < NX; ++m) e[m] = b * 32 + lane < n ? __ldcg(o + il32(b * 32 + lane, m, NX)) : T(0);
   }
 }
 
-// Down (one warp per block of 32 segments): incoming state of the lane's segment, composed from
-// the top level down, then the segment's nodes with outputs (staged like the inputs).
-template <typename T, int NX, int DIR>
-__device__ __forceinline__ void sw_down0_warp(int g, SweepTiles<T, NX>& tl, const T* __restrict__ Dn,
-                                              const T* __restrict__ Y,
-                                              const T* __restrict__ G, int64_t P, int64_t L,
-                                              const T* __restrict__ w, T s, const Levels<T>& lv,
-                                              T* __restrict__ out, T* __restrict__ bout) {
+// Down pass (one warp per block of 32 segments): incoming state of the lane's segment, composed from
+// the top level down (S <- Pre(i) S + e(i-1); backward S <- Suf(i)^T S + e(i+1)), a level's data
+// loaded while the level above it is applied; then the segment's nodes with outputs.
+template <typename T, int NX, int DIR, bool HASG>
+__device__ __forceinline__ void sw_down_warp(const SweepArgs<T>& a, int col, int g) {
   constexpr int NC = NX * NX;
-  constexpr int CH = SweepChunk<T>::CH, TS = SweepChunk<T>::TS, SEG = Seg<T>::v;
-  const int nblk0 = (lv.n[0] + 31) >> 5;
+  const Levels<T>& lv = a.lv;
   const int lane = threadIdx.x & 31;
-  if (lv.sdev) s = T(*lv.sdev);
-  const int64_t seg0 = (int64_t)g * 32;
-  const int64_t seg = seg0 + lane;
-  const bool live = seg < lv.n[0];
-  T S[NX];
+  const int64_t seg = (int64_t)g * 32 + lane;
+  const int64_t sc = seg < lv.n[0] ? seg : lv.n[0] - 1;
+  T S[NX], Mv[2][NC], ev[2][NX];
 #pragma unroll
   for (int m = 0; m < NX; ++m) S[m] = T(0);
-  for (int l = lv.nlev - 1; l >= 0 && live; --l) {
-    const int64_t i = seg >> (5 * l);
-    const int q = (int)(i & 31);
-    if (DIR == 0 ? q == 0 : q == 31) continue;  // first item of its block in sweep order
+  auto load = [&](int l, T* M, T* e) {
+    const int64_t i = sc >> (5 * l);
     const int64_t slot = (int64_t)((lv.n[l] + 31) >> 5) * 32 * NC;
-    const T* Mt = lv.m[l] + (DIR == 0 ? SL_PRE : SL_SUF) * slot;
-    const T* el = lv.e[l];
-    const int64_t ia = DIR == 0 ? i - 1 : i + 1;
-    T Mv[NC], ns[NX];
+    const T* mp = lv.m[l] + (DIR == 0 ? SL_PRE : SL_SUF) * slot + il32(i, 0, NC);
+    const int q = (int)(i & 31);
+    const int64_t ia = DIR == 0 ? (q == 0 ? i : i - 1) : (q == 31 ? i : i + 1);
+    const T* ep = lv.e[l] + col * lv.es[l] + il32(ia, 0, NX);
 #pragma unroll
-    for (int c = 0; c < NC; ++c) Mv[c] = zcol<NX>(c % NX) ? T(0) : Mt[il32(i, c, NC)];
+    for (int c = 0; c < NC; ++c) M[c] = zcol<NX>(c % NX) ? T(0) : mp[c << 5];
 #pragma unroll
-    for (int r = 0; r < NX; ++r) {
-      T a = T(0);   // (I + D) S = S + D S
+    for (int m = 0; m < NX; ++m) e[m] = ep[m << 5];
+  };
 #pragma unroll
-      for (int c = 0; c < NX; ++c)
-        if (!zcol<NX>(DIR == 0 ? c : r)) a += (DIR == 0 ? Mv[r * NX + c] : Mv[c * NX + r]) * S[c];
-      ns[r] = el[il32(ia, r, NX)] + (S[r] + a);
-    }
+  for (int l = MAXLEV - 1; l >= 0; --l) {
+    if (l >= lv.nlev) continue;
+    if (l == lv.nlev - 1) load(l, Mv[l & 1], ev[l & 1]);
+    if (l > 0) load(l - 1, Mv[(l - 1) & 1], ev[(l - 1) & 1]);
+    const int q = (int)((sc >> (5 * l)) & 31);
+    const bool first = DIR == 0 ? q == 0 : q == 31;   // first item of its block in sweep order
+    T r[NX];
+    dev_apply<T, NX, DIR == 1>(Mv[l & 1], S, r);
 #pragma unroll
-    for (int r = 0; r < NX; ++r) S[r] = ns[r];
+    for (int m = 0; m < NX; ++m) S[m] = first ? S[m] : ev[l & 1][m] + (S[m] + r[m]);
   }
-  T st[NX];
-#pragma unroll
-  for (int m = 0; m < NX; ++m) st[m] = S[m];
-  const bool wantb = DIR == 1 && bout != nullptr;
-  for (int c = 0; c < SEG / CH; ++c) {
-    const int i0 = (DIR == 0 ? c : SEG / CH - 1 - c) * CH;
-    __syncwarp();
-    stage_in<T>(Y, P, NX, L, seg0, i0, tl.a);
-    if (DIR == 0 && G) stage_in<T>(G, P, NX, L, seg0, i0, tl.b);
-    stage_in<T>(w, P, 1, L, seg0, i0, tl.w);
-    __syncwarp();
-#pragma unroll
-    for (int jj = 0; jj < CH; ++jj) {
-      const int nd = DIR == 0 ? jj : CH - 1 - jj;
-      const int64_t k = seg * SEG + i0 + nd;
-      if (live && k < L) {
-        T yin[NX], gin[NX], o[2 * NX];
-#pragma unroll
-        for (int m = 0; m < NX; ++m) {
-          yin[m] = tl.a[(m * 32 + lane) * TS + nd];
-          gin[m] = (DIR == 0 && G) ? tl.b[(m * 32 + lane) * TS + nd] : T(0);
-        }
-        const T wk = tl.w[lane * TS + nd];
-        node_step<T, NX, DIR>(Dn, k, yin, gin, T(0.5) * s * wk, st, o, true);
-        // outputs replace the inputs just read (same lane, same node)
-#pragma unroll
-        for (int m = 0; m < NX; ++m) tl.a[(m * 32 + lane) * TS + nd] = o[m];
-        if (wantb) {
-#pragma unroll
-          for (int m = 0; m < NX; ++m) tl.b[(m * 32 + lane) * TS + nd] = wk * o[NX + m];
-        }
-      }
-    }
-    __syncwarp();
-    stage_out<T>(tl.a, NX, P, L, seg0, i0, out);
-    if (wantb) stage_out<T>(tl.b, NX, P, L, seg0, i0, bout);
-  }
-  // the warp of the last block also zeroes the outputs' padding (elements L..P-1)
-  if (g == nblk0 - 1) {
+  sweep_segment<T, NX, DIR, HASG, true>(a, col, seg, S);
+  // the last block also zeroes the outputs' padding beyond the last segment
+  if (g == (lv.n[0] - 1) >> 5) {
     for (int c = 0; c < NX; ++c)
-      for (int64_t k = L + lane; k < P; k += 32) {
-        out[c * P + k] = T(0);
-        if (wantb) bout[c * P + k] = T(0);
+      for (int64_t k = (int64_t)lv.n[0] * Seg<T>::v + lane; k < a.P; k += 32) {
+        a.out[col * a.os + c * a.P + k] = T(0);
+        if (DIR == 1 && a.bout) a.bout[col * a.bs + c * a.P + k] = T(0);
       }
   }
 }
@@ -647,75 +653,21 @@ __device__ __forceinline__ void sw_down0_warp(int g, SweepTiles<T, NX>& tl, cons
 // The sweep kernels: one warp per block of 32 items, W warps per CTA (4; 1 for grids whose
 // level 0 has fewer blocks than four per SM, so that their warps spread over the SMs: each
 // warp's segments are sequential chains whose FP64 arithmetic would otherwise share one SM's
-// FP64 pipe).
-template <typename T, int NX, int DIR, int W>
-__global__ void __launch_bounds__(32 * W) k_sw_up0(const T* __restrict__ Dn, const T* __restrict__ Y, const T* __restrict__ G, int64_t P,
-                                                   int64_t L, const T* __restrict__ w, T s, Levels<T> lv) {
+// FP64 pipe); blockIdx.y the column.
+template <typename T, int NX, int DIR, bool HASG, int W>
+__global__ void __launch_bounds__(32 * W) k_sw_up(const __grid_constant__ SweepArgs<T> a) {
   pdl_wait();
-  __shared__ SweepTiles<T, NX> tiles[W];
   const int g = blockIdx.x * W + (threadIdx.x >> 5);
-  if (g >= ((lv.n[0] + 31) >> 5)) return;  // whole warps
-  sw_up0_warp<T, NX, DIR>(g, tiles[threadIdx.x >> 5], Dn, Y, G, P, L, w, s, lv);
+  if (g >= ((a.lv.n[0] + 31) >> 5)) return;  // whole warps
+  sw_up_warp<T, NX, DIR, HASG>(a, blockIdx.y, g);
 }
 
-template <typename T, int NX, int DIR, int W>
-__global__ void __launch_bounds__(32 * W) k_sw_upL(Levels<T> lv, int l) {
+template <typename T, int NX, int DIR, bool HASG, int W>
+__global__ void __launch_bounds__(32 * W) k_sw_down(const __grid_constant__ SweepArgs<T> a) {
   pdl_wait();
-  const int b = blockIdx.x * W + (threadIdx.x >> 5);
-  if (b >= ((lv.n[l] + 31) >> 5)) return;
-  sw_upL_warp<T, NX, DIR>(b, lv, l);
-}
-
-template <typename T, int NX, int DIR, int W>
-__global__ void __launch_bounds__(32 * W) k_sw_down0(const T* __restrict__ Dn, const T* __restrict__ Y, const T* __restrict__ G, int64_t P,
-                                                     int64_t L, const T* __restrict__ w, T s, Levels<T> lv,
-                                                     T* __restrict__ out, T* __restrict__ bout) {
-  pdl_wait();
-  __shared__ SweepTiles<T, NX> tiles[W];
   const int g = blockIdx.x * W + (threadIdx.x >> 5);
-  if (g >= ((lv.n[0] + 31) >> 5)) return;  // whole warps
-  sw_down0_warp<T, NX, DIR>(g, tiles[threadIdx.x >> 5], Dn, Y, G, P, L, w, s, lv, out, bout);
-}
-
-// The whole sweep in one CTA for small grids (at most two scan levels and SW1_MAXW blocks of 32
-// segments): one warp per block; the level-0 up pass, the level-1 scan by warp 0 and the down
-// pass are separated by barriers instead of launches (1 launch instead of nlev + 1; the serving
-// mix's small problems run many sweeps per Newton step).
-constexpr int SW1_MAXW = 16;
-template <typename T, int NX, int DIR>
-__global__ void __launch_bounds__(32 * SW1_MAXW) k_sw_one(const T* __restrict__ Dn, const T* __restrict__ Y, const T* __restrict__ G,
-                                                          int64_t P, int64_t L, const T* __restrict__ w, T s,
-                                                          Levels<T> lv, T* __restrict__ out, T* __restrict__ bout) {
-  pdl_wait();
-  extern __shared__ __align__(16) unsigned char sw1_smem[];
-  SweepTiles<T, NX>* tiles = reinterpret_cast<SweepTiles<T, NX>*>(sw1_smem);
-  const int warp = threadIdx.x >> 5;
-  const int nblk0 = (lv.n[0] + 31) >> 5;
-  if (warp < nblk0) sw_up0_warp<T, NX, DIR>(warp, tiles[warp], Dn, Y, G, P, L, w, s, lv);
-  __syncthreads();
-  if (lv.nlev > 1 && warp == 0) sw_upL_warp<T, NX, DIR>(0, lv, 1);
-  __syncthreads();
-  if (warp < nblk0) sw_down0_warp<T, NX, DIR>(warp, tiles[warp], Dn, Y, G, P, L, w, s, lv, out, bout);
-}
-
-// The sweep kernels keep up to four 4-warp CTAs per SM; give shared memory the whole L1 array.
-template <typename T, int NX>
-static bk_status sweep_attrs() {
-  BK_TRY_CUDA(cudaFuncSetAttribute(k_sw_up0<T, NX, 0, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-  BK_TRY_CUDA(cudaFuncSetAttribute(k_sw_up0<T, NX, 1, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-  BK_TRY_CUDA(cudaFuncSetAttribute(k_sw_down0<T, NX, 0, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-  BK_TRY_CUDA(cudaFuncSetAttribute(k_sw_down0<T, NX, 1, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-  const int sm1 = (int)(SW1_MAXW * sizeof(SweepTiles<T, NX>));
-  BK_TRY_CUDA(cudaFuncSetAttribute(k_sw_one<T, NX, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1));
-  BK_TRY_CUDA(cudaFuncSetAttribute(k_sw_one<T, NX, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1));
-  return BK_OK;
-}
-
-template <typename T>
-static bk_status sweep_attrs_nx(int nx) {
-  if (nx == 1) return sweep_attrs<T, 1>();
-  if (nx == 2) return sweep_attrs<T, 2>();
-  return sweep_attrs<T, 4>();
+  if (g >= ((a.lv.n[0] + 31) >> 5)) return;  // whole warps
+  sw_down_warp<T, NX, DIR, HASG>(a, blockIdx.y, g);
 }
 
 // The time scale the GMRES-step kernels read: the device copy for a fixed final time, none
@@ -725,66 +677,59 @@ static const double* sdev_of(const Problem* pr) { return pr->free_time ? nullptr
 template <typename T>
 static Levels<T> levels_of(const Problem* pr, const OpData& d) {
   Levels<T> lv;
-  memset(&lv, 0, sizeof(lv));
+  memset((void*)&lv, 0, sizeof(lv));
   lv.nlev = pr->nlev;
   for (int l = 0; l < pr->nlev; ++l) {
     lv.m[l] = (const T*)d.lvm[l];
     lv.o[l] = (T*)d.lvo[l];
     lv.e[l] = (T*)d.lve[l];
+    lv.es[l] = round_up(pr->lvn[l], 32) * pr->n_x;
     lv.n[l] = pr->lvn[l];
+    lv.cnt0[l] = lv.ncnt;
+    if (l > 0) lv.ncnt += (pr->lvn[l] + 31) / 32;
   }
+  lv.cnt = d.lvcnt;
   lv.sdev = sdev_of(pr);
   return lv;
 }
 
-// Sweep launch form: 0 automatic, 1 one CTA (small grids only), 2 one warp per CTA, 3 four
-// warps per CTA (BK_SWEEP_FORM overrides the automatic choice, for timing).
-static int sweep_form() {
-  static const int f = [] {
-    const char* e = getenv("BK_SWEEP_FORM");
-    const int v = e ? atoi(e) : 0;
-    return v >= 1 && v <= 3 ? v : 0;
-  }();
-  return f;
-}
-
-template <typename T, int NX, int DIR, int W>
-static bk_status run_sweep_multi(Problem* pr, OpData& d, const T* Y, const T* G, T* out, T* bout, const T* w, T s,
-                                 const Levels<T>& lv, cudaStream_t st) {
-  const int g0 = (((pr->lvn[0] + 31) >> 5) + W - 1) / W;
-  BK_TRY(launch(k_sw_up0<T, NX, DIR, W>, g0, 32 * W, 0, st, (const T*)d.Dn, Y, G, pr->P, pr->L, w, s, lv));
-  for (int l = 1; l < pr->nlev; ++l) {
-    const int gl = (((pr->lvn[l] + 31) >> 5) + W - 1) / W;
-    BK_TRY(launch(k_sw_upL<T, NX, DIR, W>, gl, 32 * W, 0, st, lv, l));
-  }
-  BK_TRY(launch(k_sw_down0<T, NX, DIR, W>, g0, 32 * W, 0, st, (const T*)d.Dn, Y, G, pr->P, pr->L, w, s, lv, out, bout));
-  return BK_OK;
-}
-
-// Full sweep: out = P^{-1} (Y, forcing G) (DIR 0) or P^{-T} Y with bout = B-tilde^T out (DIR 1).
-// Grids with at most two scan levels and 16 level-0 blocks: one launch (k_sw_one). Otherwise
-// nlev + 1 launches (the level-0 up pass, one scan per upper level, the down pass), one warp per
-// CTA while level 0 has fewer than four blocks per SM, else four. Measured orbit solves (GB300,
-// host-form GMRES, ms, one CTA / 1-warp / 4-warp CTAs): FP64 2^8 7.35 / 7.61 / 7.56, FP32 2^16
-// (1-warp range) - / 7.29 / 8.18, FP64 2^16 - / 12.84 / 13.04.
+// Full sweep of ncol columns: out = P^{-1} (Y, forcing G) (DIR 0) or P^{-T} Y with bout =
+// B-tilde^T out (DIR 1); a holds the operands, the rest is filled in here. Two launches: the up
+// pass with every scan level, and the down pass. Measured (GB300, us per KKT preconditioner, which
+// takes two sweeps; nlev + 1 launches with staged loads / this form): FP32 N = 2^12 70 / 35, 2^16
+// 78 / 42, FP64 2^14 114 / 87, 2^17 120 / 110, 2^20 586 / 512.
 template <typename T, int NX, int DIR>
-static bk_status run_sweep(Problem* pr, OpData& d, const T* Y, const T* G, T* out, T* bout, cudaStream_t st) {
+static bk_status run_sweep(Problem* pr, OpData& d, SweepArgs<T>& a, int ncol, cudaStream_t st) {
   // segment length and level data follow the problem's preconditioner precision
   BK_ARG(d.dtype == pr->pdtype && d.Dn != nullptr, "sweeps run in the preconditioner's precision only");
-  const T* w = (const T*)d.w;
-  const T s = (T)pr->s;
-  const Levels<T> lv = levels_of<T>(pr, d);
+  BK_ARG(ncol >= 1 && ncol <= std::max(1, pr->n_e), "bad sweep column count");
+  a.lv = levels_of<T>(pr, d);
+  a.Dn = (const T*)d.Dn;
+  a.w = (const T*)d.w;
+  a.P = pr->P;
+  a.L = pr->L;
+  a.s = (T)pr->s;
   const int nblk0 = (pr->lvn[0] + 31) >> 5;
-  int form = sweep_form();
-  if (form == 1 && !(pr->nlev <= 2 && nblk0 <= SW1_MAXW)) form = 0;
-  if (form == 0) form = nblk0 < 4 * 152 ? 2 : 3;
-  if (form == 1) {
-    BK_TRY(launch(k_sw_one<T, NX, DIR>, 1, 32 * nblk0, nblk0 * sizeof(SweepTiles<T, NX>), st, 
-        (const T*)d.Dn, Y, G, pr->P, pr->L, w, s, lv, out, bout));
+  uintptr_t al = (uintptr_t)a.Y | (uintptr_t)a.out | (uintptr_t)a.bout;
+  for (int c = 0; c < ncol; ++c) al |= (uintptr_t)a.G[c];
+  a.vec = (al & 15) == 0;   // pitch and column strides are multiples of 32 elements
+  auto run = [&](auto hasg) -> bk_status {
+    constexpr bool HASG = decltype(hasg)::value;
+    if (nblk0 < 4 * 152) {
+      const dim3 grid(nblk0, ncol);
+      BK_TRY(launch(k_sw_up<T, NX, DIR, HASG, 1>, grid, 32, 0, st, a));
+      BK_TRY(launch(k_sw_down<T, NX, DIR, HASG, 1>, grid, 32, 0, st, a));
+    } else {
+      const dim3 grid((nblk0 + 3) / 4, ncol);
+      BK_TRY(launch(k_sw_up<T, NX, DIR, HASG, 4>, grid, 128, 0, st, a));
+      BK_TRY(launch(k_sw_down<T, NX, DIR, HASG, 4>, grid, 128, 0, st, a));
+    }
     return BK_OK;
+  };
+  if constexpr (DIR == 0) {
+    if (a.G[0]) return run(std::true_type());
   }
-  if (form == 2) return run_sweep_multi<T, NX, DIR, 1>(pr, d, Y, G, out, bout, w, s, lv, st);
-  return run_sweep_multi<T, NX, DIR, 4>(pr, d, Y, G, out, bout, w, s, lv, st);
+  return run(std::false_type());
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1060,15 +1005,28 @@ __global__ void k_border_fix(const T* __restrict__ q, const double* __restrict__
 // ---------------------------------------------------------------------------------------------
 // KKT preconditioner elementwise kernels
 // ---------------------------------------------------------------------------------------------
-// yu_q = (r_u,q + s sum_m Ju[m][q] b_m) / (s w_k cost_uu);  g_m = sum_q Ju[m][q] yu_q
+// y_q = (r_u,q + s sum_m Ju[m][q] b_m) / (s w_k), yu = ysign y;  g_m = sum_q Ju[m][q] y_q; the
+// columns blockIdx.y of b (bs apart), yu (yus apart) and g
+template <typename T> struct PreUArgs {
+  const T* ru;   // null: zero
+  const T* b;
+  int64_t bs;
+  T* yu;
+  int64_t yus;
+  T* g[NEM];
+  T ysign;
+};
 template <typename T, int KIND>
-__global__ void k_pre_u(const T* __restrict__ xu, const T* __restrict__ w, T s, T cost_uu, const T* __restrict__ ru,
-                        const T* __restrict__ b, int64_t P, int64_t L, T* __restrict__ yu, T* __restrict__ g,
-                        T gsign, const T* __restrict__ mu, T pa, const double* __restrict__ sdev,
+__global__ void k_pre_u(const __grid_constant__ PreUArgs<T> a, const T* __restrict__ xu, const T* __restrict__ w, T s,
+                        int64_t P, int64_t L, const T* __restrict__ mu, T pa, const double* __restrict__ sdev,
                         const T* __restrict__ hbar) {
   pdl_wait();
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
   if (sdev) s = T(*sdev);
+  const T* __restrict__ ru = a.ru;
+  const T* __restrict__ b = a.b + blockIdx.y * a.bs;
+  T* __restrict__ yu = a.yu + blockIdx.y * a.yus;
+  T* __restrict__ g = a.g[blockIdx.y];
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
     if (k >= L) {
 #pragma unroll
@@ -1086,7 +1044,7 @@ __global__ void k_pre_u(const T* __restrict__ xu, const T* __restrict__ w, T s, 
     T mk[NXM];
 #pragma unroll
     for (int m = 0; m < NX; ++m) mk[m] = Dyn<KIND>::huu_needs_mu ? mu[m * P + k] : T(0);
-    const T huu = Dyn<KIND>::template pre_huu<T>(mk, s * w[k] * cost_uu, pa);
+    const T huu = Dyn<KIND>::template pre_huu<T>(mk, s * w[k], pa);
     // control bounds: the barrier's diagonal joins the (diagonal) control block, one inverse per
     // control (for two controls from one division: 1/h0 = h1 r, 1/h1 = h0 r, r = 1/(h0 h1))
     T inv[NUM];
@@ -1109,46 +1067,46 @@ __global__ void k_pre_u(const T* __restrict__ xu, const T* __restrict__ w, T s, 
     }
 #pragma unroll
     for (int q = 0; q < NU; ++q) {
-      T a = ru ? ru[q * P + k] : T(0);
+      T t = ru ? ru[q * P + k] : T(0);
 #pragma unroll
       for (int m = 0; m < NX; ++m)
-        if (Dyn<KIND>::ju_nz(m, q)) a += s * Ju[m * NU + q] * b[m * P + k];
-      y[q] = a * inv[q];
-      yu[q * P + k] = y[q];
+        if (Dyn<KIND>::ju_nz(m, q)) t += s * Ju[m * NU + q] * b[m * P + k];
+      y[q] = t * inv[q];
+      yu[q * P + k] = a.ysign * y[q];
     }
 #pragma unroll
     for (int m = 0; m < NX; ++m) {
-      T a = T(0);
+      T t = T(0);
 #pragma unroll
       for (int q = 0; q < NU; ++q)
-        if (Dyn<KIND>::ju_nz(m, q)) a += Ju[m * NU + q] * y[q];
-      g[m * P + k] = gsign * a;
+        if (Dyn<KIND>::ju_nz(m, q)) t += Ju[m * NU + q] * y[q];
+      g[m * P + k] = t;
     }
   }
 }
 
-// y_nu = S^{-1} (q[term, N] - r_nu)   (one thread)
-template <typename T>
-__global__ void k_pre_nu(const T* __restrict__ q, const T* __restrict__ rnu, const T* __restrict__ Sinv, int64_t P,
-                         int64_t L, TermSpec ts, T* __restrict__ ynu) {
-  pdl_wait();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  T rhs[NEM];
-  for (int r = 0; r < ts.n_e; ++r) rhs[r] = T(ts.ea[r]) * q[ts.idx[r] * P + (L - 1)] - rnu[r];
-  for (int r = 0; r < 32; ++r) {
-    T a = T(0);
-    if (r < ts.n_e)
-      for (int c = 0; c < ts.n_e; ++c) a += Sinv[r * ts.n_e + c] * rhs[c];
-    ynu[r] = a;
-  }
-}
-
-// y_u += HW y_nu; y_x -= Q y_nu; y_lambda -= Z y_nu
+// y_nu = S^{-1} (E q - r_nu) with q at the last node in qlast (every CTA forms it for itself; block
+// 0 writes it), then y_u += HW y_nu; y_x -= Q y_nu; y_lambda -= Z y_nu.
 template <typename T, int NX, int NU>
 __global__ void k_pre_fix(const T* __restrict__ Zc, const T* __restrict__ HWc, const T* __restrict__ Qc,
-                          const T* __restrict__ ynu, int n_e, int64_t P, int64_t L, T* __restrict__ yx,
-                          T* __restrict__ yu, T* __restrict__ yl) {
+                          const T* __restrict__ qlast, const T* __restrict__ rnu, const T* __restrict__ Sinv,
+                          const __grid_constant__ TermSpec ts, int64_t P, int64_t L, T* __restrict__ yx,
+                          T* __restrict__ yu, T* __restrict__ yl, T* __restrict__ ynu) {
   pdl_wait();
+  __shared__ T cs[NEM];
+  const int n_e = ts.n_e;
+  if (threadIdx.x < 32) {
+    const int r = threadIdx.x;
+    T t = T(0);
+    if (r < n_e) {
+#pragma unroll
+      for (int c = 0; c < NEM; ++c)
+        if (c < n_e) t += Sinv[r * n_e + c] * (T(ts.ea[c]) * qlast[ts.idx[c]] - rnu[c]);
+      cs[r] = t;
+    }
+    if (blockIdx.x == 0) ynu[r] = t;
+  }
+  __syncthreads();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
     // the node's outputs stay in registers over the n_e columns (one read and one write each)
     T ax[NX], al[NX], au[NU];
@@ -1156,8 +1114,10 @@ __global__ void k_pre_fix(const T* __restrict__ Zc, const T* __restrict__ HWc, c
     for (int m = 0; m < NX; ++m) { ax[m] = yx[m * P + k]; al[m] = yl[m * P + k]; }
 #pragma unroll
     for (int q = 0; q < NU; ++q) au[q] = yu[q * P + k];
-    for (int r = 0; r < n_e; ++r) {
-      const T c = ynu[r];
+#pragma unroll
+    for (int r = 0; r < NEM; ++r) {
+      if (r >= n_e) break;
+      const T c = cs[r];
 #pragma unroll
       for (int m = 0; m < NX; ++m) {
         ax[m] -= c * Qc[((int64_t)r * NX + m) * P + k];
@@ -1171,13 +1131,6 @@ __global__ void k_pre_fix(const T* __restrict__ Zc, const T* __restrict__ HWc, c
 #pragma unroll
     for (int q = 0; q < NU; ++q) yu[q * P + k] = au[q];
   }
-}
-
-template <typename T>
-__global__ void k_unit(T* v, int64_t n, int64_t idx) {
-  pdl_wait();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    v[i] = i == idx ? T(1) : T(0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1379,7 +1332,6 @@ template <int KIND> struct KindNX { static constexpr int nx = Dyn<KIND>::nx, nu 
 
 static bk_status alloc_opdata(Problem* pr, OpData& d, int dtype) {
   d.dtype = dtype;
-  BK_TRY(dtype == BK_F64 ? sweep_attrs_nx<double>(pr->n_x) : sweep_attrs_nx<float>(pr->n_x));
   const size_t es = dtype_size(dtype);
   const int64_t P = pr->P;
   const int nx = pr->n_x, nu = pr->n_u, ne = pr->n_e;
@@ -1395,12 +1347,22 @@ static bk_status alloc_opdata(Problem* pr, OpData& d, int dtype) {
   if (pre) {
     BK_TRY(dmalloc(&d.Dn, es * il));   // the node deviations D (K = I + D, N = 2 D)
   }
+  int64_t ncnt = 0;
   for (int l = 0; pre && l < pr->nlev; ++l) {
     const size_t npad = (size_t)round_up(pr->lvn[l], 32);
     BK_TRY(dmalloc(&d.lvm[l], es * NSLOT * npad * nx * nx));
-    BK_TRY(dmalloc(&d.lve[l], es * npad * nx));
-    if (l > 0) BK_TRY(dmalloc(&d.lvo[l], es * npad * nx));
+    const int nc = std::max(1, ne);   // the terminal Schur columns are swept side by side
+    BK_TRY(dmalloc(&d.lve[l], es * npad * nx * nc));
+    if (l > 0) {
+      BK_TRY(dmalloc(&d.lvo[l], es * npad * nx * nc));
+      ncnt += nc * ((pr->lvn[l] + 31) / 32);
+    }
   }
+  if (ncnt > 0) {
+    BK_TRY(dmalloc((void**)&d.lvcnt, sizeof(unsigned) * ncnt));
+    BK_TRY_CUDA(cudaMemset(d.lvcnt, 0, sizeof(unsigned) * ncnt));
+  }
+  if (pre) BK_TRY(dmalloc(&d.qlast, es * NEM * NXM));
   if (pre && pr->free_time) {
     BK_TRY(dmalloc(&d.brd, es * pr->kkt_len()));
     BK_TRY(dmalloc(&d.brq, es * pr->kkt_len()));
@@ -1420,7 +1382,7 @@ static bk_status alloc_opdata(Problem* pr, OpData& d, int dtype) {
 
 static void free_opdata(OpData& d) {
   if (d.plan) plan_destroy(d.plan);
-  void* ps[] = {d.xu, d.mu, d.Dn, d.Zc, d.HWc, d.Qc, d.Sinv, d.t1, d.t2, d.t3, d.brd, d.brq, d.bgam, d.hbar};
+  void* ps[] = {d.xu, d.mu, d.Dn, d.Zc, d.HWc, d.Qc, d.Sinv, d.t1, d.t2, d.t3, d.brd, d.brq, d.bgam, d.hbar, d.lvcnt, d.qlast};
   for (void* p : ps) dfree(p);
   for (int l = 0; l < MAXLEV; ++l) {
     dfree(d.lvm[l]);
@@ -1487,49 +1449,47 @@ static bk_status lin_factors(Problem* pr, OpData& d, const double* z, cudaStream
   return lin_levels<T, NX>(pr, d, st);
 }
 
-template <typename T>
-__global__ void k_negate(T* v, int64_t n) {
-  pdl_wait();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) v[i] = -v[i];
-}
-
 // Terminal Schur data of the KKT preconditioner (see precond_kkt): the launches, ending with the
-// n_e x n_e entries of S copied into pinned host memory (lin_schur_finish inverts S).
+// last-node values of the columns Q copied into pinned host memory (lin_schur_finish inverts S). The
+// n_e columns run side by side in every launch (one after another, the FP32 solve at N = 2^12 spent
+// 42 sweeps and 60 smaller launches on them).
 template <typename T, int KIND>
 static bk_status lin_schur_launch(Problem* pr, OpData& d, cudaStream_t st) {
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
   const int ne = pr->n_e;
   if (ne == 0 || !pr->has_cost) return BK_OK;
-  const int64_t P = pr->P, L = pr->L;
-  const T s = (T)pr->s;
+  BK_ARG(ne <= 3, "more than three terminal conditions");
+  const int64_t P = pr->P;
   T* Zc = (T*)d.Zc;
   T* HWc = (T*)d.HWc;
   T* Qc = (T*)d.Qc;
-  T* unit = (T*)d.t1;   // n_x * P
-  T* bz = (T*)d.t2;     // n_x * P : B-tilde^T Z_r
-  T* g = (T*)d.t3;      // n_x * P : forcing
-  for (int r = 0; r < ne; ++r) {
-    BK_TRY(launch(k_unit<T>, nblk(NX * P), 256, 0, st, unit, NX * P, (int64_t)pr->term_idx[r] * P + (L - 1)));
-    T* Z = Zc + (int64_t)r * NX * P;
-    BK_TRY((run_sweep<T, NX, 1>(pr, d, unit, nullptr, Z, bz, st)));
-    // W = Pu^T Z = -s Ju^T (B-tilde^T Z). k_pre_u with r_u = 0 and b = B-tilde^T Z gives
-    // yu = s Ju^T b / (s w) = -H~^{-1} W and g = Ju yu = -Ju H~^{-1} W.
-    T* HW = HWc + (int64_t)r * NU * P;
-    BK_TRY(launch(k_pre_u<T, KIND>, nblk(P), 256, 0, st, (const T*)d.xu, (const T*)d.w, s, (T)1, nullptr, bz, P, L, HW, g, T(1),
-                                              (const T*)d.mu, (T)pr->dyn_param(), nullptr, bar_hbar<T>(pr, d)));
-    // Q = P^{-1} Pu HW: forward sweep with Y = 0 and forcing -Ju HW = Ju (-HW) = g
-    BK_TRY(launch(k_unit<T>, nblk(NX * P), 256, 0, st, unit, NX * P, -1));
-    T* Q = Qc + (int64_t)r * NX * P;
-    BK_TRY((run_sweep<T, NX, 0>(pr, d, unit, g, Q, nullptr, st)));
-  }
-  // HWc holds -H~^{-1} W: negate it
-  BK_TRY(launch(k_negate<T>, nblk((int64_t)ne * NU * P), 256, 0, st, HWc, (int64_t)ne * NU * P));
-  // S = E Q: S[r][c] = Q_c[term_idx[r]][N], into pinned host memory
-  T* hq = reinterpret_cast<T*>(pr->red_host + 256);
-  for (int c = 0; c < ne; ++c)
-    for (int r = 0; r < ne; ++r)
-      BK_TRY_CUDA(cudaMemcpyAsync(&hq[r * ne + c], Qc + ((int64_t)c * NX + pr->term_idx[r]) * P + (L - 1), sizeof(T),
-                                  cudaMemcpyDeviceToHost, st));
+  T* const g[3] = {(T*)d.t1, (T*)d.t2, (T*)d.t3};   // forcing per column, n_x * P each
+  SweepArgs<T> a = {};
+  a.out = Zc;
+  a.os = a.bs = NX * P;
+  a.bout = Qc;   // B-tilde^T Z_r, until the forward sweep writes Q there
+  for (int r = 0; r < ne; ++r) a.unit[r] = pr->term_idx[r];
+  BK_TRY((run_sweep<T, NX, 1>(pr, d, a, ne, st)));
+  // W = Pu^T Z = -s Ju^T (B-tilde^T Z). k_pre_u with r_u = 0 and b = B-tilde^T Z gives
+  // y = s Ju^T b / (s w) = -H~^{-1} W and g = Ju y = -Ju H~^{-1} W; HWc = H~^{-1} W = -y.
+  PreUArgs<T> u = {};
+  u.b = Qc;
+  u.bs = NX * P;
+  u.yu = HWc;
+  u.yus = NU * P;
+  for (int r = 0; r < ne; ++r) u.g[r] = g[r];
+  u.ysign = T(-1);
+  BK_TRY(launch(k_pre_u<T, KIND>, dim3(nblk(P), ne), 256, 0, st, u, (const T*)d.xu, (const T*)d.w, (T)pr->s, P, pr->L,
+                (const T*)d.mu, (T)pr->dyn_param(), nullptr, bar_hbar<T>(pr, d)));
+  // Q = P^{-1} Pu HW: forward sweep with Y = 0 and forcing -Ju HW = g
+  SweepArgs<T> f = {};
+  f.out = Qc;
+  f.os = NX * P;
+  for (int r = 0; r < ne; ++r) f.G[r] = g[r];
+  f.last = (T*)d.qlast;
+  BK_TRY((run_sweep<T, NX, 0>(pr, d, f, ne, st)));
+  // S = E Q: S[r][c] = Q_c[term_idx[r]][N], from the columns' last-node values
+  BK_TRY_CUDA(cudaMemcpyAsync(pr->red_host + 256, d.qlast, sizeof(T) * ne * NX, cudaMemcpyDeviceToHost, st));
   return BK_OK;
 }
 
@@ -1539,9 +1499,10 @@ static bk_status lin_schur_finish(Problem* pr, OpData& d, cudaStream_t st) {
   std::vector<double> S(ne * ne);
   BK_TRY_CUDA(cudaStreamSynchronize(st));
   const T* hq = reinterpret_cast<const T*>(pr->red_host + 256);
-  for (int i = 0; i < ne * ne; ++i) S[i] = (double)hq[i];
+  for (int r = 0; r < ne; ++r)
+    for (int c = 0; c < ne; ++c) S[r * ne + c] = (double)hq[c * pr->n_x + pr->term_idx[r]];
   // endpoint bounds: rows ea_r (E x)_r + ec_r nu_r = r_r give (diag(ea) E Q - diag(ec)) nu =
-  // diag(ea) E x0 - r (k_pre_nu scales its E x0 by ea)
+  // diag(ea) E x0 - r (k_pre_fix scales its E x0 by ea)
   for (int r = 0; r < ne; ++r) {
     if (!(pr->has_ebounds && pr->term_bnd[r])) continue;
     for (int c = 0; c < ne; ++c) S[r * ne + c] *= pr->term_ea[r];
@@ -1726,9 +1687,12 @@ static bk_status precond_typed(Problem* pr, OpData& d, int op, const T* in, T* o
                                bool border = true) {
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NV = NX + NU;
   const int64_t P = pr->P, L = pr->L;
+  SweepArgs<T> a = {};
   if (op == BK_OP_STATE) {
-    if (!transpose) return run_sweep<T, NX, 0>(pr, d, in, nullptr, out, nullptr, st);
-    return run_sweep<T, NX, 1>(pr, d, in, nullptr, out, nullptr, st);
+    a.Y = in;
+    a.out = out;
+    if (!transpose) return run_sweep<T, NX, 0>(pr, d, a, 1, st);
+    return run_sweep<T, NX, 1>(pr, d, a, 1, st);
   }
   BK_ARG(pr->has_cost, "the KKT preconditioner needs a control cost (problem kind has none)");
   const T* rx = in;
@@ -1741,13 +1705,27 @@ static bk_status precond_typed(Problem* pr, OpData& d, int op, const T* in, T* o
   T* ynu = out + (NV + NX) * P;
   T* b = (T*)d.t1;
   T* g = (T*)d.t2;
-  BK_TRY((run_sweep<T, NX, 1>(pr, d, rx, nullptr, yl, b, st)));
-  BK_TRY(launch(k_pre_u<T, KIND>, nblk(P), 256, 0, st, (const T*)d.xu, (const T*)d.w, (T)pr->s, (T)1, ru, b, P, L, yu, g, T(1),
-                                            (const T*)d.mu, (T)pr->dyn_param(), sdev_of(pr), bar_hbar<T>(pr, d)));
-  BK_TRY((run_sweep<T, NX, 0>(pr, d, rl, g, yx, nullptr, st)));
+  a.Y = rx;
+  a.out = yl;
+  a.bout = b;
+  BK_TRY((run_sweep<T, NX, 1>(pr, d, a, 1, st)));
+  PreUArgs<T> u = {};
+  u.ru = ru;
+  u.b = b;
+  u.yu = yu;
+  u.g[0] = g;
+  u.ysign = T(1);
+  BK_TRY(launch(k_pre_u<T, KIND>, nblk(P), 256, 0, st, u, (const T*)d.xu, (const T*)d.w, (T)pr->s, P, L,
+                (const T*)d.mu, (T)pr->dyn_param(), sdev_of(pr), bar_hbar<T>(pr, d)));
+  SweepArgs<T> f = {};
+  f.Y = rl;
+  f.G[0] = g;
+  f.out = yx;
+  f.last = (T*)d.qlast;
+  BK_TRY((run_sweep<T, NX, 0>(pr, d, f, 1, st)));
   if (pr->n_e > 0) {
-    BK_TRY(launch(k_pre_nu<T>, 1, 32, 0, st, yx, rnu, (const T*)d.Sinv, P, L, term_spec(pr), ynu));
-    BK_TRY(launch(k_pre_fix<T, NX, NU>, nblk(L), 256, 0, st, (const T*)d.Zc, (const T*)d.HWc, (const T*)d.Qc, ynu, pr->n_e, P, L, yx, yu, yl));
+    BK_TRY(launch(k_pre_fix<T, NX, NU>, nblk(L), 256, 0, st, (const T*)d.Zc, (const T*)d.HWc, (const T*)d.Qc,
+                  (const T*)d.qlast, rnu, (const T*)d.Sinv, term_spec(pr), P, L, yx, yu, yl, ynu));
   } else {
     BK_TRY_CUDA(cudaMemsetAsync(ynu, 0, sizeof(T) * 32, st));
   }

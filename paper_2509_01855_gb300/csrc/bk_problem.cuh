@@ -290,8 +290,10 @@ struct OpData {
   void* Dn = nullptr;          // per-node D_k = h_k J_k K_k, K_k = (I - h_k J_k)^{-1} = I + D_k and
                                // N_k = 2 h_k J_k K_k = 2 D_k; interleaved (n_x^2 per node)
   void* lvm[MAXLEV] = {};      // per level: NSLOT matrix slots (n_x^2 per item each), working type
-  void* lvo[MAXLEV] = {};      // per level >= 1: item offsets from zero (n_x per item), per sweep
-  void* lve[MAXLEV] = {};      // per level: inclusive in-block scan values (n_x per item), per sweep
+  void* lvo[MAXLEV] = {};      // per level >= 1: item offsets from zero (n_x per item and column), per sweep
+  void* lve[MAXLEV] = {};      // per level: inclusive in-block scan values (n_x per item and column), per sweep
+  unsigned* lvcnt = nullptr;   // arrival counters of the levels' blocks (zero between sweeps)
+  void* qlast = nullptr;       // last-node values of a forward sweep, n_x per column
   // KKT preconditioner (terminal Schur data)
   void* Zc = nullptr;          // n_e state vectors   Z = P^{-T} E^T
   void* HWc = nullptr;         // n_e control vectors H~^{-1} W, W = Pu^T Z
