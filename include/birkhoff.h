@@ -181,7 +181,8 @@ bk_status bk_plan_set_dense(bk_plan* plan, int on, void* stream);
 
 /* How a plan computes its products. *path: 0 one CTA per vector (small N), 1 four-step FFT in
  * one launch (a cluster of CTAs per vector), 2 four-step FFT split into a launch per pass, 3 dense
- * product, 4 Bluestein convolution (N not a power of two above 1024). For paths 1 and 2: the
+ * product, 4 Bluestein convolution (N above 1024 that is neither a power of two nor, with a
+ * path 2 of mixed radix, 16 times a product of 2, 3 and 5). For paths 1 and 2: the
  * rows N1 and columns N2 that the real-even four-step transform keeps (half of its factors, N1 N2 =
  * N / 2) and the complex elements per CTA, for path 2 as chosen by the tile autotuner at plan
  * creation (or by the occupancy heuristic when tuning is off: environment BK_AUTOTUNE=0). Outputs

@@ -167,6 +167,17 @@ __global__ void k_stage_tw(typename V2<T>::t* stw, int log2n, int e, int len) {
   }
 }
 
+// Twiddles of one mixed-radix stage: stw[(r - 1) Ns + k] = omega_{R Ns}^{r k}.
+template <typename T>
+__global__ void k_mix_tw(typename V2<T>::t* stw, int Ns, int R) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (R - 1) * Ns; i += gridDim.x * blockDim.x) {
+    const int r = i / Ns + 1, k = i % Ns;
+    double sn, cs;
+    sincospi((double)(2 * r * k) / (double)(R * Ns), &sn, &cs);
+    stw[i] = mk2<T>((T)cs, (T)(-sn));
+  }
+}
+
 // Inter-pass twiddles of the real-even passes, [N1/2 + 1][N2/2 + 2] (2N = N1 N2; see bk_dct.cuh):
 // omega_2N^{n2 k} / 2 for a pair's first column (even positions; position 0 is column 0), times -i
 // for its second (odd positions; position 1 is column N2/2).
@@ -727,6 +738,26 @@ static bk_status build_stage_table(void** dst, int64_t n, int e, cudaStream_t st
   return BK_OK;
 }
 
+template <typename T>
+static bk_status build_mix_table(void** dst, const unsigned char* rad, int nst, cudaStream_t st) {
+  typedef typename V2<T>::t C;
+  int len = 0, Ns = 1;
+  for (int s = 0; s < nst; Ns *= rad[s++])
+    if (Ns > 1) len += (rad[s] - 1) * Ns;
+  if (len == 0) return BK_OK;
+  BK_TRY(dmalloc(dst, sizeof(C) * len));
+  C* p = (C*)*dst;
+  Ns = 1;
+  for (int s = 0; s < nst; Ns *= rad[s++]) {
+    if (Ns == 1) continue;
+    const int n = (rad[s] - 1) * Ns;
+    k_mix_tw<T><<<(n + 255) / 256, 256, 0, st>>>(p, Ns, rad[s]);
+    BK_CHECK_LAUNCH();
+    p += n;
+  }
+  return BK_OK;
+}
+
 // Tables of the plain complex layout: stage tables and the inter-pass twiddles.
 template <typename T>
 static bk_status build_fs_tables(FourStep& f, cudaStream_t st) {
@@ -782,8 +813,13 @@ static bk_status build_tables(Plan* p, cudaStream_t st) {
     if (N >= 16) BK_TRY(build_stage_table<T>(&p->stwS, N, SmallFft<T>::E, st));
   } else {
     const int e = p->split ? p->fe : SmallFft<T>::E;
-    BK_TRY(build_stage_table<T>(&p->fs.stw1, p->fs.N1, e, st));
-    BK_TRY(build_stage_table<T>(&p->fs.stw2, p->fs.N2, e, st));
+    if (p->mix) {
+      BK_TRY(build_mix_table<T>(&p->fs.stw1, p->rad1, p->nst1, st));
+      BK_TRY(build_mix_table<T>(&p->fs.stw2, p->rad2, p->nst2, st));
+    } else {
+      BK_TRY(build_stage_table<T>(&p->fs.stw1, p->fs.N1, e, st));
+      BK_TRY(build_stage_table<T>(&p->fs.stw2, p->fs.N2, e, st));
+    }
     BK_TRY(dmalloc(&p->fs.twN, sizeof(C) * p->fs.a_len()));
     k_re_tw<T><<<re_tw_blocks(p->fs), 256, 0, st>>>((C*)p->fs.twN, p->fs.N1, p->fs.N2);
     BK_CHECK_LAUNCH();
@@ -1028,6 +1064,71 @@ static bk_status configure_re(FourStep& f, int64_t N, int dtype, int fe, int nve
   return BK_OK;
 }
 
+// Mixed-radix lengths: n as radices, the odd ones first (their stage without twiddles), 0 stages when
+// n has another prime factor.
+static int mix_radices(int n, unsigned char* rad) {
+  int k = 0;
+  unsigned char r4[12];
+  int k4 = 0;
+  while (n % 5 == 0 && k < 12) { rad[k++] = 5; n /= 5; }
+  while (n % 3 == 0 && k < 12) { rad[k++] = 3; n /= 3; }
+  while (n % 4 == 0 && k4 < 12) { r4[k4++] = 4; n /= 4; }
+  if (n == 2 && k < 12) { rad[k++] = 2; n = 1; }
+  if (n != 1 || k + k4 > 12) return 0;
+  for (int i = 0; i < k4; ++i) rad[k++] = r4[i];
+  return k;
+}
+
+// Longest mixed-radix transform: two buffers of one transform in shared memory.
+static int mix_max(int dtype) { return dtype == BK_F64 ? 5120 : 10240; }
+
+// Factors 2N = N1 N2 of a mixed-radix plan: multiples of 4, N1 <= N2 as near as they come. False when N
+// has no such form (N must be 16 times a product of 2, 3 and 5: then both halves of the passes' pairing are
+// whole) or a factor is too long; Bluestein's convolution serves those, at 4 to 8 times the cost
+// (products of 4 components, convolution / mixed radix, us: FP64 N = 100000 690 / 106, FP32 122 / 25).
+static bool mix_factors(int64_t N, int dtype, int* N1, int* N2) {
+  if (N % 16 != 0 || is_pow2(N)) return false;
+  int64_t m = N / 16;
+  for (int f : {2, 3, 5})
+    while (m % f == 0) m /= f;
+  if (m != 1) return false;
+  int64_t best = 0;
+  for (int64_t a = 16; a * a <= 2 * N; a += 4)
+    if ((2 * N) % a == 0 && (2 * N / a) % 4 == 0) best = a;
+  if (best == 0 || 2 * N / best > mix_max(dtype)) return false;
+  unsigned char r[12];
+  if (mix_radices((int)best, r) == 0 || mix_radices((int)(2 * N / best), r) == 0) return false;
+  *N1 = (int)best;
+  *N2 = (int)(2 * N / best);
+  return true;
+}
+
+// Tiles of a mixed-radix plan for E complex elements per CTA (0: enough CTAs for two per SM).
+static bk_status configure_mix(Plan* p, int nvec, int Eforce) {
+  FourStep& f = p->fs;
+  if (!mix_factors(p->N, p->dtype, &f.N1, &f.N2)) {
+    set_error("mixed-radix configuration failed for N=%lld", (long long)p->N);
+    return BK_ERR_UNSUPPORTED;
+  }
+  f.n = 2 * p->N;
+  p->nst1 = mix_radices(f.N1, p->rad1);
+  p->nst2 = mix_radices(f.N2, p->rad2);
+  const int E = std::min(p->dtype == BK_F64 ? 4096 : 8192, fourstep_elems(p->dtype, p->N / 2, nvec, f.N1, f.N2 / 2, Eforce));
+  f.NB = std::max(1, std::min(E / f.N1, f.N2 / 4 + 1));
+  f.P = std::max(1, std::min(E / f.N2, f.N1 / 4 + 1));
+  f.bsA = f.N1 + f.N1 / 16 + 1;
+  f.bsB = f.N2 + f.N2 / 16 + 1;
+  const size_t csz = 2 * dtype_size(p->dtype);
+  f.smemA = csz * 2 * (size_t)f.NB * f.bsA;
+  f.smemB = csz * 2 * (size_t)f.P * f.bsB;
+  f.thrA = f.thrB = MixFft::MT;
+  if (f.smemA > FOURSTEP_SMEM_BUDGET || f.smemB > FOURSTEP_SMEM_BUDGET) {
+    set_error("mixed-radix tiles too large for N=%lld", (long long)p->N);
+    return BK_ERR_UNSUPPORTED;
+  }
+  return BK_OK;
+}
+
 // Tiles of the one-launch form: a cluster of at most 16 CTAs per vector, its column and row pairs
 // spread over all of them.
 static bk_status configure_cluster(Plan* p) {
@@ -1096,6 +1197,7 @@ static bk_status cluster_attr(F* fn, int cap) {
 template <typename T>
 bk_status re_attrs() {
   const int cap = (int)FOURSTEP_SMEM_BUDGET;
+  if constexpr (!std::is_same<T, dfl>::value) BK_TRY((re_attrs_AB<T, MixFft>(cap)));
   if constexpr (sizeof(T) == 4) {
     BK_TRY((re_attrs_AB<T, FftShape<T, 2>>(cap)));
     BK_TRY((re_attrs_AB<T, FftShape<T, 4>>(cap)));
@@ -1190,6 +1292,7 @@ static bool dense_default(int dtype, int64_t N, int nvec) {
 // Four-step shapes of a plan for E complex elements per CTA (0: the occupancy heuristic).
 static bk_status fourstep_shapes(Plan* p, int E) {
   const int nvec = p->n_comp * p->max_batch;
+  if (p->mix) return configure_mix(p, nvec, E);
   return p->split ? configure_re(p->fs, p->N, p->dtype, p->fe, nvec, E) : configure_cluster(p);
 }
 
@@ -1223,7 +1326,7 @@ static bk_status autotune_tiles(Plan* p, cudaStream_t st) {
       return fourstep_shapes(p, it->second);
     }
   }
-  const int cap = re_elems_max(p->fs, p->dtype, p->fe);
+  const int cap = p->mix ? (p->dtype == BK_F64 ? 4096 : 8192) : re_elems_max(p->fs, p->dtype, p->fe);
   const int emin = std::max(p->fs.N1, p->fs.N2);
   const size_t vbytes = dtype_size(p->dtype) * (size_t)p->pitch * nvec;
   void* vin = nullptr;
@@ -1308,13 +1411,17 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
   p->pitch = pitch;
   // N not a power of two: the FFT chain does not apply; every product is the dense one
   p->generic = !is_pow2(N) && dense_supported(N);
-  p->blue = !is_pow2(N) && !dense_supported(N);
+  {
+    int n1, n2;
+    p->mix = !is_pow2(N) && !dense_supported(N) && mix_factors(N, dtype, &n1, &n2);
+  }
+  p->blue = !is_pow2(N) && !dense_supported(N) && !p->mix;
   {
     const char* e = getenv("BK_DENSE_TEST_TIMEOUT");  // test mode of the dense kernel, as bk_plan_dense_test_timeout
     p->dtest = (e && e[0] == '1') ? 1 : 0;
   }
   p->df = dtype == BK_F64 && is_pow2(N) && N >= 256 && !weights_only && f64_df_default(N);
-  p->small = !p->generic && !p->blue && !p->df && N <= small_limit(dtype);
+  p->small = !p->generic && !p->blue && !p->mix && !p->df && N <= small_limit(dtype);
   bk_status st_ = BK_OK;
   AllocCounter counter(&p->bytes);
   do {
@@ -1343,8 +1450,8 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
       if ((st_ = dmalloc(&p->scrY, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
       if ((st_ = dmalloc(&p->scrG, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
     } else {
-      p->split = p->df || ilog2(N) >= std::min(2 * CL_MAXLOG2, split_min_log2(dtype));
-      p->fe = re_radix(N, dtype, p->df);
+      p->split = p->df || p->mix || ilog2(N) >= std::min(2 * CL_MAXLOG2, split_min_log2(dtype));
+      p->fe = p->mix ? 0 : re_radix(N, dtype, p->df);
       if ((st_ = fourstep_shapes(p, 0)) != BK_OK) break;
       const int64_t nvec = (int64_t)n_comp * max_batch;
       const size_t es = dtype_size(dtype);
@@ -1474,6 +1581,10 @@ static ReArgs<T> re_args(const Plan* p) {
   g.twA = (const C*)f.twN;
   g.rk = (const T*)p->rk;
   g.cE = (T)(2.0 / ((double)p->N + 1.0));
+  g.nst1 = p->nst1;
+  g.nst2 = p->nst2;
+  memcpy(g.rad1, p->rad1, sizeof(g.rad1));
+  memcpy(g.rad2, p->rad2, sizeof(g.rad2));
   return g;
 }
 
@@ -1488,6 +1599,9 @@ static bk_status re_launch_AF(const Plan* p, const S* src, int64_t sstride, int 
 }
 template <typename T, int K, typename S>
 static bk_status re_launch_A(const Plan* p, const S* src, int64_t sstride, int nvec, cudaStream_t st) {
+  if constexpr (!std::is_same<T, dfl>::value) {
+    if (p->mix) return re_launch_AF<T, K, MixFft>(p, src, sstride, nvec, st);
+  }
   if constexpr (sizeof(T) == 4) {
     if (p->fe == 4) return re_launch_AF<T, K, FftShape<T, 4>>(p, src, sstride, nvec, st);
     return re_launch_AF<T, K, FftShape<T, 2>>(p, src, sstride, nvec, st);
@@ -1507,6 +1621,9 @@ static bk_status re_launch_BF(const Plan* p, S* dst, int64_t dstride, int64_t ze
 }
 template <typename T, int E, typename S>
 static bk_status re_launch_B(const Plan* p, S* dst, int64_t dstride, int64_t zero_to, int nvec, T s, cudaStream_t st) {
+  if constexpr (!std::is_same<T, dfl>::value) {
+    if (p->mix) return re_launch_BF<T, E, MixFft>(p, dst, dstride, zero_to, nvec, s, st);
+  }
   if constexpr (sizeof(T) == 4) {
     if (p->fe == 4) return re_launch_BF<T, E, FftShape<T, 4>>(p, dst, dstride, zero_to, nvec, s, st);
     return re_launch_BF<T, E, FftShape<T, 2>>(p, dst, dstride, zero_to, nvec, s, st);

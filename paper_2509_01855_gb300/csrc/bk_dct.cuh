@@ -22,6 +22,9 @@
 // omega^m table indexed by n2 k1 cost one 32-byte sector per value), and holds the unpacking
 // factors 1/2 and -i/2.
 //
+// N that is 16 times a product of 2, 3 and 5 runs the same passes with N1 and N2 multiples of 4 and
+// mixed-radix FFTs.
+//
 // The second DCT's input is the integration stencil of the first one's output; pass A forms it in
 // its loads (two aligned pair loads per column pair), so a product is four passes and no stencil pass.
 #pragma once
@@ -36,6 +39,9 @@ template <typename T> struct ReArgs {
   const C* twA;    // [N1/2 + 1][RS]
   const T* rk;     // 1 / (4k), k = 0..N+1 (0 at k = 0)
   T cE;            // 2 / (N + 1)
+  // radices of the two FFT lengths (N not a power of two; bk_fft.cuh, fft_mix)
+  int nst1, nst2;
+  unsigned char rad1[12], rad2[12];
 };
 
 // Longest FFT of the one-launch form (its kernels hold an instance per length): N <= 2^17.
@@ -52,11 +58,16 @@ __device__ __noinline__ void re_fft_call(unsigned off, int log2n, int nbatch, in
                                                         reinterpret_cast<const C*>(smem + tw_off));
 }
 // F: the FFT's shape, void for the one-launch kernels' call.
+template <typename F> struct IsMix { static constexpr bool v = F::MIX; };
+template <> struct IsMix<void> { static constexpr bool v = false; };
 template <typename T, typename F>
-__device__ __forceinline__ void re_fft(typename V2<T>::t* buf, int log2n, int nbatch, int bs,
-                                       const typename V2<T>::t* stw) {
+__device__ __forceinline__ void re_fft(const ReArgs<T>& g, bool first, typename V2<T>::t* buf, typename V2<T>::t* alt,
+                                       int nbatch, int bs, const typename V2<T>::t* stw) {
   extern __shared__ __align__(16) unsigned char smem[];
-  if constexpr (std::is_void<F>::value)
+  const int log2n = first ? g.log2N1 : g.log2N2;
+  if constexpr (IsMix<F>::v)
+    fft_mix<T>(buf, alt, first ? g.N1 : g.N2, first ? g.rad1 : g.rad2, first ? g.nst1 : g.nst2, nbatch, bs, stw);
+  else if constexpr (std::is_void<F>::value)
     re_fft_call<T>((unsigned)(reinterpret_cast<unsigned char*>(buf) - smem), log2n, nbatch, bs,
                    (unsigned)(reinterpret_cast<const unsigned char*>(stw) - smem));
   else
@@ -146,7 +157,9 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
   const int p = p0 + b;
   const bool on = b < na && row0 < step;
   const bool last = p == (N2 >> 2);   // no second column
-  C* z = buf + b * bs;
+  // fft_mix alternates between two buffers: with an odd number of stages its input is the second
+  C* const alt = buf + NB * bs;
+  C* z = (IsMix<F>::v && (g.nst1 & 1) ? alt : buf) + b * bs;
   if (on && p != 0) {
     // rows j and N1 - 1 - j: x at m = j N2 + 2p - 1 and m + 1, and, reflected, at
     // i = (j + 1) N2 - 2p + 1 and i - 1 (m and i are odd)
@@ -208,7 +221,8 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
     }
   }
   __syncthreads();
-  re_fft<T, F>(buf, g.log2N1, na, bs, stw);
+  re_fft<T, F>(g, true, buf, alt, na, bs, stw);
+  z = buf + b * bs;
   if (on) {
     constexpr int LD = sizeof(T) == 8 ? 2 : 4;
     const C* tw = g.twA + 2 * p;
@@ -225,7 +239,7 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
         const int k = k0 + u * step;
         if (k > half) continue;
         const C zk = z[padi(k)];
-        const C zm = z[padi((N1 - k) & (N1 - 1))];
+        const C zm = z[padi(k == 0 ? 0 : N1 - k)];
         if (k == 0) part[p] = p == 0 ? zk.x + zk.y : T(2) * (zk.x + zk.y);
         const C sa = mk2<T>(zk.x + zm.x, zk.y - zm.y);   // Z_k + conj Z_{N1-k}
         const C sb = mk2<T>(zk.x - zm.x, zk.y + zm.y);   // Z_k - conj Z_{N1-k}
@@ -252,18 +266,19 @@ __device__ __forceinline__ void re_passB(const ReArgs<T>& g, int tile, int P, in
   const int nt = blockDim.x;
   const int N = g.N, N1 = g.N1, N2 = g.N2, h2 = N2 >> 1;
   const int na = min(P, (N1 >> 2) + 1 - q0);
+  C* const alt = buf + P * bs;
   {
     // positions 0..N2/2 of the two rows (pos 0, 1: columns 0 and N2/2, whose values are real;
     // pos >= 2: column pos - 1 and its mirror image N2 - pos + 1); threads along the rows
     const int tpr = min(nt, h2);
     const int i0 = threadIdx.x / tpr, istep = nt / tpr, ps0 = threadIdx.x - i0 * tpr;
     constexpr int LD = 4;
-    for (int i = i0; i < na; i += istep) {
+    for (int i = i0 < istep ? i0 : na; i < na; i += istep) {
       const int q = q0 + i;
       const C* ra = A + (int64_t)(q == 0 ? N1 >> 1 : 2 * q - 1) * g.RS;
       const C* rb = A + (int64_t)(2 * q) * g.RS;
       const bool two = q != (N1 >> 2);
-      C* z = buf + i * bs;
+      C* z = (IsMix<F>::v && (g.nst2 & 1) ? alt : buf) + i * bs;
       for (int ps = ps0; ps <= h2; ps += LD * tpr) {
         C a[LD], c[LD];
 #pragma unroll
@@ -300,7 +315,7 @@ __device__ __forceinline__ void re_passB(const ReArgs<T>& g, int tile, int P, in
     if (threadIdx.x == 0) *y0s = a;
   }
   __syncthreads();
-  re_fft<T, F>(buf, g.log2N2, na, bs, stw);
+  re_fft<T, F>(g, false, buf, alt, na, bs, stw);
   const T Y0 = DC ? *y0s : T(0);
   // threads along consecutive rows r = 2 q0 - 1 + c, so that each store run covers 2P consecutive
   // outputs: row r gives k = r + N1 j and, reflected, k = N1 (j + 1) - r from column N2 - 1 - j
@@ -357,7 +372,7 @@ __device__ __forceinline__ void re_passA_cta(const ReArgs<T>& g, int vec, int ti
   extern __shared__ __align__(16) unsigned char smem[];
   C* buf = reinterpret_cast<C*>(smem);
   const C* stw = g.stw1;
-  if (sizeof(T) == 4) {   // FP32: stage twiddles in shared memory after the tile
+  if (sizeof(T) == 4 && !F::MIX) {   // FP32: stage twiddles in shared memory after the tile
     C* tws = buf + (size_t)NB * bs;
     load_tw_smem<T>(tws, stw, stage_tw_len(g.log2N1, F::E));
     stw = tws;
@@ -375,7 +390,7 @@ __device__ __forceinline__ void re_passB_cta(const ReArgs<T>& g, int vec, int ti
   __shared__ T y0s;
   C* buf = reinterpret_cast<C*>(smem);
   const C* stw = g.stw2;
-  if (sizeof(T) == 4) {
+  if (sizeof(T) == 4 && !F::MIX) {
     C* tws = buf + (size_t)P * bs;
     load_tw_smem<T>(tws, stw, stage_tw_len(g.log2N2, F::E));
     stw = tws;

@@ -43,12 +43,15 @@ __host__ __device__ inline int stage_tw_len(int log2n, int e) {
 // resident CTAs per SM they are compiled for (64K registers / (threads x this) per thread).
 template <typename T, int E_> struct FftShape {
   static constexpr int E = E_, EPT = 1 << E_, MT = E_ == 4 ? 512 : (E_ == 3 ? 512 : 1024), MINB = MT == 512 ? 2 : 1;
+  static constexpr bool MIX = false;
 };
+// Launch-per-pass kernels of lengths 2^a 3^b 5^c (fft_mix).
+struct MixFft { static constexpr int E = 2, MT = 256, MINB = 2; static constexpr bool MIX = true; };
 // Radix of the launch-per-pass kernels (re_radix) and of the plain complex passes, and of the
 // one-CTA and one-launch kernels, whose few CTAs are bound by latency.
 template <typename T> struct CplxFft : FftShape<T, sizeof(T) == 4 ? 4 : 2> {};
 template <typename T> struct SmallFft : FftShape<T, 2> {};
-template <typename T> struct BigFft { static constexpr int E = std::is_same<T, dfl>::value ? 3 : 2, EPT = 16, MT = 512, MINB = 1; };
+template <typename T> struct BigFft { static constexpr int E = std::is_same<T, dfl>::value ? 3 : 2, EPT = 16, MT = 512, MINB = 1; static constexpr bool MIX = false; };
 
 // Radix-R DFT of v[0..R-1] in registers (forward, natural order in and out).
 template <typename C, typename T, int R> struct Radix;
@@ -94,6 +97,48 @@ template <typename C, typename T> struct Radix<C, T, 8> {
     v[6] = csub(e[2], o2);
     v[3] = cadd(e[3], o3);
     v[7] = csub(e[3], o3);
+  }
+};
+
+// omega_3 = -1/2 - i sqrt(3)/2.
+template <typename C, typename T> struct Radix<C, T, 3> {
+  static __device__ __forceinline__ void run(C* v) {
+    const T q = T(0.86602540378443864676372317075293618347140262690519);   // sqrt(3) / 2
+    const C t = cadd(v[1], v[2]), e = csub(v[1], v[2]);
+    C m;
+    m.x = v[0].x - T(0.5) * t.x;
+    m.y = v[0].y - T(0.5) * t.y;
+    v[0] = cadd(v[0], t);
+    v[1].x = m.x + q * e.y;
+    v[1].y = m.y - q * e.x;
+    v[2].x = m.x - q * e.y;
+    v[2].y = m.y + q * e.x;
+  }
+};
+
+// X_1,4 = v0 + c1 a1 + c2 a2 -+ i (s1 b1 + s2 b2), X_2,3 = v0 + c2 a1 + c1 a2 -+ i (s2 b1 - s1 b2)
+// with a_j = v_j + v_{5-j}, b_j = v_j - v_{5-j}, c_j + i s_j = e^{2 pi i j / 5}.
+template <typename C, typename T> struct Radix<C, T, 5> {
+  static __device__ __forceinline__ void run(C* v) {
+    const T c1 = T(0.30901699437494742410229341718281905886015458990288);
+    const T c2 = T(-0.80901699437494742410229341718281905886015458990288);
+    const T s1 = T(0.95105651629515357211643933337938214340569863412575);
+    const T s2 = T(0.58778525229247312916870595463907276859765243764314);
+    const C a1 = cadd(v[1], v[4]), b1 = csub(v[1], v[4]), a2 = cadd(v[2], v[3]), b2 = csub(v[2], v[3]);
+    C t1, t2, u1, u2;
+    t1.x = v[0].x + c1 * a1.x + c2 * a2.x;
+    t1.y = v[0].y + c1 * a1.y + c2 * a2.y;
+    t2.x = v[0].x + c2 * a1.x + c1 * a2.x;
+    t2.y = v[0].y + c2 * a1.y + c1 * a2.y;
+    u1.x = s1 * b1.x + s2 * b2.x;
+    u1.y = s1 * b1.y + s2 * b2.y;
+    u2.x = s2 * b1.x - s1 * b2.x;
+    u2.y = s2 * b1.y - s1 * b2.y;
+    v[0] = cadd(v[0], cadd(a1, a2));
+    v[1] = mk2<T>(t1.x + u1.y, t1.y - u1.x);
+    v[4] = mk2<T>(t1.x - u1.y, t1.y + u1.x);
+    v[2] = mk2<T>(t2.x + u2.y, t2.y - u2.x);
+    v[3] = mk2<T>(t2.x - u2.y, t2.y + u2.x);
   }
 };
 
@@ -310,6 +355,56 @@ __device__ __forceinline__ void fft_any(typename V2<T>::t* buf, int log2n, int n
                                         const typename V2<T>::t* __restrict__ stw) {
   if constexpr (std::is_same<T, dfl>::value) fft_rt<T, E, EPT>(buf, log2n, nbatch, bs, stw);
   else fft_ct_dispatch<T, E, EPT, LO, HI>(buf, log2n, nbatch, bs, stw);
+}
+
+// Batched forward FFT of length n = product of rad[0..nst), radices 2 to 5, over `nbatch` transforms bs
+// apart: Stockham stages between the two buffers a and b (the input in b when nst is odd, else in
+// a; the result in a), any thread count. stw: for each stage after the first, (R - 1) Ns twiddles
+// omega_{R Ns}^{r k} as in the power-of-two tables.
+template <typename T, int R>
+__device__ __forceinline__ void mix_stage(const typename V2<T>::t* src, typename V2<T>::t* dst, int n, int nbatch, int bs,
+                                          unsigned Ns, const typename V2<T>::t* __restrict__ stw) {
+  typedef typename V2<T>::t C;
+  const unsigned nb = (unsigned)n / R;
+  for (unsigned idx = threadIdx.x; idx < nb * nbatch; idx += blockDim.x) {
+    const unsigned q = idx / nb, j = idx - q * nb;
+    const unsigned jq = j / Ns, k = j - jq * Ns;
+    const C* s = src + q * bs;
+    C v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = s[padi(j + r * nb)];
+    if (Ns > 1) {
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], ldg(stw + (r - 1) * Ns + k));
+    }
+    Radix<C, T, R>::run(v);
+    C* o = dst + q * bs;
+    const unsigned d0 = jq * Ns * R + k;
+#pragma unroll
+    for (int r = 0; r < R; ++r) o[padi(d0 + r * Ns)] = v[r];
+  }
+  __syncthreads();
+}
+
+template <typename T>
+__device__ __forceinline__ void fft_mix(typename V2<T>::t* a, typename V2<T>::t* b, int n, const unsigned char* rad,
+                                        int nst, int nbatch, int bs, const typename V2<T>::t* __restrict__ stw) {
+  typedef typename V2<T>::t C;
+  C* src = (nst & 1) ? b : a;
+  C* dst = (nst & 1) ? a : b;
+  unsigned Ns = 1;
+  for (int s = 0; s < nst; ++s) {
+    const int R = rad[s];
+    if (R == 4) mix_stage<T, 4>(src, dst, n, nbatch, bs, Ns, stw);
+    else if (R == 5) mix_stage<T, 5>(src, dst, n, nbatch, bs, Ns, stw);
+    else if (R == 3) mix_stage<T, 3>(src, dst, n, nbatch, bs, Ns, stw);
+    else mix_stage<T, 2>(src, dst, n, nbatch, bs, Ns, stw);
+    if (Ns > 1) stw += (R - 1) * Ns;
+    Ns *= R;
+    C* t = src;
+    src = dst;
+    dst = t;
+  }
 }
 
 }  // namespace bk

@@ -52,6 +52,9 @@ struct Plan {
   // a launch each; else as one launch, a cluster of csize CTAs per vector.
   FourStep fs;
   int split = 0;
+  bool mix = false;           // N = 16 m, m a product of 2, 3 and 5 (not a power of two): mixed-radix
+  unsigned char rad1[12] = {}, rad2[12] = {};   // its radices of N1 and N2
+  int nst1 = 0, nst2 = 0;
   int fe = 2;                 // log2 radix of the launch-per-pass kernels
   int csize = 0, cthr = 0;
   size_t csmem = 0;

@@ -60,3 +60,19 @@ def test_longest_rows_in_double_float_and_binary64():
             _check(1 << 24, torch.float64, comps=1, path="split_four_step")
     finally:
         api.set_f64_transform(-1)
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("N", [1200, 1280, 2160, 6000, 16 * 625, 16 * 3 ** 6, 100000, 16 * 3 ** 4 * 5 ** 4])
+def test_mixed_radix_sizes(N, dtype):
+    """N = 16 m with m a product of 2, 3 and 5: every radix alone and mixed, odd and even stage counts."""
+    _check(N, dtype, path="split_four_step")
+
+
+@pytest.mark.parametrize("N", [1040, 1100, 3000, 4095, 16 * 7 * 11])
+def test_sizes_without_a_mixed_radix_form_keep_the_convolution(N):
+    _check(N, torch.float64, path="bluestein")
+
+
+def test_mixed_radix_longest():
+    _check(16 * 3 ** 4 * 5 ** 5, torch.float64, comps=1, path="split_four_step")   # N = 4050000
