@@ -426,8 +426,8 @@ __global__ void __launch_bounds__(1024)
 // omega_n^{j2 k1}; writes A[k1][j2]. Pass B: per CTA, 2P rows k1; FFT over j2 (length N2); writes
 // the outputs in natural order.
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
+template <typename T, typename F>
+__global__ void __launch_bounds__(F::MT, F::MINB)
     k_passA(const T* __restrict__ src, int64_t src_stride, typename V2<T>::t* __restrict__ Aout, int N, int N1,
             int log2N1, int N2, int NB, int bs, const typename V2<T>::t* __restrict__ stw,
             const typename V2<T>::t* __restrict__ twN, const typename V2<T>::t* __restrict__ twLo,
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
   // FP32: sub-FFT twiddles in shared memory after the tile (FP64 reads the global table)
   C* tws = buf + (size_t)NB * bs;
   const bool smem_tw = sizeof(T) == 4;
-  if (smem_tw) load_tw_smem<T>(tws, stw, stage_tw_len(log2N1, CplxFft<T>::E));
+  if (smem_tw) load_tw_smem<T>(tws, stw, stage_tw_len(log2N1, F::E));
   const int vec = blockIdx.y;
   const C* x = reinterpret_cast<const C*>(src + (int64_t)vec * src_stride);
   const int c0 = blockIdx.x * NB;
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
     }
   }
   __syncthreads();
-  fft_any<T, CplxFft<T>::E, CplxFft<T>::EPT>(buf, log2N1, NB, bs, smem_tw ? tws : stw);
+  fft_any<T, F::E, F::EPT>(buf, log2N1, NB, bs, smem_tw ? tws : stw);
   C* A = Aout + (int64_t)vec * N;
   // inter-pass twiddles omega_N^{j2 k1}, 4 independent table loads in flight per thread.
   // FP64: one table of omega_N^m (the FP64 pipe, not memory, bounds these kernels).
@@ -597,8 +597,8 @@ __global__ void __launch_bounds__(256) k_bs_post(const T* __restrict__ y, int64_
 
 // Pass B of the plain complex FFT: outputs as complex pairs in natural order; EP_CPLX_MC multiplies
 // by the spectral table and conjugates.
-template <typename T, int E>
-__global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
+template <typename T, int E, typename F>
+__global__ void __launch_bounds__(F::MT, F::MINB)
     k_passB(const typename V2<T>::t* __restrict__ Ain, T* __restrict__ dst, int64_t dst_stride, int N, int N1, int N2,
             int log2N2, int P, const typename V2<T>::t* __restrict__ stw, const typename V2<T>::t* __restrict__ tab) {
   pdl_wait();
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
   C* buf = reinterpret_cast<C*>(smem);
   C* tws = buf + (size_t)2 * P * bs;
   const bool smem_tw = sizeof(T) == 4;
-  if (smem_tw) load_tw_smem<T>(tws, stw, stage_tw_len(log2N2, CplxFft<T>::E));
+  if (smem_tw) load_tw_smem<T>(tws, stw, stage_tw_len(log2N2, F::E));
   const C* A = Ain + (int64_t)blockIdx.y * N;
   C* out = reinterpret_cast<C*>(dst + (int64_t)blockIdx.y * dst_stride);
   const int p0 = blockIdx.x * P;
@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(CplxFft<T>::MT, CplxFft<T>::MINB)
     }
   }
   __syncthreads();
-  fft_any<T, CplxFft<T>::E, CplxFft<T>::EPT>(buf, log2N2, 2 * P, bs, smem_tw ? tws : stw);
+  fft_any<T, F::E, F::EPT>(buf, log2N2, 2 * P, bs, smem_tw ? tws : stw);
   // lanes take consecutive rows, so each store run covers 2P consecutive outputs
   const int log2R = __ffs(2 * P) - 1;
   for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
@@ -760,10 +760,10 @@ static bk_status build_mix_table(void** dst, const unsigned char* rad, int nst, 
 
 // Tables of the plain complex layout: stage tables and the inter-pass twiddles.
 template <typename T>
-static bk_status build_fs_tables(FourStep& f, cudaStream_t st) {
+static bk_status build_fs_tables(FourStep& f, int e, cudaStream_t st) {
   typedef typename V2<T>::t C;
-  BK_TRY(build_stage_table<T>(&f.stw1, f.N1, CplxFft<T>::E, st));
-  BK_TRY(build_stage_table<T>(&f.stw2, f.N2, CplxFft<T>::E, st));
+  BK_TRY(build_stage_table<T>(&f.stw1, f.N1, e, st));
+  BK_TRY(build_stage_table<T>(&f.stw2, f.N2, e, st));
   const int64_t n = f.n;
   if (sizeof(T) == 8) {
     BK_TRY(dmalloc(&f.twN, sizeof(C) * n));
@@ -801,7 +801,7 @@ static bk_status build_tables(Plan* p, cudaStream_t st) {
   // FFT twiddles: single-CTA plans keep omega_N^i (direct DFT for N < 16) and the stage table of
   // N; four-step plans the stage tables of N1 and N2 and the inter-pass table.
   if (p->blue) {
-    BK_TRY(build_fs_tables<T>(p->fsM, st));
+    BK_TRY(build_fs_tables<T>(p->fsM, p->fe, st));
     BK_TRY(dmalloc(&p->chirp, sizeof(C) * N));
     k_chirp<T><<<(int)std::min<int64_t>((N + 255) / 256, 4096), 256, 0, st>>>((C*)p->chirp, N);
     BK_CHECK_LAUNCH();
@@ -968,13 +968,18 @@ static int split_min_log2(int dtype) {
 
 // Shapes of one four-step layout (tables untouched, so a built plan can be re-shaped); Eforce
 // > 0 fixes the elements per CTA (the autotuner's candidates), 0 takes fourstep_elems.
-static bk_status configure_fourstep(FourStep& f, int64_t n, int dtype, int nvec, int Eforce = 0) {
-  const int ept = dtype == BK_F64 ? CplxFft<double>::EPT : CplxFft<float>::EPT;
+// log2 radix of the plain complex passes of length n: 4 in FP32; in FP64 2 while few warps share the
+// FP64 pipes and 4 from 2^18 on, where its fewer shared-memory round trips count (products of 4
+// components, radix 4 / radix 16, us: N = 3001 61 / 127, N = 140001 1512 / 1344, N = 393217 2853 / 2433).
+static int cplx_radix(int dtype, int64_t n) { return dtype == BK_F64 && n < (int64_t(1) << 18) ? 2 : 4; }
+
+static bk_status configure_fourstep(FourStep& f, int64_t n, int dtype, int fe, int nvec, int Eforce = 0) {
+  const int ept = 1 << fe;
   const int log2n = ilog2(n);
   f.n = n;
   // balanced factors, with the rows short enough for one row pair per CTA (2 N2 / EPT threads)
   // and the columns for one column per CTA (N1 / EPT threads) under the thread cap
-  const int maxthr = dtype == BK_F64 ? CplxFft<double>::MT : CplxFft<float>::MT;
+  const int maxthr = (dtype == BK_F64 ? 4096 : 8192) / ept;
   int l2 = log2n - log2n / 2;
   while (l2 > 0 && (2 << l2) / ept > maxthr) --l2;
   f.N2 = 1 << l2;
@@ -1187,6 +1192,14 @@ static bk_status re_attrs_AB(int cap) {
   return re_attrs_B<T, F>(cap);
 }
 
+template <typename T, typename F>
+static bk_status cplx_attrs(int cap) {
+  BK_TRY(smem_attr(k_passA<T, F>, cap));
+  BK_TRY(smem_attr(k_passB<T, EP_CPLX, F>, cap));
+  BK_TRY(smem_attr(k_passB<T, EP_CPLX_MC, F>, cap));
+  return BK_OK;
+}
+
 template <typename F>
 static bk_status cluster_attr(F* fn, int cap) {
   BK_TRY(smem_attr(fn, cap));
@@ -1236,9 +1249,8 @@ bk_status set_smem_attrs(const Plan* p) {
   } else if (p->blue) {
     if constexpr (!std::is_same<T, dfl>::value) {
       const int cap = (int)FOURSTEP_SMEM_BUDGET;
-      BK_TRY(smem_attr(k_passA<T>, cap));
-      BK_TRY(smem_attr(k_passB<T, EP_CPLX>, cap));
-      BK_TRY(smem_attr(k_passB<T, EP_CPLX_MC>, cap));
+      BK_TRY((cplx_attrs<T, FftShape<T, 4>>(cap)));
+      if constexpr (sizeof(T) == 8) BK_TRY((cplx_attrs<T, FftShape<T, 2>>(cap)));
     }
   } else {
     BK_TRY(re_attrs<T>());
@@ -1444,7 +1456,8 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
       p->M = 1;
       while (p->M < 2 * N - 1) p->M *= 2;
       const int64_t nvec = (int64_t)n_comp * max_batch;
-      if ((st_ = configure_fourstep(p->fsM, p->M, dtype, (int)nvec)) != BK_OK) break;
+      p->fe = cplx_radix(dtype, p->M);
+      if ((st_ = configure_fourstep(p->fsM, p->M, dtype, p->fe, (int)nvec)) != BK_OK) break;
       const size_t csz = 2 * dtype_size(dtype);
       if ((st_ = dmalloc(&p->scrA, csz * (size_t)p->M * 2 * nvec)) != BK_OK) break;   // two M-vectors
       if ((st_ = dmalloc(&p->scrY, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
@@ -1518,17 +1531,23 @@ void plan_destroy(Plan* p) {
 // One length-M complex FFT on the plan's Bluestein layout: src (M complex per vector, as real
 // pairs) -> dst (same), through the four-step scratch A; E = EP_CPLX_MC multiplies by the
 // spectral table and conjugates in the store.
-template <typename T, int E>
-static bk_status blue_fft(const Plan* p, const T* src, T* dst, typename V2<T>::t* A, int nvec, cudaStream_t st) {
+template <typename T, int E, typename F>
+static bk_status blue_fft_F(const Plan* p, const T* src, T* dst, typename V2<T>::t* A, int nvec, cudaStream_t st) {
   typedef typename V2<T>::t C;
   const FourStep& f = p->fsM;
   const int M = (int)p->M;
-  BK_TRY(launch(k_passA<T>, dim3(f.N2 / f.NB, nvec), f.thrA, f.smemA, st, src, 2 * (int64_t)M, A, M, f.N1, ilog2(f.N1), f.N2, f.NB,
-                                                               f.bsA, (const C*)f.stw1, (const C*)f.twN,
-                                                               (const C*)f.twLo, (const C*)f.twHi, f.tw_h));
-  BK_TRY(launch(k_passB<T, E>, dim3(f.N1 / 2 / f.P, nvec), f.thrB, f.smemB, st, A, dst, 2 * (int64_t)M, M, f.N1, f.N2, ilog2(f.N2),
-                                                                     f.P, (const C*)f.stw2, (const C*)p->bh));
+  BK_TRY(launch(k_passA<T, F>, dim3(f.N2 / f.NB, nvec), f.thrA, f.smemA, st, src, 2 * (int64_t)M, A, M, f.N1, ilog2(f.N1),
+                f.N2, f.NB, f.bsA, (const C*)f.stw1, (const C*)f.twN, (const C*)f.twLo, (const C*)f.twHi, f.tw_h));
+  BK_TRY(launch(k_passB<T, E, F>, dim3(f.N1 / 2 / f.P, nvec), f.thrB, f.smemB, st, A, dst, 2 * (int64_t)M, M, f.N1, f.N2,
+                ilog2(f.N2), f.P, (const C*)f.stw2, (const C*)p->bh));
   return BK_OK;
+}
+template <typename T, int E>
+static bk_status blue_fft(const Plan* p, const T* src, T* dst, typename V2<T>::t* A, int nvec, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    if (p->fe == 2) return blue_fft_F<T, E, FftShape<T, 2>>(p, src, dst, A, nvec, st);
+  }
+  return blue_fft_F<T, E, FftShape<T, 4>>(p, src, dst, A, nvec, st);
 }
 
 // One DCT-I of length N + 1 for N not a power of two: chirp, FFT_M, spectral product, FFT_M,
@@ -1987,8 +2006,8 @@ static size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 static size_t noalloc_layout(const Plan& p, int nvec, size_t off[7]) {
   const int64_t N = p.N;
   size_t o = 0;
-  off[0] = o; o += align256(sizeof(double2) * stage_tw_len(ilog2(p.fs.N1), CplxFft<double>::E));  // stw1
-  off[1] = o; o += align256(sizeof(double2) * stage_tw_len(ilog2(p.fs.N2), CplxFft<double>::E));  // stw2
+  off[0] = o; o += align256(sizeof(double2) * stage_tw_len(ilog2(p.fs.N1), 2));  // stw1
+  off[1] = o; o += align256(sizeof(double2) * stage_tw_len(ilog2(p.fs.N2), 2));  // stw2
   off[2] = o; o += align256(sizeof(double2) * p.fs.a_len());                          // twN
   off[3] = o; o += align256(sizeof(double2) * p.fs.a_len() * nvec);                   // scrA
   off[4] = o; o += align256(sizeof(double) * (size_t)(N + 2) * nvec);                 // scrY
@@ -2057,7 +2076,7 @@ bk_status noalloc_apply(const double* v, double* out, int64_t N, int nvec, int64
   // every table is rewritten by each call: nothing in the array has to start at zero
   k_rk_table<double><<<(int)std::min<int64_t>((N + 2 + 255) / 256, 4096), 256, 0, st>>>((double*)p.rk, N + 2);
   BK_CHECK_LAUNCH();
-  constexpr int e = CplxFft<double>::E;
+  constexpr int e = 2;
   const int len1 = stage_tw_len(ilog2(p.fs.N1), e), len2 = stage_tw_len(ilog2(p.fs.N2), e);
   k_stage_tw<double><<<(len1 + 255) / 256, 256, 0, st>>>((double2*)p.fs.stw1, ilog2(p.fs.N1), e, len1);
   BK_CHECK_LAUNCH();

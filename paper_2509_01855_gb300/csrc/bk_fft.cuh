@@ -45,11 +45,14 @@ template <typename T, int E_> struct FftShape {
   static constexpr int E = E_, EPT = 1 << E_, MT = E_ == 4 ? 512 : (E_ == 3 ? 512 : 1024), MINB = MT == 512 ? 2 : 1;
   static constexpr bool MIX = false;
 };
+template <> struct FftShape<double, 4> {
+  static constexpr int E = 4, EPT = 16, MT = 256, MINB = 2;
+  static constexpr bool MIX = false;
+};
 // Launch-per-pass kernels of lengths 2^a 3^b 5^c (fft_mix).
 struct MixFft { static constexpr int E = 2, MT = 256, MINB = 2; static constexpr bool MIX = true; };
-// Radix of the launch-per-pass kernels (re_radix) and of the plain complex passes, and of the
-// one-CTA and one-launch kernels, whose few CTAs are bound by latency.
-template <typename T> struct CplxFft : FftShape<T, sizeof(T) == 4 ? 4 : 2> {};
+// Radix of the one-CTA and one-launch kernels, whose few CTAs are bound by latency (re_radix and
+// cplx_radix choose that of the launch-per-pass kernels).
 template <typename T> struct SmallFft : FftShape<T, 2> {};
 template <typename T> struct BigFft { static constexpr int E = std::is_same<T, dfl>::value ? 3 : 2, EPT = 16, MT = 512, MINB = 1; static constexpr bool MIX = false; };
 
