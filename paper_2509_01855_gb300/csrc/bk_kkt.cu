@@ -735,22 +735,68 @@ static bk_status run_sweep(Problem* pr, OpData& d, SweepArgs<T>& a, int ncol, cu
 // ---------------------------------------------------------------------------------------------
 // KKT / state operator kernels (per node, Jacobians and Hessian recomputed from (x, u, mu))
 // ---------------------------------------------------------------------------------------------
-// t = J dz per node; with a free final time (ds != null) t += (ds / s) f, so that the product
-// s B^a t adds the column d c / ds = -B^a f times ds.
+// Entries of J_x and H at the linearisation (Dyn::pack), for kinds that store them: the operator
+// kernels read them instead of forming them from (x, u, mu) at every apply, which had bound the FP64
+// ones by the FP64 pipe (one division and some 50 products per node; orbit, N = 2^18, us: k_jvp 21 ->
+// 12, k_kkt_post 47 -> 34; the whole KKT product at 2^20 734 -> 649).
 template <typename T, int KIND>
-__global__ void k_jvp(const T* __restrict__ xu, const T* __restrict__ dX, const T* __restrict__ dU, int64_t P,
-                      int64_t L, T* __restrict__ t, T pa, const T* __restrict__ ds, T inv_s) {
+__global__ void k_lin_entries(const T* __restrict__ xu, const T* __restrict__ mu, int64_t P, int64_t L, T pa,
+                              T* __restrict__ lin) {
   pdl_wait();
-  constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
-  const T dss = ds ? ds[0] * inv_s : T(0);
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
-    T x[NXM], u[NUM], Jx[NXM * NXM], Ju[NXM * NUM], fx[NXM];
+  constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NL = Dyn<KIND>::nlj + Dyn<KIND>::nlh;
+  if constexpr (NL > 0) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
+      T x[NXM], u[NUM], m_[NXM], v[NL];
+#pragma unroll
+      for (int m = 0; m < NX; ++m) { x[m] = xu[m * P + k]; m_[m] = mu[m * P + k]; }
+#pragma unroll
+      for (int q = 0; q < NU; ++q) u[q] = xu[(NX + q) * P + k];
+      Dyn<KIND>::template pack<T>(x, u, m_, pa, v);
+#pragma unroll
+      for (int i = 0; i < NL; ++i) lin[i * P + k] = v[i];
+    }
+  }
+}
+
+// J_x and J_u of node k: stored entries, or formed from (x, u).
+template <typename T, int KIND>
+__device__ __forceinline__ void node_jac(const T* __restrict__ xu, const T* __restrict__ lin, int64_t P, int64_t k, T pa,
+                                         T* Jx, T* Ju) {
+  constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NJ = Dyn<KIND>::nlj;
+  if constexpr (NJ > 0) {
+    T v[NJ];
+#pragma unroll
+    for (int i = 0; i < NJ; ++i) v[i] = lin[i * P + k];
+    Dyn<KIND>::template unpack_j<T>(v, Jx, Ju);
+  } else {
+    T x[NXM], u[NUM];
 #pragma unroll
     for (int m = 0; m < NX; ++m) x[m] = xu[m * P + k];
 #pragma unroll
     for (int q = 0; q < NU; ++q) u[q] = xu[(NX + q) * P + k];
     Dyn<KIND>::template jac<T>(x, u, Jx, Ju, pa);
-    if (ds) Dyn<KIND>::template f<T>(x, u, fx, pa);
+  }
+}
+
+// t = J dz per node; with a free final time (ds != null) t += (ds / s) f, so that the product
+// s B^a t adds the column d c / ds = -B^a f times ds.
+template <typename T, int KIND>
+__global__ void k_jvp(const T* __restrict__ xu, const T* __restrict__ dX, const T* __restrict__ dU, int64_t P,
+                      int64_t L, T* __restrict__ t, T pa, const T* __restrict__ ds, T inv_s, const T* __restrict__ lin) {
+  pdl_wait();
+  constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
+  const T dss = ds ? ds[0] * inv_s : T(0);
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
+    T Jx[NXM * NXM], Ju[NXM * NUM], fx[NXM];
+    node_jac<T, KIND>(xu, lin, P, k, pa, Jx, Ju);
+    if (ds) {
+      T x[NXM], u[NUM];
+#pragma unroll
+      for (int m = 0; m < NX; ++m) x[m] = xu[m * P + k];
+#pragma unroll
+      for (int q = 0; q < NU; ++q) u[q] = xu[(NX + q) * P + k];
+      Dyn<KIND>::template f<T>(x, u, fx, pa);
+    }
 #pragma unroll
     for (int m = 0; m < NX; ++m) {
       T a = ds ? dss * fx[m] : T(0);
@@ -786,13 +832,15 @@ __global__ void k_state_post(const T* __restrict__ chi, const T* __restrict__ Bt
 // block writes its partial of mu . (J dz) + f . Mu; the s row is -(1/s) times their sum
 // (k_free_finish), i.e. -(B^aT lambda) . (J dz) - (B^a f) . dlambda.
 template <typename T, int KIND>
-__global__ void k_kkt_post(const T* __restrict__ xu, const T* __restrict__ mu, const T* __restrict__ w, T s,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_kkt_post(const T* __restrict__ xu, const T* __restrict__ mu, const T* __restrict__ w, T s,
                            const T* __restrict__ in, const T* __restrict__ Bt, T* __restrict__ Mu, int64_t P,
                            int64_t L, TermSpec ts, T cost_uu, T* __restrict__ out, T pa, int64_t s_idx,
                            double* __restrict__ part, const double* __restrict__ sdev,
-                           const T* __restrict__ hbar) {
+                           const T* __restrict__ hbar, const T* __restrict__ lin) {
   pdl_wait();
-  constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NV = NX + NU;
+  constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NV = NX + NU, NJ = Dyn<KIND>::nlj, NH = Dyn<KIND>::nlh;
+  // with stored entries the node's (x, u, mu) are read for the free final time's terms only
+  const bool point = NJ == 0 || part != nullptr;
   __shared__ double red[32];
   // sdev: Bt and Mu arrive unscaled (B^a, B^aT products) and take the device time scale here;
   // the scaled Mu is written back (the caller's record of s B^aT dlambda)
@@ -816,8 +864,8 @@ __global__ void k_kkt_post(const T* __restrict__ xu, const T* __restrict__ mu, c
     T x[NXM], u[NUM], m_[NXM], Jx[NXM * NXM], Ju[NXM * NUM], H[(NXM + NUM) * (NXM + NUM)], dz[NXM + NUM], mp[NXM];
 #pragma unroll
     for (int m = 0; m < NX; ++m) {
-      x[m] = xu[m * P + k];
-      m_[m] = mu[m * P + k];
+      x[m] = point ? xu[m * P + k] : T(0);
+      m_[m] = point ? mu[m * P + k] : T(0);
       dz[m] = dX[m * P + k];
       mp[m] = Mu[m * P + k];
       if (sdev) {
@@ -826,9 +874,21 @@ __global__ void k_kkt_post(const T* __restrict__ xu, const T* __restrict__ mu, c
       }
     }
 #pragma unroll
-    for (int q = 0; q < NU; ++q) { u[q] = xu[(NX + q) * P + k]; dz[NX + q] = dU[q * P + k]; }
-    Dyn<KIND>::template jac<T>(x, u, Jx, Ju, pa);
-    Dyn<KIND>::template hess<T>(x, u, m_, H, pa);
+    for (int q = 0; q < NU; ++q) { u[q] = point ? xu[(NX + q) * P + k] : T(0); dz[NX + q] = dU[q * P + k]; }
+    if constexpr (NJ > 0) {
+      T v[NH];
+      node_jac<T, KIND>(xu, lin, P, k, pa, Jx, Ju);
+#pragma unroll
+      for (int i = 0; i < NH; ++i) v[i] = lin[(NJ + i) * P + k];
+      Dyn<KIND>::template unpack_h<T>(v, H);
+    } else {
+      Dyn<KIND>::template jac<T>(x, u, Jx, Ju, pa);
+      Dyn<KIND>::template hess<T>(x, u, m_, H, pa);
+    }
+    // ds / s of the free final time joins s B^aT dlambda
+    T md[NXM];
+#pragma unroll
+    for (int m = 0; m < NX; ++m) md[m] = part ? mp[m] + dss * m_[m] : mp[m];
     const T swk = s * w[k] * cost_uu;
     T hb[NUM];   // control bounds: the barrier's diagonal of the control block
 #pragma unroll
@@ -859,11 +919,11 @@ __global__ void k_kkt_post(const T* __restrict__ xu, const T* __restrict__ mu, c
         acc += dL[a * P + k];
 #pragma unroll
         for (int m = 0; m < NX; ++m)
-          if (Dyn<KIND>::jx_nz(m, a)) acc -= Jx[m * NX + a] * (mp[m] + dss * m_[m]);
+          if (Dyn<KIND>::jx_nz(m, a)) acc -= Jx[m * NX + a] * md[m];
       } else {
 #pragma unroll
         for (int m = 0; m < NX; ++m)
-          if (Dyn<KIND>::ju_nz(m, a - NX)) acc -= Ju[m * NU + (a - NX)] * (mp[m] + dss * m_[m]);
+          if (Dyn<KIND>::ju_nz(m, a - NX)) acc -= Ju[m * NU + (a - NX)] * md[m];
       }
       if (a < NX && k == L - 1) {
         // compile-time indices into the parameter struct (a run-time index would copy it to
@@ -1339,6 +1399,8 @@ static bk_status alloc_opdata(Problem* pr, OpData& d, int dtype) {
   pr->bytes += d.plan->bytes;  // the plan counted its own allocations
   BK_TRY(dmalloc(&d.xu, es * (nx + nu) * P));
   BK_TRY(dmalloc(&d.mu, es * nx * P));
+  const int nl = pr->kind == BK_ORBIT ? Dyn<BK_ORBIT>::nlj + Dyn<BK_ORBIT>::nlh : 0;
+  if (nl > 0) BK_TRY(dmalloc(&d.lin, es * nl * P));
   d.w = dtype == BK_F64 ? (void*)d.plan->w64 : d.plan->wT;
   // preconditioner data only in the working precision (an FP32 problem's FP64 side serves the
   // residual and the refinement products)
@@ -1382,7 +1444,7 @@ static bk_status alloc_opdata(Problem* pr, OpData& d, int dtype) {
 
 static void free_opdata(OpData& d) {
   if (d.plan) plan_destroy(d.plan);
-  void* ps[] = {d.xu, d.mu, d.Dn, d.Zc, d.HWc, d.Qc, d.Sinv, d.t1, d.t2, d.t3, d.brd, d.brq, d.bgam, d.hbar, d.lvcnt, d.qlast};
+  void* ps[] = {d.xu, d.mu, d.lin, d.Dn, d.Zc, d.HWc, d.Qc, d.Sinv, d.t1, d.t2, d.t3, d.brd, d.brq, d.bgam, d.hbar, d.lvcnt, d.qlast};
   for (void* p : ps) dfree(p);
   for (int l = 0; l < MAXLEV; ++l) {
     dfree(d.lvm[l]);
@@ -1571,6 +1633,12 @@ static bk_status lin_end_rows(Problem* pr, const double* z, cudaStream_t st) {
   return BK_OK;
 }
 
+template <typename T, int KIND>
+static bk_status lin_entries(Problem* pr, OpData& d, cudaStream_t st) {
+  return launch(k_lin_entries<T, KIND>, nblk(pr->L), 256, 0, st, (const T*)d.xu, (const T*)d.mu, pr->P, pr->L,
+                (T)pr->dyn_param(), (T*)d.lin);
+}
+
 // mu (nullable): s B^aT lambda at this z, known to the caller (e.g. from the residual that
 // accepted the step); it is copied instead of recomputed.
 // A BK_F32 problem builds its preconditioner data in FP32 only; the FP64 side keeps the
@@ -1607,6 +1675,13 @@ static bk_status linearize_kind(Problem* pr, const double* z, const double* mu, 
       BK_TRY(launch(k_lin_bar<float, NU>, nblk(P), 256, 0, st, z, pr->d64.plan->w64, pr->s, P, pr->L, NX, b, (float*)pr->d32.hbar));
     }
   }
+  if constexpr (Dyn<KIND>::nlj > 0) {
+    pr->lin64_stale = pr->dtype == BK_F32;
+    if (pr->dtype == BK_F32)
+      BK_TRY((lin_entries<float, KIND>(pr, pr->d32, st)));
+    else
+      BK_TRY((lin_entries<double, KIND>(pr, pr->d64, st)));
+  }
   pr->linearized = true;
   if (keep != LIN_FULL) return BK_OK;
   if (pr->n_e > 0 && pr->has_cost) {
@@ -1634,9 +1709,16 @@ static bk_status apply_typed(Problem* pr, OpData& d, int op, const T* in, T* out
   T* t1 = (T*)d.t1;
   T* t2 = (T*)d.t2;
   T* t3 = (T*)d.t3;
+  if constexpr (Dyn<KIND>::nlj > 0 && sizeof(T) == 8) {
+    if (pr->lin64_stale) {
+      BK_TRY((lin_entries<T, KIND>(pr, d, st)));
+      pr->lin64_stale = false;
+    }
+  }
   if (op == BK_OP_STATE) {
     // the product ignores t1's padding (elements L..P-1), so it is never written
-    BK_TRY(launch(k_jvp<T, KIND>, nblk(L), 256, 0, st, (const T*)d.xu, in, nullptr, P, L, t1, (T)pr->dyn_param(), nullptr, T(0)));
+    BK_TRY(launch(k_jvp<T, KIND>, nblk(L), 256, 0, st, (const T*)d.xu, in, nullptr, P, L, t1, (T)pr->dyn_param(), nullptr, T(0),
+                  (const T*)d.lin));
     const double* sd = sdev_of(pr);
     BK_TRY(plan_apply_n(d.plan, t1, t2, NX, false, sd ? 1.0 : pr->s, st));
     BK_TRY(launch(k_state_post<T, NX>, nblk(NX * P), 256, 0, st, in, t2, P, L, out, sd));
@@ -1645,7 +1727,7 @@ static bk_status apply_typed(Problem* pr, OpData& d, int op, const T* in, T* out
   const bool ft = pr->free_time;
   const T pa = (T)pr->dyn_param();
   BK_TRY(launch(k_jvp<T, KIND>, nblk(L), 256, 0, st, (const T*)d.xu, in, in + NX * P, P, L, t1, pa,
-                                          ft ? in + pr->s_idx() : nullptr, (T)(1.0 / pr->s)));
+                                          ft ? in + pr->s_idx() : nullptr, (T)(1.0 / pr->s), (const T*)d.lin));
   // fixed final time: both products unscaled, k_kkt_post applies s from the device (so that a
   // captured GMRES step does not hold s); free final time: s (which changes within a step) by value
   const double* sd = sdev_of(pr);
@@ -1654,7 +1736,7 @@ static bk_status apply_typed(Problem* pr, OpData& d, int op, const T* in, T* out
   BK_TRY(plan_apply_n(d.plan, in + (NX + NU) * P, Mu, NX, true, sd ? 1.0 : pr->s, st));
   BK_TRY(launch(k_kkt_post<T, KIND>, ft ? FT_NB : nblk(P), 256, 0, st, (const T*)d.xu, (const T*)d.mu, (const T*)d.w, (T)pr->s, in,
                                                             t2, Mu, P, L, term_spec(pr), (T)pr->cost_uu(), out, pa,
-                                                            pr->s_idx(), ft ? pr->sred : nullptr, sd, bar_hbar<T>(pr, d)));
+                                                            pr->s_idx(), ft ? pr->sred : nullptr, sd, bar_hbar<T>(pr, d), (const T*)d.lin));
   if (ft) {
     BK_TRY(launch(k_free_finish<T>, 1, 256, 0, st, pr->sred, FT_NB, -1.0 / pr->s, out + pr->s_idx()));
   }

@@ -37,11 +37,16 @@ enum { SL_A = 0, SL_M1 = 1, SL_PRE = 5, SL_SUF = 6, NSLOT = 7 };
 // ---------------------------------------------------------------------------------------------
 template <int KIND> struct Dyn;
 
+// nlj + nlh: values per node that the linearisation stores for the KKT product (pack; unpack_j and
+// unpack_h set the entries that jx_nz, ju_nz and h_nz name), 0 for kinds whose Jacobian and Hessian
+// cost less to form than to read.
+//
 // Structural nonzeros of J_x (n_x x n_x), J_u (n_x x n_u) and the Lagrangian Hessian
 // H ((n_x + n_u)^2) of a kind: the node-local kernels skip the products with structural zeros
 // (the indices are compile-time constants after unrolling, so the skipped terms and their loads
 // vanish). Kinds without a pattern take the dense one.
 struct DenseNZ {
+  static constexpr int nlj = 0, nlh = 0;
   __host__ __device__ static constexpr bool jx_nz(int, int) { return true; }
   __host__ __device__ static constexpr bool ju_nz(int, int) { return true; }
   __host__ __device__ static constexpr bool h_nz(int, int) { return true; }
@@ -53,6 +58,7 @@ __device__ inline void sincos_t(float x, float* s, float* c) { sincosf(x, s, c);
 // Minimum-energy double integrator: x = (p, v), x' = (v, u), F = u^2 / 2.
 template <> struct Dyn<BK_DBL_INT> {
   static constexpr int nx = 2, nu = 1;
+  static constexpr int nlj = 0, nlh = 0;
   // J_x = [[0, 1], [0, 0]], J_u = [0; 1], H = 0 (f is linear)
   __host__ __device__ static constexpr bool jx_nz(int r, int c) { return r == 0 && c == 1; }
   __host__ __device__ static constexpr bool ju_nz(int r, int q) { return r == 1 && q == 0; }
@@ -91,6 +97,22 @@ template <> struct Dyn<BK_ORBIT> {
   // control block of the KKT preconditioner at a node: s w_k times the running cost's curvature
   static constexpr bool huu_needs_mu = false;
   template <typename T> __device__ static T pre_huu(const T* mu, T swk, T) { return swk; }
+  // entries the KKT product reads from the linearisation: J_x (7, without the constant ones), H (5)
+  static constexpr int nlj = 7, nlh = 5;
+  template <typename T> __device__ static void pack(const T* x, const T* u, const T* mu, T pa, T* v) {
+    T Jx[16], Ju[8], H[36];
+    jac<T>(x, u, Jx, Ju, pa);
+    hess<T>(x, u, mu, H, pa);
+    v[0] = Jx[4]; v[1] = Jx[7]; v[2] = Jx[8]; v[3] = Jx[11]; v[4] = Jx[12]; v[5] = Jx[14]; v[6] = Jx[15];
+    v[7] = H[0]; v[8] = H[3]; v[9] = H[2]; v[10] = H[21]; v[11] = H[15];
+  }
+  template <typename T> __device__ static void unpack_j(const T* v, T* Jx, T* Ju) {
+    Jx[2] = 1; Jx[4] = v[0]; Jx[7] = v[1]; Jx[8] = v[2]; Jx[11] = v[3]; Jx[12] = v[4]; Jx[14] = v[5]; Jx[15] = v[6];
+    Ju[4] = 1; Ju[7] = 1;
+  }
+  template <typename T> __device__ static void unpack_h(const T* v, T* H) {
+    H[0] = v[0]; H[3] = H[18] = v[1]; H[2] = H[12] = v[2]; H[21] = v[3]; H[15] = H[20] = v[4];
+  }
   template <typename T> __device__ static void f(const T* x, const T* u, T* fx, T) {
     const T r = x[0], vr = x[2], vt = x[3];
     const T ir = T(1) / r;
@@ -154,6 +176,7 @@ template <> struct Dyn<BK_BILINEAR> : DenseNZ {
 // Minimum-time orbit transfer of Eq. ot: the same state, fixed-magnitude thrust a (sin u, cos u)
 // steered by the angle u (pa = a), cost T = t_f - t_0 with the final time free.
 template <> struct Dyn<BK_ORBIT_MT> : DenseNZ {
+  static constexpr int nlj = 0, nlh = 0;
   // the state Jacobian of BK_ORBIT (theta enters no right-hand side); J_u and H dense
   __host__ __device__ static constexpr bool jx_nz(int r, int c) { return Dyn<BK_ORBIT>::jx_nz(r, c); }
   static constexpr int nx = 4, nu = 1;
@@ -286,6 +309,7 @@ struct OpData {
   Plan* plan = nullptr;        // n_comp = n_x, max_batch = 1
   void* xu = nullptr;          // linearisation point X, U ((n_x + n_u) * P)
   void* mu = nullptr;          // mu = s (B^a)^T lambda (n_x * P)
+  void* lin = nullptr;         // stored entries of J_x and H per node ((nlj + nlh) * P)
   void* w = nullptr;           // Clenshaw-Curtis weights (L), working type
   void* Dn = nullptr;          // per-node D_k = h_k J_k K_k, K_k = (I - h_k J_k)^{-1} = I + D_k and
                                // N_k = 2 h_k J_k K_k = 2 D_k; interleaved (n_x^2 per node)
@@ -331,6 +355,7 @@ struct Problem {
   int nlev = 0;                // scan levels; level nlev - 1 has at most 32 items
   int lvn[MAXLEV] = {};        // items per level
   bool linearized = false;
+  bool lin64_stale = false;    // BK_F32 problems: d64.lin is formed when an FP64 product first needs it
   OpData d64;                  // FP64 operators (always)
   OpData d32;                  // FP32 operators (BK_F32 problems)
   double* F = nullptr;         // KKT residual scratch (FP64, kkt_len)
