@@ -1311,7 +1311,7 @@ static bk_status fourstep_shapes(Plan* p, int E) {
 // Tile autotuner of the four-step transforms. The elements per CTA E (powers of two from one
 // column and one row pair up to the thread cap) set the CTA count, shared memory per CTA and how
 // many CTAs share an SM; the best E depends on N, the vector count and the GPU. For each
-// candidate the plan is re-shaped and timed (CUDA events, one B and one B^T after a warm-up
+// candidate the plan is re-shaped and timed (CUDA events, one B and one B^T, three times after a warm-up
 // pair, on zero vectors: the kernels have no data-dependent paths); the fastest stays. Results
 // are cached per (N, dtype, vectors, SM count, device) for the process, so plans of one size
 // share one shape (and bitwise the same results). BK_AUTOTUNE=0 keeps the heuristic shape;
@@ -1357,18 +1357,20 @@ static bk_status autotune_tiles(Plan* p, cudaStream_t st) {
     if (fourstep_shapes(p, E) != BK_OK) continue;  // shape outside the thread/shared-memory caps
     r = plan_apply_n(p, vin, vout, nvec, false, p->s, st);
     if (r == BK_OK) r = plan_apply_n(p, vin, vout, nvec, true, p->s, st);
-    if (r == BK_OK && cudaEventRecord(e0, st) != cudaSuccess) r = BK_ERR_CUDA;
-    if (r == BK_OK) r = plan_apply_n(p, vin, vout, nvec, false, p->s, st);
-    if (r == BK_OK) r = plan_apply_n(p, vin, vout, nvec, true, p->s, st);
-    float ms = 0.f;
-    if (r == BK_OK && (cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-                       cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)) {
-      set_error("autotune: timing failed");
-      r = BK_ERR_CUDA;
-    }
-    if (r == BK_OK && (best == 0 || ms < best_ms)) {
-      best = E;
-      best_ms = ms;
+    for (int rep = 0; rep < 3; ++rep) {   // the least of three: one timing chose between near tiles at random
+      if (r == BK_OK && cudaEventRecord(e0, st) != cudaSuccess) r = BK_ERR_CUDA;
+      if (r == BK_OK) r = plan_apply_n(p, vin, vout, nvec, false, p->s, st);
+      if (r == BK_OK) r = plan_apply_n(p, vin, vout, nvec, true, p->s, st);
+      float ms = 0.f;
+      if (r == BK_OK && (cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+                         cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)) {
+        set_error("autotune: timing failed");
+        r = BK_ERR_CUDA;
+      }
+      if (r == BK_OK && (best == 0 || ms < best_ms)) {
+        best = E;
+        best_ms = ms;
+      }
     }
   }
   if (e0) cudaEventDestroy(e0);

@@ -1587,10 +1587,10 @@ static bk_status lin_schur_finish(Problem* pr, OpData& d, cudaStream_t st) {
       for (int q = 0; q < ne; ++q) { A[r * ne + q] -= f * A[c * ne + q]; Inv[r * ne + q] -= f * Inv[c * ne + q]; }
     }
   }
-  std::vector<T> hs(NEM * NEM, T(0));
+  // from pinned memory that is not written again before the next linearisation has synchronised
+  T* hs = reinterpret_cast<T*>(pr->red_host + 400);
   for (int i = 0; i < ne * ne; ++i) hs[i] = (T)Inv[i];
-  BK_TRY_CUDA(cudaMemcpyAsync(d.Sinv, hs.data(), sizeof(T) * ne * ne, cudaMemcpyHostToDevice, st));
-  BK_TRY_CUDA(cudaStreamSynchronize(st));
+  BK_TRY_CUDA(cudaMemcpyAsync(d.Sinv, hs, sizeof(T) * ne * ne, cudaMemcpyHostToDevice, st));
   return BK_OK;
 }
 

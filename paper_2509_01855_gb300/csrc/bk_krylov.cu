@@ -38,7 +38,15 @@
 
 namespace bk {
 
-static constexpr int DOT_BLOCKS = 608;   // 4 blocks per SM on 152 SMs, fixed for determinism
+// Blocks of the reductions over n elements: 4 per SM on 152 SMs, fewer for short vectors (8 elements
+// per thread), whose last block otherwise spent most of the kernel adding up the partials of nearly
+// empty blocks (n = 41000 in FP32, cold caches: 54 us with 608 blocks, 22 us with 21). A function of n alone, so
+// the order of the sums is fixed.
+static constexpr int DOT_BLOCKS = 608;
+static inline int dot_blocks(int64_t n) {
+  const int64_t b = (n + 2047) / 2048;
+  return (int)(b < 1 ? 1 : (b < DOT_BLOCKS ? b : DOT_BLOCKS));
+}
 static constexpr int MAXM = 100;
 
 // FP32 elements per thread summed in FP32 before each FP64 accumulation.
@@ -234,14 +242,41 @@ __global__ void __launch_bounds__(256) k_multidot(const T* __restrict__ V, int64
   multidot_body<T>(V, ld, nv, w, n, partial, out, cnt);
 }
 
+// --- device-resident Arnoldi state -----------------------------------------------------------
+// One per GMRES workspace. j counts the columns of the current cycle; the host sets the cycle up
+// (k_gm_init) and reads the first fields back at its end.
+struct GmState {
+  int j;          // columns finished in this cycle
+  int jmax;       // columns allowed in this cycle (restart length, iteration cap)
+  int m;          // restart length (row stride of H)
+  int need2;      // DGKS: second Gram-Schmidt pass wanted for the current column
+  int stop;       // the cycle is over (converged, breakdown, or jmax reached)
+  int pad;
+  double target;  // absolute residual target
+  double resid;   // |g_{j}|, the Arnoldi residual estimate after the last column
+  double hn;      // |w| after orthogonalisation, the new basis vector's scale
+  double gv[MAXM + 1], cs[MAXM], sn[MAXM], y[MAXM];
+  double H[(MAXM + 1) * MAXM];
+};
+
+// After the first Gram-Schmidt pass (one block): column j of H from h = V^T w, and the DGKS test
+// (|w|^2 after the pass below half of |w|^2 before it).
+__device__ __forceinline__ void gm_first_pass(GmState* s, const double* __restrict__ h1, const double* w2) {
+  const int j = s->j, m = s->m;
+  for (int i = threadIdx.x; i <= j; i += blockDim.x) s->H[i * m + j] = h1[i];
+  if (threadIdx.x == 0) s->need2 = w2[0] < 0.5 * h1[j + 1] ? 1 : 0;
+}
+
 // w <- alpha * w + cscale * sum_i c[i] V_i   (c on the device, FP64). With `partial`, each block
 // also writes the sum of squares of its slice of the new w and the last block to finish writes
-// their sum, |w|^2, to *sq_out (block order, as k_multidot).
+// their sum, |w|^2, to *sq_out (block order, as k_multidot) and, with `fin`, finishes the first
+// Gram-Schmidt pass (c is then h).
 template <typename T>
 __device__ __forceinline__ void multiaxpy_body(const T* __restrict__ V, int64_t ld, int nv,
                                                const double* __restrict__ c, double cscale, T* __restrict__ w,
                                                double alpha, int64_t n, double* __restrict__ partial,
-                                               double* __restrict__ sq_out, unsigned* __restrict__ cnt) {
+                                               double* __restrict__ sq_out, unsigned* __restrict__ cnt,
+                                               GmState* fin = nullptr) {
   __shared__ double cs[MAXM + 1];
   __shared__ float cs32[MAXM + 1];
   __shared__ double red[8];
@@ -362,7 +397,10 @@ __device__ __forceinline__ void multiaxpy_body(const T* __restrict__ V, int64_t 
       for (int wp = 0; wp < (int)(blockDim.x >> 5); ++wp) t += red[wp];
       partial[blockIdx.x] = t;
     }
-    if (last_block(cnt)) block_sum_column(partial, gridDim.x, 1, 0, sq_out);
+    if (last_block(cnt)) {
+      block_sum_column(partial, gridDim.x, 1, 0, sq_out);
+      if (fin) gm_first_pass(fin, c, sq_out);
+    }
   }
 }
 
@@ -375,23 +413,6 @@ __global__ void __launch_bounds__(256) k_multiaxpy(const T* __restrict__ V, int6
   pdl_wait();
   multiaxpy_body<T>(V, ld, nv, c, cscale, w, alpha, n, partial, sq_out, cnt);
 }
-
-// --- device-resident Arnoldi state -----------------------------------------------------------
-// One per GMRES workspace. j counts the columns of the current cycle; the host sets the cycle up
-// (k_gm_init) and reads the first fields back at its end.
-struct GmState {
-  int j;          // columns finished in this cycle
-  int jmax;       // columns allowed in this cycle (restart length, iteration cap)
-  int m;          // restart length (row stride of H)
-  int need2;      // DGKS: second Gram-Schmidt pass wanted for the current column
-  int stop;       // the cycle is over (converged, breakdown, or jmax reached)
-  int pad;
-  double target;  // absolute residual target
-  double resid;   // |g_{j}|, the Arnoldi residual estimate after the last column
-  double hn;      // |w| after orthogonalisation, the new basis vector's scale
-  double gv[MAXM + 1], cs[MAXM], sn[MAXM], y[MAXM];
-  double H[(MAXM + 1) * MAXM];
-};
 
 __global__ void k_gm_init(GmState* s, double beta, double target, int jmax, int m) {
   pdl_wait();
@@ -429,34 +450,22 @@ __global__ void __launch_bounds__(256) k_multiaxpy_s(const T* __restrict__ V, in
                                                      const int* __restrict__ gate, const double* __restrict__ c,
                                                      double cscale, double alpha, int64_t n,
                                                      double* __restrict__ partial, double* __restrict__ sq_out,
-                                                     unsigned* __restrict__ cnt) {
+                                                     unsigned* __restrict__ cnt, GmState* fin) {
   pdl_wait();
   if (gate && *gate == 0) return;
   const int j = s->j;
   T* w = woff >= 0 ? const_cast<T*>(V) + (int64_t)(j + woff) * ld : x;
-  multiaxpy_body<T>(V, ld, j + add, c, cscale, w, alpha, n, partial, sq_out, cnt);
+  multiaxpy_body<T>(V, ld, j + add, c, cscale, w, alpha, n, partial, sq_out, cnt, fin);
 }
 
-// After the first Gram-Schmidt pass: column j of H from h = V^T w, and the DGKS test (|w|^2
-// after the pass below half of |w|^2 before it).
-__global__ void k_gm_a(GmState* s, const double* __restrict__ h1, const double* __restrict__ w2) {
-  pdl_wait();
-  const int j = s->j, m = s->m;
-  for (int i = threadIdx.x; i <= j; i += blockDim.x) s->H[i * m + j] = h1[i];
-  if (threadIdx.x == 0) s->need2 = w2[0] < 0.5 * h1[j + 1] ? 1 : 0;
-}
-
-// Column j finished: the second pass's corrections, |w|, the Givens rotations of the column,
-// the residual estimate and the stop test; j advances. In a graph, the WHILE condition follows.
-__global__ void k_gm_b(GmState* s, const double* __restrict__ h2, const double* __restrict__ w2,
-                       cudaGraphConditionalHandle cond, int in_graph) {
-  pdl_wait();
-  if (threadIdx.x != 0) return;
+// Column j finished (one thread): the second pass's corrections, |w|, the Givens rotations of the
+// column, the residual estimate and the stop test; j advances. In a graph, the WHILE condition follows.
+__device__ void gm_column(GmState* s, const double* __restrict__ h2, double hnext, cudaGraphConditionalHandle cond,
+                          int in_graph) {
   const int j = s->j, m = s->m;
   double* H = s->H;
   if (s->need2)
     for (int i = 0; i <= j; ++i) H[i * m + j] += h2[i];
-  const double hnext = sqrt(w2[0]);
   s->hn = hnext;
   H[(j + 1) * m + j] = hnext;
   for (int i = 0; i < j; ++i) {
@@ -483,16 +492,28 @@ __global__ void k_gm_b(GmState* s, const double* __restrict__ h2, const double* 
   if (in_graph) cudaGraphSetConditional(cond, stop ? 0u : 1u);
 }
 
-// V_j <- V_j / hn (j after k_gm_b, i.e. the new basis vector), unless hn == 0.
+// End of an Arnoldi step: V_{j+1} <- w / |w| (unless |w| = 0), and the last block to finish, after
+// every block has read j, closes the column. One square root and division per block: in every
+// thread they took the FP64 pipe longer than the vector takes to move.
 template <typename T>
-__global__ void k_scale_inv_s(T* __restrict__ V, int64_t ld, const GmState* __restrict__ s, int64_t n) {
+__global__ void __launch_bounds__(256) k_gm_finish(T* __restrict__ V, int64_t ld, int64_t n, GmState* s,
+                                                   const double* __restrict__ h2, const double* __restrict__ w2,
+                                                   unsigned* __restrict__ cnt, cudaGraphConditionalHandle cond,
+                                                   int in_graph) {
   pdl_wait();
-  const double hn = s->hn;
-  if (!(hn > 0.0)) return;
-  T* v = V + (int64_t)s->j * ld;
-  const T inv = (T)(1.0 / hn);
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    v[k] = v[k] * inv;
+  __shared__ double hs, is;
+  if (threadIdx.x == 0) {
+    hs = sqrt(w2[0]);
+    is = 1.0 / hs;
+  }
+  __syncthreads();
+  if (hs > 0.0) {
+    T* v = V + (int64_t)(s->j + 1) * ld;
+    const T inv = (T)is;
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+      v[k] = v[k] * inv;
+  }
+  if (last_block(cnt) && threadIdx.x == 0) gm_column(s, h2, hs, cond, in_graph);
 }
 
 // y = H(0:j, 0:j)^{-1} g (back substitution, one thread).
@@ -545,19 +566,10 @@ __global__ void k_axpby(const T* __restrict__ x, double a, T* __restrict__ y, do
     y[k] = b == 0.0 ? aa * x[k] : aa * x[k] + bb * y[k];
 }
 
-// y <- x * (1 / c[0])  (scale by a device scalar)
-template <typename T>
-__global__ void k_scale_inv(const T* __restrict__ x, const double* __restrict__ c, T* __restrict__ y, int64_t n) {
-  pdl_wait();
-  const T inv = (T)(1.0 / c[0]);
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    y[k] = x[k] * inv;
-}
-
 template <typename T>
 static bk_status dots(const T* V, int64_t ld, int nv, const T* w, int64_t n, double* partial, double* out,
                       unsigned* cnt, cudaStream_t st) {
-  BK_TRY(launch(k_multidot<T>, DOT_BLOCKS, 256, 0, st, V, ld, nv, w, n, partial, out, cnt));
+  BK_TRY(launch(k_multidot<T>, dot_blocks(n), 256, 0, st, V, ld, nv, w, n, partial, out, cnt));
   return BK_OK;
 }
 
@@ -656,17 +668,15 @@ static bk_status arnoldi_step(const GmCtx<T>& c, int jh, bool graph, cudaGraphCo
                                        c.aux ? c.aux->n : 0));
   }
   // Gram-Schmidt (DGKS): h1 = [V_0..V_j]^T w and |w|^2 (w = V_{j+1}), w <- w - V h1 with the new
-  // |w|^2; the second pass runs (its kernels do work) only when k_gm_a asked for it.
+  // |w|^2; the second pass runs (its kernels do work) only when the first one's end asked for it.
   double* w2 = c.h2 + (MAXM + 1);
-  BK_TRY(launch(k_multidot_s<T>, DOT_BLOCKS, 256, 0, st, c.V, ld, 2, 1, c.gs, nullptr, n, c.partial, c.h1, c.cnt));
-  BK_TRY(launch(k_multiaxpy_s<T>, DOT_BLOCKS, 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, nullptr, c.h1, -1.0, 1.0, n, c.partial,
-                                               w2, c.cnt + 1));
-  BK_TRY(launch(k_gm_a, 1, 128, 0, st, c.gs, c.h1, w2));
-  BK_TRY(launch(k_multidot_s<T>, DOT_BLOCKS, 256, 0, st, c.V, ld, 1, 1, c.gs, &c.gs->need2, n, c.partial, c.h2, c.cnt));
-  BK_TRY(launch(k_multiaxpy_s<T>, DOT_BLOCKS, 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, &c.gs->need2, c.h2, -1.0, 1.0, n,
-                                               c.partial, w2, c.cnt + 1));
-  BK_TRY(launch(k_gm_b, 1, 32, 0, st, c.gs, c.h2, w2, cond, graph ? 1 : 0));
-  BK_TRY(launch(k_scale_inv_s<T>, c.g, 256, 0, st, c.V, ld, c.gs, n));
+  BK_TRY(launch(k_multidot_s<T>, dot_blocks(n), 256, 0, st, c.V, ld, 2, 1, c.gs, nullptr, n, c.partial, c.h1, c.cnt));
+  BK_TRY(launch(k_multiaxpy_s<T>, dot_blocks(n), 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, nullptr, c.h1, -1.0, 1.0, n, c.partial,
+                                               w2, c.cnt + 1, c.gs));
+  BK_TRY(launch(k_multidot_s<T>, dot_blocks(n), 256, 0, st, c.V, ld, 1, 1, c.gs, &c.gs->need2, n, c.partial, c.h2, c.cnt));
+  BK_TRY(launch(k_multiaxpy_s<T>, dot_blocks(n), 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, &c.gs->need2, c.h2, -1.0, 1.0, n,
+                                               c.partial, w2, c.cnt + 1, nullptr));
+  BK_TRY(launch(k_gm_finish<T>, c.g, 256, 0, st, c.V, ld, n, c.gs, c.h2, w2, c.cnt + 2, cond, graph ? 1 : 0));
   return BK_OK;
 }
 
@@ -859,7 +869,7 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
   // arrival counters of the one-launch reductions (k_multidot, k_multiaxpy); each launch's
   // last block resets its counter, so one clear per solve suffices
   unsigned* cnt = reinterpret_cast<unsigned*>(dvec + 3 * (MAXM + 2));
-  BK_TRY_CUDA(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned), st));
+  BK_TRY_CUDA(cudaMemsetAsync(cnt, 0, 3 * sizeof(unsigned), st));
   const int g = grid_for(n);
   weighted = weighted && op == BK_OP_KKT && o.use_precond;
   const int wz = pr->n_x + pr->n_u, wl = pr->n_x;
@@ -896,12 +906,9 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
   double resid = bnorm;
   bool first = true;
   while (true) {
-    // r = b - A x (x = 0 on the first cycle)
-    if (first) {
-      if (!weighted) {  // weighted: r already holds D b
-        BK_TRY(launch(k_axpby<T>, g, 256, 0, st, b, 1.0, r, 0.0, n));
-      }
-    } else {
+    // r = b - A x (on the first cycle x = 0: the right-hand side itself)
+    const T* src = first ? bw : r;
+    if (!first) {
       BK_TRY(op_apply(pr, d, op, x, r, st));
       BK_TRY(launch(k_axpby<T>, g, 256, 0, st, b, 1.0, r, -1.0, n));
       if (weighted) BK_TRY(wscale(r, r, 0));
@@ -916,7 +923,7 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
     first = false;
     resid = beta;
     if (beta <= target || total >= o.max_iter) break;
-    BK_TRY(launch(k_axpby<T>, g, 256, 0, st, r, 1.0 / beta, V, 0.0, n));
+    BK_TRY(launch(k_axpby<T>, g, 256, 0, st, src, 1.0 / beta, V, 0.0, n));
     const int jmax = std::min(m, o.max_iter - total);
     BK_TRY(launch(k_gm_init, 1, 128, 0, st, gs, beta, target, jmax, m));
     if (gg) {
@@ -933,10 +940,10 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
     // x += Z y (flexible form; Z = V without preconditioning), y = H^{-1} g on the device
     BK_TRY(launch(k_gm_solve, 1, 32, 0, st, gs));
     BK_TRY(launch(k_multiaxpy_s<T>, g, 256, 0, st, o.use_precond ? Zb : V, ld, 0, -1, x, gs, nullptr, gs->y, 1.0, 1.0, n,
-                                        nullptr, nullptr, nullptr));
+                                        nullptr, nullptr, nullptr, nullptr));
     if (aux) {
       BK_TRY(launch(k_multiaxpy_s<double>, grid_for(aux->n), 256, 0, st, aux->T, aux->ld, 0, -1, aux->Td, gs, nullptr, gs->y,
-                                                              1.0, 1.0, aux->n, nullptr, nullptr, nullptr));
+                                                              1.0, 1.0, aux->n, nullptr, nullptr, nullptr, nullptr));
     }
     if (gg) {
       BK_TRY_CUDA(cudaMemcpyAsync(hostbuf, gs, sizeof(GmHead), cudaMemcpyDeviceToHost, st));

@@ -470,23 +470,31 @@ static bk_status newton_impl(Problem* pr, double* z, const bk_newton_opts& o, bk
       info->kkt_solves += 1;
     } else {
       // FP32 GMRES inside FP64 iterative refinement
-      double rn0 = 0.0;
-      BK_TRY(norm2(pr, rhs, n, &rn0, st));
-      BK_TRY_CUDA(cudaMemsetAsync(d, 0, sizeof(double) * n, st));
-      BK_TRY(launch(k_axpby64, g, 256, 0, st, rhs, 1.0, r, 0.0, n));
-      for (int sweep = 0; sweep < o.max_refine; ++sweep) {
-        BK_TRY(launch(k_cast<double, float>, g, 256, 0, st, r, r32, n));
+      if (o.max_refine == 1) {   // the Newton residual checks d: one solve, no refinement residual
+        BK_TRY(launch(k_cast<double, float>, g, 256, 0, st, rhs, r32, n));
         BK_TRY(gmres(pr, pr->d32, BK_OP_KKT, r32, d32, ko, &ki, gws, st, nullptr, weighted));
         info->krylov_iterations += ki.iterations;
         info->kkt_solves += 1;
-        BK_TRY(launch(k_acc32, g, 256, 0, st, d32, d, n));
-        if (sweep + 1 == o.max_refine) break;  // last sweep: the Newton residual checks d
-        // r = rhs - K d (FP64)
-        BK_TRY(op_apply(pr, pr->d64, BK_OP_KKT, d, r, st));
-        BK_TRY(launch(k_axpby64, g, 256, 0, st, rhs, 1.0, r, -1.0, n));
-        double rn = 0.0;
-        BK_TRY(norm2(pr, r, n, &rn, st));
-        if (rn <= o.ir_rtol * rn0) break;
+        BK_TRY(launch(k_cast<float, double>, g, 256, 0, st, d32, d, n));
+      } else {
+        double rn0 = 0.0;
+        BK_TRY(norm2(pr, rhs, n, &rn0, st));
+        BK_TRY_CUDA(cudaMemsetAsync(d, 0, sizeof(double) * n, st));
+        BK_TRY(launch(k_axpby64, g, 256, 0, st, rhs, 1.0, r, 0.0, n));
+        for (int sweep = 0; sweep < o.max_refine; ++sweep) {
+          BK_TRY(launch(k_cast<double, float>, g, 256, 0, st, r, r32, n));
+          BK_TRY(gmres(pr, pr->d32, BK_OP_KKT, r32, d32, ko, &ki, gws, st, nullptr, weighted));
+          info->krylov_iterations += ki.iterations;
+          info->kkt_solves += 1;
+          BK_TRY(launch(k_acc32, g, 256, 0, st, d32, d, n));
+          if (sweep + 1 == o.max_refine) break;  // last sweep: the Newton residual checks d
+          // r = rhs - K d (FP64)
+          BK_TRY(op_apply(pr, pr->d64, BK_OP_KKT, d, r, st));
+          BK_TRY(launch(k_axpby64, g, 256, 0, st, rhs, 1.0, r, -1.0, n));
+          double rn = 0.0;
+          BK_TRY(norm2(pr, r, n, &rn, st));
+          if (rn <= o.ir_rtol * rn0) break;
+        }
       }
       if (!ft) BK_TRY(plan_apply_n(pr->d64.plan, dlam, Mud, pr->n_x, true, pr->s, st));
     }
