@@ -1164,13 +1164,12 @@ static bk_status configure_cluster(Plan* p) {
 // The dynamic shared-memory cap is a per-function setting shared by every plan, so it is set to
 // the largest size any plan of the type can request (never to one plan's own size, which would
 // lower the cap under plans created earlier).
-// Kernel attributes: the dynamic shared-memory cap (largest size any plan of the type requests)
-// and a carveout that gives shared memory the whole unified L1/shared array, so that several
-// transform CTAs stay resident per SM.
+// No carveout is preferred: the L1 that the resident CTAs' tiles leave free holds the stage twiddles
+// of the FP64 kernels (with all of the array as shared memory, 4 components, us: double-float 2^20 246,
+// 2^22 1041, FP32 2^22 339; without 225, 908, 304).
 template <typename K>
 static bk_status smem_attr(K* fn, int cap) {
   BK_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-  BK_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   return BK_OK;
 }
 

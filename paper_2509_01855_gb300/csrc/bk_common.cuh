@@ -113,7 +113,6 @@ template <typename T> __host__ __device__ __forceinline__ typename V2<T>::t mk2(
 // computed in (a plan's own or a batched launch) rounds it alike.
 __device__ __forceinline__ float dot2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
 __device__ __forceinline__ double dot2(double a, double b, double c, double d) { return __fma_rn(a, b, __dmul_rn(c, d)); }
-__device__ __forceinline__ dfl dot2(dfl a, dfl b, dfl c, dfl d) { return a * b + c * d; }
 
 // Complex product a * b.
 template <typename C> __device__ __forceinline__ C cmul(C a, C b) {

