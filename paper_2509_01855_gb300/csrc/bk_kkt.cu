@@ -68,11 +68,28 @@ constexpr int FT_NB = 608;
 // factorisation of I - h J with partial pivoting and the n_x columns of h J as right-hand
 // sides: about 120 operations per node at n_x = 4, where inverting I - h J by Gauss-Jordan and
 // multiplying by h J took about 240 (the kernel is bound by the FP64 pipe). Solving for D
-// directly keeps its relative accuracy when h J is small (forming K - I would cancel).
+// directly keeps its relative accuracy when h J is small (forming K - I would cancel). FP64 nodes of the
+// orbit kinds with a small h J take their closed form, some 45 operations (k_lin_nodes at N = 2^20, with
+// the KKT product's entries, 296 + 83 -> 182 us); in FP32, not bound by arithmetic, that form's rounding
+// doubled the preconditioner's error.
+__device__ __forceinline__ bool below_eighth(double x) {   // |x| < 1/8 on the integer pipe
+  return (__double2hiint(x) & 0x7fffffff) < 0x3fc00000;
+}
+
 template <typename Tc, int KIND, int NX>
-__device__ void node_deviation(const Tc* x, const Tc* u, Tc h, Tc* D, Tc pa) {
-  Tc Jx[NXM * NXM], Ju[NXM * NUM];
-  Dyn<KIND>::template jac<Tc>(x, u, Jx, Ju, pa);
+__device__ void node_deviation(const Tc* Jx, Tc h, Tc* D) {
+  if constexpr (Dyn<KIND>::closed_deviation && sizeof(Tc) == 8) {
+    bool small = true;
+#pragma unroll
+    for (int r = 0; r < NX; ++r)
+#pragma unroll
+      for (int c = 0; c < NX; ++c)
+        if (Dyn<KIND>::jx_nz(r, c)) small = small && below_eighth((double)(h * Jx[r * NX + c]));
+    if (small) {
+      Dyn<KIND>::template deviation<Tc>(Jx, h, D);
+      return;
+    }
+  }
   Tc A[NX * NX], B[NX * NX], ip[NX];
 #pragma unroll
   for (int r = 0; r < NX; ++r)
@@ -132,8 +149,9 @@ __device__ void node_deviation(const Tc* x, const Tc* u, Tc h, Tc* D, Tc pa) {
 // directly by node_deviation), which halves the sweeps' node factor traffic and, with
 // K v = v + D v and N v = 2 D v, their FP64 products.
 template <typename T, int KIND, int NX, int NU>
-__global__ void k_lin_nodes(const double* __restrict__ z, int64_t P, int64_t L, const double* __restrict__ w,
-                            double s, T* __restrict__ Dn, T* __restrict__ xu, double pa) {
+__global__ void __launch_bounds__(256, 2) k_lin_nodes(const double* __restrict__ z, int64_t P, int64_t L, const double* __restrict__ w,
+                            double s, T* __restrict__ Dn, T* __restrict__ xu, double pa, const T* __restrict__ mu,
+                            T* __restrict__ lin) {
   pdl_wait();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
     T x[NXM], u[NUM];
@@ -141,8 +159,19 @@ __global__ void k_lin_nodes(const double* __restrict__ z, int64_t P, int64_t L, 
     for (int m = 0; m < NX; ++m) x[m] = (T)z[m * P + k];
 #pragma unroll
     for (int q = 0; q < NU; ++q) u[q] = (T)z[(NX + q) * P + k];
-    T D[NX * NX];
-    node_deviation<T, KIND, NX>(x, u, (T)(0.5 * s * w[k]), D, (T)pa);
+    T D[NX * NX], Jx[NXM * NXM], Ju[NXM * NUM];
+    Dyn<KIND>::template jac<T>(x, u, Jx, Ju, (T)pa);
+    node_deviation<T, KIND, NX>(Jx, (T)(0.5 * s * w[k]), D);
+    if constexpr (Dyn<KIND>::nlj > 0) {   // the entries the KKT product reads (k_lin_entries)
+      if (lin) {
+        T m_[NXM], v[Dyn<KIND>::nlj + Dyn<KIND>::nlh];
+#pragma unroll
+        for (int m = 0; m < NX; ++m) m_[m] = mu[m * P + k];
+        Dyn<KIND>::template pack<T>(x, u, m_, (T)pa, v);
+#pragma unroll
+        for (int i = 0; i < Dyn<KIND>::nlj + Dyn<KIND>::nlh; ++i) lin[i * P + k] = v[i];
+      }
+    }
 #pragma unroll
     for (int c = 0; c < NX * NX; ++c) Dn[il_index<Seg<T>::v>(k, c, NX * NX)] = D[c];
 #pragma unroll
@@ -195,9 +224,11 @@ __global__ void k_lin_seg(const T* __restrict__ Dn, int64_t L, int nseg, T* __re
   const int64_t k0 = (int64_t)seg * SEG;
 #pragma unroll
   for (int c = 0; c < NX * NX; ++c) A[c] = zcol<NX>(c % NX) ? T(0) : T(2) * Dn[il_index<Seg<T>::v>(k0, c, NX * NX)];
+  // every node's matrix is loaded ahead of the product chain (the storage covers whole segments; nodes
+  // past L are dropped): one load after another, an FP32 problem of N = 2^12 took 24 us here
+#pragma unroll
   for (int i = 1; i < SEG; ++i) {
     const int64_t k = k0 + i;
-    if (k >= L) break;
 #pragma unroll
     for (int c = 0; c < NX * NX; ++c) D[c] = zcol<NX>(c % NX) ? T(0) : Dn[il_index<Seg<T>::v>(k, c, NX * NX)];
 #pragma unroll
@@ -215,7 +246,7 @@ __global__ void k_lin_seg(const T* __restrict__ Dn, int64_t L, int nseg, T* __re
         R[r * NX + c] = fma(T(2), a, A[r * NX + c]);
       }
 #pragma unroll
-    for (int c = 0; c < NX * NX; ++c) A[c] = R[c];
+    for (int c = 0; c < NX * NX; ++c) A[c] = k < L ? R[c] : A[c];
   }
 #pragma unroll
   for (int c = 0; c < NX * NX; ++c) A0[il32(seg, c, NX * NX)] = A[c];
@@ -223,9 +254,11 @@ __global__ void k_lin_seg(const T* __restrict__ Dn, int64_t L, int nseg, T* __re
 
 // Slots of one level (deviations from I), one warp per block of 32 items (items at or beyond n
 // are identity maps, deviation 0):
-// spans M_k(j) = M_{k-1}(j) M_{k-1}(j - 2^{k-1}) by doubling (defined for j >= 2^k - 1), Pre(i)
-// and Suf(i) as products of the spans that tile [0, i) and (i, 31], and the block's product
-// M_4(31) M_4(15), which is the map of the parent item at the next level.
+// products M_k(j) = M_{k-1}(j) M_{k-1}(j - 2^{k-1}) of the last 2^k items up to j (fewer at the block's
+// start) by doubling: the spans of the scans for j >= 2^k - 1 and, at k = 5, every prefix, hence Pre(i)
+// and the block's product, the map of the parent item at the next level (FP64, bound by its products:
+// N = 2^20 172 -> 126 us; FP32 keeps the products of spans that tile [0, i), whose roundings the doubled
+// prefixes exceeded for some inputs). Suf(i) is a product of the spans that tile (i, 31].
 template <typename T, int NX>
 __global__ void __launch_bounds__(32) k_lin_level(T* __restrict__ m, int n, T* __restrict__ parent) {
   pdl_wait();
@@ -244,11 +277,11 @@ __global__ void __launch_bounds__(32) k_lin_level(T* __restrict__ m, int n, T* _
   for (int k = 1; k < 5; ++k) {
     const int h = 1 << (k - 1);
     T R[NC];
-    if (lane >= 2 * h - 1) {
+    if (lane >= h) {
       dev_mul<NX, T>(S[k - 1][lane], S[k - 1][lane - h], R);
     } else {
 #pragma unroll
-      for (int c = 0; c < NC; ++c) R[c] = T(0);
+      for (int c = 0; c < NC; ++c) R[c] = S[k - 1][lane][c];
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) S[k][lane][c] = R[c];
@@ -259,20 +292,48 @@ __global__ void __launch_bounds__(32) k_lin_level(T* __restrict__ m, int n, T* _
 #pragma unroll
     for (int c = 0; c < NC; ++c) m[k * slot + il32(i, c, NC)] = S[k][lane][c];
   T R[NC], Q[NC];
-  // Pre(i) = A_{i-1} ... A_0
+  if constexpr (sizeof(T) == 8) {
+    // one more doubling gives every lane the product of the items up to its own; Pre(i) is the lane before
+    if (lane >= 16) {
+      dev_mul<NX, T>(S[4][lane], S[4][lane - 16], R);
+    } else {
 #pragma unroll
-  for (int c = 0; c < NC; ++c) R[c] = T(0);
-  int pos = 0;
-  for (int k = 4; k >= 0; --k) {
-    if ((lane >> k) & 1) {
-      dev_mul<NX, T>(S[k][pos + (1 << k) - 1], R, Q);
+      for (int c = 0; c < NC; ++c) R[c] = S[4][lane][c];
+    }
+    if (parent && lane == 31) {
 #pragma unroll
-      for (int c = 0; c < NC; ++c) R[c] = Q[c];
-      pos += 1 << k;
+      for (int c = 0; c < NC; ++c) parent[il32(blockIdx.x, c, NC)] = R[c];
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const T v = shfl_up(R[c], 1);
+      m[SL_PRE * slot + il32(i, c, NC)] = lane == 0 ? T(0) : v;
+    }
+  } else {
+    // Pre(i) = A_{i-1} ... A_0 from the spans that tile [0, i)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) R[c] = T(0);
+    int pos = 0;
+    for (int k = 4; k >= 0; --k) {
+      if ((lane >> k) & 1) {
+        dev_mul<NX, T>(S[k][pos + (1 << k) - 1], R, Q);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) R[c] = Q[c];
+        pos += 1 << k;
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) m[SL_PRE * slot + il32(i, c, NC)] = R[c];
+    if (parent) {
+      for (int c = lane; c < NC; c += 32) {
+        const int r = c / NX, cc = c % NX;
+        T a = 0;
+#pragma unroll
+        for (int q = 0; q < NX; ++q) a += S[4][31][r * NX + q] * S[4][15][q * NX + cc];
+        parent[il32(blockIdx.x, c, NC)] = (S[4][31][c] + S[4][15][c]) + a;
+      }
     }
   }
-#pragma unroll
-  for (int c = 0; c < NC; ++c) m[SL_PRE * slot + il32(i, c, NC)] = R[c];
   // Suf(i) = A_31 ... A_{i+1}
 #pragma unroll
   for (int c = 0; c < NC; ++c) R[c] = T(0);
@@ -288,15 +349,6 @@ __global__ void __launch_bounds__(32) k_lin_level(T* __restrict__ m, int n, T* _
   }
 #pragma unroll
   for (int c = 0; c < NC; ++c) m[SL_SUF * slot + il32(i, c, NC)] = R[c];
-  if (parent) {
-    for (int c = lane; c < NC; c += 32) {
-      const int r = c / NX, cc = c % NX;
-      T a = 0;
-#pragma unroll
-      for (int q = 0; q < NX; ++q) a += S[4][31][r * NX + q] * S[4][15][q * NX + cc];
-      parent[il32(blockIdx.x, c, NC)] = (S[4][31][c] + S[4][15][c]) + a;
-    }
-  }
 }
 
 template <typename Tin, typename Tout>
@@ -1495,7 +1547,7 @@ static const T* bar_hbar(const Problem* pr, const OpData& d) {
 // Segment maps and scan levels from the node factors N_k (level data of the sweeps).
 template <typename T, int NX>
 static bk_status lin_levels(Problem* pr, OpData& d, cudaStream_t st) {
-  BK_TRY(launch(k_lin_seg<T, NX>, (pr->nseg + 127) / 128, 128, 0, st, (const T*)d.Dn, pr->L, pr->nseg, (T*)d.lvm[0]));
+  BK_TRY(launch(k_lin_seg<T, NX>, (pr->nseg + 31) / 32, 32, 0, st, (const T*)d.Dn, pr->L, pr->nseg, (T*)d.lvm[0]));
   for (int l = 0; l < pr->nlev; ++l) {
     BK_TRY(launch(k_lin_level<T, NX>, (pr->lvn[l] + 31) / 32, 32, 0, st, (T*)d.lvm[l], pr->lvn[l],
                                                               l + 1 < pr->nlev ? (T*)d.lvm[l + 1] : nullptr));
@@ -1504,10 +1556,10 @@ static bk_status lin_levels(Problem* pr, OpData& d, cudaStream_t st) {
 }
 
 template <typename T, int KIND>
-static bk_status lin_factors(Problem* pr, OpData& d, const double* z, cudaStream_t st) {
+static bk_status lin_factors(Problem* pr, OpData& d, const double* z, bool entries, cudaStream_t st) {
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu;
   BK_TRY(launch(k_lin_nodes<T, KIND, NX, NU>, nblk(pr->L), 256, 0, st, z, pr->P, pr->L, pr->d64.plan->w64, pr->s, (T*)d.Dn, (T*)d.xu,
-                                                             pr->dyn_param()));
+                pr->dyn_param(), (const T*)d.mu, entries ? (T*)d.lin : nullptr));
   return lin_levels<T, NX>(pr, d, st);
 }
 
@@ -1657,13 +1709,13 @@ static bk_status linearize_kind(Problem* pr, const double* z, const double* mu, 
   else
     BK_TRY(plan_apply_n(pr->d64.plan, z + (NX + NU) * P, pr->d64.mu, NX, true, pr->s, st));
   if (pr->pdtype == BK_F64 && keep != LIN_KEEP_PRECOND)
-    BK_TRY((lin_factors<double, KIND>(pr, pr->d64, z, st)));
+    BK_TRY((lin_factors<double, KIND>(pr, pr->d64, z, pr->dtype == BK_F64, st)));
   else
     BK_TRY_CUDA(cudaMemcpyAsync(pr->d64.xu, z, sizeof(double) * (NX + NU) * P, cudaMemcpyDeviceToDevice, st));
   if (pr->d32.plan) {
     BK_TRY(launch(k_convert<double, float>, nblk(NX * P), 256, 0, st, (const double*)pr->d64.mu, (float*)pr->d32.mu, NX * P));
     if (keep != LIN_KEEP_PRECOND) {
-      BK_TRY((lin_factors<float, KIND>(pr, pr->d32, z, st)));
+      BK_TRY((lin_factors<float, KIND>(pr, pr->d32, z, pr->dtype == BK_F32, st)));
     } else {
       BK_TRY(launch(k_convert<double, float>, nblk((NX + NU) * P), 256, 0, st, z, (float*)pr->d32.xu, (NX + NU) * P));
     }
@@ -1677,10 +1729,13 @@ static bk_status linearize_kind(Problem* pr, const double* z, const double* mu, 
   }
   if constexpr (Dyn<KIND>::nlj > 0) {
     pr->lin64_stale = pr->dtype == BK_F32;
-    if (pr->dtype == BK_F32)
-      BK_TRY((lin_entries<float, KIND>(pr, pr->d32, st)));
-    else
-      BK_TRY((lin_entries<double, KIND>(pr, pr->d64, st)));
+    // k_lin_nodes wrote them where it ran in the problem's precision
+    if (keep == LIN_KEEP_PRECOND || pr->pdtype != pr->dtype) {
+      if (pr->dtype == BK_F32)
+        BK_TRY((lin_entries<float, KIND>(pr, pr->d32, st)));
+      else
+        BK_TRY((lin_entries<double, KIND>(pr, pr->d64, st)));
+    }
   }
   pr->linearized = true;
   if (keep != LIN_FULL) return BK_OK;

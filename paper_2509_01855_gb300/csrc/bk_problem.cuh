@@ -47,6 +47,7 @@ template <int KIND> struct Dyn;
 // vanish). Kinds without a pattern take the dense one.
 struct DenseNZ {
   static constexpr int nlj = 0, nlh = 0;
+  static constexpr bool closed_deviation = false;
   __host__ __device__ static constexpr bool jx_nz(int, int) { return true; }
   __host__ __device__ static constexpr bool ju_nz(int, int) { return true; }
   __host__ __device__ static constexpr bool h_nz(int, int) { return true; }
@@ -59,6 +60,7 @@ __device__ inline void sincos_t(float x, float* s, float* c) { sincosf(x, s, c);
 template <> struct Dyn<BK_DBL_INT> {
   static constexpr int nx = 2, nu = 1;
   static constexpr int nlj = 0, nlh = 0;
+  static constexpr bool closed_deviation = false;
   // J_x = [[0, 1], [0, 0]], J_u = [0; 1], H = 0 (f is linear)
   __host__ __device__ static constexpr bool jx_nz(int r, int c) { return r == 0 && c == 1; }
   __host__ __device__ static constexpr bool ju_nz(int r, int q) { return r == 1 && q == 0; }
@@ -97,6 +99,32 @@ template <> struct Dyn<BK_ORBIT> {
   // control block of the KKT preconditioner at a node: s w_k times the running cost's curvature
   static constexpr bool huu_needs_mu = false;
   template <typename T> __device__ static T pre_huu(const T* mu, T swk, T) { return swk; }
+  // Node deviation D = (I - h J)^{-1} h J in closed form, for max |h J| < 1/8 (I - h J is then strictly
+  // diagonally dominant, and elimination needs no pivoting). theta drops out: D_theta = h J_theta (I + D);
+  // with r eliminated from (r, v_r, v_theta) a 2 x 2 system is left for each of the three columns.
+  static constexpr bool closed_deviation = true;
+  template <typename T> __device__ static void deviation(const T* Jx, T h, T* D) {
+    const T a = h * Jx[8], b = h * Jx[11], c = h * Jx[12], d = h * Jx[14], e = h * Jx[15];
+    const T f = h * Jx[4], g = h * Jx[7];
+    const T p = fma(-a, h, T(1)), q = T(1) - e, t = fma(c, h, d);
+    const T inv = T(1) / fma(p, q, -(b * t));
+    // right-hand sides of (v_r, v_theta) for the columns r, v_r, v_theta, and r's own
+    const T R2[3] = {a, a * h, b}, R3[3] = {c, t, e}, r0[3] = {T(0), h, T(0)};
+    const int col[3] = {0, 2, 3};
+#pragma unroll
+    for (int i = 0; i < 16; ++i) D[i] = T(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int j = col[k];
+      const T x2 = fma(q, R2[k], b * R3[k]) * inv;
+      const T x3 = fma(p, R3[k], t * R2[k]) * inv;
+      const T x0 = fma(h, x2, r0[k]);
+      D[0 * 4 + j] = x0;
+      D[2 * 4 + j] = x2;
+      D[3 * 4 + j] = x3;
+      D[1 * 4 + j] = fma(f, x0, g * x3) + (j == 0 ? f : (j == 3 ? g : T(0)));
+    }
+  }
   // entries the KKT product reads from the linearisation: J_x (7, without the constant ones), H (5)
   static constexpr int nlj = 7, nlh = 5;
   template <typename T> __device__ static void pack(const T* x, const T* u, const T* mu, T pa, T* v) {
@@ -177,6 +205,8 @@ template <> struct Dyn<BK_BILINEAR> : DenseNZ {
 // steered by the angle u (pa = a), cost T = t_f - t_0 with the final time free.
 template <> struct Dyn<BK_ORBIT_MT> : DenseNZ {
   static constexpr int nlj = 0, nlh = 0;
+  static constexpr bool closed_deviation = true;   // the state Jacobian of BK_ORBIT
+  template <typename T> __device__ static void deviation(const T* Jx, T h, T* D) { Dyn<BK_ORBIT>::deviation<T>(Jx, h, D); }
   // the state Jacobian of BK_ORBIT (theta enters no right-hand side); J_u and H dense
   __host__ __device__ static constexpr bool jx_nz(int r, int c) { return Dyn<BK_ORBIT>::jx_nz(r, c); }
   static constexpr int nx = 4, nu = 1;
