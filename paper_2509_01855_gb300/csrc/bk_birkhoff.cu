@@ -346,7 +346,7 @@ __device__ void dct1_block(const T* __restrict__ X, int kind, T* __restrict__ Y,
   }
   __syncthreads();
   if (N >= 16) {
-    fft_any<T, SmallFft<T>::E, SmallFft<T>::EPT, 4, 12>(buf, log2N, 1, pad_stride(N), stw);
+    fft_any<T, SmallFft<T>::E, SmallFft<T>::EPT, 4, sizeof(T) == 8 ? 9 : 12>(buf, log2N, 1, pad_stride(N), stw);
   } else {
     // N = 4 or 8: direct DFT (tw holds omega_N^i, n_tab = N)
     C zk = mk2<T>(T(0), T(0));
@@ -412,7 +412,7 @@ __device__ __forceinline__ void small_body(int vec, const Us<T>* __restrict__ in
 }
 
 template <typename T, bool TRANS>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 1024)
     k_birkhoff_small(const Us<T>* __restrict__ in, Us<T>* __restrict__ out, int N, int log2N, int64_t pitch,
                      T s, const typename V2<T>::t* __restrict__ tw, const typename V2<T>::t* __restrict__ stw,
                      const typename V2<T>::t* __restrict__ tpost, StencilTab<T> tb) {
@@ -680,7 +680,7 @@ __device__ __forceinline__ int batch_job(const Batch<J>& b, int cta) {
 }
 
 template <typename T, bool TRANS>
-__global__ void __launch_bounds__(1024) k_small_batch(const __grid_constant__ Batch<SmallJob<T>> b) {
+__global__ void __launch_bounds__(sizeof(T) == 8 ? 256 : 1024) k_small_batch(const __grid_constant__ Batch<SmallJob<T>> b) {
   pdl_wait();
   const int q = batch_job(b, blockIdx.x);
   const SmallJob<T>& J = b.j[q];
@@ -892,13 +892,13 @@ static bk_status compute_weights(Plan* p, cudaStream_t st) {
 #endif  // BK_TRANSFORM_KERNEL_UNIT
 
 // Largest N run by the single-CTA kernel (one CTA per vector): 256 in FP64, whose single CTA runs
-// on one SM's FP64 pipe, 4096 in FP32. Measured (4 components, warm, us per product, one CTA /
-// cluster): FP64 2^8 18.6 / 24.7, 2^10 35.1 / 26.8; FP32 2^11 13.5 / 15.5, 2^12 16.7 / 17.2.
-// BK_SMALL_MAX_LOG2 overrides it for tuning (at least 2^4; at most the shared-memory limit of
-// 4096). The four-step kernels need N >= 128.
-static int small_default(int dtype) { return dtype == BK_F64 ? 256 : 4096; }
+// on one SM's FP64 pipe, 2048 in FP32. Measured (4 components, us per product, one CTA / cluster): FP64
+// 2^8 12.0 / 18.1, 2^9 19.8 / 18.2; FP32 2^11 10.2 / 11.6, 2^12 14.3 / 12.9. BK_SMALL_MAX_LOG2
+// overrides it for tuning (at least 2^4; at most 512 in FP64, 4096 in FP32). The four-step kernels
+// need N >= 128.
+static int small_default(int dtype) { return dtype == BK_F64 ? 256 : 2048; }
 static int small_limit(int dtype) {
-  const int cap = 4096;
+  const int cap = dtype == BK_F64 ? 512 : 4096;
   const char* e = getenv("BK_SMALL_MAX_LOG2");
   if (e) {
     const long v = atol(e);
@@ -952,22 +952,20 @@ static int fourstep_elems(int dtype, int64_t n, int nvec, int N1, int N2, int Ef
   return (int)std::min<int64_t>(E, cap);
 }
 
-// Smallest log2 N whose four passes run as a launch each instead of as one cluster launch: 14 in
-// FP64, whose sixteen CTAs per vector leave most FP64 pipes idle, 15 in FP32. Measured (4
-// components, warm, us per product, cluster / launch per pass): FP64 2^12 30.9 / 40.2, 2^13 39.1 /
-// 42.2, 2^14 49.4 / 45.3, 2^15 72 / 46.3; FP32 2^13 21.3 / 26.9, 2^14 22.8 / 25.8, 2^16 49.0 / 30.7.
-// BK_SPLIT_MIN_LOG2 overrides it for tuning.
-static int split_min_log2(int dtype) {
+// Whether the four passes run as a launch each instead of as one cluster launch: from 2^13 on, and in FP64
+// from 2^12 with more than 8 vectors, whose sixteen CTAs per vector then share FP64 pipes. Measured
+// (us per product, cluster / launch per pass): FP64, 4 components, 2^11 20.5 / 24.5, 2^12 23.8 / 31.1, 2^13 31.7 /
+// 32.1, 2^14 47.0 / 34.2; 16 components 2^10 21.6 / 25.2, 2^12 36.4 / 30.8; FP32 2^12 12.9 / 15.5,
+// 2^13 17.1 / 15.5, 2^14 20.5 / 16.5. BK_SPLIT_MIN_LOG2 sets the border for tuning.
+static bool split_passes(int dtype, int64_t N, int nvec) {
   const char* e = getenv("BK_SPLIT_MIN_LOG2");
   if (e) {
     const long v = atol(e);
-    if (v >= 7 && v <= 30) return (int)v;
+    if (v >= 7 && v <= 30) return ilog2(N) >= std::min((int)v, 2 * CL_MAXLOG2);
   }
-  return dtype == BK_F64 ? 14 : 15;
+  return N >= 8192 || (dtype == BK_F64 && N >= 4096 && nvec > 8);
 }
 
-// Shapes of one four-step layout (tables untouched, so a built plan can be re-shaped); Eforce
-// > 0 fixes the elements per CTA (the autotuner's candidates), 0 takes fourstep_elems.
 // log2 radix of the plain complex passes of length n: 4 in FP32; in FP64 2 while few warps share the
 // FP64 pipes and 4 from 2^18 on, where its fewer shared-memory round trips count (products of 4
 // components, radix 4 / radix 16, us: N = 3001 61 / 127, N = 140001 1512 / 1344, N = 393217 2853 / 2433).
@@ -1141,9 +1139,11 @@ static bk_status configure_cluster(Plan* p) {
   re_factors(f, p->N);
   p->csize = std::min(16, f.N2 / 4);
   const int maxthr = 512;
+  const int ept = p->dtype == BK_F64 ? SmallFft<double>::EPT : SmallFft<float>::EPT;
+  const int e = p->dtype == BK_F64 ? SmallFft<double>::E : SmallFft<float>::E;
   auto per = [&](int pairs, int n) {   // pairs per CTA, in as few equal rounds as the thread cap allows
     const int each = (pairs + p->csize - 1) / p->csize;
-    const int rounds = (int)(((int64_t)each * n / SmallFft<float>::EPT + maxthr - 1) / maxthr);
+    const int rounds = (int)(((int64_t)each * n / ept + maxthr - 1) / maxthr);
     return (each + rounds - 1) / rounds;
   };
   f.NB = per(f.N2 / 4 + 1, f.N1);
@@ -1151,9 +1151,8 @@ static bk_status configure_cluster(Plan* p) {
   f.bsA = re_stride(p->dtype, f.N1, f.NB);
   f.bsB = re_stride(p->dtype, f.N2, f.P);
   const size_t csz = 2 * dtype_size(p->dtype);
-  p->csmem = csz * (size_t)(std::max(f.NB * f.bsA, f.P * f.bsB) + stage_tw_len(ilog2(f.N1), SmallFft<float>::E) +
-                               stage_tw_len(ilog2(f.N2), SmallFft<float>::E));
-  p->cthr = std::max(128, round_threads(std::max(f.NB * f.N1, f.P * f.N2) / SmallFft<float>::EPT));
+  p->csmem = csz * (size_t)(std::max(f.NB * f.bsA, f.P * f.bsB) + stage_tw_len(ilog2(f.N1), e) + stage_tw_len(ilog2(f.N2), e));
+  p->cthr = std::max(128, round_threads(std::max(f.NB * f.N1, f.P * f.N2) / ept));
   if (p->csmem > FOURSTEP_SMEM_BUDGET || p->cthr > maxthr) {
     set_error("cluster configuration failed for N=%lld", (long long)p->N);
     return BK_ERR_UNSUPPORTED;
@@ -1239,7 +1238,7 @@ template <typename T>
 bk_status set_smem_attrs(const Plan* p) {
   if (p->small) {
     if constexpr (!std::is_same<T, dfl>::value) {
-      const int cap = (int)smem_small<T>(4096);
+      const int cap = (int)smem_small<T>(p->dtype == BK_F64 ? 512 : 4096);
       BK_TRY(smem_attr(k_birkhoff_small<T, false>, cap));
       BK_TRY(smem_attr(k_birkhoff_small<T, true>, cap));
       BK_TRY(smem_attr(k_small_batch<T, false>, cap));
@@ -1452,7 +1451,7 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
     }
     if (p->small) {
       p->smemS = dtype == BK_F64 ? smem_small<double>(N) : smem_small<float>(N);
-      p->thrS = round_threads(N / SmallFft<float>::EPT);
+      p->thrS = round_threads(std::max<int64_t>(N / (dtype == BK_F64 ? SmallFft<double>::EPT : SmallFft<float>::EPT), std::min<int64_t>(N, 256)));
     } else if (p->blue) {
       p->M = 1;
       while (p->M < 2 * N - 1) p->M *= 2;
@@ -1464,7 +1463,7 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
       if ((st_ = dmalloc(&p->scrY, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
       if ((st_ = dmalloc(&p->scrG, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
     } else {
-      p->split = p->df || p->mix || ilog2(N) >= std::min(2 * CL_MAXLOG2, split_min_log2(dtype));
+      p->split = p->df || p->mix || split_passes(dtype, N, n_comp * max_batch);
       p->fe = p->mix ? 0 : re_radix(N, dtype, p->df);
       if ((st_ = fourstep_shapes(p, 0)) != BK_OK) break;
       const int64_t nvec = (int64_t)n_comp * max_batch;
@@ -1825,8 +1824,8 @@ static bk_status launch_passes_batch(const Plan* const* ps, const void* const* v
   return BK_OK;
 }
 
-// fs_*: the four-step plans of radix 4. With launch-per-pass plans among them, the one-launch plans
-// join those launches (the same tiles and arithmetic, so the same results; beside the longer plans
+// fs_*: the four-step plans of radix 4. With launch-per-pass plans among them, FP32 one-launch plans
+// join those launches (the same radix and arithmetic, so the same results; beside the longer plans
 // they take no time of their own: sizes 2^8..2^16 of 4 FP32 components 79 -> 53 us in all).
 template <typename T>
 bk_status apply_batch_impl(const Plan* const* small_p, const void* const* small_v, void* const* small_o,
@@ -1837,8 +1836,24 @@ bk_status apply_batch_impl(const Plan* const* small_p, const void* const* small_
   bool split = false;
   for (int i = 0; i < nfs; ++i) split = split || fs_p[i]->split;
   if (!split) return launch_fourstep_batch<T>(fs_p, fs_v, fs_o, fs_n, nfs, trans, st);
-  return trans ? launch_passes_batch<T, true>(fs_p, fs_v, fs_o, fs_n, nfs, st)
-               : launch_passes_batch<T, false>(fs_p, fs_v, fs_o, fs_n, nfs, st);
+  auto passes = [&](const Plan* const* p, const void* const* v, void* const* o, const int* nv, int n) -> bk_status {
+    return trans ? launch_passes_batch<T, true>(p, v, o, nv, n, st) : launch_passes_batch<T, false>(p, v, o, nv, n, st);
+  };
+  if constexpr (SmallFft<T>::E == FftShape<T, 2>::E) {
+    return passes(fs_p, fs_v, fs_o, fs_n, nfs);
+  } else {
+    std::vector<const Plan*> p[2];
+    std::vector<const void*> v[2];
+    std::vector<void*> o[2];
+    std::vector<int> nv[2];
+    for (int i = 0; i < nfs; ++i) {
+      const int w = fs_p[i]->split ? 1 : 0;
+      p[w].push_back(fs_p[i]); v[w].push_back(fs_v[i]); o[w].push_back(fs_o[i]); nv[w].push_back(fs_n[i]);
+    }
+    if (!p[0].empty())
+      BK_TRY(launch_fourstep_batch<T>(p[0].data(), v[0].data(), o[0].data(), nv[0].data(), (int)p[0].size(), trans, st));
+    return passes(p[1].data(), v[1].data(), o[1].data(), nv[1].data(), (int)p[1].size());
+  }
 }
 
 #ifndef BK_TRANSFORM_KERNEL_UNIT

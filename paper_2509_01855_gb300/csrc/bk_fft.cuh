@@ -11,7 +11,8 @@
 // instructions per point as radix 16 (28 per 4 points and 2 bits against 220 per 16 points and 4
 // bits), so radix 4 with 4 values per thread spreads the same work over four times the warps
 // (products of 4 components, radix 16 / radix 4, us: N = 2^10 55 / 27, 2^14 90 / 47, 2^16 122 / 70).
-// FP32 while latency bounds it: radix 4 as well (2^14 35 / 26, 2^16 47 / 31, 2^18 50 / 41); from
+// The few CTAs of the one-CTA and one-launch FP64 kernels go on to radix 2 (2^8 13.0 / 12.0, 2^12 26.4 /
+// 23.8 radix 4 / radix 2). FP32 while latency bounds it: radix 4 as well (2^14 35 / 26, 2^16 47 / 31, 2^18 50 / 41); from
 // 2^19 on, bound by issue and shared memory: radix 16 (2^20 87 / 81). Double-float: radix 8, whose
 // code and registers are half of radix 16's (2^18 130 / 90, 2^20 339 / 260 radix 16 / radix 8).
 //
@@ -53,7 +54,7 @@ template <> struct FftShape<double, 4> {
 struct MixFft { static constexpr int E = 2, MT = 256, MINB = 2; static constexpr bool MIX = true; };
 // Radix of the one-CTA and one-launch kernels, whose few CTAs are bound by latency (re_radix and
 // cplx_radix choose that of the launch-per-pass kernels).
-template <typename T> struct SmallFft : FftShape<T, 2> {};
+template <typename T> struct SmallFft : FftShape<T, sizeof(T) == 8 ? 1 : 2> {};
 template <typename T> struct BigFft { static constexpr int E = std::is_same<T, dfl>::value ? 3 : 2, EPT = 16, MT = 512, MINB = 1; static constexpr bool MIX = false; };
 
 // Radix-R DFT of v[0..R-1] in registers (forward, natural order in and out).
@@ -197,7 +198,7 @@ __device__ __forceinline__ void stage_ct(typename V2<T>::t* __restrict__ buf, in
                                          const typename V2<T>::t* __restrict__ stw) {
   typedef typename V2<T>::t C;
   constexpr int log2R = R == 16 ? 4 : (R == 8 ? 3 : (R == 4 ? 2 : 1));
-  constexpr int log2EPT = EPT == 16 ? 4 : (EPT == 8 ? 3 : 2);
+  constexpr int log2EPT = EPT == 16 ? 4 : (EPT == 8 ? 3 : (EPT == 4 ? 2 : 1));
   constexpr int PER = EPT / R;
   constexpr int LOG2TP = LOG2N - log2EPT;
   constexpr int nTP = 1 << LOG2TP;
@@ -294,7 +295,7 @@ __device__ __forceinline__ void stage_rt(typename V2<T>::t* __restrict__ buf, in
                                          const typename V2<T>::t* __restrict__ stw, int log2n, int log2ns) {
   typedef typename V2<T>::t C;
   constexpr int log2R = R == 16 ? 4 : (R == 8 ? 3 : (R == 4 ? 2 : 1));
-  constexpr int log2EPT = EPT == 16 ? 4 : (EPT == 8 ? 3 : 2);
+  constexpr int log2EPT = EPT == 16 ? 4 : (EPT == 8 ? 3 : (EPT == 4 ? 2 : 1));
   constexpr int PER = EPT / R;
   const int log2tp = log2n - log2EPT;
   const int ntp = 1 << log2tp;
