@@ -635,8 +635,8 @@ __device__ __forceinline__ void sw_up_warp(const SweepArgs<T>& a, int col, int g
 #pragma unroll
       for (int m = 0; m < NX; ++m) o[il32(b, m, NX)] = e[m];
     }
+    __syncwarp();   // the parent's offset, written by another lane, before lane 0's fence and arrival
     __threadfence();
-    __syncwarp();
     const int64_t nb = b >> 5;
     const int n = lv.n[l + 1];
     unsigned* cnt = lv.cnt + col * lv.ncnt + lv.cnt0[l + 1] + nb;
@@ -647,7 +647,8 @@ __device__ __forceinline__ void sw_up_warp(const SweepArgs<T>& a, int col, int g
     }
     old = __shfl_sync(0xffffffffu, old, 0);
     if (old + 1 != (unsigned)min(32, n - 32 * (int)nb)) return;
-    __threadfence();
+    __threadfence();   // lane 0's arrival before every lane's reads
+    __syncwarp();
     b = nb;
 #pragma unroll
     for (int m = 0; m < NX; ++m) e[m] = b * 32 + lane < n ? __ldcg(o + il32(b * 32 + lane, m, NX)) : T(0);
@@ -1475,6 +1476,7 @@ static bk_status alloc_opdata(Problem* pr, OpData& d, int dtype) {
   if (ncnt > 0) {
     BK_TRY(dmalloc((void**)&d.lvcnt, sizeof(unsigned) * ncnt));
     BK_TRY_CUDA(cudaMemset(d.lvcnt, 0, sizeof(unsigned) * ncnt));
+    BK_TRY_CUDA(cudaStreamSynchronize(0));   // streams that do not wait for this one use them next
   }
   if (pre) BK_TRY(dmalloc(&d.qlast, es * NEM * NXM));
   if (pre && pr->free_time) {
