@@ -160,6 +160,8 @@ __device__ bool last_block(unsigned* cnt) {
   return last;
 }
 
+// Bounded in FP64 by the FP64 pipe (one FMA per operand; n = 10.5e6, cold caches, us: |w|^2 46 -> 26, two
+// columns 63 -> 49 with the trees and registers below), in FP32 by memory.
 // out[i] = V_i . w (i < nv), FP64 sums: each block writes partial[b * nv + i] for its slice and
 // the last block to finish adds the partials of every column in block order (one launch, the
 // result independent of scheduling).
@@ -167,6 +169,9 @@ template <typename T>
 __device__ __forceinline__ void multidot_body(const T* __restrict__ V, int64_t ld, int nv, const T* __restrict__ w,
                                               int64_t n, double* __restrict__ partial, double* __restrict__ out,
                                               unsigned* __restrict__ cnt) {
+  // columns side by side: in FP64 4, whose 64 registers leave four blocks per SM (8 columns took 128; the
+  // pipe, not a second read of w, bounds them)
+  constexpr int G = sizeof(T) == 8 ? 4 : 8;
   __shared__ double red[8][8];
   // slices of a multiple of 4 elements, so that 16-byte loads start on a slice boundary
   const int64_t chunk = ((n + gridDim.x - 1) / gridDim.x + 3) & ~int64_t(3);
@@ -174,22 +179,22 @@ __device__ __forceinline__ void multidot_body(const T* __restrict__ V, int64_t l
   const int64_t hi = lo + chunk < n ? lo + chunk : n;
   const bool vec = ((reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(w) |
                      (uintptr_t)(ld * (int64_t)sizeof(T))) & 15) == 0;
-  for (int i0 = 0; i0 < nv; i0 += 8) {
-    const int ng = nv - i0 < 8 ? nv - i0 : 8;
+  for (int i0 = 0; i0 < nv; i0 += G) {
+    const int ng = nv - i0 < G ? nv - i0 : G;
     const T* Vg = V + (int64_t)i0 * ld;
-    double acc[8];
+    double acc[G];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.0;
+    for (int q = 0; q < G; ++q) acc[q] = 0.0;
     if (vec) {
       switch (ng) {
         case 1: dot_group_vec<T, 1>(Vg, ld, w, lo, hi, acc); break;
         case 2: dot_group_vec<T, 2>(Vg, ld, w, lo, hi, acc); break;
         case 3: dot_group_vec<T, 3>(Vg, ld, w, lo, hi, acc); break;
         case 4: dot_group_vec<T, 4>(Vg, ld, w, lo, hi, acc); break;
-        case 5: dot_group_vec<T, 5>(Vg, ld, w, lo, hi, acc); break;
-        case 6: dot_group_vec<T, 6>(Vg, ld, w, lo, hi, acc); break;
-        case 7: dot_group_vec<T, 7>(Vg, ld, w, lo, hi, acc); break;
-        default: dot_group_vec<T, 8>(Vg, ld, w, lo, hi, acc); break;
+        case 5: if constexpr (G >= 5) dot_group_vec<T, 5>(Vg, ld, w, lo, hi, acc); break;
+        case 6: if constexpr (G >= 6) dot_group_vec<T, 6>(Vg, ld, w, lo, hi, acc); break;
+        case 7: if constexpr (G >= 7) dot_group_vec<T, 7>(Vg, ld, w, lo, hi, acc); break;
+        default: if constexpr (G >= 8) dot_group_vec<T, 8>(Vg, ld, w, lo, hi, acc); break;
       }
     } else {
       switch (ng) {
@@ -197,14 +202,16 @@ __device__ __forceinline__ void multidot_body(const T* __restrict__ V, int64_t l
         case 2: dot_group<T, 2>(Vg, ld, w, lo, hi, acc); break;
         case 3: dot_group<T, 3>(Vg, ld, w, lo, hi, acc); break;
         case 4: dot_group<T, 4>(Vg, ld, w, lo, hi, acc); break;
-        case 5: dot_group<T, 5>(Vg, ld, w, lo, hi, acc); break;
-        case 6: dot_group<T, 6>(Vg, ld, w, lo, hi, acc); break;
-        case 7: dot_group<T, 7>(Vg, ld, w, lo, hi, acc); break;
-        default: dot_group<T, 8>(Vg, ld, w, lo, hi, acc); break;
+        case 5: if constexpr (G >= 5) dot_group<T, 5>(Vg, ld, w, lo, hi, acc); break;
+        case 6: if constexpr (G >= 6) dot_group<T, 6>(Vg, ld, w, lo, hi, acc); break;
+        case 7: if constexpr (G >= 7) dot_group<T, 7>(Vg, ld, w, lo, hi, acc); break;
+        default: if constexpr (G >= 8) dot_group<T, 8>(Vg, ld, w, lo, hi, acc); break;
       }
     }
+    // the group's own columns only: a tree over all 8 took 40 FP64 instructions per warp, 64 cycles each
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < G; ++q) {
+      if (q >= ng) break;
       double a = acc[q];
       for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
       if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][q] = a;
@@ -235,7 +242,7 @@ __device__ __forceinline__ void multidot_body(const T* __restrict__ V, int64_t l
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_multidot(const T* __restrict__ V, int64_t ld, int nv, const T* __restrict__ w,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 4 : 0) k_multidot(const T* __restrict__ V, int64_t ld, int nv, const T* __restrict__ w,
                                                   int64_t n, double* __restrict__ partial, double* __restrict__ out,
                                                   unsigned* __restrict__ cnt) {
   pdl_wait();
@@ -267,16 +274,71 @@ __device__ __forceinline__ void gm_first_pass(GmState* s, const double* __restri
   if (threadIdx.x == 0) s->need2 = w2[0] < 0.5 * h1[j + 1] ? 1 : 0;
 }
 
-// w <- alpha * w + cscale * sum_i c[i] V_i   (c on the device, FP64). With `partial`, each block
-// also writes the sum of squares of its slice of the new w and the last block to finish writes
-// their sum, |w|^2, to *sq_out (block order, as k_multidot) and, with `fin`, finishes the first
-// Gram-Schmidt pass (c is then h).
-template <typename T>
+// FP64 elements c = tid, tid + stride, ... (16 bytes each) of w <- w + sum_{i < nv} cs_i V_i; with SQ the
+// sum of their squares is added to sq. NV > 0: nv as a constant, two elements' loads in flight together.
+// Bounded by the FP64 pipe (one FMA per operand takes longer than its 8 bytes from HBM), so neither
+// the unit factor of w nor an unwanted square is multiplied: n = 10.5e6, nv = 1,
+// cold caches: 91 -> 49 us with the squares, 82 -> 36 us without.
+template <int NV, bool SQ>
+__device__ __forceinline__ void axpy_chunks(const double* __restrict__ V, int64_t ld, int nv, const double* cs, double2* w,
+                                          int64_t nc, double& sq) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t ld2 = ld >> 1;
+  const double2* V2 = reinterpret_cast<const double2*>(V);
+  const int m = NV > 0 ? NV : nv;
+  constexpr int U = NV > 0 ? 2 : 1;
+  int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  for (; c + (U - 1) * stride < nc; c += U * stride) {
+    double2 a[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) a[u] = w[c + u * stride];
+#pragma unroll
+    for (int i = 0; i < m; ++i) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const double2 v = V2[i * ld2 + c + u * stride];
+        a[u].x = fma(cs[i], v.x, a[u].x);
+        a[u].y = fma(cs[i], v.y, a[u].y);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      w[c + u * stride] = a[u];
+      if (SQ) sq = fma(a[u].y, a[u].y, fma(a[u].x, a[u].x, sq));
+    }
+  }
+  if (U > 1 && c < nc) {
+    double2 a = w[c];
+    for (int i = 0; i < m; ++i) {
+      const double2 v = V2[i * ld2 + c];
+      a.x = fma(cs[i], v.x, a.x);
+      a.y = fma(cs[i], v.y, a.y);
+    }
+    w[c] = a;
+    if (SQ) sq = fma(a.y, a.y, fma(a.x, a.x, sq));
+  }
+}
+template <bool SQ>
+__device__ __forceinline__ void axpy_nv(const double* __restrict__ V, int64_t ld, int nv, const double* cs, double2* w,
+                                             int64_t nc, double& sq) {
+  switch (nv) {
+    case 1: axpy_chunks<1, SQ>(V, ld, nv, cs, w, nc, sq); break;
+    case 2: axpy_chunks<2, SQ>(V, ld, nv, cs, w, nc, sq); break;
+    case 3: axpy_chunks<3, SQ>(V, ld, nv, cs, w, nc, sq); break;
+    default: axpy_chunks<0, SQ>(V, ld, nv, cs, w, nc, sq); break;
+  }
+}
+
+// w <- w + cscale * sum_i c[i] V_i   (c on the device, FP64). With SQ each block also writes the sum
+// of squares of its slice of the new w to `partial` and the last block to finish writes their sum,
+// |w|^2, to *sq_out (block order, as k_multidot) and, with `fin`, finishes the first Gram-Schmidt
+// pass (c is then h).
+template <typename T, bool SQ>
 __device__ __forceinline__ void multiaxpy_body(const T* __restrict__ V, int64_t ld, int nv,
                                                const double* __restrict__ c, double cscale, T* __restrict__ w,
-                                               double alpha, int64_t n, double* __restrict__ partial,
+                                               int64_t n, double* __restrict__ partial,
                                                double* __restrict__ sq_out, unsigned* __restrict__ cnt,
-                                               GmState* fin = nullptr) {
+                                               GmState* fin) {
   __shared__ double cs[MAXM + 1];
   __shared__ float cs32[MAXM + 1];
   __shared__ double red[8];
@@ -297,30 +359,14 @@ __device__ __forceinline__ void multiaxpy_body(const T* __restrict__ V, int64_t 
     const int64_t nc = n / VW;
     VT* wv = reinterpret_cast<VT*>(w);
     if constexpr (sizeof(T) == 8) {
-      for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc; c += stride) {
-        const VT wk = wv[c];
-        double ax = alpha == 0.0 ? 0.0 : alpha * wk.x, ay = alpha == 0.0 ? 0.0 : alpha * wk.y;
-        for (int i = 0; i < nv; ++i) {
-          const VT v = reinterpret_cast<const VT*>(V + (int64_t)i * ld)[c];
-          ax += cs[i] * v.x;
-          ay += cs[i] * v.y;
-        }
-        VT o;
-        o.x = ax;
-        o.y = ay;
-        wv[c] = o;
-        sq += ax * ax;
-        sq += ay * ay;
-      }
+      axpy_nv<SQ>(V, ld, nv, cs, wv, nc, sq);
     } else {
-      const float al = (float)alpha;
       int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
       while (c < nc) {
         float s32 = 0.f;
         for (int it = 0; it < RUN32 / VW && c < nc; ++it, c += stride) {
           const VT wk = wv[c];
-          float a0 = alpha == 0.0 ? 0.f : al * wk.x, a1 = alpha == 0.0 ? 0.f : al * wk.y;
-          float a2 = alpha == 0.0 ? 0.f : al * wk.z, a3 = alpha == 0.0 ? 0.f : al * wk.w;
+          float a0 = wk.x, a1 = wk.y, a2 = wk.z, a3 = wk.w;
           for (int i = 0; i < nv; ++i) {
             const VT v = reinterpret_cast<const VT*>(V + (int64_t)i * ld)[c];
             a0 = fmaf(cs32[i], v.x, a0);
@@ -334,24 +380,21 @@ __device__ __forceinline__ void multiaxpy_body(const T* __restrict__ V, int64_t 
           o.z = a2;
           o.w = a3;
           wv[c] = o;
-          s32 = fmaf(a0, a0, s32);
-          s32 = fmaf(a1, a1, s32);
-          s32 = fmaf(a2, a2, s32);
-          s32 = fmaf(a3, a3, s32);
+          if (SQ) s32 = fmaf(a3, a3, fmaf(a2, a2, fmaf(a1, a1, fmaf(a0, a0, s32))));
         }
-        sq += (double)s32;
+        if (SQ) sq += (double)s32;
       }
     }
     // the last n mod VW elements one by one
     for (int64_t k = nc * VW + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += stride) {
-      T a = alpha == 0.0 ? T(0) : T(alpha) * w[k];
+      T a = w[k];
       for (int i = 0; i < nv; ++i) a += (sizeof(T) == 8 ? T(cs[i]) : T(cs32[i])) * V[(int64_t)i * ld + k];
       w[k] = a;
-      sq += (double)a * (double)a;
+      if (SQ) sq += (double)a * (double)a;
     }
   } else if constexpr (sizeof(T) == 8) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += stride) {
-      double a = alpha == 0.0 ? 0.0 : alpha * w[k];
+      double a = w[k];
       int i = 0;
       for (; i + 4 <= nv; i += 4) {
         const double v0 = V[(int64_t)i * ld + k], v1 = V[(int64_t)(i + 1) * ld + k];
@@ -363,15 +406,14 @@ __device__ __forceinline__ void multiaxpy_body(const T* __restrict__ V, int64_t 
       }
       for (; i < nv; ++i) a += cs[i] * V[(int64_t)i * ld + k];
       w[k] = a;
-      sq += a * a;
+      if (SQ) sq += a * a;
     }
   } else {
-    const float al = (float)alpha;
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     while (k < n) {
       float s32 = 0.f;
       for (int it = 0; it < RUN32 && k < n; ++it, k += stride) {
-        float a = alpha == 0.0 ? 0.f : al * (float)w[k];
+        float a = (float)w[k];
         int i = 0;
         for (; i + 4 <= nv; i += 4) {
           const float v0 = V[(int64_t)i * ld + k], v1 = V[(int64_t)(i + 1) * ld + k];
@@ -383,12 +425,12 @@ __device__ __forceinline__ void multiaxpy_body(const T* __restrict__ V, int64_t 
         }
         for (; i < nv; ++i) a = fmaf(cs32[i], (float)V[(int64_t)i * ld + k], a);
         w[k] = (T)a;
-        s32 = fmaf(a, a, s32);
+        if (SQ) s32 = fmaf(a, a, s32);
       }
-      sq += (double)s32;
+      if (SQ) sq += (double)s32;
     }
   }
-  if (partial) {
+  if constexpr (SQ) {
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
     __syncthreads();
@@ -402,16 +444,6 @@ __device__ __forceinline__ void multiaxpy_body(const T* __restrict__ V, int64_t 
       if (fin) gm_first_pass(fin, c, sq_out);
     }
   }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_multiaxpy(const T* __restrict__ V, int64_t ld, int nv,
-                                                   const double* __restrict__ c, double cscale, T* __restrict__ w,
-                                                   double alpha, int64_t n, double* __restrict__ partial,
-                                                   double* __restrict__ sq_out = nullptr,
-                                                   unsigned* __restrict__ cnt = nullptr) {
-  pdl_wait();
-  multiaxpy_body<T>(V, ld, nv, c, cscale, w, alpha, n, partial, sq_out, cnt);
 }
 
 __global__ void k_gm_init(GmState* s, double beta, double target, int jmax, int m) {
@@ -432,7 +464,7 @@ __global__ void k_gm_init(GmState* s, double beta, double target, int jmax, int 
 
 // V_i . w for i < j + add, w = V_{j + woff} (j from the state); skipped when *gate == 0.
 template <typename T>
-__global__ void __launch_bounds__(256) k_multidot_s(const T* __restrict__ V, int64_t ld, int add, int woff,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 4 : 0) k_multidot_s(const T* __restrict__ V, int64_t ld, int add, int woff,
                                                     const GmState* __restrict__ s, const int* __restrict__ gate,
                                                     int64_t n, double* __restrict__ partial, double* __restrict__ out,
                                                     unsigned* __restrict__ cnt) {
@@ -442,20 +474,20 @@ __global__ void __launch_bounds__(256) k_multidot_s(const T* __restrict__ V, int
   multidot_body<T>(V, ld, j + add, V + (int64_t)(j + woff) * ld, n, partial, out, cnt);
 }
 
-// w <- alpha w + cscale sum_{i < j + add} c_i V_i with w = V_{j + woff} (woff >= 0) or the
+// w <- w + cscale sum_{i < j + add} c_i V_i with w = V_{j + woff} (woff >= 0) or the
 // fixed vector x (woff < 0); skipped when *gate == 0.
-template <typename T>
+template <typename T, bool SQ>
 __global__ void __launch_bounds__(256) k_multiaxpy_s(const T* __restrict__ V, int64_t ld, int add, int woff,
                                                      T* __restrict__ x, const GmState* __restrict__ s,
                                                      const int* __restrict__ gate, const double* __restrict__ c,
-                                                     double cscale, double alpha, int64_t n,
+                                                     double cscale, int64_t n,
                                                      double* __restrict__ partial, double* __restrict__ sq_out,
                                                      unsigned* __restrict__ cnt, GmState* fin) {
   pdl_wait();
   if (gate && *gate == 0) return;
   const int j = s->j;
   T* w = woff >= 0 ? const_cast<T*>(V) + (int64_t)(j + woff) * ld : x;
-  multiaxpy_body<T>(V, ld, j + add, c, cscale, w, alpha, n, partial, sq_out, cnt, fin);
+  multiaxpy_body<T, SQ>(V, ld, j + add, c, cscale, w, n, partial, sq_out, cnt, fin);
 }
 
 // Column j finished (one thread): the second pass's corrections, |w|, the Givens rotations of the
@@ -510,8 +542,22 @@ __global__ void __launch_bounds__(256) k_gm_finish(T* __restrict__ V, int64_t ld
   if (hs > 0.0) {
     T* v = V + (int64_t)(s->j + 1) * ld;
     const T inv = (T)is;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-      v[k] = v[k] * inv;
+    typedef typename Vec16<T>::t VT;
+    constexpr int VW = Vec16<T>::n;   // the basis vectors are 16-byte aligned (n = 10.5e6 in FP64 45 -> 38 us)
+    const int64_t nc = n / VW, tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    VT* vv = reinterpret_cast<VT*>(v);
+#pragma unroll 2
+    for (int64_t c = tid; c < nc; c += (int64_t)gridDim.x * blockDim.x) {
+      VT a = vv[c];
+      a.x *= inv;
+      a.y *= inv;
+      if constexpr (VW == 4) {
+        a.z *= inv;
+        a.w *= inv;
+      }
+      vv[c] = a;
+    }
+    if (tid < n - nc * VW) v[nc * VW + tid] *= inv;
   }
   if (last_block(cnt) && threadIdx.x == 0) gm_column(s, h2, hs, cond, in_graph);
 }
@@ -671,10 +717,10 @@ static bk_status arnoldi_step(const GmCtx<T>& c, int jh, bool graph, cudaGraphCo
   // |w|^2; the second pass runs (its kernels do work) only when the first one's end asked for it.
   double* w2 = c.h2 + (MAXM + 1);
   BK_TRY(launch(k_multidot_s<T>, dot_blocks(n), 256, 0, st, c.V, ld, 2, 1, c.gs, nullptr, n, c.partial, c.h1, c.cnt));
-  BK_TRY(launch(k_multiaxpy_s<T>, dot_blocks(n), 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, nullptr, c.h1, -1.0, 1.0, n, c.partial,
+  BK_TRY(launch(k_multiaxpy_s<T, true>, dot_blocks(n), 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, nullptr, c.h1, -1.0, n, c.partial,
                                                w2, c.cnt + 1, c.gs));
   BK_TRY(launch(k_multidot_s<T>, dot_blocks(n), 256, 0, st, c.V, ld, 1, 1, c.gs, &c.gs->need2, n, c.partial, c.h2, c.cnt));
-  BK_TRY(launch(k_multiaxpy_s<T>, dot_blocks(n), 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, &c.gs->need2, c.h2, -1.0, 1.0, n,
+  BK_TRY(launch(k_multiaxpy_s<T, true>, dot_blocks(n), 256, 0, st, c.V, ld, 1, 1, nullptr, c.gs, &c.gs->need2, c.h2, -1.0, n,
                                                c.partial, w2, c.cnt + 1, nullptr));
   BK_TRY(launch(k_gm_finish<T>, c.g, 256, 0, st, c.V, ld, n, c.gs, c.h2, w2, c.cnt + 2, cond, graph ? 1 : 0));
   return BK_OK;
@@ -939,11 +985,11 @@ static bk_status gmres_impl(Problem* pr, OpData& d, int op, const T* b, T* x, co
     }
     // x += Z y (flexible form; Z = V without preconditioning), y = H^{-1} g on the device
     BK_TRY(launch(k_gm_solve, 1, 32, 0, st, gs));
-    BK_TRY(launch(k_multiaxpy_s<T>, g, 256, 0, st, o.use_precond ? Zb : V, ld, 0, -1, x, gs, nullptr, gs->y, 1.0, 1.0, n,
+    BK_TRY(launch(k_multiaxpy_s<T, false>, g, 256, 0, st, o.use_precond ? Zb : V, ld, 0, -1, x, gs, nullptr, gs->y, 1.0, n,
                                         nullptr, nullptr, nullptr, nullptr));
     if (aux) {
-      BK_TRY(launch(k_multiaxpy_s<double>, grid_for(aux->n), 256, 0, st, aux->T, aux->ld, 0, -1, aux->Td, gs, nullptr, gs->y,
-                                                              1.0, 1.0, aux->n, nullptr, nullptr, nullptr, nullptr));
+      BK_TRY(launch(k_multiaxpy_s<double, false>, grid_for(aux->n), 256, 0, st, aux->T, aux->ld, 0, -1, aux->Td, gs, nullptr, gs->y,
+                                                              1.0, aux->n, nullptr, nullptr, nullptr, nullptr));
     }
     if (gg) {
       BK_TRY_CUDA(cudaMemcpyAsync(hostbuf, gs, sizeof(GmHead), cudaMemcpyDeviceToHost, st));
