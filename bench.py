@@ -44,6 +44,9 @@ FALLBACK_HBM_GBS = 6800.0
 # FP64 FMA rate of GB300: 152 SMs x 2 FP64 FMA / clk x 2 flop x 2.07 GHz = 1.26 TFLOP/s
 # (nominal 1.25 TFLOP/s); the transforms of the FP64 path are bound by it, not by HBM.
 FP64_PEAK_TFLOPS = 1.25
+# From N = 2^18 they run in double-float arithmetic: about 10 FP32 instructions per operation (11 per
+# sum, 8 per product), issued at 37.4e12 lane instructions/s (the measured 74.8 TFLOP/s of FP32 FMAs).
+DOUBLE_FLOAT_PEAK_TFLOPS = 3.74
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12   # 80.5 TFLOP/s nominal FFMA
 
 
@@ -277,7 +280,7 @@ def run_newton(args, rank, world, dist):
 
 
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
-TRANSFORM_SOURCES = ("bk_birkhoff.cu", "bk_fft.cuh", "bk_plan.cuh", "bk_common.cuh")
+TRANSFORM_SOURCES = ("bk_birkhoff.cu", "bk_fft.cuh", "bk_dct.cuh", "bk_plan.cuh", "bk_common.cuh")
 
 
 def transform_source_hash():
@@ -854,8 +857,13 @@ def main():
     # roofline of the dominant unit: the 4-component Birkhoff apply (four transform passes)
     ams, abytes, aflops = measure_apply(N, dt)
     if dt == torch.float64:
-        peak, unit, achieved = FP64_PEAK_TFLOPS, "TFLOP/s", aflops / ams / 1e9
-        bound = "alu"
+        bound, unit, achieved = "alu", "TFLOP/s", aflops / ams / 1e9
+        from paper_2509_01855_gb300 import api
+        pl = api.Plan(N, n_comp=4, dtype=dt, t0=0.0, tf=TF)
+        df = pl.f64_mode() == 1
+        pl.close()
+        peak, alu = ((DOUBLE_FLOAT_PEAK_TFLOPS, "double-float operations at the measured FP32 rate (10 FP32 instructions each)") if df
+                     else (FP64_PEAK_TFLOPS, "FP64 FMA nominal 1.25 TFLOP/s (2 FP64 FMA/clk/SM)"))
     else:
         peak, unit, achieved = hbm_peak, "GB/s", abytes / ams / 1e6
         bound = "hbm"
@@ -864,7 +872,7 @@ def main():
                         "traffic_source": "profiles/traffic.json",
                         "kernel": "birkhoff_apply N=2^%d x4 components (%s)" % (args.N, dtype_name),
                         "algorithmic": {"bytes": abytes, "flops": aflops},
-                        "peak_source": ("FP64 FMA nominal 1.25 TFLOP/s (2 FP64 FMA/clk/SM)" if bound == "alu"
+                        "peak_source": (alu if bound == "alu"
                                         else "MEASURED_PEAKS.json hbm_gbs (%s)" % peak_kind)}
     line["apply"] = {"ms": ams, "gbs": abytes / ams / 1e6, "tflops": aflops / ams / 1e9, "N": N,
                      "n_comp": 4, "dtype": dtype_name}

@@ -51,7 +51,7 @@ namespace bk {
 
 // The kernels compute in T and keep their internal real vectors (the stage buffers between the
 // two DCTs) in T; the caller's vectors are User<T> (binary64 for double-float arithmetic, whose
-// products convert the input once in k_to_arith and the output in the last epilogue).
+// products convert the input in the first pass's loads and the output in the last pass's stores).
 template <typename T> using Us = typename User<T>::t;
 // Conversion of a stored element S to the arithmetic type T and back (identity when S == T).
 template <typename T, typename S> struct Cv;
@@ -921,8 +921,6 @@ static int round_threads(int64_t t) {  // whole warps
 
 static constexpr size_t FOURSTEP_SMEM_BUDGET = 192 * 1024;
 
-// Complex elements one four-step CTA transforms (its tile: NB columns of N1 in pass A, 2P rows
-// of N2 in pass B; 16 per thread). BK_FOURSTEP_ELEMS overrides the default (tuning).
 static int sm_count() {
   static int n = 0;
   if (n == 0) {
@@ -933,7 +931,7 @@ static int sm_count() {
   return n;
 }
 
-// Complex elements per four-step CTA (16 per thread): enough CTAs for two per SM over the plan's
+// Complex elements per CTA of a pass: enough CTAs for two per SM over the plan's
 // vectors, at least one column of N1 and one row pair of 2 N2, at most the thread cap. Small
 // transforms thus run many one-warp CTAs instead of a few full ones (at 2^14 x 4 components the
 // full-size tiles gave 16 CTAs per pass). BK_FOURSTEP_ELEMS fixes it (tuning).
@@ -1279,8 +1277,8 @@ extern template bk_status blue_spectrum<float>(Plan* p, cudaStream_t st);
 // FP64 plans of N >= 2^18 compute their transforms in double-float arithmetic (bk_df.cuh) unless
 // switched off: bk_set_f64_transform(0) for plans created afterwards, or the environment variable
 // BK_F64_DF=0 (read at plan creation); bk_set_f64_transform(1) extends it to every FP64 plan with
-// N >= 256. Measured products (4 components, warm, us, FP64 / double-float): 2^18 206 / 122, 2^20
-// 736 / 363; below 2^18 the passes are latency-bound and the double-float instructions lengthen them.
+// N >= 256. Measured products (4 components, warm, us, FP64 / double-float): 2^17 103 / 54, 2^18 195 /
+// 79, 2^20 705 / 225. Below 2^18 the plans keep binary64's accuracy (relative errors 4e-16 against 8e-15).
 #ifndef BK_TRANSFORM_KERNEL_UNIT
 static std::atomic<int> g_f64_df{-1};
 static bool f64_df_default(int64_t N) {
@@ -1826,7 +1824,8 @@ static bk_status launch_passes_batch(const Plan* const* ps, const void* const* v
 
 // fs_*: the four-step plans of radix 4. With launch-per-pass plans among them, FP32 one-launch plans
 // join those launches (the same radix and arithmetic, so the same results; beside the longer plans
-// they take no time of their own: sizes 2^8..2^16 of 4 FP32 components 79 -> 53 us in all).
+// they take no time of their own: sizes 2^8..2^16 of 4 FP32 components, before dependent launches,
+// 79 -> 53 us in all).
 template <typename T>
 bk_status apply_batch_impl(const Plan* const* small_p, const void* const* small_v, void* const* small_o,
                            const int* small_n, int nsmall, const Plan* const* fs_p, const void* const* fs_v,
