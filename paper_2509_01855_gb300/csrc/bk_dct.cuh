@@ -252,7 +252,7 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
 // Epilogue kinds of pass B:
 //   EP_STORE     : stage[k] = R_k / N                        (after the first DCT, forward)
 //   EP_STORE_TRN : stage[k] = (R_k - R_0) / (4k), 0 at k = 0 (after the first DCT, transpose)
-//   EP_FWD_OUT   : out[k] = s (R_k - R_0)                    (after the second DCT, forward)
+//   EP_FWD_OUT   : out[k] = s (R_k - R_0), 0 at k = 0        (after the second DCT, forward)
 //   EP_TRN_OUT   : out[k] = (s/N) W_k R_k                    (after the second DCT, transpose)
 // Pass B of row pairs [tile P, tile P + P) of one vector.
 template <typename T, int E, bool CG, typename F, typename S>
@@ -329,7 +329,7 @@ __device__ __forceinline__ void re_passB(const ReArgs<T>& g, int tile, int P, in
   auto val = [&](T v, int k, T rk) {
     if (E == EP_STORE) return v * invN;
     if (E == EP_STORE_TRN) return (v - Y0) * rk;
-    if (E == EP_FWD_OUT) return s * (v - Y0);
+    if (E == EP_FWD_OUT) return s * (v - (k == 0 ? v : Y0));   // Y0's sum rounds apart from the row's R_0
     return (k == 0 || k == N ? sN : T(2) * sN) * v;
   };
   if (j0 < step && (mid || r < (N1 >> 1))) {
