@@ -125,7 +125,8 @@ bk_status birkhoff_apply(const bk_plan* plan, const void* v, void* out, int batc
  *   plans, v, out, batch   host arrays of `count` entries (1 <= count <= 4096); v[i], out[i]
  *                          device arrays as for birkhoff_apply; v[i] == out[i] is allowed, but
  *                          different entries' vectors must not overlap
- * A four-step plan may appear only once per call (it owns the scratch its passes use); all
+ * A four-step plan in the shared launches may appear only once per call (it owns the scratch its
+ * passes use), except that later entries of an FP64 plan with N >= 2^17 run their own launches; all
  * plans must have the same dtype. BK_ERR_ARG otherwise, before any work is queued. */
 bk_status birkhoff_apply_batch(const bk_plan* const* plans, const void* const* v, void* const* out,
                                const int* batch, int count, int trans, void* stream);

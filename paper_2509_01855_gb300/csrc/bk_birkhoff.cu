@@ -1951,7 +1951,9 @@ bk_status plan_apply(const Plan* p, const void* v, void* out, int batch, bool tr
 
 // Products of several plans of one precision, N free per plan: small plans in one launch, four-step
 // plans of radix 4 in another, or in one launch per pass where one of them needs it (each per
-// BATCH_MAX plans), every other plan (dense, Bluestein, radix 8 and 16) by its own launches.
+// BATCH_MAX plans), every other plan (dense, Bluestein, radix 8 and 16) by its own launches. The shared
+// launches use a four-step plan's scratch once, so a plan comes in them once; the later entries of an
+// FP64 plan of N >= 2^17 follow as launches of their own, those of a shorter one are refused.
 bk_status plan_apply_batch(const Plan* const* ps, const void* const* v, void* const* out, const int* batch, int count,
                            bool trans, cudaStream_t st) {
   BK_ARG(ps != nullptr && v != nullptr && out != nullptr && batch != nullptr, "NULL argument");
@@ -1977,7 +1979,12 @@ bk_status plan_apply_batch(const Plan* const* ps, const void* const* v, void* co
     } else if (p->small) {
       sp.push_back(p); sv.push_back(v[i]); so.push_back(out[i]); sn.push_back(nv);
     } else {
-      for (const Plan* q : fp) BK_ARG(q != p, "entry %d: a four-step plan may appear once per batch (its scratch)", i);
+      const bool again = std::find(fp.begin(), fp.end(), p) != fp.end();
+      if (again && dtype == BK_F64 && p->N >= (int64_t(1) << 17)) {   // as the double-float plans of that size
+        op.push_back(p); ov.push_back(v[i]); oo.push_back(out[i]); on.push_back(nv);
+        continue;
+      }
+      BK_ARG(!again, "entry %d: a four-step plan may appear once per batch (its scratch)", i);
       fp.push_back(p); fv.push_back(v[i]); fo.push_back(out[i]); fn.push_back(nv);
     }
   }
