@@ -82,7 +82,9 @@ uint64_t bk_launch_count(void);
  *              (about 4-8x the work of the nearest power of two)
  *   n_comp     components per batch item (>= 1)
  *   max_batch  largest `batch` later passed to birkhoff_apply / birkhoff_apply_T (>= 1); the
- *              plan's scratch is sized for max_batch * n_comp vectors
+ *              plan's scratch is sized for max_batch * n_comp vectors and serves one call at a
+ *              time. Products need none, and may overlap on any streams and threads, at powers
+ *              of two N <= 256 (BK_F64 in binary64) and N <= 4096 (BK_F32), not dense
  *   dtype      arithmetic and storage type
  *   t0, tf     time interval, tf != t0 (s = (tf - t0) / 2 scales B)
  *   pitch      distance in elements between component blocks; 0 = default (L rounded up to

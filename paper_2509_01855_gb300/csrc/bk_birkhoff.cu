@@ -893,7 +893,7 @@ static bk_status compute_weights(Plan* p, cudaStream_t st) {
 
 // Largest N run by the single-CTA kernel (one CTA per vector): 256 in FP64, whose single CTA runs
 // on one SM's FP64 pipe, 2048 in FP32. Measured (4 components, us per product, one CTA / cluster): FP64
-// 2^8 12.0 / 18.1, 2^9 19.8 / 18.2; FP32 2^11 10.2 / 11.6, 2^12 14.3 / 12.9. BK_SMALL_MAX_LOG2
+// 2^8 12.0 / 18.1, 2^9 19.8 / 18.2; FP32 2^11 10.2 / 11.6, 2^12 14.3 / 13.8 (transposed 14.6 / 13.9). BK_SMALL_MAX_LOG2
 // overrides it for tuning (at least 2^4; at most 512 in FP64, 4096 in FP32). The four-step kernels
 // need N >= 128.
 static int small_default(int dtype) { return dtype == BK_F64 ? 256 : 2048; }
@@ -920,6 +920,7 @@ static int round_threads(int64_t t) {  // whole warps
 }
 
 static constexpr size_t FOURSTEP_SMEM_BUDGET = 192 * 1024;
+static size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 static int sm_count() {
   static int n = 0;
@@ -953,13 +954,14 @@ static int fourstep_elems(int dtype, int64_t n, int nvec, int N1, int N2, int Ef
 // Whether the four passes run as a launch each instead of as one cluster launch: from 2^13 on, and in FP64
 // from 2^12 with more than 8 vectors, whose sixteen CTAs per vector then share FP64 pipes. Measured
 // (us per product, cluster / launch per pass): FP64, 4 components, 2^11 20.5 / 24.5, 2^12 23.8 / 31.1, 2^13 31.7 /
-// 32.1, 2^14 47.0 / 34.2; 16 components 2^10 21.6 / 25.2, 2^12 36.4 / 30.8; FP32 2^12 12.9 / 15.5,
-// 2^13 17.1 / 15.5, 2^14 20.5 / 16.5. BK_SPLIT_MIN_LOG2 sets the border for tuning.
+// 32.1, 2^14 47.0 / 34.2; 16 components 2^10 21.6 / 25.2, 2^12 36.4 / 30.8; FP32 2^12 13.8 / 15.5,
+// 2^13 17.1 / 15.5, 2^14 20.5 / 16.5 (2^13 and 2^14 with the exchange in global memory, where 2^12 took 12.9). BK_SPLIT_MIN_LOG2 sets the border for tuning.
 static bool split_passes(int dtype, int64_t N, int nvec) {
   const char* e = getenv("BK_SPLIT_MIN_LOG2");
   if (e) {
     const long v = atol(e);
-    if (v >= 7 && v <= 30) return ilog2(N) >= std::min((int)v, 2 * CL_MAXLOG2);
+    // FP32 one-launch plans keep their exchange area in shared memory: N <= 2^13
+    if (v >= 7 && v <= 30) return ilog2(N) >= std::min((int)v, dtype == BK_F32 ? 14 : 2 * CL_MAXLOG2);
   }
   return N >= 8192 || (dtype == BK_F64 && N >= 4096 && nvec > 8);
 }
@@ -1028,6 +1030,17 @@ static void re_factors(FourStep& f, int64_t N) {
   f.n = 2 * N;
   f.N1 = 1 << (l / 2);
   f.N2 = 1 << (l - l / 2);
+}
+
+// Scratch of the passes of nvec FP32 vectors: A, the stage buffer and the shares of R_0. A launch-per-pass
+// plan of radix 4 keeps that of up to GUEST_VECTORS vectors of N = 4096 for the one-launch plans that
+// join its launches in a batch; its own scratch serves one call at a time anyway.
+static constexpr int GUEST_VECTORS = 64;
+static size_t re_scratch_f32(int64_t N, int64_t nvec) {
+  FourStep f;
+  re_factors(f, N);
+  return align256(2 * sizeof(float) * (size_t)f.a_len() * nvec) + align256(sizeof(float) * (size_t)(N + 2) * nvec) +
+         align256(sizeof(float) * (size_t)f.pairs() * nvec);
 }
 
 static bool re_big(const FourStep& f, int dtype) { return dtype == BK_F64 && f.N2 > 4096; }
@@ -1150,6 +1163,13 @@ static bk_status configure_cluster(Plan* p) {
   f.bsB = re_stride(p->dtype, f.N2, f.P);
   const size_t csz = 2 * dtype_size(p->dtype);
   p->csmem = csz * (size_t)(std::max(f.NB * f.bsA, f.P * f.bsB) + stage_tw_len(ilog2(f.N1), e) + stage_tw_len(ilog2(f.N2), e));
+  if (p->dtype == BK_F32) {   // the exchange area: rows of A that this CTA's pass B reads, stage block, shares
+    const int tiles = ((f.N1 / 4 + f.P) / f.P + p->csize - 1) / p->csize;
+    p->cex = (int)align256(p->csmem);
+    p->cexY = p->cex + (int)align256(csz * (size_t)tiles * f.P * 2 * f.RS());
+    p->cexP = p->cexY + (int)align256(sizeof(float) * (size_t)(p->N / p->csize + 2));
+    p->csmem = p->cexP + align256(sizeof(float) * (size_t)f.pairs());
+  }
   p->cthr = std::max(128, round_threads(std::max(f.NB * f.N1, f.P * f.N2) / ept));
   if (p->csmem > FOURSTEP_SMEM_BUDGET || p->cthr > maxthr) {
     set_error("cluster configuration failed for N=%lld", (long long)p->N);
@@ -1466,9 +1486,15 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
       if ((st_ = fourstep_shapes(p, 0)) != BK_OK) break;
       const int64_t nvec = (int64_t)n_comp * max_batch;
       const size_t es = dtype_size(dtype);
-      if ((st_ = dmalloc(&p->scrA, 2 * es * (size_t)p->fs.a_len() * nvec)) != BK_OK) break;
-      if ((st_ = dmalloc(&p->scrY, es * (size_t)(N + 2) * nvec)) != BK_OK) break;
-      if ((st_ = dmalloc(&p->part, es * (size_t)p->fs.pairs() * nvec)) != BK_OK) break;
+      if (p->split || dtype == BK_F64) {   // FP32 one-launch plans exchange in shared memory
+        if ((st_ = dmalloc(&p->scrA, 2 * es * (size_t)p->fs.a_len() * nvec)) != BK_OK) break;
+        if ((st_ = dmalloc(&p->scrY, es * (size_t)(N + 2) * nvec)) != BK_OK) break;
+        if ((st_ = dmalloc(&p->part, es * (size_t)p->fs.pairs() * nvec)) != BK_OK) break;
+      }
+      if (p->split && dtype == BK_F32 && p->fe == 2) {
+        p->guest_bytes = (size_t)std::min<int64_t>(nvec, GUEST_VECTORS) * re_scratch_f32(4096, 1);
+        if ((st_ = dmalloc(&p->guest, p->guest_bytes)) != BK_OK) break;
+      }
     }
     st_ = dtype == BK_F64 ? (p->df ? build_tables<dfl>(p, st) : build_tables<double>(p, st)) : build_tables<float>(p, st);
     if (st_ != BK_OK) break;
@@ -1516,6 +1542,7 @@ void plan_destroy(Plan* p) {
   dfree(p->scrY);
   dfree(p->scrG);
   dfree(p->part);
+  dfree(p->guest);
   dfree(p->t_nodes);
   dfree(p->dA[0]);
   dfree(p->dA[1]);
@@ -1669,6 +1696,10 @@ static ReJob<T> re_job(const Plan* p, const void* in, void* out, int nvec, T s) 
   J.P = p->fs.P;
   J.bsB = p->fs.bsB;
   J.nvec = nvec;
+  J.ex = p->cex;
+  J.exY = p->cexY;
+  J.exP = p->cexP;
+  J.csz = p->csize;
   return J;
 }
 
@@ -1786,10 +1817,11 @@ static bk_status launch_fourstep_batch(const Plan* const* ps, const void* const*
   return BK_OK;
 }
 
-// Four-step plans of radix 4 in the launch-per-pass form, one launch per pass for all of them.
+// Four-step plans of radix 4 in the launch-per-pass form, one launch per pass for all of them. guest[i]:
+// scratch for entry i when its plan has none of its own (FP32 one-launch plans), else null.
 template <typename T, bool TRANS>
 static bk_status launch_passes_batch(const Plan* const* ps, const void* const* vin, void* const* vout, const int* nv,
-                                     int n, cudaStream_t st) {
+                                     unsigned char* const* guest, int n, cudaStream_t st) {
   typedef FftShape<T, 2> F;
   for (int c0 = 0; c0 < n; c0 += BATCH_MAX) {
     Batch<ReJob<T>> a, b;
@@ -1801,16 +1833,25 @@ static bk_status launch_passes_batch(const Plan* const* ps, const void* const* v
     for (int q = 0; q < a.njob; ++q) {
       const Plan* p = ps[c0 + q];
       const FourStep& f = p->fs;
-      a.j[q] = b.j[q] = re_job<T>(p, vin[c0 + q], vout[c0 + q], nv[c0 + q], (T)p->s);
+      ReJob<T>& J = a.j[q];
+      J = re_job<T>(p, vin[c0 + q], vout[c0 + q], nv[c0 + q], (T)p->s);
+      if (guest[c0 + q]) {   // laid out as re_scratch_f32 counts it
+        unsigned char* m = guest[c0 + q];
+        J.A = reinterpret_cast<typename V2<T>::t*>(m);
+        m += align256(2 * sizeof(T) * (size_t)J.astride * J.nvec);
+        J.Y = reinterpret_cast<T*>(m);
+        J.part = reinterpret_cast<T*>(m + align256(sizeof(T) * (size_t)J.ystride * J.nvec));
+      }
+      b.j[q] = J;
       a.start[q] = ca;
       b.start[q] = cb;
       ca += nv[c0 + q] * ((f.pairs() + f.NB - 1) / f.NB);
       cb += nv[c0 + q] * ((f.N1 / 4 + f.P) / f.P);
-      // a one-launch plan's shared memory and threads hold either of its passes' tiles
+      // a one-launch plan's threads and shared memory before its exchange area hold either pass's tiles
       thrA = std::max(thrA, p->split ? f.thrA : p->cthr);
       thrB = std::max(thrB, p->split ? f.thrB : p->cthr);
-      smA = std::max(smA, p->split ? f.smemA : p->csmem);
-      smB = std::max(smB, p->split ? f.smemB : p->csmem);
+      smA = std::max(smA, p->split ? f.smemA : (size_t)p->cex);
+      smB = std::max(smB, p->split ? f.smemB : (size_t)p->cex);
     }
     a.start[a.njob] = ca;
     b.start[b.njob] = cb;
@@ -1823,36 +1864,47 @@ static bk_status launch_passes_batch(const Plan* const* ps, const void* const* v
 }
 
 // fs_*: the four-step plans of radix 4. With launch-per-pass plans among them, FP32 one-launch plans
-// join those launches (the same radix and arithmetic, so the same results; beside the longer plans
-// they take no time of their own: sizes 2^8..2^16 of 4 FP32 components, before dependent launches,
-// 79 -> 53 us in all).
+// join those launches on scratch that these plans lend (the same radix and arithmetic, so the same
+// results; beside the longer plans they take no time of their own: sizes 2^8..2^16 of 4 FP32
+// components, before dependent launches, 79 -> 53 us in all); those that find none left, and the FP64
+// ones, of another radix, take their one launch.
 template <typename T>
 bk_status apply_batch_impl(const Plan* const* small_p, const void* const* small_v, void* const* small_o,
                            const int* small_n, int nsmall, const Plan* const* fs_p, const void* const* fs_v,
                            void* const* fs_o, const int* fs_n, int nfs, bool trans, cudaStream_t st) {
   if (nsmall > 0) BK_TRY(launch_small_batch<T>(small_p, small_v, small_o, small_n, nsmall, trans, st));
-  if (nfs == 0) return BK_OK;
-  bool split = false;
-  for (int i = 0; i < nfs; ++i) split = split || fs_p[i]->split;
-  if (!split) return launch_fourstep_batch<T>(fs_p, fs_v, fs_o, fs_n, nfs, trans, st);
-  auto passes = [&](const Plan* const* p, const void* const* v, void* const* o, const int* nv, int n) -> bk_status {
-    return trans ? launch_passes_batch<T, true>(p, v, o, nv, n, st) : launch_passes_batch<T, false>(p, v, o, nv, n, st);
-  };
-  if constexpr (SmallFft<T>::E == FftShape<T, 2>::E) {
-    return passes(fs_p, fs_v, fs_o, fs_n, nfs);
-  } else {
-    std::vector<const Plan*> p[2];
-    std::vector<const void*> v[2];
-    std::vector<void*> o[2];
-    std::vector<int> nv[2];
-    for (int i = 0; i < nfs; ++i) {
-      const int w = fs_p[i]->split ? 1 : 0;
-      p[w].push_back(fs_p[i]); v[w].push_back(fs_v[i]); o[w].push_back(fs_o[i]); nv[w].push_back(fs_n[i]);
+  std::vector<const Plan*> p[2];   // 0: one launch, 1: launch per pass
+  std::vector<const void*> v[2];
+  std::vector<void*> o[2];
+  std::vector<int> nv[2];
+  std::vector<unsigned char*> guest;
+  int lender = 0;   // the launch-per-pass plan that lends next, and the bytes it has lent
+  size_t lent = 0;
+  for (int i = 0; i < nfs; ++i) {
+    unsigned char* g = nullptr;
+    int w = fs_p[i]->split ? 1 : 0;
+    if constexpr (SmallFft<T>::E == FftShape<T, 2>::E) {
+      if (w == 0) {
+        const size_t need = re_scratch_f32(fs_p[i]->N, fs_n[i]);
+        while (lender < nfs && lent + need > fs_p[lender]->guest_bytes) {
+          ++lender;
+          lent = 0;
+        }
+        if (lender < nfs) {
+          g = static_cast<unsigned char*>(fs_p[lender]->guest) + lent;
+          lent += need;
+          w = 1;
+        }
+      }
     }
-    if (!p[0].empty())
-      BK_TRY(launch_fourstep_batch<T>(p[0].data(), v[0].data(), o[0].data(), nv[0].data(), (int)p[0].size(), trans, st));
-    return passes(p[1].data(), v[1].data(), o[1].data(), nv[1].data(), (int)p[1].size());
+    p[w].push_back(fs_p[i]); v[w].push_back(fs_v[i]); o[w].push_back(fs_o[i]); nv[w].push_back(fs_n[i]);
+    if (w == 1) guest.push_back(g);
   }
+  if (!p[0].empty())
+    BK_TRY(launch_fourstep_batch<T>(p[0].data(), v[0].data(), o[0].data(), nv[0].data(), (int)p[0].size(), trans, st));
+  if (p[1].empty()) return BK_OK;
+  return (trans ? launch_passes_batch<T, true> : launch_passes_batch<T, false>)(
+      p[1].data(), v[1].data(), o[1].data(), nv[1].data(), guest.data(), (int)p[1].size(), st);
 }
 
 #ifndef BK_TRANSFORM_KERNEL_UNIT
@@ -1952,8 +2004,8 @@ bk_status plan_apply(const Plan* p, const void* v, void* out, int batch, bool tr
 // Products of several plans of one precision, N free per plan: small plans in one launch, four-step
 // plans of radix 4 in another, or in one launch per pass where one of them needs it (each per
 // BATCH_MAX plans), every other plan (dense, Bluestein, radix 8 and 16) by its own launches. The shared
-// launches use a four-step plan's scratch once, so a plan comes in them once; the later entries of an
-// FP64 plan of N >= 2^17 follow as launches of their own, those of a shorter one are refused.
+// launches use a four-step plan's scratch once, so a plan that has some comes in them once; the later
+// entries of an FP64 plan of N >= 2^17 follow as launches of their own, those of a shorter one are refused.
 bk_status plan_apply_batch(const Plan* const* ps, const void* const* v, void* const* out, const int* batch, int count,
                            bool trans, cudaStream_t st) {
   BK_ARG(ps != nullptr && v != nullptr && out != nullptr && batch != nullptr, "NULL argument");
@@ -1979,7 +2031,8 @@ bk_status plan_apply_batch(const Plan* const* ps, const void* const* v, void* co
     } else if (p->small) {
       sp.push_back(p); sv.push_back(v[i]); so.push_back(out[i]); sn.push_back(nv);
     } else {
-      const bool again = std::find(fp.begin(), fp.end(), p) != fp.end();
+      // FP32 one-launch plans have no scratch to share
+      const bool again = (p->split || dtype == BK_F64) && std::find(fp.begin(), fp.end(), p) != fp.end();
       if (again && dtype == BK_F64 && p->N >= (int64_t(1) << 17)) {   // as the double-float plans of that size
         op.push_back(p); ov.push_back(v[i]); oo.push_back(out[i]); on.push_back(nv);
         continue;
@@ -2021,8 +2074,6 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 // Device address of g_noalloc_scratch per device (host code cannot use the symbol itself).
 static void* g_noalloc_ptr[NOALLOC_MAX_DEV] = {nullptr};
 static std::mutex g_noalloc_mu;
-
-static size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 // Bytes of the scratch layout for N (FP64) and nvec vectors, and the sub-buffer offsets.
 static size_t noalloc_layout(const Plan& p, int nvec, size_t off[7]) {

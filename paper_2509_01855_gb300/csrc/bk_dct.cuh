@@ -74,7 +74,7 @@ __device__ __forceinline__ void re_fft(const ReArgs<T>& g, bool first, typename 
     fft_any<T, F::E, F::EPT>(buf, log2n, nbatch, bs, stw);
 }
 
-// Loads that bypass L1 (CG: data other CTAs of the running kernel wrote) or not.
+// Loads that bypass L1 (CG: data other CTAs of the running kernel wrote to global memory) or not.
 template <bool CG> __device__ __forceinline__ float ldr(const float* p) { return CG ? __ldcg(p) : *p; }
 template <bool CG> __device__ __forceinline__ double ldr(const double* p) { return CG ? __ldcg(p) : *p; }
 template <bool CG> __device__ __forceinline__ dfl ldr(const dfl* p) {
@@ -109,24 +109,66 @@ __device__ __forceinline__ void st2(dfl2* p, dfl2 a, dfl2 b) {
   q[1] = make_float4(b.x.hi, b.x.lo, b.y.hi, b.y.lo);
 }
 
+// Where a pass finds element m of a vector and row k of A: in global memory, or (FP32 one-launch form)
+// spread over the exchange areas of the cluster's CTAs. Row k of A is kept by the CTA whose pass B reads
+// it (tile = pair / P, rank = tile mod csize), so pass A writes to all CTAs and pass B reads its own;
+// the stage buffer is cut into csz blocks of 2^sh elements (the last two more); the shares of R_0 go to
+// every CTA, so that the last pass touches no other CTA's memory.
+template <typename S> __device__ __forceinline__ S* at(S* x, int m) { return x + m; }
+template <typename T> __device__ __forceinline__ void put_share(T* part, int p, T v) { part[p] = v; }
+template <typename C> __device__ __forceinline__ C* row(C* A, int k, int RS) { return A + (int64_t)k * RS; }
+
+// The address of the same shared variable in CTA `rank` of the cluster.
+template <typename P> __device__ __forceinline__ P* cluster_map(P* p, unsigned rank) {
+  unsigned long long r;
+  asm("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"((unsigned long long)p), "r"(rank));
+  return reinterpret_cast<P*>(r);
+}
+struct ClusterStage {
+  float* base;
+  int sh, csz;
+};
+struct ClusterRows {
+  float2* base;
+  int P, csize, half;
+};
+struct ClusterShares {
+  float* base;
+  int csize;
+};
+__device__ __forceinline__ float* at(const ClusterShares& c, int p) { return c.base + p; }
+__device__ __forceinline__ void put_share(const ClusterShares& c, int p, float v) {
+  for (int o = 0; o < c.csize; ++o) cluster_map(c.base, o)[p] = v;
+}
+__device__ __forceinline__ float* at(const ClusterStage& y, int m) {
+  const int o = min(m >> y.sh, y.csz - 1);
+  return cluster_map(y.base, o) + (m - (o << y.sh));
+}
+__device__ __forceinline__ float2* row(const ClusterRows& a, int k, int RS) {
+  const int q = k == a.half ? 0 : (k + 1) >> 1;   // its pair: rows 2q - 1 and 2q (q = 0: N1/2 and 0)
+  const int second = k != a.half && !(k & 1);
+  const int tile = q / a.P, o = tile % a.csize;
+  return cluster_map(a.base, o) + (((tile / a.csize) * a.P + (q - tile * a.P)) * 2 + second) * RS;
+}
+
 // Second-DCT input x_m from the stage buffer Y, any m (see stencil_fwd / stencil_trn; ST_TRN's
 // buffer holds T_k = (Y_k - Y_0) / (4k), for which the transposed stencil is T_{m-1} - T_{m+1}).
-template <typename T, int K, bool CG>
-__device__ __forceinline__ T re_stencil(const T* Y, int m, const ReArgs<T>& g) {
+template <typename T, int K, bool CG, typename X>
+__device__ __forceinline__ T re_stencil(X Y, int m, const ReArgs<T>& g) {
   const int N = g.N;
   if (K == ST_FWD) {
     if (m == 0) return T(0);
-    if (m == N) return -ldr<CG>(Y + N - 1) * (T(2) * g.rk[N]);
+    if (m == N) return -ldr<CG>(at(Y, N - 1)) * (T(2) * g.rk[N]);
     if (m == N - 1) {
-      const T yN = ldr<CG>(Y + N);
+      const T yN = ldr<CG>(at(Y, N));
       const T a = T(0.5) * g.rk[N - 1] - T(0.5) * g.rk[N + 1];
-      return dot2(yN, a, -ldr<CG>(Y + N - 2), g.rk[N - 1]);
+      return dot2(yN, a, -ldr<CG>(at(Y, N - 2)), g.rk[N - 1]);
     }
-    return (ldr<CG>(Y + m + 1) - ldr<CG>(Y + m - 1)) * g.rk[m];
+    return (ldr<CG>(at(Y, m + 1)) - ldr<CG>(at(Y, m - 1))) * g.rk[m];
   }
-  if (m == 0) return T(-2) * ldr<CG>(Y + 1);
-  if (m == N) return ldr<CG>(Y + N - 1) * g.cE;
-  return ldr<CG>(Y + m - 1) - ldr<CG>(Y + m + 1);
+  if (m == 0) return T(-2) * ldr<CG>(at(Y, 1));
+  if (m == N) return ldr<CG>(at(Y, N - 1)) * g.cE;
+  return ldr<CG>(at(Y, m - 1)) - ldr<CG>(at(Y, m + 1));
 }
 
 // 1 / (4k), k >= 1: correctly rounded either way (4k is exact in binary32 for k <= 2^24); the FP32
@@ -142,10 +184,9 @@ template <> __device__ __forceinline__ float re_rk<float>(const ReArgs<float>& g
 // depend on the tile or the thread count. A thread keeps one pair and steps over its rows, so that
 // its addresses are one base plus constant strides (per-element index arithmetic was half of the
 // FP32 kernel's instructions).
-template <typename T, int K, bool CG, typename F, typename S>
-__device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, int bs, const S* x,
-                                         typename V2<T>::t* A, T* part, typename V2<T>::t* buf,
-                                         const typename V2<T>::t* stw) {
+template <typename T, int K, bool CG, typename F, typename S, typename X, typename AP, typename PP>
+__device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, int bs, X x, AP A, PP part,
+                                         typename V2<T>::t* buf, const typename V2<T>::t* stw) {
   typedef typename V2<T>::t C;
   typedef Cv<T, S> CV;
   const int N = g.N, N1 = g.N1, N2 = g.N2, half = N1 >> 1;
@@ -172,8 +213,8 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
         if (j >= half) continue;
         const int m = j * N2 + 2 * p - 1, i = (j + 1) * N2 - 2 * p + 1;
         if constexpr (K == IN_PLAIN || K == IN_WINV) {
-          d[u] = mk2<T>(CV::in(x[m]), last ? T(0) : CV::in(x[m + 1]));
-          r[u] = mk2<T>(CV::in(x[i]), last ? T(0) : CV::in(x[i - 1]));
+          d[u] = mk2<T>(CV::in(*at(x, m)), last ? T(0) : CV::in(*at(x, m + 1)));
+          r[u] = mk2<T>(CV::in(*at(x, i)), last ? T(0) : CV::in(*at(x, i - 1)));
           if (K == IN_WINV) {
             d[u].x = T(0.5) * d[u].x;
             d[u].y = T(0.5) * d[u].y;
@@ -181,10 +222,10 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
             r[u].y = T(0.5) * r[u].y;
           }
         } else {
-          const C a0 = ldc<CG>(reinterpret_cast<const C*>(x + m - 1));   // x_{m-1}, x_m
-          const C a1 = ldc<CG>(reinterpret_cast<const C*>(x + m + 1));   // x_{m+1}, x_{m+2}
-          const C c0 = ldc<CG>(reinterpret_cast<const C*>(x + i - 1));   // x_{i-1}, x_i
-          const T hi = ldr<CG>(x + i + 1), lo = ldr<CG>(x + i - 2);
+          const C a0 = ldc<CG>(reinterpret_cast<const C*>(at(x, m - 1)));   // x_{m-1}, x_m
+          const C a1 = ldc<CG>(reinterpret_cast<const C*>(at(x, m + 1)));   // x_{m+1}, x_{m+2}
+          const C c0 = ldc<CG>(reinterpret_cast<const C*>(at(x, i - 1)));   // x_{i-1}, x_i
+          const T hi = ldr<CG>(at(x, i + 1)), lo = ldr<CG>(at(x, i - 2));
           if (K == ST_FWD) {
             d[u] = mk2<T>((a1.x - a0.x) * re_rk<T>(g, m), (a1.y - a0.y) * re_rk<T>(g, m + 1));
             r[u] = mk2<T>((hi - c0.x) * re_rk<T>(g, i), (c0.y - lo) * re_rk<T>(g, i - 1));
@@ -209,7 +250,7 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
       const int ma = n1 * N2, mb = ma + (N2 >> 1);
       const int ia = ma <= N ? ma : 2 * N - ma, ib = mb <= N ? mb : 2 * N - mb;
       if constexpr (K == IN_PLAIN || K == IN_WINV) {
-        T a = CV::in(x[ia]), c = CV::in(x[ib]);
+        T a = CV::in(*at(x, ia)), c = CV::in(*at(x, ib));
         if (K == IN_WINV) {
           if (ia != 0 && ia != N) a = T(0.5) * a;
           c = T(0.5) * c;
@@ -226,7 +267,6 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
   if (on) {
     constexpr int LD = sizeof(T) == 8 ? 2 : 4;
     const C* tw = g.twA + 2 * p;
-    C* Ap = A + 2 * p;
     for (int k0 = row0; k0 <= half; k0 += LD * step) {
       C wa[LD], wb[LD];
 #pragma unroll
@@ -240,10 +280,10 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
         if (k > half) continue;
         const C zk = z[padi(k)];
         const C zm = z[padi(k == 0 ? 0 : N1 - k)];
-        if (k == 0) part[p] = p == 0 ? zk.x + zk.y : T(2) * (zk.x + zk.y);
+        if (k == 0) put_share(part, p, p == 0 ? zk.x + zk.y : T(2) * (zk.x + zk.y));
         const C sa = mk2<T>(zk.x + zm.x, zk.y - zm.y);   // Z_k + conj Z_{N1-k}
         const C sb = mk2<T>(zk.x - zm.x, zk.y + zm.y);   // Z_k - conj Z_{N1-k}
-        st2(Ap + (int64_t)k * g.RS, cmul(sa, wa[u]), cmul(sb, wb[u]));
+        st2(row(A, k, g.RS) + 2 * p, cmul(sa, wa[u]), cmul(sb, wb[u]));
       }
     }
   }
@@ -255,9 +295,9 @@ __device__ __forceinline__ void re_passA(const ReArgs<T>& g, int tile, int NB, i
 //   EP_FWD_OUT   : out[k] = s (R_k - R_0), 0 at k = 0        (after the second DCT, forward)
 //   EP_TRN_OUT   : out[k] = (s/N) W_k R_k                    (after the second DCT, transpose)
 // Pass B of row pairs [tile P, tile P + P) of one vector.
-template <typename T, int E, bool CG, typename F, typename S>
-__device__ __forceinline__ void re_passB(const ReArgs<T>& g, int tile, int P, int bs, const typename V2<T>::t* A,
-                                         S* out, int64_t zero_to, const T* part, typename V2<T>::t* buf,
+template <typename T, int E, bool CG, typename F, typename S, typename X, typename AP, typename PP>
+__device__ __forceinline__ void re_passB(const ReArgs<T>& g, int tile, int P, int bs, AP A, X out, int64_t zero_to,
+                                         PP part, typename V2<T>::t* buf,
                                          const typename V2<T>::t* stw, T* y0s, T s, T invN) {
   typedef typename V2<T>::t C;
   typedef Cv<T, S> CV;
@@ -275,8 +315,8 @@ __device__ __forceinline__ void re_passB(const ReArgs<T>& g, int tile, int P, in
     constexpr int LD = 4;
     for (int i = i0 < istep ? i0 : na; i < na; i += istep) {
       const int q = q0 + i;
-      const C* ra = A + (int64_t)(q == 0 ? N1 >> 1 : 2 * q - 1) * g.RS;
-      const C* rb = A + (int64_t)(2 * q) * g.RS;
+      const C* ra = row(A, q == 0 ? N1 >> 1 : 2 * q - 1, g.RS);
+      const C* rb = row(A, 2 * q, g.RS);
       const bool two = q != (N1 >> 2);
       C* z = (IsMix<F>::v && (g.nst2 & 1) ? alt : buf) + i * bs;
       for (int ps = ps0; ps <= h2; ps += LD * tpr) {
@@ -308,7 +348,7 @@ __device__ __forceinline__ void re_passB(const ReArgs<T>& g, int tile, int P, in
     for (int i = threadIdx.x; i < np; i += 128) {
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        if (i + 32 * u < np) acc[u] += ldr<CG>(part + i + 32 * u);
+        if (i + 32 * u < np) acc[u] += ldr<CG>(at(part, i + 32 * u));
     }
     T a = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     for (int o = 16; o > 0; o >>= 1) a += shfl_xor(a, o);
@@ -353,13 +393,13 @@ __device__ __forceinline__ void re_passB(const ReArgs<T>& g, int tile, int P, in
         const int j = jj + u * step;
         if (j >= h2) continue;
         const int kd = r + N1 * j, km = N1 * (j + 1) - r;
-        out[kd] = CV::out(val(vd[u], kd, rd[u]));
-        if (!mid && (!zero || j == h2 - 1)) out[km] = CV::out(val(vm[u], km, rm[u]));
+        *at(out, kd) = CV::out(val(vd[u], kd, rd[u]));
+        if (!mid && (!zero || j == h2 - 1)) *at(out, km) = CV::out(val(vm[u], km, rm[u]));
       }
     }
   }
   if ((E == EP_FWD_OUT || E == EP_TRN_OUT) && tile == 0) {
-    for (int64_t m = N + 1 + threadIdx.x; m < zero_to; m += nt) out[m] = S(0);
+    for (int64_t m = N + 1 + threadIdx.x; m < zero_to; m += nt) *at(out, m) = S(0);
   }
 }
 
@@ -418,8 +458,10 @@ __global__ void __launch_bounds__(F::MT, F::MINB)
 }
 
 // ---- all four passes of a vector in one launch: one cluster of CTAs per vector ------------------
-// The passes exchange A and the stage buffer through global memory (L2), separated by cluster
-// barriers (release / acquire) in place of launches; reads of exchanged data bypass L1.
+// The passes exchange A, the stage buffer and the shares of R_0, separated by cluster barriers
+// (release / acquire) in place of launches. FP32: in shared memory, spread over the exchange areas of the
+// cluster's CTAs, so that such a plan owns no scratch and any number of its products may run at a time,
+// on any streams. FP64: through global memory (L2), with reads that bypass L1.
 template <typename T> struct ReJob {
   typedef typename V2<T>::t C;
   ReArgs<T> g;
@@ -431,10 +473,15 @@ template <typename T> struct ReJob {
   T* part;
   T s, invN;
   int NB, bsA, P, bsB, nvec;
+  int ex, exY, exP, csz;   // FP32 one-launch form: byte offsets of A's rows, the stage block and the
+                           // shares in a CTA's shared memory; blocks of the stage buffer
 };
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 
 template <typename T, bool TRANS>
@@ -443,6 +490,9 @@ __device__ __forceinline__ void re_cluster_body(const ReJob<T>& J, int vec, int 
   typedef Us<T> U;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ T y0s;
+  constexpr bool DS = sizeof(T) == 4;   // exchange in shared memory
+  constexpr bool CG = !DS;
+  if (DS) cluster_arrive();   // waited for below: every CTA of the cluster runs before another writes to it
   const ReArgs<T>& g = J.g;
   C* tw1 = reinterpret_cast<C*>(smem);
   const int l1 = stage_tw_len(g.log2N1, SmallFft<T>::E), l2 = stage_tw_len(g.log2N2, SmallFft<T>::E);
@@ -452,30 +502,37 @@ __device__ __forceinline__ void re_cluster_body(const ReJob<T>& J, int vec, int 
   load_tw_smem<T>(tw2, g.stw2, l2);
   const U* in = J.in + vec * J.pitch;
   U* out = J.out + vec * J.pitch;
-  C* A = J.A + vec * J.astride;
-  T* Y = J.Y + vec * J.ystride;
-  T* part = J.part + (int64_t)vec * ((g.N2 >> 2) + 1);
   const int ta = ((g.N2 >> 2) + J.NB) / J.NB;   // tiles of the N2/4 + 1 column pairs
   const int tb = ((g.N1 >> 2) + J.P) / J.P;     // tiles of the N1/4 + 1 row pairs
-  for (int t = rank; t < ta; t += csize) {
-    re_passA<T, TRANS ? IN_WINV : IN_PLAIN, true, void, U>(g, t, J.NB, J.bsA, in, A, part, buf, tw1);
-    __syncthreads();
-  }
-  cluster_barrier();
-  for (int t = rank; t < tb; t += csize) {
-    re_passB<T, TRANS ? EP_STORE_TRN : EP_STORE, true, void, T>(g, t, J.P, J.bsB, A, Y, 0, part, buf, tw2, &y0s, J.s, J.invN);
-    __syncthreads();
-  }
-  cluster_barrier();
-  for (int t = rank; t < ta; t += csize) {
-    re_passA<T, TRANS ? ST_TRN : ST_FWD, true, void, T>(g, t, J.NB, J.bsA, Y, A, part, buf, tw1);
-    __syncthreads();
-  }
-  cluster_barrier();
-  for (int t = rank; t < tb; t += csize) {
-    re_passB<T, TRANS ? EP_TRN_OUT : EP_FWD_OUT, true, void, U>(g, t, J.P, J.bsB, A, out, J.pitch, part, buf, tw2, &y0s, J.s,
-                                                          J.invN);
-    __syncthreads();
+  auto passes = [&](auto A, auto Y, auto part) {
+    for (int t = rank; t < ta; t += csize) {
+      re_passA<T, TRANS ? IN_WINV : IN_PLAIN, CG, void, U>(g, t, J.NB, J.bsA, in, A, part, buf, tw1);
+      __syncthreads();
+    }
+    cluster_barrier();
+    for (int t = rank; t < tb; t += csize) {
+      re_passB<T, TRANS ? EP_STORE_TRN : EP_STORE, CG, void, T>(g, t, J.P, J.bsB, A, Y, 0, part, buf, tw2, &y0s, J.s, J.invN);
+      __syncthreads();
+    }
+    cluster_barrier();
+    for (int t = rank; t < ta; t += csize) {
+      re_passA<T, TRANS ? ST_TRN : ST_FWD, CG, void, T>(g, t, J.NB, J.bsA, Y, A, part, buf, tw1);
+      __syncthreads();
+    }
+    cluster_barrier();
+    for (int t = rank; t < tb; t += csize) {
+      re_passB<T, TRANS ? EP_TRN_OUT : EP_FWD_OUT, CG, void, U>(g, t, J.P, J.bsB, A, out, J.pitch, part, buf, tw2, &y0s, J.s,
+                                                            J.invN);
+      __syncthreads();
+    }
+  };
+  if constexpr (DS) {
+    const ClusterRows A = {reinterpret_cast<C*>(smem + J.ex), J.P, csize, g.N1 >> 1};
+    const ClusterStage Y = {reinterpret_cast<T*>(smem + J.exY), __clz(J.csz) - __clz(g.N), J.csz};
+    cluster_wait();
+    passes(A, Y, ClusterShares{reinterpret_cast<T*>(smem + J.exP), csize});
+  } else {
+    passes(J.A + vec * J.astride, J.Y + vec * J.ystride, J.part + (int64_t)vec * ((g.N2 >> 2) + 1));
   }
 }
 

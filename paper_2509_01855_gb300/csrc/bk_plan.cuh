@@ -58,9 +58,13 @@ struct Plan {
   int fe = 2;                 // log2 radix of the launch-per-pass kernels
   int csize = 0, cthr = 0;
   size_t csmem = 0;
+  int cex = 0, cexY = 0, cexP = 0;   // FP32: offsets of the exchange area's parts in shared memory
+  void* guest = nullptr;      // FP32 launch-per-pass plans: scratch lent to one-launch plans of a batch
+  size_t guest_bytes = 0;
   void* tpost = nullptr;      // (cos, sin)(pi k / N), k = 0..N/2 (working type; not four-step)
   void* rk = nullptr;         // 1 / (4k), k = 0..N+1 (working type; rk[0] = 0)
-  void* scrA = nullptr;       // scratch between passes A and B, fs.a_len() complex per vector
+  void* scrA = nullptr;       // scratch between passes A and B, fs.a_len() complex per vector (none of these
+                              // three in FP32 one-launch plans)
   void* scrY = nullptr;       // stage buffer between the two DCTs, N + 2 per vector (Bluestein N + 1)
   void* scrG = nullptr;       // Bluestein: second-DCT input (stencil output), N + 1 per vector
   void* part = nullptr;       // pass-A shares of R_0, fs.pairs() per vector
