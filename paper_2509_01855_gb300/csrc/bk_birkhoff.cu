@@ -1224,6 +1224,42 @@ static bk_status cluster_attr(F* fn, int cap) {
 }
 
 template <typename T>
+static bk_status cluster_attrs(int cap) {
+  BK_TRY(cluster_attr(k_re_cluster<T, false>, cap));
+  BK_TRY(cluster_attr(k_re_cluster<T, true>, cap));
+  BK_TRY(cluster_attr(k_re_cluster_batch<T, false>, cap));
+  BK_TRY(cluster_attr(k_re_cluster_batch<T, true>, cap));
+  return BK_OK;
+}
+
+// Whether the device (or the partition of it that the context has) holds a cluster of csize CTAs of
+// every one-launch kernel, at the largest thread count a batch may launch them with.
+template <typename T>
+bool clusters_held(int csize, size_t smem) {
+  if (cluster_attrs<T>((int)FOURSTEP_SMEM_BUDGET) != BK_OK) return false;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(csize);
+  cfg.blockDim = dim3(512);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)csize;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  auto held = [&](auto* k) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      n = 0;
+    }
+    return n > 0;
+  };
+  return held(k_re_cluster<T, false>) && held(k_re_cluster<T, true>) && held(k_re_cluster_batch<T, false>) &&
+         held(k_re_cluster_batch<T, true>);
+}
+
+template <typename T>
 bk_status re_attrs() {
   const int cap = (int)FOURSTEP_SMEM_BUDGET;
   if constexpr (!std::is_same<T, dfl>::value) BK_TRY((re_attrs_AB<T, MixFft>(cap)));
@@ -1235,10 +1271,7 @@ bk_status re_attrs() {
     BK_TRY((re_attrs_B<T, BigFft<T>>(cap)));
   }
   if constexpr (!std::is_same<T, dfl>::value) {
-    BK_TRY(cluster_attr(k_re_cluster<T, false>, cap));
-    BK_TRY(cluster_attr(k_re_cluster<T, true>, cap));
-    BK_TRY(cluster_attr(k_re_cluster_batch<T, false>, cap));
-    BK_TRY(cluster_attr(k_re_cluster_batch<T, true>, cap));
+    BK_TRY(cluster_attrs<T>(cap));
     typedef FftShape<T, 2> F;
     BK_TRY(smem_attr(k_re_passA_batch<T, false, false, F>, cap));
     BK_TRY(smem_attr(k_re_passA_batch<T, false, true, F>, cap));
@@ -1282,6 +1315,8 @@ static int64_t blue_max(int dtype) { return dtype == BK_F64 ? (int64_t(1) << 22)
 // compiled in bk_birkhoff_f64.cu and bk_birkhoff_f32.cu, in parallel with this unit.
 extern template bk_status set_smem_attrs<double>(const Plan* p);
 extern template bk_status re_attrs<double>();
+extern template bool clusters_held<double>(int, size_t);
+extern template bool clusters_held<float>(int, size_t);
 extern template bk_status set_smem_attrs<float>(const Plan* p);
 extern template bk_status set_smem_attrs<dfl>(const Plan* p);
 template <typename T> bk_status blue_spectrum(Plan* p, cudaStream_t st);
@@ -1408,6 +1443,27 @@ bool plan_n_supported(int64_t N, int dtype) {
   return N >= 4 && (is_pow2(N) ? N <= (int64_t(1) << 24) : (dense_supported(N) || N <= blue_max(dtype)));
 }
 
+// Whether the one-launch form of the plan's size can run on the current device; asked once per device and
+// shape. BK_MAX_CLUSTER (read at plan creation) sets the largest cluster instead, for tuning and tests.
+static bool cluster_form_held(const Plan* p) {
+  Plan q;
+  q.N = p->N;
+  q.dtype = p->dtype;
+  if (configure_cluster(&q) != BK_OK) return false;
+  const char* e = getenv("BK_MAX_CLUSTER");
+  if (e) return q.csize <= atoi(e);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int, size_t>, bool> seen;
+  std::lock_guard<std::mutex> lk(mu);
+  const auto key = std::make_tuple(dev, q.dtype, q.csize, q.csmem);
+  auto it = seen.find(key);
+  if (it == seen.end())
+    it = seen.emplace(key, q.dtype == BK_F64 ? clusters_held<double>(q.csize, q.csmem) : clusters_held<float>(q.csize, q.csmem)).first;
+  return it->second;
+}
+
 bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtype, double t0, double tf, int64_t pitch,
                       cudaStream_t st) {
   return plan_create_arith(out, N, n_comp, max_batch, dtype, t0, tf, pitch, st, false);
@@ -1452,6 +1508,12 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
   }
   p->df = dtype == BK_F64 && is_pow2(N) && N >= 256 && !weights_only && f64_df_default(N);
   p->small = !p->generic && !p->blue && !p->mix && !p->df && N <= small_limit(dtype);
+  const bool fourstep = !p->generic && !p->blue && !p->small;
+  p->split = fourstep && (p->df || p->mix || split_passes(dtype, N, n_comp * max_batch));
+  if (fourstep && !p->split && !cluster_form_held(p)) {
+    p->small = dtype == BK_F32 && N <= 4096;   // the other form without scratch
+    p->split = !p->small;
+  }
   bk_status st_ = BK_OK;
   AllocCounter counter(&p->bytes);
   do {
@@ -1481,7 +1543,6 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
       if ((st_ = dmalloc(&p->scrY, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
       if ((st_ = dmalloc(&p->scrG, dtype_size(dtype) * (size_t)(N + 1) * nvec)) != BK_OK) break;
     } else {
-      p->split = p->df || p->mix || split_passes(dtype, N, n_comp * max_batch);
       p->fe = p->mix ? 0 : re_radix(N, dtype, p->df);
       if ((st_ = fourstep_shapes(p, 0)) != BK_OK) break;
       const int64_t nvec = (int64_t)n_comp * max_batch;

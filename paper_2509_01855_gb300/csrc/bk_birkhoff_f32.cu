@@ -8,6 +8,7 @@
 namespace bk {
 
 template bk_status set_smem_attrs<float>(const Plan* p);
+template bool clusters_held<float>(int, size_t);
 template bk_status blue_spectrum<float>(Plan* p, cudaStream_t st);
 template bk_status apply_batch_impl<float>(const Plan* const*, const void* const*, void* const*, const int*, int,
                                         const Plan* const*, const void* const*, void* const*, const int*, int, bool,

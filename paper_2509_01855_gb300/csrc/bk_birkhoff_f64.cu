@@ -8,6 +8,7 @@
 namespace bk {
 
 template bk_status set_smem_attrs<double>(const Plan* p);
+template bool clusters_held<double>(int, size_t);
 template bk_status re_attrs<double>();
 template bk_status blue_spectrum<double>(Plan* p, cudaStream_t st);
 template bk_status apply_batch_impl<double>(const Plan* const*, const void* const*, void* const*, const int*, int,
