@@ -836,58 +836,103 @@ static bk_status build_tables(Plan* p, cudaStream_t st) {
 }
 
 #ifndef BK_TRANSFORM_KERNEL_UNIT
-static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_batch, int dtype, double t0, double tf,
-                                   int64_t pitch, cudaStream_t st, bool weights_only);
-
-__global__ void k_unit_last(double* e, int64_t L, int64_t pitch) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < pitch; i += (int64_t)gridDim.x * blockDim.x)
-    e[i] = (i == L - 1) ? 1.0 : 0.0;
+// Clenshaw-Curtis weights (the last row of B^a) in closed form, each to its own relative accuracy. With
+// theta = pi k / N, w_k = (c / N) [1 - sum_{j <= N/2}'' 2 cos(2 j theta) / (4 j^2 - 1)] (c = 1 at the ends,
+// 2 inside). The series taken to infinity is (pi/2) sin theta, and its remainder, with 2 / (4 j^2 - 1) =
+// int_0^1 x^{2j-2} (1 - x^2) dx summed as a geometric series under the integral and x = e^{-t/N}, is
+//   T = (1/N) int_0^inf e^{-t} e^{t/N} u^2 (1 + r) / (2 (u^2 + 4 r sin^2 theta)) dt       (N even),
+//   T = (1/N) int_0^inf e^{-t} cos theta u^2 / (u^2 + 4 r sin^2 theta) dt                  (N odd),
+// u = 1 - r, r = e^{-2t/N}, so that N w_k / c = (pi/2) sin theta + (-1)^k T. The integrand's poles lie near
+// t = +- i pi k: from k = 32 on five Gauss-Laguerre nodes give T to 3e-18 of the weight, from k = 1024 on its
+// leading term in 1 / sin^2 theta does (past 1.6e5 T is below 1e-17 of it); below, the trapezoidal rule in
+// y, t = exp(y - e^{-y}), at 96 points (one warp per weight). The ends are 1 / (N^2 - 1) and 1 / N^2.
+// (The transposed product with e_N, used before, has its absolute rounding in every weight: the weights next to
+// the ends, which the KKT preconditioner's control block divides by, were off by some N ulp. It also needed a
+// binary64 plan, 0.3 ms at N = 2^20, which FP32 lengths above 2^22 do not have.)
+__device__ __forceinline__ void put_weight(double v, int64_t k, int64_t N, double* w, float* wT) {
+  w[k] = w[N - k] = v;
+  if (wT) wT[k] = wT[N - k] = (float)v;
 }
-__global__ void k_d2f(const double* a, float* b, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    b[i] = (float)a[i];
-}
 
-// The end weights of an even N are 1 / (N^2 - 1) exactly. The transpose product gives them to its
-// absolute rounding, N times larger relative to them than to the others, and the control block of
-// the KKT preconditioner divides by them.
-__global__ void k_weight_ends(double* w, int64_t N) {
-  if (threadIdx.x < 2) w[threadIdx.x * N] = 1.0 / ((double)N * (double)N - 1.0);
-}
-
-// Clenshaw-Curtis weights as the last row of B^a: w = (B^a)^T e_N, computed in binary64 with the
-// transpose product itself (O(N log N)). FP32 and double-float plans use a temporary binary64 plan.
-static bk_status compute_weights(Plan* p, cudaStream_t st) {
-  const int64_t L = p->L;
-  Plan* q = p;
-  Plan* tmp = nullptr;
-  if (p->dtype != BK_F64 || p->df) {
-    BK_TRY(plan_create_arith(&tmp, p->N, 1, 1, BK_F64, 0.0, 2.0, 0, st, true));
-    q = tmp;
+__global__ void __launch_bounds__(256) k_weights(double* __restrict__ w, float* __restrict__ wT, int64_t N, int64_t pitch) {
+  // nodes and weights of the Gauss-Laguerre rule (zeros t of L_5, t / (36 L_6(t)^2))
+  const double gt[5] = {0.26356031971814091020, 1.4134030591065167922, 3.5964257710407220812, 7.0858100058588375569,
+                        12.640800844275782659};
+  const double gw[5] = {0.52175561058280865248, 0.39866681108317592745, 0.075942449681707595388,
+                        0.0036117586799220484545, 0.000023369972385776227891};
+  __shared__ double su[5], sr[5], sc[5], lead;   // u^2, 4 r, and the numerator of each node
+  const bool odd = N & 1;
+  if (threadIdx.x < 5) {
+    const int i = threadIdx.x;
+    const double u = -expm1(-2.0 * gt[i] / (double)N), r = 1.0 - u;
+    su[i] = u * u;
+    sr[i] = 4.0 * r;
+    sc[i] = gw[i] * u * u * (odd ? 1.0 : 0.5 * (1.0 + r) * exp(gt[i] / (double)N));
   }
-  double* e = nullptr;
-  bk_status r = dmalloc((void**)&e, sizeof(double) * q->pitch);
-  if (r == BK_OK) r = dmalloc((void**)&p->w64, sizeof(double) * q->pitch);
-  if (r == BK_OK) {
-    k_unit_last<<<(int)((q->pitch + 255) / 256), 256, 0, st>>>(e, L, q->pitch);
-    note_launch();
-    r = cudaGetLastError() == cudaSuccess ? plan_apply_n(q, e, p->w64, 1, true, 1.0, st) : BK_ERR_CUDA;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = 0.0;
+    for (int i = 0; i < 5; ++i) a += sc[i] / sr[i];
+    lead = a;
   }
-  if (r == BK_OK && p->N % 2 == 0) {
-    k_weight_ends<<<1, 32, 0, st>>>(p->w64, p->N);
-    note_launch();
-  }
-  if (r == BK_OK && p->dtype == BK_F32) {
-    r = dmalloc(&p->wT, sizeof(float) * L);
-    if (r == BK_OK) {
-      k_d2f<<<(int)((L + 255) / 256), 256, 0, st>>>(p->w64, (float*)p->wT, L);
-      note_launch();
+  __syncthreads();
+  const double iN = 1.0 / (double)N;
+  const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k = 32 + id; k <= N / 2; k += nt) {
+    const double x = (double)k / (double)N;
+    const double s = sinpi(x);
+    double v = 1.5707963267948966192 * s;
+    if (k < 163840) {
+      const double s2 = s * s;
+      double T = 0.0;
+      if (k >= 1024) {
+        T = lead / s2;
+      } else {
+        for (int i = 0; i < 5; ++i) T += sc[i] / fma(sr[i], s2, su[i]);
+      }
+      T *= odd ? iN * cospi(x) : iN;
+      v = (k & 1) ? v - T : v + T;
     }
+    put_weight(2.0 * v / (double)N, k, N, w, wT);
   }
-  if (r == BK_OK && cudaStreamSynchronize(st) != cudaSuccess) { set_error("weights: sync failed"); r = BK_ERR_CUDA; }
-  dfree(e);
-  if (tmp) plan_destroy(tmp);
-  return r;
+  for (int64_t k = N + 1 + id; k < pitch; k += nt) w[k] = 0.0;
+}
+
+// Weights k = blockIdx.x < 32 from either end; one warp.
+__global__ void __launch_bounds__(32) k_weight_ends(double* __restrict__ w, float* __restrict__ wT, int64_t N) {
+  const int64_t k = blockIdx.x;
+  if (k > N / 2) return;
+  const double n = (double)N;
+  const bool odd = N & 1;
+  if (k == 0) {
+    if (threadIdx.x == 0) put_weight(odd ? 1.0 / (n * n) : 1.0 / ((n - 1.0) * (n + 1.0)), 0, N, w, wT);
+    return;
+  }
+  double s, c;
+  sincospi((double)k / n, &s, &c);
+  const double h = 0.125;
+  double T = 0.0;
+  for (int i = threadIdx.x; i < 96; i += 32) {
+    const double y = -4.5 + h * i, ey = exp(-y), t = exp(y - ey);
+    const double u = -expm1(-2.0 * t / n), r = 1.0 - u;
+    const double q = odd ? c : 0.5 * (1.0 + r);
+    const double e = exp(odd ? -t : -t * (n - 1.0) / n);
+    T += h * t * (1.0 + ey) * e * q * u * u / fma(4.0 * r, s * s, u * u);
+  }
+  for (int o = 16; o > 0; o >>= 1) T += __shfl_xor_sync(0xffffffffu, T, o);
+  T /= n;
+  const double v = 1.5707963267948966192 * s;
+  if (threadIdx.x == 0) put_weight(2.0 * ((k & 1) ? v - T : v + T) / n, k, N, w, wT);
+}
+
+static bk_status compute_weights(Plan* p, cudaStream_t st) {
+  BK_TRY(dmalloc((void**)&p->w64, sizeof(double) * p->pitch));
+  if (p->dtype == BK_F32) BK_TRY(dmalloc(&p->wT, sizeof(float) * p->L));
+  k_weights<<<(int)std::min<int64_t>((p->N / 2 + 256) / 256, 4096), 256, 0, st>>>(p->w64, (float*)p->wT, p->N, p->pitch);
+  BK_CHECK_LAUNCH();
+  k_weight_ends<<<32, 32, 0, st>>>(p->w64, (float*)p->wT, p->N);
+  BK_CHECK_LAUNCH();
+  return BK_OK;
 }
 #endif  // BK_TRANSFORM_KERNEL_UNIT
 
@@ -1466,13 +1511,6 @@ static bool cluster_form_held(const Plan* p) {
 
 bk_status plan_create(Plan** out, int64_t N, int n_comp, int max_batch, int dtype, double t0, double tf, int64_t pitch,
                       cudaStream_t st) {
-  return plan_create_arith(out, N, n_comp, max_batch, dtype, t0, tf, pitch, st, false);
-}
-
-// weights_only: a plan for compute_weights' one product, in binary64, with the default tiles and
-// without weights of its own.
-static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_batch, int dtype, double t0, double tf,
-                                   int64_t pitch, cudaStream_t st, bool weights_only) {
   *out = nullptr;
   BK_ARG(plan_n_supported(N, dtype),
          "N must be a power of two in [4, 2^24] or any N in [4, %lld] (this precision), got %lld",
@@ -1506,7 +1544,7 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
     const char* e = getenv("BK_DENSE_TEST_TIMEOUT");  // test mode of the dense kernel, as bk_plan_dense_test_timeout
     p->dtest = (e && e[0] == '1') ? 1 : 0;
   }
-  p->df = dtype == BK_F64 && is_pow2(N) && N >= 256 && !weights_only && f64_df_default(N);
+  p->df = dtype == BK_F64 && is_pow2(N) && N >= 256 && f64_df_default(N);
   p->small = !p->generic && !p->blue && !p->mix && !p->df && N <= small_limit(dtype);
   const bool fourstep = !p->generic && !p->blue && !p->small;
   p->split = fourstep && (p->df || p->mix || split_passes(dtype, N, n_comp * max_batch));
@@ -1566,7 +1604,6 @@ static bk_status plan_create_arith(Plan** out, int64_t N, int n_comp, int max_ba
     st_ = dtype == BK_F64 ? (p->df ? set_smem_attrs<dfl>(p) : set_smem_attrs<double>(p)) : set_smem_attrs<float>(p);
     if (st_ != BK_OK) break;
     if (p->blue && (st_ = dtype == BK_F64 ? blue_spectrum<double>(p, st) : blue_spectrum<float>(p, st)) != BK_OK) break;
-    if (weights_only) break;
     if ((st_ = compute_weights(p, st)) != BK_OK) break;
     if (p->split && autotune_enabled()) {
       if ((st_ = autotune_tiles(p, st)) != BK_OK) break;
