@@ -407,12 +407,20 @@ template <typename T> struct SweepArgs {
 template <typename T> struct V16;
 template <> struct V16<float> { typedef float4 t; static constexpr int n = 4; };
 template <> struct V16<double> { typedef double2 t; static constexpr int n = 2; };
+// A vector's components to and from an array of the element's own alignment.
+__device__ __forceinline__ void put16(float4 t, float* v) { v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; }
+__device__ __forceinline__ void put16(double2 t, double* v) { v[0] = t.x; v[1] = t.y; }
+__device__ __forceinline__ float4 get16(const float* v) { return make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ double2 get16(const double* v) { return make_double2(v[0], v[1]); }
 template <typename T, int N>
 __device__ __forceinline__ void ld_run(const T* __restrict__ p, bool vec, T* v) {
   if (vec) {
     typedef typename V16<T>::t VT;
 #pragma unroll
-    for (int q = 0; q < N / V16<T>::n; ++q) *reinterpret_cast<VT*>(v + q * V16<T>::n) = reinterpret_cast<const VT*>(p)[q];
+    for (int q = 0; q < N / V16<T>::n; ++q) {
+      const VT t = reinterpret_cast<const VT*>(p)[q];
+      put16(t, v + q * V16<T>::n);
+    }
   } else {
 #pragma unroll
     for (int q = 0; q < N; ++q) v[q] = p[q];
@@ -423,7 +431,7 @@ __device__ __forceinline__ void st_run(T* p, bool vec, const T* v) {
   if (vec) {
     typedef typename V16<T>::t VT;
 #pragma unroll
-    for (int q = 0; q < N / V16<T>::n; ++q) reinterpret_cast<VT*>(p)[q] = *reinterpret_cast<const VT*>(v + q * V16<T>::n);
+    for (int q = 0; q < N / V16<T>::n; ++q) reinterpret_cast<VT*>(p)[q] = get16(v + q * V16<T>::n);
   } else {
 #pragma unroll
     for (int q = 0; q < N; ++q) p[q] = v[q];
