@@ -794,7 +794,8 @@ static bk_status run_sweep(Problem* pr, OpData& d, SweepArgs<T>& a, int ncol, cu
 }
 
 // ---------------------------------------------------------------------------------------------
-// KKT / state operator kernels (per node, Jacobians and Hessian recomputed from (x, u, mu))
+// KKT / state operator kernels (per node; Jacobians and Hessian from the stored entries, or recomputed
+// from (x, u, mu))
 // ---------------------------------------------------------------------------------------------
 // Entries of J_x and H at the linearisation (Dyn::pack), for kinds that store them: the operator
 // kernels read them instead of forming them from (x, u, mu) at every apply, which had bound the FP64
@@ -819,12 +820,12 @@ __global__ void k_lin_entries(const T* __restrict__ xu, const T* __restrict__ mu
   }
 }
 
-// J_x and J_u of node k: stored entries, or formed from (x, u).
-template <typename T, int KIND>
+// J_x and J_u of node k: stored entries (ST), or formed from (x, u).
+template <typename T, int KIND, bool ST>
 __device__ __forceinline__ void node_jac(const T* __restrict__ xu, const T* __restrict__ lin, int64_t P, int64_t k, T pa,
                                          T* Jx, T* Ju) {
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NJ = Dyn<KIND>::nlj;
-  if constexpr (NJ > 0) {
+  if constexpr (ST) {
     T v[NJ];
 #pragma unroll
     for (int i = 0; i < NJ; ++i) v[i] = lin[i * P + k];
@@ -841,7 +842,7 @@ __device__ __forceinline__ void node_jac(const T* __restrict__ xu, const T* __re
 
 // t = J dz per node; with a free final time (ds != null) t += (ds / s) f, so that the product
 // s B^a t adds the column d c / ds = -B^a f times ds.
-template <typename T, int KIND>
+template <typename T, int KIND, bool ST>
 __global__ void k_jvp(const T* __restrict__ xu, const T* __restrict__ dX, const T* __restrict__ dU, int64_t P,
                       int64_t L, T* __restrict__ t, T pa, const T* __restrict__ ds, T inv_s, const T* __restrict__ lin) {
   pdl_wait();
@@ -849,7 +850,7 @@ __global__ void k_jvp(const T* __restrict__ xu, const T* __restrict__ dX, const 
   const T dss = ds ? ds[0] * inv_s : T(0);
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < L; k += (int64_t)gridDim.x * blockDim.x) {
     T Jx[NXM * NXM], Ju[NXM * NUM], fx[NXM];
-    node_jac<T, KIND>(xu, lin, P, k, pa, Jx, Ju);
+    node_jac<T, KIND, ST>(xu, lin, P, k, pa, Jx, Ju);
     if (ds) {
       T x[NXM], u[NUM];
 #pragma unroll
@@ -892,7 +893,7 @@ __global__ void k_state_post(const T* __restrict__ chi, const T* __restrict__ Bt
 // Free final time (part != null): the gradient rows add ds d g / ds = -(ds / s) J^T mu, and each
 // block writes its partial of mu . (J dz) + f . Mu; the s row is -(1/s) times their sum
 // (k_free_finish), i.e. -(B^aT lambda) . (J dz) - (B^a f) . dlambda.
-template <typename T, int KIND>
+template <typename T, int KIND, bool ST>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_kkt_post(const T* __restrict__ xu, const T* __restrict__ mu, const T* __restrict__ w, T s,
                            const T* __restrict__ in, const T* __restrict__ Bt, T* __restrict__ Mu, int64_t P,
                            int64_t L, TermSpec ts, T cost_uu, T* __restrict__ out, T pa, int64_t s_idx,
@@ -901,7 +902,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_kkt_post(const 
   pdl_wait();
   constexpr int NX = Dyn<KIND>::nx, NU = Dyn<KIND>::nu, NV = NX + NU, NJ = Dyn<KIND>::nlj, NH = Dyn<KIND>::nlh;
   // with stored entries the node's (x, u, mu) are read for the free final time's terms only
-  const bool point = NJ == 0 || part != nullptr;
+  const bool point = !ST || part != nullptr;
   __shared__ double red[32];
   // sdev: Bt and Mu arrive unscaled (B^a, B^aT products) and take the device time scale here;
   // the scaled Mu is written back (the caller's record of s B^aT dlambda)
@@ -936,9 +937,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_kkt_post(const 
     }
 #pragma unroll
     for (int q = 0; q < NU; ++q) { u[q] = point ? xu[(NX + q) * P + k] : T(0); dz[NX + q] = dU[q * P + k]; }
-    if constexpr (NJ > 0) {
+    if constexpr (ST) {
       T v[NH];
-      node_jac<T, KIND>(xu, lin, P, k, pa, Jx, Ju);
+      node_jac<T, KIND, ST>(xu, lin, P, k, pa, Jx, Ju);
 #pragma unroll
       for (int i = 0; i < NH; ++i) v[i] = lin[(NJ + i) * P + k];
       Dyn<KIND>::template unpack_h<T>(v, H);
@@ -1461,7 +1462,9 @@ static bk_status alloc_opdata(Problem* pr, OpData& d, int dtype) {
   BK_TRY(dmalloc(&d.xu, es * (nx + nu) * P));
   BK_TRY(dmalloc(&d.mu, es * nx * P));
   const int nl = pr->kind == BK_ORBIT ? Dyn<BK_ORBIT>::nlj + Dyn<BK_ORBIT>::nlh : 0;
-  if (nl > 0) BK_TRY(dmalloc(&d.lin, es * nl * P));
+  // stored entries in the working precision only: the FP64 side of an FP32 problem, which applies the
+  // operator once per refinement sweep, forms them in the product
+  if (nl > 0 && dtype == pr->dtype) BK_TRY(dmalloc(&d.lin, es * nl * P));
   d.w = dtype == BK_F64 ? (void*)d.plan->w64 : d.plan->wT;
   // preconditioner data only in the working precision (an FP32 problem's FP64 side serves the
   // residual and the refinement products)
@@ -1738,7 +1741,6 @@ static bk_status linearize_kind(Problem* pr, const double* z, const double* mu, 
     }
   }
   if constexpr (Dyn<KIND>::nlj > 0) {
-    pr->lin64_stale = pr->dtype == BK_F32;
     // k_lin_nodes wrote them where it ran in the problem's precision
     if (keep == LIN_KEEP_PRECOND || pr->pdtype != pr->dtype) {
       if (pr->dtype == BK_F32)
@@ -1774,16 +1776,13 @@ static bk_status apply_typed(Problem* pr, OpData& d, int op, const T* in, T* out
   T* t1 = (T*)d.t1;
   T* t2 = (T*)d.t2;
   T* t3 = (T*)d.t3;
-  if constexpr (Dyn<KIND>::nlj > 0 && sizeof(T) == 8) {
-    if (pr->lin64_stale) {
-      BK_TRY((lin_entries<T, KIND>(pr, d, st)));
-      pr->lin64_stale = false;
-    }
-  }
+  // with stored entries (lin), or without: the FP64 side of an FP32 problem, never an FP32 one
+  constexpr bool KEPT = Dyn<KIND>::nlj > 0, ALT = KEPT && sizeof(T) == 4;
+  const T* lin = (const T*)d.lin;
   if (op == BK_OP_STATE) {
     // the product ignores t1's padding (elements L..P-1), so it is never written
-    BK_TRY(launch(k_jvp<T, KIND>, nblk(L), 256, 0, st, (const T*)d.xu, in, nullptr, P, L, t1, (T)pr->dyn_param(), nullptr, T(0),
-                  (const T*)d.lin));
+    BK_TRY(launch(lin ? k_jvp<T, KIND, KEPT> : k_jvp<T, KIND, ALT>, nblk(L), 256, 0, st, (const T*)d.xu, in, nullptr, P, L, t1, (T)pr->dyn_param(), nullptr, T(0),
+                  lin));
     const double* sd = sdev_of(pr);
     BK_TRY(plan_apply_n(d.plan, t1, t2, NX, false, sd ? 1.0 : pr->s, st));
     BK_TRY(launch(k_state_post<T, NX>, nblk(NX * P), 256, 0, st, in, t2, P, L, out, sd));
@@ -1791,17 +1790,17 @@ static bk_status apply_typed(Problem* pr, OpData& d, int op, const T* in, T* out
   }
   const bool ft = pr->free_time;
   const T pa = (T)pr->dyn_param();
-  BK_TRY(launch(k_jvp<T, KIND>, nblk(L), 256, 0, st, (const T*)d.xu, in, in + NX * P, P, L, t1, pa,
-                                          ft ? in + pr->s_idx() : nullptr, (T)(1.0 / pr->s), (const T*)d.lin));
+  BK_TRY(launch(lin ? k_jvp<T, KIND, KEPT> : k_jvp<T, KIND, ALT>, nblk(L), 256, 0, st, (const T*)d.xu, in, in + NX * P, P, L, t1, pa,
+                                          ft ? in + pr->s_idx() : nullptr, (T)(1.0 / pr->s), lin));
   // fixed final time: both products unscaled, k_kkt_post applies s from the device (so that a
   // captured GMRES step does not hold s); free final time: s (which changes within a step) by value
   const double* sd = sdev_of(pr);
   BK_TRY(plan_apply_n(d.plan, t1, t2, NX, false, sd ? 1.0 : pr->s, st));
   T* Mu = mu_out ? mu_out : t3;
   BK_TRY(plan_apply_n(d.plan, in + (NX + NU) * P, Mu, NX, true, sd ? 1.0 : pr->s, st));
-  BK_TRY(launch(k_kkt_post<T, KIND>, ft ? FT_NB : nblk(P), 256, 0, st, (const T*)d.xu, (const T*)d.mu, (const T*)d.w, (T)pr->s, in,
+  BK_TRY(launch(lin ? k_kkt_post<T, KIND, KEPT> : k_kkt_post<T, KIND, ALT>, ft ? FT_NB : nblk(P), 256, 0, st, (const T*)d.xu, (const T*)d.mu, (const T*)d.w, (T)pr->s, in,
                                                             t2, Mu, P, L, term_spec(pr), (T)pr->cost_uu(), out, pa,
-                                                            pr->s_idx(), ft ? pr->sred : nullptr, sd, bar_hbar<T>(pr, d), (const T*)d.lin));
+                                                            pr->s_idx(), ft ? pr->sred : nullptr, sd, bar_hbar<T>(pr, d), lin));
   if (ft) {
     BK_TRY(launch(k_free_finish<T>, 1, 256, 0, st, pr->sred, FT_NB, -1.0 / pr->s, out + pr->s_idx()));
   }

@@ -339,7 +339,7 @@ struct OpData {
   Plan* plan = nullptr;        // n_comp = n_x, max_batch = 1
   void* xu = nullptr;          // linearisation point X, U ((n_x + n_u) * P)
   void* mu = nullptr;          // mu = s (B^a)^T lambda (n_x * P)
-  void* lin = nullptr;         // stored entries of J_x and H per node ((nlj + nlh) * P)
+  void* lin = nullptr;         // stored entries of J_x and H per node ((nlj + nlh) * P; working precision only)
   void* w = nullptr;           // Clenshaw-Curtis weights (L), working type
   void* Dn = nullptr;          // per-node D_k = h_k J_k K_k, K_k = (I - h_k J_k)^{-1} = I + D_k and
                                // N_k = 2 h_k J_k K_k = 2 D_k; interleaved (n_x^2 per node)
@@ -385,7 +385,6 @@ struct Problem {
   int nlev = 0;                // scan levels; level nlev - 1 has at most 32 items
   int lvn[MAXLEV] = {};        // items per level
   bool linearized = false;
-  bool lin64_stale = false;    // BK_F32 problems: d64.lin is formed when an FP64 product first needs it
   OpData d64;                  // FP64 operators (always)
   OpData d32;                  // FP32 operators (BK_F32 problems)
   double* F = nullptr;         // KKT residual scratch (FP64, kkt_len)
