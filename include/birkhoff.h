@@ -75,11 +75,13 @@ uint64_t bk_launch_count(void);
  *              with N <= 1024 to the dense product: BK_F32 on the tensor cores, BK_F64 on the
  *              CUDA cores); any other N <= 1024 takes the dense product in both precisions (B^a
  *              formed once in FP64 from its definition: Chebyshev coefficients of the Lagrange
- *              basis times the closed-form integrals of T_k, Eq. intChebPoly=); any other
- *              N > 1024 computes each DCT-I's length-N DFT by Bluestein's identity as a circular
- *              convolution of length M (a power of two, M >= 2N - 1) on the four-step FFT, with
- *              the chirp exp(-i pi j^2 / N) and the convolution kernel's spectrum as plan tables
- *              (about 4-8x the work of the nearest power of two)
+ *              basis times the closed-form integrals of T_k, Eq. intChebPoly=); N > 1024 that is
+ *              16 times a product of 2, 3 and 5 takes the FFT chain with mixed radices (factors of
+ *              2N of at most 5120 in BK_F64, 10240 in BK_F32); any other N > 1024 computes each
+ *              DCT-I's length-N DFT by Bluestein's identity as a circular convolution of length M
+ *              (a power of two, M >= 2N - 1) on the four-step FFT, with the chirp
+ *              exp(-i pi j^2 / N) and the convolution kernel's spectrum as plan tables (about 4-8x
+ *              the work of the nearest power of two)
  *   n_comp     components per batch item (>= 1)
  *   max_batch  largest `batch` later passed to birkhoff_apply / birkhoff_apply_T (>= 1); the
  *              plan's scratch is sized for max_batch * n_comp vectors and serves one call at a
@@ -103,7 +105,9 @@ bk_status bk_plan_info(const bk_plan* plan, int64_t* N, int64_t* L, int64_t* pit
                        int* dtype);
 
 /* Copy the L node times t_j (FP64) and the L Clenshaw-Curtis weights w_j (FP64, tau-domain,
- * sum 2; last row of B^a per the remark after Eq. Ba=10) to HOST arrays; either may be NULL.
+ * sum 2; last row of B^a per the remark after Eq. Ba=10; for N on the FFT chain or Bluestein's
+ * convolution in closed form, each within a few units in its last place) to HOST arrays; either
+ * may be NULL.
  * Synchronous. */
 bk_status bk_plan_grid(const bk_plan* plan, double* t_host, double* w_host);
 
@@ -120,10 +124,11 @@ bk_status birkhoff_apply(const bk_plan* plan, const void* v, void* out, int batc
 /* B v (trans = 0) or B^T v (trans = 1) for `count` plans of one dtype whose N may all differ,
  * e.g. the requests of a serving batch: entry i computes out[i] = B_i v[i] for batch[i]
  * vectors of plans[i], exactly as birkhoff_apply(_T)(plans[i], v[i], out[i], batch[i]) would
- * (bitwise the same values). Plans on the single-CTA path run in one launch, four-step plans (up
- * to 2^18 in FP32, 2^17 in FP64) in another, or in one launch per pass (four) when one of them is
- * on the launch-per-pass path, each per 16 plans; dense, Bluestein and longer plans run their own
- * launches within the call.
+ * (bitwise the same values). Plans on the single-CTA path run in one launch, one-launch four-step
+ * plans in another, launch-per-pass ones (powers of two up to 2^18 in FP32, 2^17 in FP64) in one
+ * launch per pass (four), each per 16 plans; beside launch-per-pass plans, FP32 one-launch plans
+ * (N = 4096) join their launches while the scratch those lend suffices. Dense, Bluestein,
+ * mixed-radix and longer plans run their own launches within the call.
  *   plans, v, out, batch   host arrays of `count` entries (1 <= count <= 4096); v[i], out[i]
  *                          device arrays as for birkhoff_apply; v[i] == out[i] is allowed, but
  *                          different entries' vectors must not overlap

@@ -147,8 +147,8 @@ def birkhoff_apply_T(plan, v, out, batch=None, stream=None):
 
 
 def birkhoff_apply_batch(plans, vs, outs, batches=None, trans=False, stream=None):
-    """out_i = B_i v_i (or B_i^T v_i) for plans of one dtype and any mix of N, in one call (one
-    launch per pass for the plans on the single-CTA and unsplit four-step paths)."""
+    """out_i = B_i v_i (or B_i^T v_i) for plans of one dtype and any mix of N, in one call: shared
+    launches for the single-CTA and the four-step plans (include/birkhoff.h says which)."""
     n = len(plans)
     if not (len(vs) == n and len(outs) == n) or n == 0:
         raise ValueError("plans, vs and outs must have the same non-zero length")

@@ -2043,8 +2043,8 @@ static bk_status problem_set_params(Problem* pr, const double* params, int npara
 // FP64 problems keep an FP64 preconditioner unless asked for an FP32 one: bk_set_f64_precond(1)
 // for problems created afterwards, or the environment variable BK_F64_PC32=1 (read at creation).
 // The FP32 sweeps are 2-3x faster, but on the orbit solve at N = 2^20 (forcing-term inner
-// tolerances down to 1e-12) flexible GMRES needed 19 instead of 11 iterations, and the solve took
-// 56.9 instead of 50.5 ms, so FP64 stays the default.
+// tolerances down to 1e-12) flexible GMRES needs 19 instead of 11 iterations, and the solve takes
+// 30.6 instead of 26.7 ms, so FP64 stays the default.
 static std::atomic<int> g_f64_pc32{-1};
 static bool f64_precond32(int64_t N) {
   (void)N;

@@ -15,7 +15,7 @@ struct FourStep {
   int NB = 0, P = 0;
   int bsA = 0, bsB = 0;       // batch strides in shared memory (complex elements)
   size_t smemA = 0, smemB = 0;
-  int thrA = 256, thrB = 256; // threads of the pass kernels (16 complex values each)
+  int thrA = 256, thrB = 256; // threads of the pass kernels
   void* stw1 = nullptr;       // stage twiddle table of the length-N1 FFT
   void* stw2 = nullptr;       // stage twiddle table of the length-N2 FFT
   void* twN = nullptr;        // real-even: the [N1/2 + 1][N2/2 + 2] table; else omega_n^m, m < n (FP64)

@@ -21,7 +21,7 @@ constexpr int NUM = 2;   // largest control dimension
 constexpr int NEM = 4;   // largest terminal-condition count
 // Nodes per sweep segment (one lane each) for the working precision: shorter segments in FP64,
 // where the sweep is bound by dependent FP64 latency and more lanes help (measured: 8 vs 16
-// nodes, KKT preconditioner at 2^20 0.75 vs 0.84 ms), 16 in FP32 (one 32-byte staging chunk).
+// nodes, KKT preconditioner at 2^20 0.75 vs 0.84 ms), 16 in FP32 (two 32-byte runs).
 template <typename T> struct Seg { static constexpr int v = sizeof(T) == 8 ? 8 : 16; };
 inline int seg_nodes(int dtype) { return dtype == BK_F64 ? Seg<double>::v : Seg<float>::v; }
 // Scan levels of the preconditioner sweep: level 0 items are segments, level l + 1 items are
